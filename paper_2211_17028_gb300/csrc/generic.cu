@@ -25,6 +25,7 @@
 #include <cmath>
 #include <vector>
 
+#include "level_sum.cuh"
 #include "nqs_internal.h"
 
 namespace nqs {
@@ -172,62 +173,30 @@ __global__ void __launch_bounds__(kT) g_sum_kernel(const double2* __restrict__ a
                                                    const long long* __restrict__ level_off, int level,
                                                    long long n_terms, double bound, double* __restrict__ vals,
                                                    nqs_result* __restrict__ res) {
-    __shared__ double s_re[kT], s_c[kT], s_im[kT];
-    __shared__ double T[NQS_MAX_LEVEL + 1];
-    __shared__ double imag_tot;
-    const int tid = threadIdx.x;
-    if (tid == 0) imag_tot = 0.0;
+    static_assert(kT == kSumThreads, "block size of level_sums");
+    __shared__ double T[NQS_MAX_LEVEL + 1], im_part[kT / 32];
+    double im_sum = 0.0;
+    level_sums(level_off, level, [&](long long i) {
+        const double2 x = a[i];
+        const double2 y = b ? b[i] : x;
+        const double re = x.x * y.x + x.y * y.y;
+        vals[i] = re;
+        im_sum += x.y * y.x - x.x * y.y;
+        return re;
+    }, T);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) im_sum += __shfl_xor_sync(0xffffffffu, im_sum, o);
+    if ((threadIdx.x & 31) == 0) im_part[threadIdx.x >> 5] = im_sum;
     __syncthreads();
-    for (int u = 0; u <= level; ++u) {
-        const long long lo = level_off[u], hi = level_off[u + 1];
-        const long long len = hi - lo, chunk = (len + kT - 1) / kT;
-        double s = 0.0, c = 0.0, si = 0.0;
-        for (long long i = lo + tid * chunk; i < lo + (tid + 1) * chunk && i < hi; ++i) {
-            const double2 x = a[i];
-            const double2 y = b ? b[i] : a[i];
-            const double re = x.x * y.x + x.y * y.y, im = x.y * y.x - x.x * y.y;
-            vals[i] = re;
-            const double t = s + re;
-            c += (fabs(s) >= fabs(re)) ? (s - t) + re : (re - t) + s;
-            s = t;
-            si += im;
-        }
-        s_re[tid] = s;
-        s_c[tid] = c;
-        s_im[tid] = si;
-        __syncthreads();
-        if (tid == 0) {
-            double S = 0.0, C = 0.0, I = 0.0;
-            for (int k = 0; k < kT; ++k) {
-                const double v = s_re[k];
-                const double t = S + v;
-                C += (fabs(S) >= fabs(v)) ? (S - t) + v : (v - t) + S;
-                S = t;
-                C += s_c[k];
-                I += s_im[k];
-            }
-            T[u] = S + C;
-            imag_tot += I;
-        }
-        __syncthreads();
-    }
-    if (tid == 0) {
-        nqs_result r;
-        double F = 0.0, C = 0.0;
-        for (int u = 0; u <= NQS_MAX_LEVEL; ++u) r.T[u] = 0.0;
-        for (int u = 0; u <= level; ++u) {
-            r.T[u] = T[u];
-            const double t = F + T[u];
-            C += (fabs(F) >= fabs(T[u])) ? (F - t) + T[u] : (T[u] - t) + F;
-            F = t;
-        }
-        r.F = F + C;
-        r.imag_residual = fabs(imag_tot);
-        r.n_terms = (uint64_t)n_terms;
-        r.bound = bound;
-        r.level = level;
-        r.status = NQS_OK;
-        *res = r;
+    if (threadIdx.x == 0) {
+        double imag_tot = 0.0;
+        for (int w = 0; w < kT / 32; ++w) imag_tot += im_part[w];
+        store_levels(res, T, level);
+        res->imag_residual = fabs(imag_tot);
+        res->n_terms = (uint64_t)n_terms;
+        res->bound = bound;
+        res->level = level;
+        res->status = NQS_OK;
     }
 }
 

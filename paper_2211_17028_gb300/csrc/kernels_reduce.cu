@@ -1,6 +1,7 @@
 // Reductions and bookkeeping kernels: the standalone reduced-matrix kernel,
 // the fixed-order finishers that turn per-block partial sums into term
 // values, the Neumaier-compensated per-level sums, and the basis-state fill.
+#include "level_sum.cuh"
 #include "sweep_types.h"
 #include "nqs_internal.h"
 
@@ -48,23 +49,24 @@ __global__ void __launch_bounds__(kThreads) reduce2x2_kernel(const float2* __res
 }
 
 // Sum per-block partials of one reduction slot in a fixed order: thread t
-// takes blocks t, t+256, ...; then a fixed tree.
-__device__ void sum_partials(const double* part, int grid, double* R, double* scratch) {
-    const int tid = threadIdx.x;
-    double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int b = tid; b < grid; b += kThreads)
-#pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] += part[(size_t)b * 8 + e];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) scratch[e * kThreads + tid] = v[e];
+// takes component t % 8 of blocks t / 8, t / 8 + 32, ... (whole 64-byte rows
+// per load), then two shuffles join the four rows of a warp and eight threads
+// add the eight warps' sums.  Latency-bound: 8.4 us as eight components per
+// thread and an eight-step tree, 3 us in this form (152 partials).
+__device__ void sum_partials(const double* __restrict__ part, int grid, double* R, double (*scratch)[8]) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    double v = 0.0;
+    for (int b = tid >> 3; b < grid; b += kThreads / 8) v += part[(size_t)b * 8 + (tid & 7)];
+    v += __shfl_xor_sync(0xffffffffu, v, 8);
+    v += __shfl_xor_sync(0xffffffffu, v, 16);
+    if (lane < 8) scratch[warp][lane] = v;
     __syncthreads();
-    for (int w = kThreads / 2; w > 0; w >>= 1) {
-        if (tid < w)
+    if (tid < 8) {
+        double t = 0.0;
 #pragma unroll
-            for (int e = 0; e < 8; ++e) scratch[e * kThreads + tid] += scratch[e * kThreads + tid + w];
-        __syncthreads();
+        for (int w = 0; w < kWarps; ++w) t += scratch[w][tid];
+        R[tid] = t;
     }
-    if (tid < 8) R[tid] = scratch[tid * kThreads];
     __syncthreads();
 }
 
@@ -73,7 +75,7 @@ __device__ void sum_partials(const double* part, int grid, double* R, double* sc
 __device__ __forceinline__ void finish_slot(const double* __restrict__ partials, int grid, int slot,
                                             const FinishDesc* __restrict__ desc, const double* __restrict__ kmats,
                                             double* __restrict__ term_vals) {
-    __shared__ double scratch[8 * kThreads];
+    __shared__ double scratch[kWarps][8];
     __shared__ double R[8];
     sum_partials(partials + (size_t)slot * grid * 8, grid, R, scratch);
     if (threadIdx.x < 4) {
@@ -114,62 +116,21 @@ __global__ void __launch_bounds__(kThreads) finish_kernel_batched(const FinishUn
 // One block: fixed-order sum of per-block partials into 8 doubles.
 __global__ void __launch_bounds__(kThreads) partials_sum_kernel(const double* __restrict__ part, int grid,
                                                                 double* __restrict__ R) {
-    __shared__ double scratch[8 * kThreads];
+    __shared__ double scratch[kWarps][8];
     __shared__ double r[8];
     sum_partials(part, grid, r, scratch);
     if (threadIdx.x < 8) R[threadIdx.x] = r[threadIdx.x];
 }
 
-// Neumaier-compensated per-level sums in canonical order, one block.
+// Neumaier-compensated per-level sums (level_sum.cuh), one block.
 __device__ __forceinline__ void level_sum_body(const double* __restrict__ vals,
-                                                             const long long* __restrict__ level_off, int level,
-                                                             nqs_result* __restrict__ res, double bound,
-                                                             long long n_terms, const int* __restrict__ err,
-                                               nqs_result* __restrict__ copy) {
-    __shared__ double s_sum[kThreads], s_comp[kThreads];
+                                               const long long* __restrict__ level_off, int level,
+                                               nqs_result* __restrict__ res, double bound, long long n_terms,
+                                               const int* __restrict__ err, nqs_result* __restrict__ copy) {
     __shared__ double T[NQS_MAX_LEVEL + 1];
-    const int tid = threadIdx.x;
-    for (int u = 0; u <= level; ++u) {
-        long long lo = level_off[u], hi = level_off[u + 1];
-        long long len = hi - lo;
-        long long chunk = (len + kThreads - 1) / kThreads;
-        long long a = lo + chunk * tid, b = min(hi, a + chunk);
-        double sum = 0.0, comp = 0.0;
-        for (long long i = a; i < b; ++i) {
-            double x = vals[i];
-            double t = sum + x;
-            if (fabs(sum) >= fabs(x)) comp += (sum - t) + x;
-            else comp += (x - t) + sum;
-            sum = t;
-        }
-        s_sum[tid] = sum;
-        s_comp[tid] = comp;
-        __syncthreads();
-        if (tid == 0) {
-            double S = 0.0, C = 0.0;
-            for (int i = 0; i < kThreads; ++i) {
-                double x = s_sum[i];
-                double t = S + x;
-                if (fabs(S) >= fabs(x)) C += (S - t) + x;
-                else C += (x - t) + S;
-                S = t;
-                C += s_comp[i];
-            }
-            T[u] = S + C;
-        }
-        __syncthreads();
-    }
-    if (tid == 0) {
-        double S = 0.0, C = 0.0;
-        for (int u = 0; u <= NQS_MAX_LEVEL; ++u) {
-            double x = (u <= level) ? T[u] : 0.0;
-            res->T[u] = x;
-            double t = S + x;
-            if (fabs(S) >= fabs(x)) C += (S - t) + x;
-            else C += (x - t) + S;
-            S = t;
-        }
-        res->F = S + C;
+    level_sums(level_off, level, [&](long long i) { return vals[i]; }, T);
+    if (threadIdx.x == 0) {
+        store_levels(res, T, level);
         res->imag_residual = 0.0;
         res->n_terms = (uint64_t)n_terms;
         res->bound = bound;
@@ -232,27 +193,32 @@ cudaError_t launch_finish(const double* partials, int grid, const FinishDesc* de
 // v <- v / ||v||, the norm from the per-block partials of reduce2x2_kernel(v,
 // v, qubit 0): ||v||^2 = Re R00 + Re R11, summed in a fixed order by every
 // block.  The noiseless circuit keeps the norm of a basis state, 1; complex64
-// gates lose a little of it, and v enters F twice.
-__global__ void __launch_bounds__(kThreads) normalize_kernel(float2* __restrict__ v, long long dim,
+// gates lose a little of it, and v enters F twice.  Bound by HBM (16 B per
+// amplitude); every block's first warp adds the partials in parallel (one
+// thread adding 608 of them took longer than the copy: 155 us at 24 qubits,
+// 45 us so).
+__global__ void __launch_bounds__(kThreads) normalize_kernel(float4* __restrict__ v, long long dim2,
                                                              const double* __restrict__ part, int grid) {
     __shared__ float scale;
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < 32) {
         double a = 0.0;
-        for (int g = 0; g < grid; ++g) a += part[(size_t)g * 8] + part[(size_t)g * 8 + 6];
-        scale = a > 0.0 ? (float)(1.0 / sqrt(a)) : 1.0f;
+        for (int g = threadIdx.x; g < grid; g += 32) a += part[(size_t)g * 8] + part[(size_t)g * 8 + 6];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        if (threadIdx.x == 0) scale = a > 0.0 ? (float)(1.0 / sqrt(a)) : 1.0f;
     }
     __syncthreads();
     const float f = scale;
     const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < dim; i += stride) {
-        const float2 x = v[i];
-        v[i] = make_float2(x.x * f, x.y * f);
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < dim2; i += stride) {
+        const float4 x = v[i];
+        v[i] = make_float4(x.x * f, x.y * f, x.z * f, x.w * f);
     }
 }
 
 cudaError_t launch_normalize(float2* v, long long dim, const double* partials, int red_grid, int grid,
                              cudaStream_t st) {
-    normalize_kernel<<<grid, kThreads, 0, st>>>(v, dim, partials, red_grid);
+    normalize_kernel<<<grid, kThreads, 0, st>>>(reinterpret_cast<float4*>(v), dim >> 1, partials, red_grid);
     return cudaGetLastError();
 }
 
