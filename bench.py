@@ -441,7 +441,7 @@ def run_nqs(args):
     fills = nqs.nqs_get_kernel_stats(h, 2)
     multi = nqs.nqs_get_kernel_stats(h, 3)    # branch-group passes (several states)
     single = nqs.nqs_get_kernel_stats(h, 4)   # single-state passes
-    kname = "nqs_pass (generated per pass)" if nqs.nqs_get_info(h)["jit_launches"] > 0 else "sweep_kernel"
+    kname = "nqs_pass (generated per pass)" if nqs.nqs_get_info(h)["jit_launches"] > 0 else "unit_sweep_kernel"
     dom, dom_name = (multi, kname + ", 3-state branch-group passes") if multi["total_ms"] >= single["total_ms"] \
         else (single, kname + ", single-state passes")
     nqs.nqs_set_profiling(h, 0)
@@ -569,7 +569,7 @@ def kernel_source_sha(jit=False):
     """Hash of the source that defines the timed sweep kernel: the pass
     generator when pass-specialised kernels ran, else the interpreting kernel."""
     import hashlib
-    p = os.path.join(ROOT, "paper_2211_17028_gb300", "csrc", "jit.cpp" if jit else "kernels_sweep_body.cuh")
+    p = os.path.join(ROOT, "paper_2211_17028_gb300", "csrc", "jit.cpp" if jit else "kernels_units.cu")
     return hashlib.sha256(open(p, "rb").read()).hexdigest()[:16]
 
 

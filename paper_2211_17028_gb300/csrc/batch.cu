@@ -28,9 +28,8 @@ int cuda_ok(cudaError_t e) { return e == cudaSuccess ? NQS_OK : NQS_ERR_CUDA; }
 // One launch of the batched sequence.
 struct Group {
     enum Kind { SWEEP, FINISH, FILL, SUM, SINGLE, MEMSET } kind;
-    int S = 1, RB = 4;
     size_t units = 0;      // byte offset of the unit array in the device blob
-    size_t begins = 0;     // byte offset of the block-begin array
+    size_t begins = 0;     // byte offset of the block-begin array (sweeps: the unit of every block)
     int n_units = 0, total = 0;
     size_t smem = 0;
     int h = -1;            // SINGLE / MEMSET: which circuit
@@ -68,9 +67,7 @@ void free_plan(BatchPlan* p, void* stream) {
 size_t state_bytes_needed(const Handle& h, int level) {
     const int N = (int)h.factors.size();
     const int lvl = std::min(level, N);
-    int n_group = 0;
-    for (int d = 1; d < lvl; ++d) n_group += (d == 1) ? 3 : 9;
-    return ((size_t)std::max(N, 1) + 1 + n_group) * ((size_t)8 << h.plan.n);
+    return ((size_t)std::max(N, 1) + 1 + group_states(h, lvl, false)) * ((size_t)8 << h.plan.n);
 }
 
 // Build the round-grouped launch sequence of the circuits [first, last) and
@@ -96,8 +93,9 @@ int build_plan(BatchPlan& P, int first, int last, void* stream) {
     size_t rounds = 0;
     for (int k = first; k < last; ++k) rounds = std::max(rounds, P.engines[k]->launches.size());
     for (size_t r = 0; r < rounds; ++r) {
-        std::vector<PassArgs> sweep_units[4][5];     // [S][RB]
-        std::vector<int> sweep_ctas[4][5];
+        // the round's sweep passes, longest blocks first (the short ones fill the
+        // last wave)
+        std::vector<std::pair<const Engine*, const Launch*>> sweeps;
         std::vector<FinishUnit> fin;
         std::vector<int> fin_blocks;
         std::vector<FillUnit> fills;
@@ -107,18 +105,17 @@ int build_plan(BatchPlan& P, int first, int last, void* stream) {
             if (r >= E.launches.size()) continue;
             const Launch& l = E.launches[r];
             const Handle& h = *P.hs[k];
-            if (l.kind == L_PASS && l.rt) {
-                sweep_units[l.S][l.rb].push_back(l.args);
-                sweep_ctas[l.S][l.rb].push_back(l.grid);
+            if (l.kind == L_PASS && l.units()) {
+                sweeps.push_back({&E, &l});
             } else if (l.kind == L_FINISH) {
                 FinishUnit u{};
                 u.partials = E.partials;
-                u.desc = E.desc_dev + l.desc_off;
+                u.slots = E.slots_dev + l.slot_off;
                 u.kmats = E.kmats_dev;
                 u.vals = E.term_vals;
-                u.grid = l.fin_grid;
+                u.n_slots = l.n_slots;
                 fin.push_back(u);
-                fin_blocks.push_back(l.n_red);
+                fin_blocks.push_back(finish_blocks(l.n_slots));
             } else if (l.kind == L_FILL) {
                 FillUnit u{};
                 u.dst = l.dst;
@@ -144,28 +141,33 @@ int build_plan(BatchPlan& P, int first, int last, void* stream) {
                 P.seq.push_back(g);
             }
         }
-        for (int S = 1; S <= 3; ++S)
-            for (int RB = 3; RB <= 4; ++RB) {
-                auto& units = sweep_units[S][RB];
-                if (units.empty()) continue;
-                std::vector<int> begins(units.size() + 1, 0);
-                int max_words = 0, max_ev = 0;
-                for (size_t u = 0; u < units.size(); ++u) {
-                    begins[u + 1] = begins[u] + sweep_ctas[S][RB][u];
-                    max_words = std::max(max_words, units[u].prog_words);
-                    max_ev = std::max(max_ev, units[u].n_events);
+        if (!sweeps.empty()) {
+            auto tiles_per_block = [](const std::pair<const Engine*, const Launch*>& x) {
+                return x.first->units[x.second->unit_off].n_tiles / x.second->ctas;
+            };
+            std::stable_sort(sweeps.begin(), sweeps.end(), [&](const auto& x, const auto& y) {
+                return tiles_per_block(x) > tiles_per_block(y);
+            });
+            std::vector<SweepUnit> units;
+            std::vector<int> block_unit;
+            Group g;
+            g.kind = Group::SWEEP;
+            for (const auto& x : sweeps) {
+                const Launch& l = *x.second;
+                for (int k = 0; k < l.n_units; ++k) {
+                    SweepUnit u = x.first->units[l.unit_off + k];
+                    u.cta_begin = (int)block_unit.size();
+                    block_unit.insert(block_unit.end(), l.ctas, (int)units.size());
+                    units.push_back(u);
                 }
-                Group g;
-                g.kind = Group::SWEEP;
-                g.S = S;
-                g.RB = RB;
-                g.units = blob.put(units.data(), units.size() * sizeof(PassArgs));
-                g.begins = blob.put(begins.data(), begins.size() * sizeof(int));
-                g.n_units = (int)units.size();
-                g.total = begins.back();
-                g.smem = sweep_smem_bytes(S, RB, max_words, max_ev);
-                P.seq.push_back(g);
+                g.smem = std::max(g.smem, l.smem);
             }
+            g.units = blob.put(units.data(), units.size() * sizeof(SweepUnit));
+            g.begins = blob.put(block_unit.data(), block_unit.size() * sizeof(int));
+            g.n_units = (int)units.size();
+            g.total = (int)block_unit.size();
+            P.seq.push_back(g);
+        }
         if (!fin.empty()) {
             std::vector<int> begins(fin.size() + 1, 0);
             for (size_t u = 0; u < fin.size(); ++u) begins[u + 1] = begins[u] + fin_blocks[u];
@@ -223,8 +225,8 @@ int run_plan(BatchPlan& P, cudaStream_t st) {
                 rc = cuda_ok(cudaMemsetAsync(P.engines[g.h]->err_dev, 0, sizeof(int), st));
                 break;
             case Group::SWEEP:
-                rc = cuda_ok(launch_sweep_batched(g.S, g.RB, (const PassArgs*)(base + g.units),
-                                                  (const int*)(base + g.begins), g.n_units, g.total, g.smem, st));
+                rc = cuda_ok(launch_units((const SweepUnit*)(base + g.units), (const int*)(base + g.begins), 0, g.total,
+                                          g.smem, st));
                 break;
             case Group::FINISH:
                 rc = cuda_ok(launch_finish_batched((const FinishUnit*)(base + g.units), (const int*)(base + g.begins),

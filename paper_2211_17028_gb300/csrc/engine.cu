@@ -29,6 +29,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <functional>
 #include <map>
 #include <vector>
 
@@ -97,7 +98,7 @@ static int jit_staging_buffers() {
 
 
 
-// Program of one register-resident launch, appended to `prog` (16-byte
+// Program of one pass for the generated kernels, appended to `prog` (16-byte
 // words): the phases, one 16-byte record per operation, then the matrices.
 // The operations (execution order) are grouped into phases: a phase gathers
 // consecutive operations whose dense qubits fit in the RB register qubits;
@@ -286,8 +287,8 @@ Run make_run(const Plan& plan, const std::vector<PassSpec>& segs, RunType rt, bo
                         rp.ev_site.push_back(o.site);
                     }
                     if (spawn && fac[o.site].m > 0) {
-                        fl |= FL_SPAWN | (fac[o.site].m << 16);
-                        rp.spawn_site = o.site;
+                        fl |= FL_SPAWN | (fac[o.site].m << 16) | ((int)rp.spawn_sites.size() << 24);
+                        rp.spawn_sites.push_back(o.site);
                     }
                     first_site_done = 1;
                 }
@@ -313,7 +314,79 @@ Run make_run(const Plan& plan, const std::vector<PassSpec>& segs, RunType rt, bo
 }
 
 // ------------------------------------------------------------------ schedule
+
+// Branch-group states of one depth held at a time.  Groups of one depth are
+// swept together, all their states in one launch per pass (a 20-qubit
+// state has 256 tiles: three states alone fill the chip 1.3 times, and a
+// 13-qubit one has two tiles).  256 MiB of states is 8192 tiles, 27 times the
+// resident blocks: more groups at once gain nothing.
+constexpr size_t kGroupBytes = (size_t)256 << 20;
+// the passes of a sweep that spawns may hold several sites (fewer passes) when
+// the children of a whole pass fit in this much
+constexpr size_t kSpawnBytes = (size_t)2 << 30;
+// per-block partial sums held before a finisher launch is put in
+constexpr size_t kPartialDoubles = (size_t)4 << 20;
+
+// Sizes of the branch-group buffers: states per depth (1 .. level - 1).
+struct GroupPlan {
+    bool grouped = false;              // spawning sweeps use passes of several sites
+    int sites = 1;                     // most spawning sites of such a pass
+    std::vector<size_t> cap;           // states of depth d
+    size_t chunk = 1;                  // groups of one depth that may spawn together
+    size_t total() const {
+        size_t t = 0;
+        for (size_t c : cap) t += c;
+        return t;
+    }
+};
+
+static GroupPlan group_plan(const Plan& plan, const std::vector<Factors>& fac, int level, bool generated,
+                            bool small) {
+    GroupPlan g;
+    g.cap.assign(std::max(1, level), 0);
+    if (level < 2) return g;
+    const size_t sb = sizeof(float2) << plan.n;
+    const size_t N = fac.size();
+    for (const PassSpec& ps : plan.free_passes) {
+        int c = 0;
+        for (int i = ps.op_begin; i < ps.op_end; ++i)
+            c += plan.ops[i].type == OP_SITE && fac[plan.ops[i].site].m > 0;
+        g.sites = std::max(g.sites, c);
+    }
+    const size_t pass_states = 3 * (size_t)g.sites + 9 * (size_t)g.sites * (level - 2);
+    // generated kernels spawn at one site per pass and sweep one group per launch
+    g.grouped = !generated && !small && pass_states * sb <= kSpawnBytes;
+    if (!g.grouped) g.sites = 1;
+    const size_t room = (generated || small) ? 0 : kGroupBytes / sb;
+    // C(N, d) 3^d states of depth d exist in all
+    double all = 3.0 * N;
+    for (int d = 1; d < level; ++d) {
+        const size_t least = (d == 1 ? 3 : 9) * (size_t)g.sites;
+        const size_t most = (size_t)std::min(all, 1e9);
+        g.cap[d] = std::max(least, std::min(room, most) / 3 * 3);
+        all *= 3.0 * (double)(N > (size_t)d ? N - d : 0) / (d + 1);
+    }
+    g.chunk = std::max<size_t>(1, room / (9 * (size_t)g.sites));
+    return g;
+}
+
+size_t group_states(const Handle& h, int level, bool generated) {
+    return group_plan(h.plan, h.factors, std::min(level, (int)h.factors.size()), generated, false).total();
+}
+
 namespace {
+
+enum PassKind { P_TILE, P_UNIT, P_GEN };
+
+// S sibling states spawned at site s_last (state s carries the s-th kept
+// factor there); `prefix` holds the earlier insertions.  They sweep from
+// operation `start` of pass `pass` on.
+struct Group {
+    std::vector<std::pair<int, int>> prefix;
+    int s_last = -1, S = 1;
+    float2* buf = nullptr;             // S consecutive states
+    int pass = 0, start = 0;
+};
 
 struct Builder {
     Handle& h;
@@ -323,21 +396,25 @@ struct Builder {
     TermIndex ti;
     Tables tab;
     std::vector<DevOp> dops;
-    std::vector<uint4> prog;          // programs of the register-resident launches
+    std::vector<uint4> prog;          // programs of the unit and generated launches
     bool too_big = false;             // a launch would not fit in shared memory
-    bool rt = false;                  // register-resident kernel (tile of exactly 12 qubits)
-    bool use_jit = false;             // passes will get pass-specialised kernels
-    std::vector<FinishDesc> descs;
+    PassKind kind = P_TILE;
+    std::vector<FinishSlot> slots;
     std::vector<Launch> L;
-    size_t partial_doubles = 0;
+    std::vector<SweepUnit> units;     // pointers into prog / partials / tables patched after layout
+    std::vector<size_t> unit_prog, unit_part;
+    std::vector<char> unit_bd;
+    std::map<std::pair<int, int>, UnitProgram> programs;   // by (first device op, count)
+    size_t partial_top = 0, partial_doubles = 0;
+    size_t finished = 0;              // slots already given to a finisher launch
     long long dim;
     // device buffers (resolved after allocation)
     float2* main_buf = nullptr;
     float2* work_buf = nullptr;                     // spaced checkpoints: block recomputation
     std::vector<float2*> phi;                       // checkpoint table (spaced: ring per site, then boundary per site)
     std::vector<float2*> bd;                        // spaced checkpoints: phi at the last site of each block
-    std::vector<std::vector<float2*>> group_bufs;   // per depth (1..level-1)
-    float2** ckpt_dev = nullptr;
+    GroupPlan gp;
+    std::vector<float2*> group_buf;                 // per depth (1..level-1)
     Run run_ideal, run_bwd, run_mat;   // run_mat: per-block phi recomputation (spaced checkpoints)
     std::vector<Run> run_fwd;    // per depth
 
@@ -365,23 +442,9 @@ struct Builder {
         return *std::min_element(rp.lin.begin(), rp.lin.end()) > last_site_pos;
     }
 
-    int grid_for(int S, int RB, long long tiles, int prog_words, int n_events) {
-        int per_sm;
-        if (rt) {
-            per_sm = sweep_blocks_per_sm(S, RB, sweep_smem_bytes(S, RB, prog_words, n_events));
-        } else {
-            size_t smem = (size_t)S * (1 << plan.k) * sizeof(float2);
-            per_sm = tile_pass_blocks_per_sm(S, smem);
-        }
-        long long g = (long long)per_sm * E.sm_count;
-        return (int)std::max<long long>(1, std::min<long long>(g, tiles));
-    }
-
-    PassArgs pass_args(const RunPass& rp, int start, int S) {
+    PassArgs pass_args(const RunPass& rp, int start) {
         PassArgs a{};
-        a.ops = nullptr;
         a.n_ops = rp.n_ops - start;
-        a.mats = nullptr;
         a.n = plan.n;
         a.k = rp.k;
         a.c = rp.c;
@@ -389,166 +452,324 @@ struct Builder {
         for (int j = 0; j < kTileSlots; ++j) a.local[j] = rp.local[j];
         for (int j = 0; j < kMaxQ; ++j) a.nonlocal[j] = rp.nonlocal[j];
         a.n_tiles = 1ll << (plan.n - rp.k);
-        a.ckpt = ckpt_dev;
         return a;
     }
 
-    void add_pass(const RunPass& rp, int start, int S, const float2* const* in, float2* const* out,
-                  float2* const* spawn, int n_spawn) {
-        if (rp.n_ops - start <= 0 && in[0] == out[0]) return;
-        Launch l;
-        l.kind = L_PASS;
-        l.S = S;
-        l.args = pass_args(rp, start, S);
-        l.op_index = rp.op_off + start;
-        l.rt = rt;
-        if (rt) {
-            // pass-specialised multi-state passes hold 16 amplitudes per state and
-            // thread (more work per instruction stream, registers for early phi loads)
-            l.rb = plan.k == kWideTileQ ? 4
-                   : (S > 1 && h.opt_rb_multi) ? h.opt_rb_multi : (S > 1 && use_jit) ? 4 : sweep_reg_bits(S);
-            ProgInfo pi = build_program(dops, rp.op_off + start, rp.n_ops - start, l.rb, tab, prog, plan.k);
-            l.prog_index = pi.words_begin;
-            l.args.prog_words = pi.n_words;
-            l.args.ops_word = pi.ops_word;
-            l.args.mats_word = pi.mats_word;
-            l.args.n_phases = pi.n_phases;
-            // static shared memory of the kernel stays below 4 KiB (13-qubit tiles:
-            // staging and two re-layout tiles of 64 KiB and the reduction slots)
-            if (plan.k == kWideTileQ) {
-                if ((size_t)3 * (8 << kWideTileQ) + (size_t)l.args.n_events * S * 16 * 64 + 4096 > E.smem_optin)
-                    too_big = true;
-            } else if (sweep_smem_bytes(S, l.rb, pi.n_words, l.args.n_events) + 4096 > E.smem_optin) {
-                too_big = true;
-            }
-        }
-        for (int s = 0; s < S; ++s) {
-            l.args.in[s] = in[s];
-            l.args.out[s] = out[s];
-        }
-        for (int i = 0; i < n_spawn; ++i) l.args.spawn[i] = spawn[i];
-        l.seq = rt && use_jit && S > 1 && (jit_seq_enabled() || plan.k == kWideTileQ);
-        // state-sequential generated passes: two 256-thread blocks per SM (13-qubit
-        // tiles: one 512-thread block)
-        const long long per_sm = plan.k == kWideTileQ ? 1 : jit_blocks_per_sm();
-        l.grid = (l.seq || (rt && use_jit && S == 1))
-                     ? (int)std::max<long long>(1, std::min<long long>(per_sm * E.sm_count, l.args.n_tiles))
-                     : grid_for(S, l.rb, l.args.n_tiles, l.args.prog_words, l.args.n_events);
-        l.smem = (size_t)S * (1 << plan.k) * sizeof(float2);
-        partial_doubles = std::max(partial_doubles, (size_t)std::max(1, l.args.n_events) * S * l.grid * 8);
-        // algorithmic bytes: state load + store, phi reads, checkpoint and spawn writes
-        double b = 16.0 * dim * S;
+    // finisher launch for the slots collected since the last one
+    void flush_finish() {
+        if (finished == slots.size()) return;
+        Launch f;
+        f.kind = L_FINISH;
+        f.slot_off = finished;
+        f.n_slots = (int)(slots.size() - finished);
+        finished = slots.size();
+        partial_top = 0;
+        L.push_back(f);
+    }
+    // room for a launch's partial sums; earlier ones are finished first when full
+    size_t take_partials(size_t need) {
+        if (partial_top > 0 && partial_top + need > kPartialDoubles) flush_finish();
+        const size_t at = partial_top;
+        partial_top += need;
+        partial_doubles = std::max(partial_doubles, partial_top);
+        return at;
+    }
+
+    // Algorithmic bytes and operation counts of one group's part of a launch:
+    // state load and store, phi reads, checkpoint and spawn writes.
+    void count(Launch& l, const RunPass& rp, int start, int S, bool first) {
         int n_red = 0, n_save = 0, n_sp = 0;
         for (int o = start; o < rp.n_ops; ++o) {
             const DevOp& d = dops[rp.op_off + o];
-            if (d.type >= OP_G1 && d.type <= OP_SITE) ++l.op_counts[d.type - OP_G1];
+            if (first && d.type >= OP_G1 && d.type <= OP_SITE) ++l.op_counts[d.type - OP_G1];
             if (d.type != OP_SITE) continue;
             if (d.flags & FL_REDUCE) ++n_red;
             if (d.flags & FL_SAVE) ++n_save;
             if (d.flags & FL_SPAWN) n_sp += (d.flags >> 16) & 0xff;
         }
-        b += 8.0 * dim * (n_red + n_save + (double)n_sp * S);
-        l.bytes = b;
-        l.op_counts[5] = n_red;
-        l.op_counts[6] = n_sp * S;
-        l.op_counts[7] = n_save;
-        L.push_back(l);
+        l.bytes += 16.0 * dim * S + 8.0 * dim * (n_red + n_save + (double)n_sp * S);
+        if (first) l.op_counts[5] = n_red;
+        l.op_counts[6] += n_sp * S;
+        l.op_counts[7] += n_save;
     }
 
-    // finisher for the last pass launch: slot (event e, state s) -> term ranks
+    // slots of the reductions a group makes from operation `start` on: event e
+    // of state s has its sums at part + (e * stride + s * one) doubles
     template <typename RankFn>
-    void add_finish(const RunPass& rp, int start, int S, RankFn rank_of) {
-        const Launch& pl = L.back();
-        int n_ev = (int)rp.ev_site.size();
-        if (n_ev == 0) return;
-        // events executed in this launch
-        std::vector<char> executed(n_ev, 0);
+    void add_slots(const RunPass& rp, int start, int s, size_t part, size_t stride, int grid, RankFn rank_of) {
         for (int o = start; o < rp.n_ops; ++o) {
             const DevOp& d = dops[rp.op_off + o];
-            if (d.type == OP_SITE && (d.flags & FL_REDUCE)) executed[(d.flags >> 8) & 0xff] = 1;
+            if (d.type != OP_SITE || !(d.flags & FL_REDUCE)) continue;
+            const int e = (d.flags >> 8) & 0xff;
+            FinishSlot f{};
+            f.part = part + e * stride;
+            f.grid = grid;
+            bool any = false;
+            for (int i = 0; i < 4; ++i) {
+                f.d[i] = FinishDesc{-1, 0, 0};
+                rank_of(rp.ev_site[e], s, i, f.d[i]);
+                any = any || f.d[i].rank >= 0;
+            }
+            if (any) slots.push_back(f);
         }
-        Launch f;
-        f.kind = L_FINISH;
-        f.n_red = n_ev * S;
-        f.fin_grid = pl.grid;
-        f.desc_off = descs.size();
-        for (int e = 0; e < n_ev; ++e)
+    }
+
+    // ---- launches --------------------------------------------------------
+    // One pass over several groups: open_launch, then add_group for each, then
+    // close_launch.  Unit launches collect every state; the tile and generated
+    // kernels sweep one group per launch.
+    Launch cur;
+    size_t first_unit = 0;
+
+    void open_launch() {
+        cur = Launch();
+        cur.kind = L_PASS;
+        first_unit = units.size();
+    }
+
+    struct SlotReq {
+        size_t unit;
+        const RunPass* rp;
+        int start, s;
+        std::function<void(int, int, int, FinishDesc&)> rank;
+    };
+    std::vector<SlotReq> reqs;
+
+    // rank(site, state, factor index 0..3, desc) names the terms of a reduction
+    void add_group(const RunPass& rp, int start, int S, const float2* in, float2* out, float2* spawn, bool bd_table,
+                   const std::function<void(int, int, int, FinishDesc&)>& rank) {
+        if (rp.n_ops - start <= 0 && in == out) return;
+        const int n_sp = [&] {
+            int c = 0;
+            for (int o = start; o < rp.n_ops; ++o) c += (dops[rp.op_off + o].flags & FL_SPAWN) != 0 &&
+                                                        dops[rp.op_off + o].type == OP_SITE;
+            return c;
+        }();
+        if (kind == P_UNIT) {
+            const std::pair<int, int> key(rp.op_off + start, rp.n_ops - start);
+            auto it = programs.find(key);
+            if (it == programs.end())
+                it = programs.emplace(key, assemble_unit(dops, key.first, key.second, rp.local, plan.n, tab.mats, prog))
+                         .first;
+            const UnitProgram& pi = it->second;
+            cur.max_words = std::max(cur.max_words, pi.words);
+            cur.max_events = std::max(cur.max_events, pi.n_events);
+            cur.n_phases = std::max(cur.n_phases, pi.n_phases);
+            const int sp_first = rp.spawn_sites.empty() ? 0 : (int)rp.spawn_sites.size() - n_sp;
+            for (int s = 0; s < S; ++s) {
+                SweepUnit u{};
+                u.in = in + (size_t)s * dim;
+                u.out = out + (size_t)s * dim;
+                // slot k of the pass (the executed ones are the last n_sp)
+                u.spawn = spawn ? spawn + (size_t)s * 3 * n_sp * dim - (ptrdiff_t)3 * sp_first * dim : nullptr;
+                u.n_tiles = (int)(1ll << (plan.n - rp.k));
+                u.n = plan.n;
+                units.push_back(u);
+                unit_prog.push_back((size_t)pi.word);
+                unit_part.push_back((size_t)pi.n_events);   // events until the launch is closed
+                unit_bd.push_back(bd_table);
+                if (rank) reqs.push_back({units.size() - 1, &rp, start, s, rank});
+            }
+            cur.S = std::max(cur.S, S);
+            count(cur, rp, start, S, units.size() - first_unit == (size_t)S);
+            return;
+        }
+        Launch l;
+        l.kind = L_PASS;
+        l.S = S;
+        l.args = pass_args(rp, start);
+        l.op_index = rp.op_off + start;
+        l.bd_table = bd_table;
+        if (kind == P_GEN) {
+            l.gen = true;
+            l.rb = plan.k == kWideTileQ ? 4 : (S > 1 && h.opt_rb_multi) ? h.opt_rb_multi : 4;
+            ProgInfo pi = build_program(dops, rp.op_off + start, rp.n_ops - start, l.rb, tab, prog, plan.k);
+            l.prog_index = pi.words_begin;
+            l.args.prog_words = pi.n_words;
+            l.args.ops_word = pi.ops_word;
+            l.args.mats_word = pi.mats_word;
+            l.args.n_phases = l.n_phases = pi.n_phases;
+            l.seq = S > 1 && (jit_seq_enabled() || plan.k == kWideTileQ);
+            // state-sequential generated passes: two 256-thread blocks per SM (13-qubit
+            // tiles: one 512-thread block); all states in registers: one block
+            const long long per_sm = (plan.k == kWideTileQ || (S > 1 && !l.seq)) ? 1 : jit_blocks_per_sm();
+            l.grid = (int)std::max<long long>(1, std::min<long long>(per_sm * E.sm_count, l.args.n_tiles));
+            // static shared memory of the kernel stays below 4 KiB
+            const size_t tile = (size_t)8 << plan.k;
+            const size_t need = (plan.k == kWideTileQ || l.seq || S == 1 ? 3 * tile : 2 * S * tile) +
+                                (size_t)l.args.n_events * S * 16 * 64 + 4096;
+            if (need > E.smem_optin) too_big = true;
+        } else {
+            l.smem = (size_t)S * (1 << plan.k) * sizeof(float2);
+            const long long per_sm = tile_pass_blocks_per_sm(S, l.smem);
+            l.grid = (int)std::max<long long>(1, std::min<long long>(per_sm * E.sm_count, l.args.n_tiles));
+        }
+        for (int s = 0; s < S; ++s) {
+            l.args.in[s] = in + (size_t)s * dim;
+            l.args.out[s] = out + (size_t)s * dim;
+            if (spawn)
+                for (int i = 0; i < 3; ++i) l.args.spawn[3 * s + i] = spawn + (size_t)(3 * s + i) * dim;
+        }
+        l.part_off = take_partials((size_t)l.args.n_events * S * l.grid * 8);
+        count(l, rp, start, S, true);
+        L.push_back(l);
+        if (rank)
             for (int s = 0; s < S; ++s)
-                for (int i = 0; i < 4; ++i) {
-                    FinishDesc d{-1, 0, 0};
-                    if (executed[e]) rank_of(rp.ev_site[e], s, i, d);
-                    descs.push_back(d);
-                }
-        L.push_back(f);
+                add_slots(rp, start, s, l.part_off + (size_t)s * l.grid * 8, (size_t)S * l.grid * 8, l.grid, rank);
+    }
+
+    void close_launch() {
+        if (kind != P_UNIT || units.size() == first_unit) return;
+        cur.unit_off = (int)first_unit;
+        cur.n_units = (int)(units.size() - first_unit);
+        cur.smem = unit_smem_bytes(cur.max_words, cur.max_events);
+        if (cur.smem + 4096 > E.smem_optin) {   // static shared memory stays below 4 KiB
+            too_big = true;
+            return;
+        }
+        const int per_sm = unit_blocks_per_sm(cur.smem);
+        cur.ctas = unit_ctas(cur.n_units, units[first_unit].n_tiles, per_sm * E.sm_count);
+        cur.grid = cur.ctas * cur.n_units;
+        size_t need = 0;
+        for (size_t u = first_unit; u < units.size(); ++u) need += unit_part[u] * cur.ctas * 8;
+        size_t at = take_partials(need);
+        cur.part_off = at;
+        for (size_t u = first_unit; u < units.size(); ++u) {
+            const size_t mine = unit_part[u] * cur.ctas * 8;
+            unit_part[u] = at;
+            units[u].ctas = cur.ctas;
+            units[u].cta_begin = (int)(u - first_unit) * cur.ctas;
+            at += mine;
+        }
+        L.push_back(cur);
+        for (const SlotReq& r : reqs)
+            add_slots(*r.rp, r.start, r.s, unit_part[r.unit], (size_t)cur.ctas * 8, cur.ctas, r.rank);
+        reqs.clear();
+    }
+
+    // a pass over one state alone
+    void add_single(const RunPass& rp, const float2* in, float2* out, float2* spawn, bool bd_table,
+                    const std::function<void(int, int, int, FinishDesc&)>& rank) {
+        open_launch();
+        add_group(rp, 0, 1, in, out, spawn, bd_table, rank);
+        close_launch();
     }
 
     int kmat_off(int site, int factor) { return site * 32 + factor * 8; }
 
-    // Group of S sibling states spawned at site `s_last` (state s carries the
-    // s-th kept factor there); `prefix` holds the earlier insertions.  The
-    // group sweeps from the operation after the site to the end of the
-    // circuit, reducing against phi_t at every later site t; when the level
-    // allows, it spawns children at each site into the next depth's buffers
-    // (3 per state) and recurses depth first.
-    void dfs_group(int depth, const std::vector<std::pair<int, int>>& prefix, int s_last, int S,
-                   const std::vector<float2*>& bufs) {
-        const Run& run = run_fwd[depth];
-        int pos = plan.site_pos[s_last];
-        int pi = -1, start = 0;
-        for (size_t p = 0; p < run.passes.size() && pi < 0; ++p) {
+    // terms of a reduction at site t of state s of a group
+    std::function<void(int, int, int, FinishDesc&)> group_rank(const Group& g, int depth) {
+        const std::vector<std::pair<int, int>> prefix = g.prefix;
+        const int s_last = g.s_last;
+        return [this, prefix, s_last, depth](int t, int s, int i, FinishDesc& d) {
+            const Factors& ft = h.factors[t];
+            if (i == 0 || i > ft.m || depth + 1 > level) return;
+            int sites[NQS_MAX_LEVEL + 1], fp[NQS_MAX_LEVEL + 1], k = 0;
+            for (const auto& pr : prefix) {
+                sites[k] = pr.first;
+                fp[k++] = pr.second;
+            }
+            sites[k] = s_last;
+            fp[k++] = s;
+            sites[k] = t;
+            fp[k++] = i - 1;
+            d.rank = (long long)ti.rank(k, sites, fp);
+            d.kmat = kmat_off(t, ft.keep[i - 1]);
+        };
+    }
+
+    // first operation of a sweep after linear position `pos`
+    bool locate(const Run& run, int pos, Group& g) const {
+        for (size_t p = 0; p < run.passes.size(); ++p) {
             const RunPass& rp = run.passes[p];
             for (int o = 0; o < rp.n_ops; ++o)
                 if (rp.lin[o] > pos) {
-                    pi = (int)p;
-                    start = o;
-                    break;
+                    g.pass = (int)p;
+                    g.start = o;
+                    return true;
                 }
         }
-        if (pi < 0) {
-            // nothing after the site: the branch states are final, nothing to reduce
-            return;
+        return false;
+    }
+
+    // Children of a group's states at the sites a pass spawns at, laid out from
+    // `base` on as [state][site][factor].
+    void make_children(const RunPass& rp, int start, const Group* parent, int S, float2* base, int depth,
+                       std::vector<Group>& out, const std::function<bool(int)>& owns) {
+        std::vector<int> at;
+        for (int o = start; o < rp.n_ops; ++o) {
+            const DevOp& d = dops[rp.op_off + o];
+            if (d.type == OP_SITE && (d.flags & FL_SPAWN)) at.push_back(d.site);
         }
-        const bool can_spawn = depth + 1 < (int)group_bufs.size();
-        for (size_t p = pi; p < run.passes.size(); ++p) {
-            const RunPass& rp = run.passes[p];
-            if (after_last(rp)) break;
-            int st = (p == (size_t)pi) ? start : 0;
-            bool spawns = can_spawn && rp.spawn_site >= 0 && rp.lin.size() > 0;
-            // a spawn before `st` (partial first pass) does not execute
-            if (spawns) {
-                int sp_pos = plan.site_pos[rp.spawn_site];
-                if (sp_pos <= pos) spawns = false;
-            }
-            std::vector<float2*> child;
-            if (spawns)
-                for (int i = 0; i < S * 3; ++i) child.push_back(group_bufs[depth + 1][i]);
-            add_pass(rp, st, S, (const float2* const*)bufs.data(), bufs.data(),
-                     child.empty() ? nullptr : child.data(), (int)child.size());
-            add_finish(rp, st, S, [&](int t, int s, int i, FinishDesc& d) {
-                const Factors& ft = h.factors[t];
-                if (i == 0 || i > ft.m || depth + 1 > level) return;
-                std::vector<std::pair<int, int>> terms = prefix;
-                terms.push_back({s_last, s});
-                terms.push_back({t, i - 1});
-                std::sort(terms.begin(), terms.end());
-                int sites[NQS_MAX_LEVEL + 1], fp[NQS_MAX_LEVEL + 1];
-                for (size_t j = 0; j < terms.size(); ++j) {
-                    sites[j] = terms[j].first;
-                    fp[j] = terms[j].second;
+        for (int s = 0; s < S; ++s)
+            for (size_t j = 0; j < at.size(); ++j) {
+                Group c;
+                if (parent) {
+                    c.prefix = parent->prefix;
+                    c.prefix.push_back({parent->s_last, s});
                 }
-                d.rank = (long long)ti.rank((int)terms.size(), sites, fp);
-                d.kmat = kmat_off(t, ft.keep[i - 1]);
-            });
-            if (spawns) {
-                int t = rp.spawn_site;
-                for (int s = 0; s < S; ++s) {
-                    std::vector<std::pair<int, int>> pre = prefix;
-                    pre.push_back({s_last, s});
-                    std::vector<float2*> cb(group_bufs[depth + 1].begin() + 3 * s,
-                                            group_bufs[depth + 1].begin() + 3 * s + 3);
-                    dfs_group(depth + 1, pre, t, h.factors[t].m, cb);
-                }
+                c.s_last = at[j];
+                c.S = h.factors[at[j]].m;
+                c.buf = base + (size_t)(s * at.size() + j) * 3 * dim;
+                if (owns && !owns(at[j])) continue;
+                if (locate(run_fwd[depth], plan.site_pos[at[j]], c)) out.push_back(c);
             }
+    }
+
+    int spawn_count(const RunPass& rp, int start) const {
+        int c = 0;
+        for (int o = start; o < rp.n_ops; ++o) {
+            const DevOp& d = dops[rp.op_off + o];
+            c += d.type == OP_SITE && (d.flags & FL_SPAWN) != 0;
+        }
+        return c;
+    }
+
+    // Groups of one depth swept together to the end of the circuit, every
+    // pass one launch over all their states, reducing against phi_t at every
+    // later site t; when the level allows, each pass spawns children into the
+    // next depth's buffers, which are swept (recursively) whenever those are full.
+    void sweep_groups(int depth, const std::vector<Group>& groups) {
+        const bool spawns = depth + 1 < level;
+        const size_t chunk = spawns ? gp.chunk : groups.size();
+        const Run& run = run_fwd[depth];
+        for (size_t g0 = 0; g0 < groups.size(); g0 += chunk) {
+            const size_t g1 = std::min(groups.size(), g0 + chunk);
+            std::vector<Group> children;
+            size_t used = 0;   // child states in use
+            int p0 = (int)run.passes.size();
+            for (size_t g = g0; g < g1; ++g) p0 = std::min(p0, groups[g].pass);
+            for (size_t p = p0; p < run.passes.size(); ++p) {
+                const RunPass& rp = run.passes[p];
+                if (after_last(rp)) break;
+                auto start_of = [&](const Group& g) { return (int)p == g.pass ? g.start : (int)p < g.pass ? -1 : 0; };
+                if (spawns) {
+                    size_t need = 0;
+                    for (size_t g = g0; g < g1; ++g)
+                        if (start_of(groups[g]) >= 0)
+                            need += (size_t)groups[g].S * 3 * spawn_count(rp, start_of(groups[g]));
+                    if (used + need > gp.cap[depth + 1] && !children.empty()) {
+                        sweep_groups(depth + 1, children);
+                        children.clear();
+                        used = 0;
+                    }
+                }
+                open_launch();
+                for (size_t g = g0; g < g1; ++g) {
+                    const Group& gr = groups[g];
+                    const int st = start_of(gr);
+                    if (st < 0) continue;
+                    const int n_sp = spawns ? spawn_count(rp, st) : 0;
+                    float2* child = n_sp ? group_buf[depth + 1] + used * dim : nullptr;
+                    add_group(rp, st, gr.S, gr.buf, gr.buf, child, false, group_rank(gr, depth));
+                    if (n_sp) {
+                        make_children(rp, st, &gr, gr.S, child, depth + 1, children, nullptr);
+                        used += (size_t)gr.S * 3 * n_sp;
+                    }
+                }
+                close_launch();
+            }
+            if (!children.empty()) sweep_groups(depth + 1, children);
         }
     }
 
@@ -572,28 +793,20 @@ struct Builder {
         return b;
     }
 
-    // The group of states spawned at site s sweeps through block c, reducing
-    // against the block's recomputed phi (level 2).
-    void group_block(int s, int c, int k, const std::vector<int>& blk) {
+    // The groups spawned in block b sweep through block c, reducing against
+    // the block's recomputed phi (level 2).
+    void groups_block(const std::vector<Group>& groups, int c, const std::vector<int>& blk) {
         const Run& run = run_fwd[1];
-        const int pos = plan.site_pos[s];
-        const int S = h.factors[s].m;
-        if (S == 0) return;
-        float2* bufs[3] = {group_bufs[1][3 * (s % k)], group_bufs[1][3 * (s % k) + 1], group_bufs[1][3 * (s % k) + 2]};
         for (size_t p = 0; p < run.passes.size(); ++p) {
             if (blk[p] != c) continue;
             const RunPass& rp = run.passes[p];
-            int st = 0;
-            while (st < rp.n_ops && rp.lin[st] <= pos) ++st;
-            if (st >= rp.n_ops) continue;
-            add_pass(rp, st, S, (const float2* const*)bufs, bufs, nullptr, 0);
-            add_finish(rp, st, S, [&](int t, int si, int i, FinishDesc& d) {
-                const Factors& ft = h.factors[t];
-                if (i == 0 || i > ft.m) return;
-                int sites[2] = {s, t}, fp[2] = {si, i - 1};
-                d.rank = (long long)ti.rank(2, sites, fp);
-                d.kmat = kmat_off(t, ft.keep[i - 1]);
-            });
+            open_launch();
+            for (const Group& g : groups) {
+                int st = 0;
+                while (st < rp.n_ops && rp.lin[st] <= plan.site_pos[g.s_last]) ++st;
+                if (st < rp.n_ops) add_group(rp, st, g.S, g.buf, g.buf, nullptr, false, group_rank(g, 1));
+            }
+            close_launch();
         }
     }
 
@@ -616,9 +829,7 @@ struct Builder {
             bool first_in = true;
             for (size_t p = 0; p < run_mat.passes.size(); ++p) {
                 if (bm[p] != c || before_first(run_mat.passes[p])) continue;
-                const float2* in[1] = {first_in ? bd[c] : work_buf};
-                float2* out[1] = {work_buf};
-                add_pass(run_mat.passes[p], 0, 1, in, out, nullptr, 0);
+                add_single(run_mat.passes[p], first_in ? bd[c] : work_buf, work_buf, nullptr, false, nullptr);
                 first_in = false;
             }
             ring_block = c;
@@ -626,25 +837,27 @@ struct Builder {
         bool first = true;
         for (int b = 0; b < nb; ++b) {
             materialize(b);
+            std::vector<Group> mine;
             for (size_t p = 0; p < fwd0.passes.size(); ++p) {
                 if (b0[p] != b) continue;
                 const RunPass& rp = fwd0.passes[p];
-                const float2* in[1] = {(first && ext) ? ext : main_buf};
-                float2* out[1] = {main_buf};
+                float2* sp = nullptr;
+                if (groups && !rp.spawn_sites.empty()) {   // passes of one site each
+                    const int s = rp.spawn_sites[0];
+                    sp = group_buf[1] + (size_t)3 * (s % k) * dim;
+                    Group g;
+                    g.s_last = s;
+                    g.S = h.factors[s].m;
+                    g.buf = sp;
+                    if (owns_group(s)) mine.push_back(g);
+                }
+                add_single(rp, (first && ext) ? ext : main_buf, main_buf, sp, false, main_rank);
                 first = false;
-                float2* sp[3];
-                int n_sp = 0;
-                if (groups && rp.spawn_site >= 0)
-                    for (int i = 0; i < 3; ++i) sp[n_sp++] = group_bufs[1][3 * (rp.spawn_site % k) + i];
-                add_pass(rp, 0, 1, in, out, n_sp ? sp : nullptr, n_sp);
-                add_finish(rp, 0, 1, main_rank);
             }
             if (!groups) continue;
-            const int s_lo = b * k, s_hi = std::min(N, (b + 1) * k);
             for (int c = b; c < nb; ++c) {
                 materialize(c);
-                for (int s = s_lo; s < s_hi; ++s)
-                    if (owns_group(s)) group_block(s, c, k, b1);
+                groups_block(mine, c, b1);
             }
         }
     }
@@ -671,6 +884,7 @@ void engine_release(Engine& E, void* stream) {
     E.buf_bytes = E.aux_bytes = 0;
     E.level = -1;
     E.launches.clear();
+    E.units.clear();
     E.jit.clear();
     E.jit_launches = 0;
     E.jit_state = 0;
@@ -722,9 +936,10 @@ int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* 
     for (int s = 0; s < N; ++s) m[s] = h.factors[s].m;
     B.ti.build(m, level);
 
-    B.rt = plan.k == kMaxTileQ || E.wide;
-    B.use_jit = want_jit && B.rt && jit_available();
-    if (want_jit && B.rt && !B.use_jit) E.jit_state = -1;   // NVRTC missing: the interpreting kernel runs
+    const bool rt = plan.k == kMaxTileQ || E.wide;
+    const bool use_jit = want_jit && rt && jit_available() && !E.jit_failed;
+    if (want_jit && rt && !use_jit) E.jit_state = -1;   // NVRTC missing: the precompiled kernel runs
+    B.kind = use_jit ? P_GEN : rt ? P_UNIT : P_TILE;
     // finisher factor table (complex128)
     B.tab.kmats.assign((size_t)std::max(N, 1) * 32, 0.0);
     for (int s = 0; s < N; ++s)
@@ -745,17 +960,20 @@ int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* 
     // ring of `spacing` slots whenever a sweep enters the block.
     const size_t sbytes = (size_t)B.dim * sizeof(float2);
     int n_phi = std::max(N, 1);
-    int n_group = 0;
-    for (int d = 1; d < level; ++d) n_group += (d == 1) ? 3 : 9;
     int spacing = 0;
     if (h.opt_spacing > 0 && h.opt_spacing < N) {
         if (level > 2) return NQS_ERR_UNSUPPORTED;
         spacing = h.opt_spacing;
     }
-    size_t n_states = (size_t)n_phi + 1 + n_group;
+    size_t n_states = 0;
     if (spacing == 0) {
-        E.buf_bytes = n_states * sbytes;
-        E.buf = dev_alloc(E.buf_bytes, stream);
+        // groups swept together when the memory allows, else one at a time
+        for (int small = B.kind != P_UNIT; small < 2 && !E.buf; ++small) {
+            B.gp = group_plan(plan, h.factors, level, B.kind != P_UNIT, small != 0);
+            n_states = (size_t)n_phi + 1 + B.gp.total();
+            E.buf_bytes = n_states * sbytes;
+            E.buf = dev_alloc(E.buf_bytes, stream);
+        }
         if (!E.buf) {
             E.buf_bytes = 0;
             if (h.opt_spacing != 0 || level > 2 || N < 2) return NQS_ERR_NOMEM;
@@ -774,14 +992,14 @@ int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* 
     E.spacing = spacing;
     E.n_states = n_states;
     float2* base = (float2*)E.buf;
-    B.group_bufs.assign(std::max(1, level), {});
+    B.group_buf.assign(std::max(2, level), nullptr);
     if (spacing == 0) {
         for (int s = 0; s < n_phi; ++s) B.phi.push_back(base + (size_t)s * B.dim);
         B.main_buf = base + (size_t)n_phi * B.dim;
         size_t next = (size_t)n_phi + 1;
         for (int d = 1; d < level; ++d) {
-            int cnt = (d == 1) ? 3 : 9;
-            for (int i = 0; i < cnt; ++i) B.group_bufs[d].push_back(base + (next++) * B.dim);
+            B.group_buf[d] = base + next * B.dim;
+            next += B.gp.cap[d];
         }
     } else {
         const int nb = (N + spacing - 1) / spacing;
@@ -791,14 +1009,12 @@ int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* 
         for (int j = 0; j < spacing; ++j) ring.push_back(base + (next++) * B.dim);
         B.main_buf = base + (next++) * B.dim;
         B.work_buf = base + (next++) * B.dim;
-        if (level >= 2)
-            for (int i = 0; i < 3 * spacing; ++i) B.group_bufs[1].push_back(base + (next++) * B.dim);
+        if (level >= 2) B.group_buf[1] = base + next * B.dim;   // 3 * spacing states
         for (int s = 0; s < N; ++s) B.phi.push_back(ring[s % spacing]);
         for (int s = 0; s < N; ++s) B.phi.push_back(bd[s / spacing]);
         B.bd = bd;
     }
 
-    // runs: the register-resident kernel needs a tile of exactly 12 qubits
     bool need_ideal = v->kind == NQS_STATE_IDEAL;
     if (need_ideal) B.run_ideal = make_run(plan, plan.free_passes, RT_IDEAL, false, false, false, h.factors, B.tab, B.dops);
     std::vector<char> block_last;
@@ -810,7 +1026,7 @@ int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* 
         for (int d = 0; d < depths; ++d) {
             bool spawn = d + 2 <= level;
             bool reduce = (level == 0) ? (d == 0) : (d + 1 <= level);
-            B.run_fwd.push_back(make_run(plan, spawn ? plan.sitecut_passes : plan.free_passes, RT_FWD,
+            B.run_fwd.push_back(make_run(plan, spawn && !B.gp.grouped ? plan.sitecut_passes : plan.free_passes, RT_FWD,
                                          reduce && N > 0, spawn, level == 0, h.factors, B.tab, B.dops));
         }
     } else {
@@ -829,10 +1045,7 @@ int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* 
     }
 
     // --- schedule (device pointers to aux tables are patched after layout) ---
-    B.ckpt_dev = nullptr;
     float2* mainb = B.main_buf;
-    const float2* in1[3];
-    float2* out1[3];
 
     auto init_state = [&](const nqs_state* st, float2* dst, bool& external, const float2*& ext) {
         external = false;
@@ -857,9 +1070,7 @@ int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* 
             const float2* pp = nullptr;
             init_state(psi, mainb, pe, pp);
             for (size_t p = 0; p < B.run_ideal.passes.size(); ++p) {
-                in1[0] = (p == 0 && pe) ? pp : mainb;
-                out1[0] = mainb;
-                B.add_pass(B.run_ideal.passes[p], 0, 1, in1, out1, nullptr, 0);
+                B.add_single(B.run_ideal.passes[p], (p == 0 && pe) ? pp : mainb, mainb, nullptr, false, nullptr);
             }
             if (B.run_ideal.passes.empty() && pe) {
                 Launch l;
@@ -891,10 +1102,7 @@ int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* 
         if (N > 0) {
             for (size_t p = 0; p < B.run_bwd.passes.size(); ++p) {
                 if (p > 0 && B.before_first(B.run_bwd.passes[p])) break;
-                in1[0] = (p == 0 && ext) ? ext_ptr : mainb;
-                out1[0] = mainb;
-                B.add_pass(B.run_bwd.passes[p], 0, 1, in1, out1, nullptr, 0);
-                if (spacing > 0) B.L.back().bd_table = true;
+                B.add_single(B.run_bwd.passes[p], (p == 0 && ext) ? ext_ptr : mainb, mainb, nullptr, spacing > 0, nullptr);
             }
         } else {
             // N = 0: keep v in the single phi slot for the final inner product
@@ -934,37 +1142,38 @@ int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* 
         const float2* ext_ptr = nullptr;
         init_state(psi, mainb, ext, ext_ptr);
         const Run& run = B.run_fwd[0];
+        std::vector<Group> children;
+        size_t used = 0;
         for (size_t p = 0; p < run.passes.size(); ++p) {
             const RunPass& rp = run.passes[p];
             if (N > 0 && p > 0 && B.after_last(rp)) break;
-            in1[0] = (p == 0 && ext) ? ext_ptr : mainb;
-            out1[0] = mainb;
-            std::vector<float2*> sp;
-            if (level >= 2 && rp.spawn_site >= 0)
-                for (int i = 0; i < 3; ++i) sp.push_back(B.group_bufs[1][i]);
-            B.add_pass(rp, 0, 1, in1, out1, sp.empty() ? nullptr : sp.data(), (int)sp.size());
-            B.add_finish(rp, 0, 1, main_rank);
-            if (level >= 2 && rp.spawn_site >= 0 && owns_group(rp.spawn_site)) {
-                int s = rp.spawn_site;
-                B.dfs_group(1, {}, s, h.factors[s].m, B.group_bufs[1]);
+            const int n_sp = level >= 2 ? B.spawn_count(rp, 0) : 0;
+            if (n_sp && used + 3 * (size_t)n_sp > B.gp.cap[1]) {
+                B.sweep_groups(1, children);
+                children.clear();
+                used = 0;
+            }
+            float2* sp = n_sp ? B.group_buf[1] + used * B.dim : nullptr;
+            B.add_single(rp, (p == 0 && ext) ? ext_ptr : mainb, mainb, sp, false, main_rank);
+            if (n_sp) {
+                B.make_children(rp, 0, nullptr, 1, sp, 1, children, owns_group);
+                used += 3 * (size_t)n_sp;
             }
         }
+        if (!children.empty()) B.sweep_groups(1, children);
         if (N == 0) {
             Launch l;
             l.kind = L_REDUCE2;
             l.src = B.phi[0];
             l.dst = mainb;
             l.grid = std::max(1, std::min<int>(E.sm_count * 4, (int)std::max<long long>(1, B.dim / (2 * kThreads * 16))));
-            B.partial_doubles = std::max(B.partial_doubles, (size_t)l.grid * 8);
+            l.part_off = B.take_partials((size_t)l.grid * 8);
             B.L.push_back(l);
-            Launch f;
-            f.kind = L_FINISH;
-            f.n_red = 1;
-            f.fin_grid = l.grid;
-            f.desc_off = B.descs.size();
-            B.descs.push_back({0, 0, 0});
-            for (int i = 1; i < 4; ++i) B.descs.push_back({-1, 0, 0});
-            B.L.push_back(f);
+            FinishSlot f{};
+            f.part = l.part_off;
+            f.grid = l.grid;
+            for (int i = 0; i < 4; ++i) f.d[i] = FinishDesc{i == 0 ? 0 : -1, 0, 0};
+            B.slots.push_back(f);
         }
     } else {
         bool ext = false;
@@ -972,6 +1181,7 @@ int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* 
         init_state(psi, mainb, ext, ext_ptr);
         B.spaced_forward(spacing, ext ? ext_ptr : nullptr, main_rank, owns_group);
     }
+    B.flush_finish();
     {
         Launch l;
         l.kind = L_SUM;
@@ -982,11 +1192,11 @@ int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* 
         return NQS_ERR_UNSUPPORTED;
     }
     // pass-specialised kernels for the register-resident passes
-    if (B.use_jit) {
+    if (use_jit) {
         std::vector<JitPass*> todo;
         std::vector<Launch*> owner;
         for (auto& l : B.L) {
-            if (l.kind != L_PASS || !l.rt) continue;
+            if (l.kind != L_PASS || !l.gen) continue;
             std::unique_ptr<JitPass> jp(new JitPass());
             jp->S = l.S;
             jp->k = plan.k;
@@ -1018,29 +1228,35 @@ int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* 
             E.jit_state = 1;
         } else {
             E.jit.clear();
-            E.jit_state = todo.empty() ? 0 : -1;
-            if (!todo.empty() && std::getenv("NQS_JIT_VERBOSE")) std::fprintf(stderr, "nqs jit: %s\n", err.c_str());
-            if (E.wide) {   // the interpreting kernel needs 12-qubit tiles
-                E.wide_failed = true;
+            E.jit_state = 0;
+            if (!todo.empty()) {
+                // 12-qubit tiles first, then the precompiled kernel
+                if (std::getenv("NQS_JIT_VERBOSE")) std::fprintf(stderr, "nqs jit: %s\n", err.c_str());
+                (E.wide ? E.wide_failed : E.jit_failed) = true;
                 engine_release(E, stream);
                 return build_schedule(h, E, psi, v, level, stream, allow_jit);
             }
         }
     }
 
-    // --- aux allocation: ops, mats, ckpt table, kmats, descs, partials, term values, level offsets, result
+    // --- aux allocation: ops, mats, ckpt table, programs, units, kmats, slots, partials, term values, level
+    // offsets, result
+    const bool tile_kernel = B.kind == P_TILE;   // reads operations and matrices from device tables
+    const size_t n_dops = tile_kernel ? B.dops.size() : 0, n_mats = tile_kernel ? B.tab.mats.size() : 0;
+    const size_t n_prog = B.kind == P_UNIT ? B.prog.size() : 0;
     auto align = [](size_t x) { return (x + 255) & ~(size_t)255; };
     size_t off_ops = 0;
-    size_t off_mats = align(off_ops + B.dops.size() * sizeof(DevOp) + 1);
-    size_t off_ckpt = align(off_mats + B.tab.mats.size() * sizeof(float2) + 1);
-    size_t off_phase = align(off_ckpt + B.phi.size() * sizeof(float2*));
-    size_t off_err = align(off_phase + B.prog.size() * sizeof(uint4) + 1);
-    size_t off_kmat = align(off_err + sizeof(int));
-    size_t off_desc = align(off_kmat + B.tab.kmats.size() * sizeof(double));
-    size_t off_part = align(off_desc + B.descs.size() * sizeof(FinishDesc) + 1);
+    size_t off_mats = align(off_ops + n_dops * sizeof(DevOp) + 1);
+    size_t off_ckpt = align(off_mats + n_mats * sizeof(float2) + 1);
+    size_t off_prog = align(off_ckpt + B.phi.size() * sizeof(float2*));
+    size_t off_unit = align(off_prog + n_prog * sizeof(uint4) + 1);
+    size_t off_kmat = align(off_unit + B.units.size() * sizeof(SweepUnit) + 1);
+    size_t off_slot = align(off_kmat + B.tab.kmats.size() * sizeof(double));
+    size_t off_loff = align(off_slot + B.slots.size() * sizeof(FinishSlot) + 1);
+    size_t off_err = align(off_loff + (level + 2) * sizeof(long long));   // up to here: uploaded in one copy
+    size_t off_part = align(off_err + sizeof(int));
     size_t off_vals = align(off_part + std::max<size_t>(B.partial_doubles, 8) * sizeof(double));
-    size_t off_loff = align(off_vals + std::max<uint64_t>(B.ti.total, 1) * sizeof(double));
-    size_t off_res = align(off_loff + (level + 2) * sizeof(long long));
+    size_t off_res = align(off_vals + std::max<uint64_t>(B.ti.total, 1) * sizeof(double));
     E.aux_bytes = align(off_res + sizeof(nqs_result));
     E.aux = dev_alloc(E.aux_bytes, stream);
     if (!E.aux) {
@@ -1050,34 +1266,44 @@ int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* 
     }
     char* ab = (char*)E.aux;
     DevOp* dops_dev = (DevOp*)(ab + off_ops);
-    B.ckpt_dev = (float2**)(ab + off_ckpt);
     float2* mats_dev = (float2*)(ab + off_mats);
     float2** ckpt_dev = (float2**)(ab + off_ckpt);
-    uint4* prog_dev = (uint4*)(ab + off_phase);
+    uint4* prog_dev = (uint4*)(ab + off_prog);
+    E.units_dev = (SweepUnit*)(ab + off_unit);
     E.err_dev = (int*)(ab + off_err);
     E.kmats_dev = (double*)(ab + off_kmat);
-    E.desc_dev = (FinishDesc*)(ab + off_desc);
+    E.slots_dev = (FinishSlot*)(ab + off_slot);
     E.partials = (double*)(ab + off_part);
     E.term_vals = (double*)(ab + off_vals);
     E.level_off_dev = (long long*)(ab + off_loff);
     E.res_dev = (nqs_result*)(ab + off_res);
+    for (size_t u = 0; u < B.units.size(); ++u) {
+        SweepUnit& x = B.units[u];
+        x.prog = prog_dev + B.unit_prog[u];
+        x.ckpt = ckpt_dev + (B.unit_bd[u] ? N : 0);
+        x.ckpt_fwd = nullptr;
+        x.partials = E.partials + B.unit_part[u];
+        x.err = E.err_dev;
+    }
 
     cudaStream_t st = (cudaStream_t)stream;
     std::vector<long long> loff(level + 2);
     for (int u = 0; u <= level + 1; ++u) loff[u] = (long long)B.ti.level_offset[u];
     int rc = NQS_OK;
-    E.upload_bytes = 0;
-    auto up = [&](void* dst, const void* src, size_t bytes) {
-        if (bytes && rc == NQS_OK) rc = cuda_err(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st));
-        E.upload_bytes += bytes;
+    std::vector<char> blob(off_err, 0);
+    auto put = [&](size_t off, const void* src, size_t bytes) {
+        if (bytes) std::memcpy(blob.data() + off, src, bytes);
     };
-    up(dops_dev, B.dops.data(), B.dops.size() * sizeof(DevOp));
-    up(mats_dev, B.tab.mats.data(), B.tab.mats.size() * sizeof(float2));
-    up(ckpt_dev, B.phi.data(), B.phi.size() * sizeof(float2*));
-    up(prog_dev, B.prog.data(), B.prog.size() * sizeof(uint4));
-    up(E.kmats_dev, B.tab.kmats.data(), B.tab.kmats.size() * sizeof(double));
-    up(E.desc_dev, B.descs.data(), B.descs.size() * sizeof(FinishDesc));
-    up(E.level_off_dev, loff.data(), loff.size() * sizeof(long long));
+    put(off_ops, B.dops.data(), n_dops * sizeof(DevOp));
+    put(off_mats, B.tab.mats.data(), n_mats * sizeof(float2));
+    put(off_ckpt, B.phi.data(), B.phi.size() * sizeof(float2*));
+    put(off_prog, B.prog.data(), n_prog * sizeof(uint4));
+    put(off_unit, B.units.data(), B.units.size() * sizeof(SweepUnit));
+    put(off_kmat, B.tab.kmats.data(), B.tab.kmats.size() * sizeof(double));
+    put(off_slot, B.slots.data(), B.slots.size() * sizeof(FinishSlot));
+    put(off_loff, loff.data(), loff.size() * sizeof(long long));
+    E.upload_bytes = blob.size();
+    rc = cuda_err(cudaMemcpyAsync(ab, blob.data(), blob.size(), cudaMemcpyHostToDevice, st));
     if (rc == NQS_OK) rc = cuda_err(cudaMemsetAsync(E.term_vals, 0, std::max<uint64_t>(B.ti.total, 1) * sizeof(double), st));
     // the uploads read pageable host memory: make sure they completed before the builder goes away
     if (rc == NQS_OK) rc = cuda_err(cudaStreamSynchronize(st));
@@ -1087,15 +1313,15 @@ int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* 
     }
     // rebase pass arguments onto the device tables
     for (auto& l : B.L) {
-        if (l.kind != L_PASS) continue;
-        l.args.ops = dops_dev + l.op_index;
-        l.args.prog = l.rt ? prog_dev + l.prog_index : nullptr;
+        if (l.kind != L_PASS || l.units()) continue;
+        l.args.ops = tile_kernel ? dops_dev + l.op_index : nullptr;
         l.args.err = E.err_dev;
         l.args.mats = mats_dev;
         l.args.ckpt = ckpt_dev + (l.bd_table ? N : 0);
-        l.args.partials = E.partials;
+        l.args.partials = E.partials + l.part_off;
     }
     E.launches = std::move(B.L);
+    E.units = std::move(B.units);
     E.level = level;
     E.psi_kind = psi->kind;
     E.v_kind = v->kind;
@@ -1121,9 +1347,9 @@ int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* 
     return NQS_OK;
 }
 
-int launch_pass(const Launch& l, cudaStream_t st) {
+static int launch_pass(const Engine& E, const Launch& l, cudaStream_t st) {
+    if (l.units()) return cuda_err(launch_units(E.units_dev + l.unit_off, nullptr, l.ctas, l.grid, l.smem, st));
     if (l.jit) return cuda_err(jit_launch(*l.jit, l.grid, l.args, st));
-    if (l.rt) return cuda_err(launch_sweep(l.S, l.rb, l.grid, l.args, st));
     return cuda_err(launch_tile_pass(l.S, l.grid, l.smem, l.args, st));
 }
 
@@ -1132,15 +1358,15 @@ int run_launch(Handle& h, Engine& E, const Launch& l, cudaStream_t st) {
     const long long dim = 1ll << h.plan.n;
     const int fill_grid = (int)std::max<long long>(1, std::min<long long>(E.sm_count * 8, dim / 512));
     switch (l.kind) {
-        case L_PASS: return launch_pass(l, st);
+        case L_PASS: return launch_pass(E, l, st);
         case L_FINISH:
             return cuda_err(
-                launch_finish(E.partials, l.fin_grid, E.desc_dev + l.desc_off, E.kmats_dev, E.term_vals, l.n_red, st));
+                launch_finish(E.partials, E.slots_dev + l.slot_off, E.kmats_dev, E.term_vals, l.n_slots, st));
         case L_FILL: return cuda_err(launch_basis_fill(l.dst, dim, l.bits, fill_grid, st));
         case L_COPY:
             return cuda_err(cudaMemcpyAsync(l.dst, l.src, dim * sizeof(float2), cudaMemcpyDeviceToDevice, st));
         case L_REDUCE2:   // bits holds the qubit
-            return cuda_err(launch_reduce2x2(l.src, l.dst, h.plan.n, (int)l.bits, E.partials, l.grid, st));
+            return cuda_err(launch_reduce2x2(l.src, l.dst, h.plan.n, (int)l.bits, E.partials + l.part_off, l.grid, st));
         case L_SUM:
             return cuda_err(launch_level_sum(E.term_vals, E.level_off_dev, E.eff_level, E.res_dev, E.bound, E.n_terms,
                                              E.err_dev, st));
@@ -1264,8 +1490,8 @@ int engine_launch_list(const Handle& h, nqs_launch_info* out, size_t cap, size_t
         o.kind = (int32_t)l.kind;
         if (l.kind == L_PASS) {
             o.states = l.S;
-            o.reg_qubits = l.rt ? l.rb : 0;
-            o.phases = l.rt ? l.args.n_phases : 0;
+            o.reg_qubits = l.units() ? kUnitRB : l.gen ? l.rb : 0;
+            o.phases = l.n_phases;
             o.grid = l.grid;
             for (int c = 0; c < 8; ++c) o.ops[c] = l.op_counts[c];
             o.jit = l.jit ? 1 : 0;

@@ -11,6 +11,7 @@
 #include "jit.h"
 #include "nqs_internal.h"
 #include "sweep_types.h"
+#include "unit_program.h"
 
 namespace nqs {
 
@@ -22,8 +23,7 @@ struct RunPass {
     int nonlocal[kMaxQ] = {};
     std::vector<int> lin;            // linear op index of each device op
     std::vector<int> ev_site;        // site of reduction event e
-    int spawn_site = -1;             // site that spawns in this pass (at most one)
-    int phase_off = 0, n_phases = 0; // register-resident phases (device phase buffer)
+    std::vector<int> spawn_sites;    // sites that spawn in this pass, in execution order
 };
 
 struct Run {
@@ -34,17 +34,25 @@ enum LaunchKind { L_PASS, L_FINISH, L_FILL, L_COPY, L_REDUCE2, L_SUM, L_NORMALIZ
 
 struct Launch {
     LaunchKind kind;
-    int S = 1;
+    int S = 1;                       // states of a branch group (1: single-state sweeps)
+    // pass, generated or tile kernel: one group of S states
     PassArgs args{};
     int op_index = 0;                // offset of the first device op (rebased onto the device table)
     int prog_index = 0;              // offset (16-byte words) of the launch's program
-    bool rt = false;                 // register-resident kernel
-    int rb = 4;                      // its register qubits
+    int rb = 4;                      // register qubits
     int grid = 0;
     size_t smem = 0;
+    JitPass* jit = nullptr;          // pass-specialised kernel (owned by the engine)
+    bool gen = false;                // runs a pass-specialised kernel
+    bool seq = false;                // multi-state pass-specialised kernel sweeps its states one at a time
+    // pass, unit kernel: n_units states of any number of groups, `grid` blocks in all
+    int unit_off = 0, n_units = 0, ctas = 0;
+    int max_words = 0, max_events = 0, n_phases = 0;
+    size_t part_off = 0;             // partial sums of the launch (doubles)
     // finisher
-    int n_red = 0, fin_grid = 0;
-    size_t desc_off = 0;
+    int n_slots = 0;
+    size_t slot_off = 0;
+    int fin_grid = 0;                // blocks of the reduction a normalisation reads
     // fill / copy
     float2* dst = nullptr;
     const float2* src = nullptr;
@@ -52,8 +60,7 @@ struct Launch {
     double bytes = 0;                // algorithmic bytes (pass kernels)
     bool bd_table = false;           // pass saves through the block-boundary checkpoint table
     int op_counts[8] = {};           // pass: G1, G2, D1, D2, sites, reductions, spawned states, saves
-    JitPass* jit = nullptr;          // pass-specialised kernel (owned by the engine), or the interpreter
-    bool seq = false;                // multi-state pass-specialised kernel sweeps its states one at a time
+    bool units() const { return n_units > 0; }
 };
 
 struct Engine {
@@ -77,7 +84,9 @@ struct Engine {
     long long* level_off_dev = nullptr;
     double* term_vals = nullptr;
     nqs_result* res_dev = nullptr;
-    FinishDesc* desc_dev = nullptr;
+    FinishSlot* slots_dev = nullptr;
+    SweepUnit* units_dev = nullptr;
+    std::vector<SweepUnit> units;    // host copy of the unit table (the batch executor regroups it)
     double* partials = nullptr;
     double* kmats_dev = nullptr;
     int* err_dev = nullptr;
@@ -101,6 +110,7 @@ struct Engine {
     Plan wide_plan;                  // the plan re-cut for 13-qubit tiles (generated kernels)
     bool wide = false;               // the current schedule runs on wide_plan
     bool wide_failed = false;        // a wide schedule's kernels could not be built: 12-qubit tiles
+    bool jit_failed = false;         // the generated kernels could not be built: the precompiled one
 };
 
 
@@ -146,6 +156,8 @@ int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* 
                    bool allow_jit = true);
 int run_schedule(Handle& h, Engine& E, cudaStream_t st);
 int run_launch(Handle& h, Engine& E, const Launch& l, cudaStream_t st);
-int launch_pass(const Launch& l, cudaStream_t st);
+// device bytes of the branch-group state buffers a schedule allocates beside
+// its checkpoints and main state (the batch executor packs waves with it)
+size_t group_states(const Handle& h, int level, bool generated);
 
 }  // namespace nqs

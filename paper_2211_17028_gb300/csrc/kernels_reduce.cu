@@ -48,38 +48,31 @@ __global__ void __launch_bounds__(kThreads) reduce2x2_kernel(const float2* __res
     }
 }
 
-// Sum per-block partials of one reduction slot in a fixed order: thread t
-// takes component t % 8 of blocks t / 8, t / 8 + 32, ... (whole 64-byte rows
-// per load), then two shuffles join the four rows of a warp and eight threads
-// add the eight warps' sums.  Latency-bound: 8.4 us as eight components per
-// thread and an eight-step tree, 3 us in this form (152 partials).
-__device__ void sum_partials(const double* __restrict__ part, int grid, double* R, double (*scratch)[8]) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+// One warp per reduction slot: the per-block partial sums in a fixed order
+// (lane l takes component l % 8 of blocks l / 8, l / 8 + 4, ...: whole 64-byte
+// rows per load, four loads in flight; two shuffles join the four rows), then
+// X = |sum_ab K[a][b] R[a][b]|^2 for each factor of the slot.  Latency-bound;
+// one launch serves all reductions since the last one (as a launch behind
+// every pass it was 109 launches of 8.4 us in a 20-qubit level-2 call).
+__device__ __forceinline__ void finish_slot(const double* __restrict__ partials, const FinishSlot& s,
+                                            const double* __restrict__ kmats, double* __restrict__ term_vals,
+                                            double* R) {
+    const int lane = threadIdx.x & 31;
+    const double* const part = partials + s.part + (lane & 7);
     double v = 0.0;
-    for (int b = tid >> 3; b < grid; b += kThreads / 8) v += part[(size_t)b * 8 + (tid & 7)];
+    int b = lane >> 3;
+    for (; b + 12 < s.grid; b += 16) {
+        const double p0 = part[(size_t)b * 8], p1 = part[(size_t)(b + 4) * 8];
+        const double p2 = part[(size_t)(b + 8) * 8], p3 = part[(size_t)(b + 12) * 8];
+        v += (p0 + p1) + (p2 + p3);
+    }
+    for (; b < s.grid; b += 4) v += part[(size_t)b * 8];
     v += __shfl_xor_sync(0xffffffffu, v, 8);
     v += __shfl_xor_sync(0xffffffffu, v, 16);
-    if (lane < 8) scratch[warp][lane] = v;
-    __syncthreads();
-    if (tid < 8) {
-        double t = 0.0;
-#pragma unroll
-        for (int w = 0; w < kWarps; ++w) t += scratch[w][tid];
-        R[tid] = t;
-    }
-    __syncthreads();
-}
-
-// One block per reduction slot (event, state): R from the partials, then
-// X = |sum_ab K[a][b] R[a][b]|^2 for each factor of the slot.
-__device__ __forceinline__ void finish_slot(const double* __restrict__ partials, int grid, int slot,
-                                            const FinishDesc* __restrict__ desc, const double* __restrict__ kmats,
-                                            double* __restrict__ term_vals) {
-    __shared__ double scratch[kWarps][8];
-    __shared__ double R[8];
-    sum_partials(partials + (size_t)slot * grid * 8, grid, R, scratch);
-    if (threadIdx.x < 4) {
-        FinishDesc d = desc[slot * 4 + threadIdx.x];
+    if (lane < 8) R[lane] = v;
+    __syncwarp();
+    if (lane < 4) {
+        const FinishDesc d = s.d[lane];
         if (d.rank >= 0) {
             const double* K = kmats + d.kmat;
             double re = 0, im = 0;
@@ -93,16 +86,19 @@ __device__ __forceinline__ void finish_slot(const double* __restrict__ partials,
     }
 }
 
-__global__ void __launch_bounds__(kThreads) finish_kernel(const double* __restrict__ partials, int grid,
-                                                          const FinishDesc* __restrict__ desc,
+__global__ void __launch_bounds__(kThreads) finish_kernel(const double* __restrict__ partials,
+                                                          const FinishSlot* __restrict__ slots,
                                                           const double* __restrict__ kmats,
-                                                          double* __restrict__ term_vals) {
-    finish_slot(partials, grid, blockIdx.x, desc, kmats, term_vals);
+                                                          double* __restrict__ term_vals, int n_slots) {
+    __shared__ double R[kWarps][8];
+    const int warp = threadIdx.x >> 5, slot = blockIdx.x * kWarps + warp;
+    if (slot < n_slots) finish_slot(partials, slots[slot], kmats, term_vals, R[warp]);
 }
 
 // finishers of many circuits: unit u owns blocks [blk_begin[u], blk_begin[u+1])
 __global__ void __launch_bounds__(kThreads) finish_kernel_batched(const FinishUnit* __restrict__ units,
                                                                   const int* __restrict__ blk_begin, int n_units) {
+    __shared__ double R[kWarps][8];
     int lo = 0, hi = n_units;
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
@@ -110,16 +106,29 @@ __global__ void __launch_bounds__(kThreads) finish_kernel_batched(const FinishUn
         else hi = mid;
     }
     const FinishUnit u = units[lo];
-    finish_slot(u.partials, u.grid, (int)blockIdx.x - blk_begin[lo], u.desc, u.kmats, u.vals);
+    const int warp = threadIdx.x >> 5, slot = ((int)blockIdx.x - blk_begin[lo]) * kWarps + warp;
+    if (slot < u.n_slots) finish_slot(u.partials, u.slots[slot], u.kmats, u.vals, R[warp]);
 }
 
 // One block: fixed-order sum of per-block partials into 8 doubles.
 __global__ void __launch_bounds__(kThreads) partials_sum_kernel(const double* __restrict__ part, int grid,
                                                                 double* __restrict__ R) {
+    // thread t takes component t % 8 of blocks t / 8, t / 8 + 32, ...; two
+    // shuffles join the rows of a warp, eight threads add the warps' sums
     __shared__ double scratch[kWarps][8];
-    __shared__ double r[8];
-    sum_partials(part, grid, r, scratch);
-    if (threadIdx.x < 8) R[threadIdx.x] = r[threadIdx.x];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    double v = 0.0;
+    for (int b = tid >> 3; b < grid; b += kThreads / 8) v += part[(size_t)b * 8 + (tid & 7)];
+    v += __shfl_xor_sync(0xffffffffu, v, 8);
+    v += __shfl_xor_sync(0xffffffffu, v, 16);
+    if (lane < 8) scratch[warp][lane] = v;
+    __syncthreads();
+    if (tid < 8) {
+        double t = 0.0;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) t += scratch[w][tid];
+        R[tid] = t;
+    }
 }
 
 // Neumaier-compensated per-level sums (level_sum.cuh), one block.
@@ -184,9 +193,11 @@ cudaError_t launch_reduce2x2(const float2* phi, const float2* chi, int n, int q,
     return cudaGetLastError();
 }
 
-cudaError_t launch_finish(const double* partials, int grid, const FinishDesc* desc, const double* kmats,
-                          double* vals, int n_red, cudaStream_t st) {
-    finish_kernel<<<n_red, kThreads, 0, st>>>(partials, grid, desc, kmats, vals);
+int finish_blocks(int n_slots) { return (n_slots + kWarps - 1) / kWarps; }
+
+cudaError_t launch_finish(const double* partials, const FinishSlot* slots, const double* kmats, double* vals,
+                          int n_slots, cudaStream_t st) {
+    finish_kernel<<<finish_blocks(n_slots), kThreads, 0, st>>>(partials, slots, kmats, vals, n_slots);
     return cudaGetLastError();
 }
 

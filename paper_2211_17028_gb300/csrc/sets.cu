@@ -53,8 +53,8 @@ struct SetsState {
     std::vector<std::pair<int, int>> mat_pass;   // (first op in mat_ops, count) per pass, reversed order
     std::vector<int> mat_seg;         // segment index of each entry of mat_pass
     std::vector<int> mat_block;       // block of each entry of mat_pass
-    float2* g1[3] = {};
-    float2* g2[9] = {};
+    float2* g1 = nullptr;             // three states spawned at the first site
+    float2* g2 = nullptr;             // nine spawned at the second
     float2** phi_tab = nullptr;
     float2** chi_tab = nullptr;
     double* kmats = nullptr;
@@ -73,10 +73,31 @@ size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct Prog {
     std::vector<DevOp> dops;          // shared-memory tile kernel
-    std::vector<uint4> prog;          // register-resident kernel
-    std::vector<FinishDesc> descs;
+    std::vector<uint4> prog;          // unit kernel
+    std::vector<SweepUnit> units;
+    std::vector<size_t> unit_prog, unit_part;
+    std::vector<char> unit_bd;
+    std::vector<FinishSlot> slots;
     std::vector<Launch> L;
-    size_t partial_doubles = 8;
+    size_t partial_doubles = 8, partial_top = 0, finished = 0;
+    size_t take_partials(size_t need) {
+        if (partial_top > 0 && partial_top + need > ((size_t)4 << 20)) flush_finish();
+        const size_t at = partial_top;
+        partial_top += need;
+        partial_doubles = std::max(partial_doubles, partial_top);
+        return at;
+    }
+    // finisher launch for the slots collected since the last one
+    void flush_finish() {
+        if (finished == slots.size()) return;
+        Launch f;
+        f.kind = L_FINISH;
+        f.slot_off = finished;
+        f.n_slots = (int)(slots.size() - finished);
+        finished = slots.size();
+        partial_top = 0;
+        L.push_back(f);
+    }
 };
 
 // DevOps of the forward direction for linear ops [a, b) of pass `ps`, with
@@ -116,15 +137,55 @@ int pass_of(const std::vector<PassSpec>& segs, int lin) {
     return -1;
 }
 
-// one sweep launch over custom DevOps of one pass
-void add_launch(Prog& G, const Plan& plan, const SetsState& S, const PassSpec& ps, int nstates,
-                std::vector<DevOp> ops, const float2* const* in, float2* const* out, float2* const* spawn,
-                int n_spawn) {
+// One sweep launch over custom DevOps of one pass; the states and the buffers
+// they spawn into are consecutive from in, out and spawn on.  Returns the
+// offset of the partial sums of state 0, event 0; `step` receives the distance
+// between states and between events, `grid` the blocks of a state.
+struct PartLayout {
+    size_t base = 0, state = 0, event = 0;
+    int grid = 0;
+};
+
+PartLayout add_launch(Prog& G, const Plan& plan, const SetsState& S, const PassSpec& ps, int nstates,
+                      const std::vector<DevOp>& ops, const float2* in, float2* out, float2* spawn, bool bd_table) {
+    const size_t dim = (size_t)1 << plan.n;
     Launch l;
+    PartLayout pl;
     l.kind = L_PASS;
     l.S = nstates;
+    const long long n_tiles = 1ll << (plan.n - plan.k);
+    if (plan.k == kMaxTileQ) {
+        int local[kMaxTileQ];
+        for (int j = 0; j < kMaxTileQ; ++j) local[j] = ps.local[j];
+        const UnitProgram pi = assemble_unit(ops, 0, (int)ops.size(), local, plan.n, S.tab.mats, G.prog);
+        l.n_phases = pi.n_phases;
+        l.smem = unit_smem_bytes(pi.words, pi.n_events);
+        l.unit_off = (int)G.units.size();
+        l.n_units = nstates;
+        l.ctas = unit_ctas(nstates, n_tiles, unit_blocks_per_sm(l.smem) * S.sm_count);
+        l.grid = l.ctas * nstates;
+        pl.grid = l.ctas;
+        pl.event = (size_t)l.ctas * 8;
+        pl.state = pl.event * pi.n_events;
+        pl.base = G.take_partials(pl.state * nstates);
+        for (int s = 0; s < nstates; ++s) {
+            SweepUnit u{};
+            u.in = in + s * dim;
+            u.out = out + s * dim;
+            u.spawn = spawn ? spawn + 3 * s * dim : nullptr;
+            u.n_tiles = (int)n_tiles;
+            u.n = plan.n;
+            u.ctas = l.ctas;
+            u.cta_begin = s * l.ctas;
+            G.units.push_back(u);
+            G.unit_prog.push_back((size_t)pi.word);
+            G.unit_part.push_back(pl.base + s * pl.state);
+            G.unit_bd.push_back(bd_table);
+        }
+        G.L.push_back(l);
+        return pl;
+    }
     PassArgs& a = l.args;
-    a = PassArgs{};
     a.n = plan.n;
     a.k = plan.k;
     a.c = plan.c;
@@ -140,89 +201,46 @@ void add_launch(Prog& G, const Plan& plan, const SetsState& S, const PassSpec& p
     int nl = 0;
     for (int q = 0; q < plan.n; ++q)
         if (!is_local[q]) a.nonlocal[nl++] = q;
-    a.n_tiles = 1ll << (plan.n - plan.k);
+    a.n_tiles = n_tiles;
     for (int s = 0; s < nstates; ++s) {
-        a.in[s] = in[s];
-        a.out[s] = out[s];
+        a.in[s] = in + s * dim;
+        a.out[s] = out + s * dim;
+        if (spawn)
+            for (int i = 0; i < 3; ++i) a.spawn[3 * s + i] = spawn + (3 * s + i) * dim;
     }
-    for (int i = 0; i < n_spawn; ++i) a.spawn[i] = spawn[i];
-    l.rt = plan.k == kMaxTileQ;
-    int per_sm;
-    if (l.rt) {
-        l.rb = sweep_reg_bits(nstates);
-        ProgInfo pi = build_program(ops, 0, (int)ops.size(), l.rb, S.tab, G.prog);
-        l.prog_index = pi.words_begin;
-        a.prog_words = pi.n_words;
-        a.ops_word = pi.ops_word;
-        a.mats_word = pi.mats_word;
-        a.n_phases = pi.n_phases;
-        per_sm = sweep_blocks_per_sm(nstates, l.rb, sweep_smem_bytes(nstates, l.rb, pi.n_words, n_ev));
-    } else {
-        l.op_index = (int)G.dops.size();
-        G.dops.insert(G.dops.end(), ops.begin(), ops.end());
-        a.n_ops = (int)ops.size();
-        l.smem = (size_t)nstates * (1 << plan.k) * sizeof(float2);
-        per_sm = tile_pass_blocks_per_sm(nstates, l.smem);
-    }
-    l.grid = (int)std::max<long long>(1, std::min<long long>((long long)per_sm * S.sm_count, a.n_tiles));
-    G.partial_doubles = std::max(G.partial_doubles, (size_t)std::max(1, n_ev) * nstates * l.grid * 8);
+    l.bd_table = bd_table;
+    l.op_index = (int)G.dops.size();
+    G.dops.insert(G.dops.end(), ops.begin(), ops.end());
+    a.n_ops = (int)ops.size();
+    l.smem = (size_t)nstates * (1 << plan.k) * sizeof(float2);
+    l.grid = (int)std::max<long long>(1, std::min<long long>((long long)tile_pass_blocks_per_sm(nstates, l.smem) * S.sm_count, n_tiles));
+    pl.grid = l.grid;
+    pl.state = (size_t)l.grid * 8;
+    pl.event = pl.state * nstates;
+    pl.base = l.part_off = G.take_partials(pl.event * n_ev);
     G.L.push_back(l);
+    return pl;
 }
 
-// finisher for the last launch: its single reduction event, `nstates` slots;
-// slot st, factor position f -> value index rank_of(st, f)
+// slot of one reduction (site, state): factor position f -> value index rank_of(f)
 template <typename R>
-void add_finish(Prog& G, int nstates, int site, const std::vector<Factors>& fac, R rank_of) {
-    const Launch& pl = G.L.back();
-    Launch f;
-    f.kind = L_FINISH;
-    f.n_red = nstates;
-    f.fin_grid = pl.grid;
-    f.desc_off = G.descs.size();
+void add_slot(Prog& G, size_t part, int grid, int site, const std::vector<Factors>& fac, R rank_of) {
     const Factors& ft = fac[site];
-    for (int st = 0; st < nstates; ++st)
-        for (int i = 0; i < 4; ++i) {
-            FinishDesc d{-1, 0, 0};
-            if (i >= 1 && i <= ft.m) {
-                d.rank = rank_of(st, i - 1);
-                d.kmat = site * 32 + ft.keep[i - 1] * 8;
-            }
-            G.descs.push_back(d);
-        }
-    G.L.push_back(f);
-}
-
-// finisher for the last launch with several reduction events (sites in
-// launch order); slot (event e, state st), factor position f -> rank_of(site, st, f)
-template <typename R>
-void add_finish_events(Prog& G, int nstates, const std::vector<int>& ev_sites, const std::vector<Factors>& fac,
-                       R rank_of) {
-    const Launch& pl = G.L.back();
-    Launch f;
-    f.kind = L_FINISH;
-    f.n_red = (int)ev_sites.size() * nstates;
-    f.fin_grid = pl.grid;
-    f.desc_off = G.descs.size();
-    for (int t : ev_sites) {
-        const Factors& ft = fac[t];
-        for (int st = 0; st < nstates; ++st)
-            for (int i = 0; i < 4; ++i) {
-                FinishDesc d{-1, 0, 0};
-                if (i >= 1 && i <= ft.m) {
-                    d.rank = rank_of(t, st, i - 1);
-                    d.kmat = t * 32 + ft.keep[i - 1] * 8;
-                }
-                G.descs.push_back(d);
-            }
+    FinishSlot f{};
+    f.part = part;
+    f.grid = grid;
+    for (int i = 0; i < 4; ++i) {
+        f.d[i] = FinishDesc{-1, 0, 0};
+        if (i >= 1 && i <= ft.m) f.d[i] = FinishDesc{(long long)rank_of(i - 1), site * 32 + ft.keep[i - 1] * 8, 0};
     }
-    G.L.push_back(f);
+    G.slots.push_back(f);
 }
 
 // sweep `nstates` states over the linear ops (a, b]; site t gets flag_of(t)
 // (which may spawn only at b); every launch with reductions gets its finisher
 template <typename FlagFn, typename RankFn>
 void sweep_range(Prog& G, const Handle& h, const SetsState& S, int a, int b, FlagFn flag_of, int nstates,
-                 float2* const* states, float2* const* spawn, int n_spawn, RankFn rank_of) {
+                 float2* states, float2* spawn, RankFn rank_of) {
     const Plan& plan = h.plan;
     for (int p = pass_of(S.fsegs, a + 1); p >= 0 && p < (int)S.fsegs.size(); ++p) {
         const PassSpec& ps = S.fsegs[p];
@@ -241,12 +259,15 @@ void sweep_range(Prog& G, const Handle& h, const SetsState& S, int a, int b, Fla
             }
             auto ops = emit_range(plan, S, ps, c0, c1, flag_of, h.factors);
             const bool last_chunk = has_last && c1 == hi;
-            add_launch(G, plan, S, ps, nstates, ops, (const float2* const*)states, states,
-                       last_chunk ? spawn : nullptr, last_chunk ? n_spawn : 0);
-            std::vector<int> ev;
-            for (const DevOp& d : ops)
-                if (d.type == OP_SITE && (d.flags & FL_REDUCE)) ev.push_back(d.site);
-            if (!ev.empty()) add_finish_events(G, nstates, ev, h.factors, rank_of);
+            const PartLayout pl = add_launch(G, plan, S, ps, nstates, ops, states, states, last_chunk ? spawn : nullptr, false);
+            int ev = 0;
+            for (const DevOp& d : ops) {
+                if (d.type != OP_SITE || !(d.flags & FL_REDUCE)) continue;
+                for (int st = 0; st < nstates; ++st)
+                    add_slot(G, pl.base + ev * pl.event + st * pl.state, pl.grid, d.site, h.factors,
+                             [&](int f) { return rank_of(d.site, st, f); });
+                ++ev;
+            }
             c0 = c1;
         }
         if (has_last) break;
@@ -254,11 +275,12 @@ void sweep_range(Prog& G, const Handle& h, const SetsState& S, int a, int b, Fla
 }
 
 int upload_and_run(Handle& h, SetsState& S, Prog& G, size_t extra_bytes, void** extra, cudaStream_t st) {
-    // per-call buffer: device ops, programs, descriptors, partials, extra
-    const size_t o_ops = 0;
-    const size_t o_prog = align256(o_ops + G.dops.size() * sizeof(DevOp) + 1);
-    const size_t o_desc = align256(o_prog + G.prog.size() * sizeof(uint4) + 1);
-    const size_t o_part = align256(o_desc + G.descs.size() * sizeof(FinishDesc) + 1);
+    G.flush_finish();
+    // per-call buffer: device ops, programs, units, finisher slots, partials, extra
+    const size_t o_prog = align256(G.dops.size() * sizeof(DevOp) + 1);
+    const size_t o_unit = align256(o_prog + G.prog.size() * sizeof(uint4) + 1);
+    const size_t o_slot = align256(o_unit + G.units.size() * sizeof(SweepUnit) + 1);
+    const size_t o_part = align256(o_slot + G.slots.size() * sizeof(FinishSlot) + 1);
     const size_t o_extra = align256(o_part + G.partial_doubles * sizeof(double));
     const size_t need = align256(o_extra + extra_bytes + 1);
     if (need > S.call_bytes) {
@@ -271,31 +293,39 @@ int upload_and_run(Handle& h, SetsState& S, Prog& G, size_t extra_bytes, void** 
         if (!S.call) return NQS_ERR_NOMEM;
     }
     char* base = (char*)S.call;
+    Engine E;   // a throwaway engine view carrying the pointers run_launch reads
+    E.sm_count = S.sm_count;
+    E.partials = (double*)(base + o_part);
+    E.slots_dev = (FinishSlot*)(base + o_slot);
+    E.units_dev = (SweepUnit*)(base + o_unit);
+    E.kmats_dev = S.kmats;
+    E.err_dev = S.err;
+    for (size_t u = 0; u < G.units.size(); ++u) {
+        SweepUnit& x = G.units[u];
+        x.prog = (const uint4*)(base + o_prog) + G.unit_prog[u];
+        x.ckpt = G.unit_bd[u] ? S.phi_bd_tab : S.phi_tab;
+        x.ckpt_fwd = S.chi_tab;
+        x.partials = E.partials + G.unit_part[u];
+        x.err = S.err;
+    }
     int rc = NQS_OK;
     auto up = [&](size_t off, const void* src, size_t bytes) {
         if (bytes && rc == NQS_OK) rc = cuda_err(cudaMemcpyAsync(base + off, src, bytes, cudaMemcpyHostToDevice, st));
     };
-    up(o_ops, G.dops.data(), G.dops.size() * sizeof(DevOp));
+    up(0, G.dops.data(), G.dops.size() * sizeof(DevOp));
     up(o_prog, G.prog.data(), G.prog.size() * sizeof(uint4));
-    up(o_desc, G.descs.data(), G.descs.size() * sizeof(FinishDesc));
+    up(o_unit, G.units.data(), G.units.size() * sizeof(SweepUnit));
+    up(o_slot, G.slots.data(), G.slots.size() * sizeof(FinishSlot));
     if (rc == NQS_OK && extra_bytes) rc = cuda_err(cudaMemsetAsync(base + o_extra, 0, extra_bytes, st));
     if (rc == NQS_OK) rc = cuda_err(cudaStreamSynchronize(st));   // pageable sources
     if (rc != NQS_OK) return rc;
     if (extra) *extra = base + o_extra;
-    // a throwaway engine view carrying the pointers run_launch reads
-    Engine E;
-    E.sm_count = S.sm_count;
-    E.partials = (double*)(base + o_part);
-    E.desc_dev = (FinishDesc*)(base + o_desc);
-    E.kmats_dev = S.kmats;
-    E.err_dev = S.err;
     for (Launch& l : G.L) {
-        if (l.kind == L_PASS) {
-            l.args.ops = (const DevOp*)(base + o_ops) + l.op_index;
-            l.args.prog = l.rt ? (const uint4*)(base + o_prog) + l.prog_index : nullptr;
+        if (l.kind == L_PASS && !l.units()) {
+            l.args.ops = (const DevOp*)base + l.op_index;
             l.args.ckpt = l.bd_table ? S.phi_bd_tab : S.phi_tab;
             l.args.ckpt_fwd = S.chi_tab;
-            l.args.partials = E.partials;
+            l.args.partials = E.partials + l.part_off;
             l.args.err = S.err;
         }
     }
@@ -371,8 +401,8 @@ int engine_prepare_sets(Handle& h, const nqs_state* psi, const nqs_state* v, voi
         S.work_mat = b + (next++) * dim;
         next++;   // spare (keeps the count of spaced_states)
     }
-    for (int i = 0; i < 3; ++i) S.g1[i] = b + (next++) * dim;
-    for (int i = 0; i < 9; ++i) S.g2[i] = b + (next++) * dim;
+    S.g1 = b + next * dim;
+    S.g2 = S.g1 + 3 * dim;
 
     // matrices: forward factors for every op (and adjoints for the backward runs)
     std::vector<char> block_last, block_first;
@@ -468,8 +498,6 @@ int engine_prepare_sets(Handle& h, const nqs_state* psi, const nqs_state* v, voi
 
     // checkpoint sweeps: (ideal v) -> backward saving phi -> forward saving chi
     Prog G;
-    const float2* in1[1];
-    float2* out1[1];
     auto run_passes = [&](const Run& run, const std::vector<PassSpec>& segs, const float2* first_in, bool bwd,
                           bool save_fwd) {
         for (size_t p = 0; p < run.passes.size(); ++p) {
@@ -484,11 +512,8 @@ int engine_prepare_sets(Handle& h, const nqs_state* psi, const nqs_state* v, voi
             for (DevOp& d : ops)
                 if (d.type == OP_SITE && save_fwd)
                     d.flags = FL_APPLY | ((!k || block_first[d.site]) ? FL_SAVE_FWD : 0) | (d.flags & FL_KDIAG);
-            in1[0] = (p == 0 && first_in) ? first_in : S.main;
-            out1[0] = S.main;
             const PassSpec& ps = segs[bwd ? run.passes.size() - 1 - p : p];
-            add_launch(G, plan, S, ps, 1, ops, in1, out1, nullptr, 0);
-            if (bwd) G.L.back().bd_table = true;
+            add_launch(G, plan, S, ps, 1, ops, (p == 0 && first_in) ? first_in : S.main, S.main, nullptr, bwd);
         }
     };
     auto fill = [&](const nqs_state* st8, const float2*& ext) {
@@ -517,7 +542,7 @@ int engine_prepare_sets(Handle& h, const nqs_state* psi, const nqs_state* v, voi
     // the matrices of the device table: programs index their own copies, the
     // shared-memory tile kernel reads the table
     for (Launch& l : G.L)
-        if (l.kind == L_PASS) l.args.mats = mats_dev;
+        if (l.kind == L_PASS && !l.units()) l.args.mats = mats_dev;
     rc = upload_and_run(h, S, G, 0, nullptr, st);
     if (rc == NQS_OK) rc = cuda_err(cudaStreamSynchronize(st));
     if (rc != NQS_OK) {
@@ -564,9 +589,8 @@ int engine_eval_sets(Handle& h, int k, const int* sets, size_t m, double* W_out,
             if (S.mat_block[p] != c) continue;
             std::vector<DevOp> ops(S.mat_ops.begin() + S.mat_pass[p].first,
                                    S.mat_ops.begin() + S.mat_pass[p].first + S.mat_pass[p].second);
-            const float2* in[1] = {first_in ? S.phi[c] : S.work_mat};
-            float2* out[1] = {S.work_mat};
-            add_launch(G, plan, S, S.segs[S.mat_seg[p]], 1, ops, in, out, nullptr, 0);
+            add_launch(G, plan, S, S.segs[S.mat_seg[p]], 1, ops, first_in ? S.phi[c] : S.work_mat, S.work_mat, nullptr,
+                       false);
             first_in = false;
         }
         ring_block = c;
@@ -582,14 +606,13 @@ int engine_eval_sets(Handle& h, int k, const int* sets, size_t m, double* W_out,
         c.dst = S.work;
         c.src = S.chi[s1 / K];
         G.L.push_back(c);
-        float2* w[1] = {S.work};
-        sweep_range(G, h, S, plan.site_pos[first] - 1, plan.site_pos[s1] - 1, [](int) { return FL_APPLY; }, 1, w,
-                    nullptr, 0, [](int, int, int) { return -1ll; });
+        sweep_range(G, h, S, plan.site_pos[first] - 1, plan.site_pos[s1] - 1, [](int) { return FL_APPLY; }, 1, S.work,
+                    nullptr, [](int, int, int) { return -1ll; });
         return S.work;
     };
     // sweep `states` from linear op `from` through the reduction sites of
     // `slots` (site -> value slot base), one checkpoint block at a time
-    auto reduce_through = [&](int from, const std::map<int, long long>& slots, int nst, float2* const* states,
+    auto reduce_through = [&](int from, const std::map<int, long long>& slots, int nst, float2* states,
                               int mult) {
         int pos = from;
         for (auto it = slots.begin(); it != slots.end();) {
@@ -599,7 +622,7 @@ int engine_eval_sets(Handle& h, int k, const int* sets, size_t m, double* W_out,
             materialize(blk);
             const int last = std::prev(end)->first;
             sweep_range(G, h, S, pos, plan.site_pos[last],
-                        [&](int t) { return FL_APPLY | (slots.count(t) ? FL_REDUCE : 0); }, nst, states, nullptr, 0,
+                        [&](int t) { return FL_APPLY | (slots.count(t) ? FL_REDUCE : 0); }, nst, states, nullptr,
                         [&](int t, int st, int f) { return slots.at(t) + st * mult + f; });
             pos = plan.site_pos[last];
             it = end;
@@ -622,9 +645,9 @@ int engine_eval_sets(Handle& h, int k, const int* sets, size_t m, double* W_out,
                 const long long npairs = 1ll << (plan.n - 1);
                 l.grid = (int)std::max<long long>(
                     1, std::min<long long>((long long)S.sm_count * 4, (npairs + 16ll * kThreads - 1) / (16ll * kThreads)));
-                G.partial_doubles = std::max(G.partial_doubles, (size_t)l.grid * 8);
+                l.part_off = G.take_partials((size_t)l.grid * 8);
                 G.L.push_back(l);
-                add_finish(G, 1, s1, h.factors, [&](int, int f) { return base + f; });
+                add_slot(G, l.part_off, l.grid, s1, h.factors, [&](int f) { return base + f; });
             }
             i = i1;
             continue;
@@ -635,9 +658,8 @@ int engine_eval_sets(Handle& h, int k, const int* sets, size_t m, double* W_out,
         const PassSpec& ps1 = S.fsegs[pass_of(S.fsegs, p1)];
         {
             auto ops = emit_range(plan, S, ps1, p1, p1 + 1, [&](int) { return FL_SPAWN; }, h.factors);
-            const float2* in[1] = {chi_of(s1)};
-            float2* out[1] = {S.scratch};
-            add_launch(G, plan, S, ps1, 1, ops, in, out, S.g1, 3);
+            const float2* chi = chi_of(s1);
+            add_launch(G, plan, S, ps1, 1, ops, chi, S.scratch, S.g1, false);
         }
         if (k == 2) {
             std::map<int, long long> base2;   // second site -> value slots of its set
@@ -652,7 +674,7 @@ int engine_eval_sets(Handle& h, int k, const int* sets, size_t m, double* W_out,
             size_t r2 = r;
             while (r2 < i1 && at(r2, 1) == s2) ++r2;
             // carry the first group to s2 (K_0 there), spawning the nine states
-            sweep_range(G, h, S, pos, p2, [&](int t) { return FL_APPLY | (t == s2 ? FL_SPAWN : 0); }, m1, S.g1, S.g2, 9,
+            sweep_range(G, h, S, pos, p2, [&](int t) { return FL_APPLY | (t == s2 ? FL_SPAWN : 0); }, m1, S.g1, S.g2,
                         [](int, int, int) { return -1ll; });
             pos = p2;
             std::map<int, long long> base3;   // third site -> value slots of its set
@@ -662,7 +684,7 @@ int engine_eval_sets(Handle& h, int k, const int* sets, size_t m, double* W_out,
                 for (int g = 0; g < m1; ++g) {
                     std::map<int, long long> bg = base3;
                     for (auto& e : bg) e.second += g * 9;
-                    reduce_through(p2, bg, m2, S.g2 + 3 * g, 3);
+                    reduce_through(p2, bg, m2, S.g2 + (size_t)3 * g * ((size_t)1 << plan.n), 3);
                 }
             } else {
                 // one block at a time for all three groups, so each block's phi is recomputed once
@@ -675,7 +697,7 @@ int engine_eval_sets(Handle& h, int k, const int* sets, size_t m, double* W_out,
                     for (int g = 0; g < m1; ++g) {
                         std::map<int, long long> bg = part;
                         for (auto& e : bg) e.second += g * 9;
-                        reduce_through(gpos[g], bg, m2, S.g2 + 3 * g, 3);
+                        reduce_through(gpos[g], bg, m2, S.g2 + (size_t)3 * g * ((size_t)1 << plan.n), 3);
                         gpos[g] = plan.site_pos[std::prev(end)->first];
                     }
                     it = end;
@@ -686,7 +708,7 @@ int engine_eval_sets(Handle& h, int k, const int* sets, size_t m, double* W_out,
         i = i1;
     }
     for (Launch& l : G.L)
-        if (l.kind == L_PASS) l.args.mats = mats_dev;
+        if (l.kind == L_PASS && !l.units()) l.args.mats = mats_dev;
     void* vals = nullptr;
     int rc = upload_and_run(h, S, G, m * 27 * sizeof(double), &vals, st);   // value slots start at zero
     if (rc != NQS_OK) return rc;

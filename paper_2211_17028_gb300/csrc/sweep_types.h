@@ -30,7 +30,7 @@ enum : int {
     FL_KDIAG = 32     // K_0 is diagonal
 };
 
-// location of a qubit inside the register-resident layout of a phase
+// location of a qubit inside the layout of a phase
 //   0..3   register bit i (amplitude index r within the thread)
 //   8..15  thread bit (threadIdx.x bit l - 8)
 //   -1     outside the tile (bit read from the tile's base index)
@@ -46,7 +46,7 @@ struct DevOp {
     int la, lb;      // locations of q0, q1 in the phase layout (register-resident kernel)
 };
 
-// One phase of a pass in the register-resident kernel: which tile positions
+// One phase of a pass of the generated kernels: which tile positions
 // sit in registers (R), in the lane bits (L) and in the warp bits (W).
 struct DevPhase {
     signed char R[kRegBits];
@@ -57,7 +57,7 @@ struct DevPhase {
     int pad2[2];
 };
 
-// Compact operation record of the register-resident kernel (16 bytes).
+// Compact operation record of the generated kernels' programs (16 bytes).
 struct OpRec {
     unsigned char type, la, lb, flags;   // la, lb: location codes (register bit, LOC_THREAD + bit, 0xff outside)
     unsigned char qa, qb, ev, nspawn;    // qubits; reduction event; spawned factors
@@ -68,9 +68,7 @@ struct OpRec {
 struct PassArgs {
     const DevOp* ops;
     int n_ops;
-    const DevPhase* phases;   // shared-memory tile kernel: unused
-    int n_phases;
-    const uint4* prog;        // register-resident kernel: phases, op records, matrices
+    int n_phases;             // generated kernels: the program they were made from
     int prog_words, ops_word, mats_word;
     const float2* mats;
     int n, k, c;
@@ -93,13 +91,21 @@ struct FinishDesc {
     int pad;
 };
 
+// One reduction of one state: its per-block partial sums and the terms they give
+struct FinishSlot {
+    unsigned long long part;   // offset (doubles) of the first block's sums
+    int grid;                  // blocks
+    int pad;
+    FinishDesc d[4];
+};
+
 // batched bookkeeping units (one per circuit of a batch round)
 struct FinishUnit {
     const double* partials;
-    const FinishDesc* desc;
+    const FinishSlot* slots;
     const double* kmats;
     double* vals;
-    int grid;
+    int n_slots;
     int pad;
 };
 
@@ -122,6 +128,7 @@ struct SumUnit {
 };
 
 // ---------------------------------------------------------------- helpers
+#ifdef __CUDACC__
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
     return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
@@ -131,26 +138,18 @@ __device__ __forceinline__ float2 cfma(float2 a, float2 b, float2 c) {   // a*b 
 __device__ __forceinline__ int insert0(int p, int pos) {
     return ((p >> pos) << (pos + 1)) | (p & ((1 << pos) - 1));
 }
+#endif
 
 // ---------------------------------------------------------------- launchers
 // shared-memory tile kernel (any tile width up to 12 qubits)
 int tile_pass_blocks_per_sm(int S, size_t smem);
 cudaError_t launch_tile_pass(int S, int grid, size_t smem, const PassArgs& P, cudaStream_t st);
-// register-resident kernel with TMA prefetch (tile width exactly 12 qubits)
-int sweep_reg_bits(int S);
-int sweep_blocks_per_sm(int S, int RB, size_t smem);
-size_t sweep_smem_bytes(int S, int RB, int prog_words, int n_events);
-cudaError_t launch_sweep(int S, int RB, int grid, const PassArgs& P, cudaStream_t st);
-cudaError_t launch_bounded_wait_probe(int* status, cudaStream_t st);
-// the passes of many circuits in one launch: unit u runs on blocks
-// [cta_begin[u], cta_begin[u+1]) (device arrays); all units share S and RB
-cudaError_t launch_sweep_batched(int S, int RB, const PassArgs* units, const int* cta_begin, int n_units,
-                                 int total_ctas, size_t smem, cudaStream_t st);
 // reductions, finishers, fills
 cudaError_t launch_reduce2x2(const float2* phi, const float2* chi, int n, int q, double* partials, int grid,
                              cudaStream_t st);
-cudaError_t launch_finish(const double* partials, int grid, const FinishDesc* desc, const double* kmats,
-                          double* vals, int n_red, cudaStream_t st);
+cudaError_t launch_finish(const double* partials, const FinishSlot* slots, const double* kmats, double* vals,
+                          int n_slots, cudaStream_t st);
+int finish_blocks(int n_slots);
 cudaError_t launch_partials_sum(const double* part, int grid, double* R, cudaStream_t st);
 cudaError_t launch_normalize(float2* v, long long dim, const double* partials, int red_grid, int grid,
                              cudaStream_t st);

@@ -1,0 +1,99 @@
+// Programs of the unit sweep kernel (kernels_units.cu): the operations of one
+// pass, assembled on the host for one 12-qubit tile of one state.
+//
+// A program is an array of 16-byte words: a header, the phases, one record
+// per operation, then the matrices.  The assembler (unit_program.cpp) decides
+// everything that does not depend on the tile: which diagonal factors are
+// pending at each operation, where they have to be multiplied into the
+// amplitudes, and which constants fold into a matrix.  The kernel keeps no
+// flags of its own.
+#pragma once
+
+#include <cstdint>
+#include <vector>
+
+#include "sweep_types.h"
+
+namespace nqs {
+
+constexpr int kUnitRB = 4;                      // register qubits: 16 amplitudes per thread
+constexpr int kUnitThreads = 1 << (kMaxTileQ - kUnitRB);
+constexpr int kUnitSlots = 8;                   // checkpoint pointers of a pass (reductions, saves)
+constexpr int kNoLoc = 31;                      // location of an absent bit (always 0)
+
+// Operation codes; a code in a family of four is FAMILY + register bit.
+enum UnitOp : int {
+    UO_G1 = 0,      // dense one-qubit matrix
+    UO_G1H = 4,     // the same, taking the pending ratio of its register bit
+    UO_FLB = 8,     // multiply the pending ratio of one register bit into the amplitudes
+    UO_HP = 12,     // scalar *= m[2c], ratio *= m[2c + 1], c = the bit at location a
+    UO_HR = 16,     // ratio *= m[c]
+    UO_SITE = 20,   // noise site
+    UO_SC = 24,     // scalar *= m[c], c = the bits at locations a, b
+    UO_FLS = 25,    // multiply the pending scalar into the amplitudes
+    UO_FLA = 26,    // multiply the scalar and all four ratios into the amplitudes
+    UO_DD = 27,     // + pair index: amplitudes with both register bits *= m[0]
+    UO_G2 = 33,     // + pair index: dense two-qubit matrix, index 2 * b(low) + b(high)
+    UO_DP = 39,     // amplitudes *= m[2c + bit b of r]
+    UO_DG = 40      // amplitudes *= m[2 * bit a of r + bit b of r]
+};
+
+// pairs of register bits (i < j) in the order 01 02 03 12 13 23
+inline int unit_pair(int i, int j) { return i == 0 ? j - 1 : i == 1 ? j + 1 : 5; }
+
+struct UnitRec {               // 16 bytes
+    unsigned char code, a, b, flags;
+    unsigned char ev, nspawn, sp, pad0;   // reduction / checkpoint slot, spawned factors, spawn slot
+    unsigned short mat, site;
+    unsigned int pad;
+};
+
+struct UnitPhase {             // 96 bytes
+    unsigned short lane_j[32]; // tile index bits of a lane
+    unsigned short warp_j[8];  // tile index bits of a warp
+    unsigned short reg_j[4];   // tile index bit of each register bit
+    unsigned short op_begin, op_end;
+    unsigned short pad[2];
+};
+
+struct UnitHeader {            // 64 bytes
+    unsigned int n_phases, n_ops, ops_word, mats_word;
+    unsigned long long nl_mask;             // qubits outside the tile
+    unsigned int n_events, words;
+    unsigned char local[12];                // tile qubits, ascending
+    unsigned char n_slots, pad[3];
+    unsigned short slot_site[kUnitSlots];   // site of each checkpoint slot (bit 15: forward table)
+};
+
+struct UnitProgram {
+    int word = 0, words = 0, n_phases = 0, n_events = 0;
+};
+
+// Assemble dops[off .. off + n) (execution order) on the tile qubits `local`
+// of an n_qubits-wide state, appending to `out`; mats is the float2 table the
+// operations index.
+UnitProgram assemble_unit(const std::vector<DevOp>& dops, int off, int n, const int* local, int n_qubits,
+                          const std::vector<float2>& mats, std::vector<uint4>& out);
+
+// One state swept through one pass: `ctas` consecutive blocks share its tiles.
+struct SweepUnit {
+    const float2* in;
+    float2* out;
+    float2* spawn;             // spawned state (slot k, factor i) at spawn + ((3 k + i) << n)
+    const uint4* prog;
+    float2* const* ckpt;       // phi_s
+    float2* const* ckpt_fwd;   // chi_s
+    double* partials;          // [event][cta][8]
+    int* err;
+    int n_tiles, n, cta_begin, ctas;
+};
+
+size_t unit_smem_bytes(int max_words, int max_events);
+int unit_blocks_per_sm(size_t smem);
+// blk: unit of every block, or null when every unit has `ctas` blocks
+cudaError_t launch_units(const SweepUnit* units, const int* blk, int ctas, int total_ctas, size_t smem,
+                         cudaStream_t st);
+// Blocks per unit of a launch of n_units units of n_tiles tiles each.
+int unit_ctas(int n_units, long long n_tiles, int slots);
+
+}  // namespace nqs
