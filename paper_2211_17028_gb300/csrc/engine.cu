@@ -1348,7 +1348,7 @@ int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* 
 }
 
 static int launch_pass(const Engine& E, const Launch& l, cudaStream_t st) {
-    if (l.units()) return cuda_err(launch_units(E.units_dev + l.unit_off, nullptr, l.ctas, l.grid, l.smem, st));
+    if (l.units()) return cuda_err(launch_units(l.S == 1, E.units_dev + l.unit_off, nullptr, l.ctas, l.grid, l.smem, st));
     if (l.jit) return cuda_err(jit_launch(*l.jit, l.grid, l.args, st));
     return cuda_err(launch_tile_pass(l.S, l.grid, l.smem, l.args, st));
 }

@@ -85,26 +85,38 @@ bool op_is_diag(const HostOp& o) { return o.type == OP_D1 || o.type == OP_D2; }
 // are both diagonal; a noise site commutes with nothing on its qubit (the
 // branch states it spawns and the reduction it makes see the state at its
 // place) and sites keep their relative order.  Returns the count taken.
-int take_pass(const Plan& p, const std::vector<int>& rest, const std::vector<char>& tile, int max_sites, int max_ops,
+struct OpMask {
+    uint64_t q = 0;      // its qubits
+    bool diag = false, site = false;
+};
+
+std::vector<OpMask> op_masks(const Plan& p) {
+    std::vector<OpMask> m(p.ops.size());
+    for (size_t i = 0; i < m.size(); ++i) {
+        const HostOp& o = p.ops[i];
+        m[i].q = (1ull << o.q0) | (o.q1 >= 0 ? 1ull << o.q1 : 0ull);
+        m[i].diag = op_is_diag(o);
+        m[i].site = o.type == OP_SITE;
+    }
+    return m;
+}
+
+int take_pass(const std::vector<OpMask>& ops, const std::vector<int>& rest, uint64_t tile, int max_sites, int max_ops,
               std::vector<int>* taken, std::vector<int>* kept) {
-    std::vector<char> blk_diag(p.n, 0), blk_any(p.n, 0);
+    uint64_t blk_diag = 0, blk_any = 0;   // qubits of the diagonal / other operations skipped
     bool site_skipped = false;
     int sites = 0, cnt = 0;
     for (int idx : rest) {
-        const HostOp& o = p.ops[idx];
-        const int qs[2] = {o.q0, o.q1};
-        const int nq = o.q1 >= 0 ? 2 : 1;
-        const bool d = op_is_diag(o), site = o.type == OP_SITE;
-        bool ok = !(site && site_skipped) && cnt < max_ops && !(site && sites >= max_sites);
-        for (int j = 0; j < nq && ok; ++j)
-            if (blk_any[qs[j]] || (!d && blk_diag[qs[j]]) || (!d && !tile[qs[j]])) ok = false;
+        const OpMask& o = ops[idx];
+        const bool ok = cnt < max_ops && !(o.site && (site_skipped || sites >= max_sites)) && !(o.q & blk_any) &&
+                        (o.diag || !(o.q & (blk_diag | ~tile)));
         if (ok) {
-            sites += site;
+            sites += o.site;
             ++cnt;
             if (taken) taken->push_back(idx);
         } else {
-            for (int j = 0; j < nq; ++j) (d ? blk_diag : blk_any)[qs[j]] = 1;
-            site_skipped = site_skipped || site;
+            (o.diag ? blk_diag : blk_any) |= o.q;
+            site_skipped = site_skipped || o.site;
             if (kept) kept->push_back(idx);
         }
     }
@@ -125,52 +137,35 @@ void lookahead_order(Plan& p, int max_sites, int max_ops, std::vector<PassSpec>&
     std::vector<int> rest(nops), order;
     for (int i = 0; i < nops; ++i) rest[i] = i;
     order.reserve(nops);
+    const std::vector<OpMask> masks = op_masks(p);
     while (!rest.empty()) {
-        std::vector<char> tile(p.n, 0);
-        int count = 0;
-        auto add = [&](int q) {
-            if (q >= 0 && !tile[q]) {
-                tile[q] = 1;
-                ++count;
-            }
-        };
-        for (int q = 0; q < p.c; ++q) add(q);
-        const HostOp& first = p.ops[rest[0]];
-        if (!op_is_diag(first)) {
-            add(first.q0);
-            add(first.q1);
-        }
+        uint64_t tile = (1ull << p.c) - 1;
+        if (!masks[rest[0]].diag) tile |= masks[rest[0]].q;
         // candidates: dense qubits of the operations near the front
-        std::vector<char> cand(p.n, 0);
-        for (size_t i = 0; i < rest.size() && i < 512; ++i) {
-            const HostOp& o = p.ops[rest[i]];
-            if (op_is_diag(o)) continue;
-            cand[o.q0] = 1;
-            if (o.q1 >= 0) cand[o.q1] = 1;
-        }
-        while (count < p.k) {
-            int best = -1, best_v = -1;
-            for (int q = 0; q < p.n; ++q) {
-                if (tile[q] || !cand[q]) continue;
-                tile[q] = 1;
-                const int v = take_pass(p, rest, tile, max_sites, max_ops, nullptr, nullptr);
-                tile[q] = 0;
+        uint64_t cand = 0;
+        for (size_t i = 0; i < rest.size() && i < 512; ++i)
+            if (!masks[rest[i]].diag) cand |= masks[rest[i]].q;
+        while (__builtin_popcountll(tile) < p.k && (cand & ~tile)) {
+            uint64_t best = 0;
+            int best_v = -1;
+            for (uint64_t left = cand & ~tile; left; left &= left - 1) {
+                const uint64_t q = left & (~left + 1);
+                const int v = take_pass(masks, rest, tile | q, max_sites, max_ops, nullptr, nullptr);
                 if (v > best_v) {
                     best_v = v;
                     best = q;
                 }
             }
-            if (best < 0) break;
-            add(best);
+            tile |= best;
         }
         std::vector<int> keep;
         PassSpec ps;
         ps.op_begin = (int)order.size();
-        take_pass(p, rest, tile, max_sites, max_ops, &order, &keep);
+        take_pass(masks, rest, tile, max_sites, max_ops, &order, &keep);
         ps.op_end = (int)order.size();
-        for (int q = 0; q < p.n && count < p.k; ++q) add(q);
+        for (int q = 0; q < p.n && __builtin_popcountll(tile) < p.k; ++q) tile |= 1ull << q;
         for (int q = 0; q < p.n; ++q)
-            if (tile[q]) ps.local.push_back(q);
+            if (tile >> q & 1) ps.local.push_back(q);
         passes.push_back(ps);
         rest.swap(keep);
     }

@@ -43,36 +43,124 @@ __device__ __forceinline__ int relay_map(int j) { return j + (j >> 4) + (j >> 8)
 __device__ __forceinline__ int stage_map(int j) { return j + 2 * (j >> 5) + 2 * (j >> 9); }
 constexpr int kRelayAmps = kAmps + (kAmps >> 4) + (kAmps >> 8);
 constexpr int kStageAmps = kAmps + 2 * (kAmps >> 5) + 2 * (kAmps >> 9);
-constexpr size_t kFixedSmem = ((size_t)kStageAmps + 2 * kRelayAmps) * sizeof(float2);
+constexpr int kRelayBufs = 2;
+constexpr int kBlocksPerSm = 2;
+constexpr size_t kFixedSmem = ((size_t)kStageAmps + kRelayBufs * kRelayAmps) * sizeof(float2);
 
-template <int I>
-__device__ __forceinline__ void u_g1(float2 (&x)[kE], float2 m0, float2 m1, float2 m2, float2 m3) {
-    const float2 p0 = make_float2(m0.x, m0.x), q0 = make_float2(-m0.y, m0.y);
-    const float2 p1 = make_float2(m1.x, m1.x), q1 = make_float2(-m1.y, m1.y);
-    const float2 p2 = make_float2(m2.x, m2.x), q2 = make_float2(-m2.y, m2.y);
-    const float2 p3 = make_float2(m3.x, m3.x), q3 = make_float2(-m3.y, m3.y);
+// An amplitude is one 64-bit register pair (re in the low word) and every
+// product on it a packed FP32x2 operation written as such: kept as two floats,
+// every operation moved its sixteen amplitudes between register pairs (half of
+// all instructions issued, 7470 per warp and tile of 27 gates).
+typedef unsigned long long c64;
+
+__device__ __forceinline__ c64 pk(float lo, float hi) {
+    c64 v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
+    return v;
+}
+__device__ __forceinline__ float2 unpk(c64 v) {
+    float2 f;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(v));
+    return f;
+}
+__device__ __forceinline__ c64 swp(c64 v) {
+    const float2 f = unpk(v);
+    return pk(f.y, f.x);
+}
+__device__ __forceinline__ c64 mul2(c64 a, c64 b) {
+    c64 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ c64 fma2(c64 a, c64 b, c64 c) {
+    c64 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+// A complex factor m as the two packed operands of a product:
+//   m a = (m.x, m.x) * (a.x, a.y) + (-m.y, m.y) * (a.y, a.x)
+struct Fac {
+    c64 p, q;
+};
+__device__ __forceinline__ Fac fac(float2 m) { return Fac{pk(m.x, m.x), pk(-m.y, m.y)}; }
+// (the products in the order of cmul and cfma)
+__device__ __forceinline__ c64 mulc(Fac m, c64 a) { return fma2(m.p, a, mul2(m.q, swp(a))); }
+__device__ __forceinline__ c64 fmac(Fac m, c64 a, c64 acc) { return fma2(m.p, a, fma2(m.q, swp(a), acc)); }
+// m times f
+__device__ __forceinline__ Fac times(Fac m, float2 f) {
+    return fac(cmul(make_float2(unpk(m.p).x, unpk(m.q).y), f));
+}
+__device__ __forceinline__ Fac times_real(Fac m, float f) { return Fac{mul2(pk(f, f), m.p), mul2(pk(f, f), m.q)}; }
+__device__ __forceinline__ Fac ld_fac(const float2* m) {
+    const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(m);
+    return Fac{v.x, v.y};
+}
+
+// y0 = m0 a + m1 b, y1 = m2 a + m3 b on register bit I.  A state swept alone
+// adds the products as cfma(m0, a, cmul(m1, b)), the states of a branch group
+// in the order (m0 a, m1 b): both orders are kept, so results do not depend on
+// which kernel sweeps them.
+template <int I, bool SINGLE>
+__device__ __forceinline__ void u_dense(c64 (&x)[kE], const Fac (&k)[4]) {
 #pragma unroll
     for (int r = 0; r < kE; ++r) {
         if (r & (1 << I)) continue;
-        const int r1 = r | (1 << I);
-        const float2 a = x[r], b = x[r1];
-        const float2 as = make_float2(a.y, a.x), bs = make_float2(b.y, b.x);
-        float2 y0 = __fmul2_rn(p0, a);
-        float2 y1 = __fmul2_rn(p2, a);
-        y0 = __ffma2_rn(q0, as, y0);
-        y1 = __ffma2_rn(q2, as, y1);
-        y0 = __ffma2_rn(p1, b, y0);
-        y1 = __ffma2_rn(p3, b, y1);
-        y0 = __ffma2_rn(q1, bs, y0);
-        y1 = __ffma2_rn(q3, bs, y1);
+        const c64 a = x[r], b = x[r | (1 << I)];
+        const c64 as = swp(a), bs = swp(b);
+        c64 y0, y1;
+        if (SINGLE) {
+            y1 = fma2(k[2].p, a, fma2(k[2].q, as, fma2(k[3].p, b, mul2(k[3].q, bs))));
+            y0 = fma2(k[0].p, a, fma2(k[0].q, as, fma2(k[1].p, b, mul2(k[1].q, bs))));
+        } else {
+            y1 = fma2(k[3].q, bs, fma2(k[3].p, b, fma2(k[2].q, as, mul2(k[2].p, a))));
+            y0 = fma2(k[1].q, bs, fma2(k[1].p, b, fma2(k[0].q, as, mul2(k[0].p, a))));
+        }
         x[r] = y0;
-        x[r1] = y1;
+        x[r | (1 << I)] = y1;
     }
+}
+
+// pending factors: a scalar and a pair per register bit
+struct Pend {
+    float2 d, h[kUnitRB][2];
+};
+
+// the dense gate of a record: its matrix with the pending factors it takes
+template <int I, bool SINGLE>
+__device__ __forceinline__ void u_gate(c64 (&x)[kE], const UnitRec& op, const float2* __restrict__ m, Pend& P,
+                                       uint32_t bits) {
+    Fac k[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) k[e] = ld_fac(m + 2 * e);
+    if (op.flags & UF_SCALAR) {
+        if (op.flags & UF_REAL) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) k[e] = times_real(k[e], P.d.x);
+        } else {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) k[e] = times(k[e], P.d);
+        }
+        P.d = make_float2(1.f, 0.f);
+    }
+    if (op.flags & UF_PAIR) {
+        k[0] = times(k[0], P.h[I][0]);
+        k[2] = times(k[2], P.h[I][0]);
+        k[1] = times(k[1], P.h[I][1]);
+        k[3] = times(k[3], P.h[I][1]);
+        P.h[I][0] = P.h[I][1] = make_float2(1.f, 0.f);
+    }
+    if (op.flags & UF_SIGN) {
+        const float f = (__popc(bits & op.mask) & 1) ? -1.f : 1.f;
+        k[1] = times_real(k[1], f);
+        k[3] = times_real(k[3], f);
+    }
+    u_dense<I, SINGLE>(x, k);
 }
 
 // A dense two-qubit gate reads its matrix anew for every quadruple: 32 held
 // entries next to the amplitudes would spill (these gates are rare: the
-// planner turns controlled gates into diagonals wherever it can).
+// planner turns controlled gates into diagonals wherever it can).  The pending
+// scalar, then the product of the pairs (first qubit's first), multiply each entry.
 __device__ __forceinline__ float2 lds_again(const float2* p) {
     float2 v;
     asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(smem_u32(p)));
@@ -80,90 +168,145 @@ __device__ __forceinline__ float2 lds_again(const float2* p) {
 }
 
 template <int I0, int I1>
-__device__ __forceinline__ void u_g2(float2 (&x)[kE], const float2* __restrict__ m) {
+__device__ __forceinline__ void u_g2(c64 (&x)[kE], const UnitRec& op, const float2* __restrict__ m, Pend& P) {
+    float2 f[4];
+    const bool pair = op.flags & UF_PAIR, scal = op.flags & UF_SCALAR;
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+        f[c] = op.a ? cmul(P.h[I1][c & 1], P.h[I0][c >> 1]) : cmul(P.h[I0][c >> 1], P.h[I1][c & 1]);
+    auto entry = [&](int q, int c) {
+        float2 e = lds_again(m + 4 * q + c);
+        if (scal) e = cmul(e, P.d);
+        if (pair) e = cmul(e, f[c]);
+        return fac(e);
+    };
 #pragma unroll
     for (int r = 0; r < kE; ++r) {
         if (r & ((1 << I0) | (1 << I1))) continue;
         const int idx[4] = {r, r | (1 << I1), r | (1 << I0), r | (1 << I0) | (1 << I1)};
-        float2 v[4];
+        c64 v[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) v[q] = x[idx[q]];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            float2 y = cmul(lds_again(m + 4 * q), v[0]);
-            y = cfma(lds_again(m + 4 * q + 1), v[1], y);
-            y = cfma(lds_again(m + 4 * q + 2), v[2], y);
-            y = cfma(lds_again(m + 4 * q + 3), v[3], y);
-            x[idx[q]] = y;
+            c64 y = mulc(entry(q, 0), v[0]);
+            if (op.a) {   // columns in the order of the gate's own qubits
+                y = fmac(entry(q, 2), v[2], y);
+                y = fmac(entry(q, 1), v[1], y);
+            } else {
+                y = fmac(entry(q, 1), v[1], y);
+                y = fmac(entry(q, 2), v[2], y);
+            }
+            x[idx[q]] = fmac(entry(q, 3), v[3], y);
         }
     }
+    P.d = make_float2(1.f, 0.f);
+    P.h[I0][0] = P.h[I0][1] = P.h[I1][0] = P.h[I1][1] = make_float2(1.f, 0.f);
+}
+
+// amplitudes *= f0 or f1 by register bit I
+template <int I>
+__device__ __forceinline__ void u_by_bit(c64 (&x)[kE], float2 f0, float2 f1) {
+    const Fac k0 = fac(f0), k1 = fac(f1);
+#pragma unroll
+    for (int r = 0; r < kE; ++r) x[r] = mulc((r >> I & 1) ? k1 : k0, x[r]);
 }
 
 template <int I>
-__device__ __forceinline__ void u_flush_bit(float2 (&x)[kE], float2 f) {
+__device__ __forceinline__ void u_flush_sign(c64 (&x)[kE], float h) {
+    const c64 f = pk(h, h);
 #pragma unroll
     for (int r = 0; r < kE; ++r)
-        if (r & (1 << I)) x[r] = cmul(f, x[r]);
+        if (r & (1 << I)) x[r] = mul2(f, x[r]);
 }
 
 template <int I0, int I1>
-__device__ __forceinline__ void u_both(float2 (&x)[kE], float2 f) {
+__device__ __forceinline__ void u_negate(c64 (&x)[kE]) {
 #pragma unroll
     for (int r = 0; r < kE; ++r)
-        if ((r >> I0 & 1) && (r >> I1 & 1)) x[r] = cmul(f, x[r]);
+        if ((r >> I0 & 1) && (r >> I1 & 1)) x[r] = mul2(pk(-1.f, -1.f), x[r]);
 }
 
-// layout of a phase: tile index bits of the thread and of each register bit
-struct Lay {
-    int jT, jR[kUnitRB];
-};
-
-__device__ __forceinline__ void load_lay(Lay& L, const UnitPhase& ph, int lane, int warp) {
-    L.jT = ph.lane_j[lane] | ph.warp_j[warp];
+template <int I0, int I1>
+__device__ __forceinline__ void u_diag2(c64 (&x)[kE], const float2* __restrict__ m) {
 #pragma unroll
-    for (int i = 0; i < kUnitRB; ++i) L.jR[i] = ph.reg_j[i];
+    for (int c = 0; c < 4; ++c) {
+        const Fac f = fac(m[c]);
+#pragma unroll
+        for (int r = 0; r < kE; ++r)
+            if (2 * (r >> I0 & 1) + (r >> I1 & 1) == c) x[r] = mulc(f, x[r]);
+    }
+}
+
+// tile index bits of the thread in a phase (those of the register bits are
+// read again where they are used: held, they would spill)
+__device__ __forceinline__ int thread_j(const UnitPhase& ph, int lane, int warp) {
+    return ph.lane_j[lane] | ph.warp_j[warp];
+}
+
+// the tile's registers to or from a buffer under an additive index map
+template <bool STORE, typename Map>
+__device__ __forceinline__ void move_tile(c64 (&x)[kE], float2* buf, const UnitPhase& ph, int jT, Map map) {
+    c64* const w = reinterpret_cast<c64*>(buf) + map(jT);
+    int o[kUnitRB];
+#pragma unroll
+    for (int i = 0; i < kUnitRB; ++i) o[i] = map(ph.reg_j[i]);
+#pragma unroll
+    for (int r = 0; r < kE; ++r) {
+        c64* const a =
+            w + (((r & 1) ? o[0] : 0) + ((r & 2) ? o[1] : 0) + ((r & 4) ? o[2] : 0) + ((r & 8) ? o[3] : 0));
+        if (STORE) *a = x[r];
+        else x[r] = *a;
+    }
 }
 
 __device__ __forceinline__ unsigned long long glob(const unsigned long long* hi_off, int j) {
     return hi_off[j >> 5] | (unsigned long long)(j & 31);
 }
 
+// Addresses of a thread's amplitudes in a state: sums over the register bits.
+struct Addr {
+    unsigned long long lo[4], hi[4];   // offsets of the bit pairs 0-1 and 2-3
+    __device__ __forceinline__ Addr(const unsigned long long* hi_off, const UnitPhase& ph, unsigned long long at) {
+        unsigned long long g[kUnitRB];
+#pragma unroll
+        for (int i = 0; i < kUnitRB; ++i) g[i] = glob(hi_off, ph.reg_j[i]);
+        lo[0] = 0;
+        lo[1] = g[0];
+        lo[2] = g[1];
+        lo[3] = g[0] + g[1];
+        hi[0] = at;
+        hi[1] = at + g[2];
+        hi[2] = at + g[3];
+        hi[3] = hi[1] + g[3];
+    }
+    __device__ __forceinline__ unsigned long long operator()(int r) const { return hi[r >> 2] + lo[r & 3]; }
+};
+
 template <int I>
-__device__ __forceinline__ void u_site(const UnitRec& op, const float2* __restrict__ m, float2 (&x)[kE],
-                                       const Lay& L, const SweepUnit& u, const unsigned long long* hi_off,
+__device__ __forceinline__ void u_site(const UnitRec& op, const float2* __restrict__ m, c64 (&x)[kE],
+                                       const UnitPhase& ph, int jT, const SweepUnit& u, const unsigned long long* hi_off,
                                        float2* const* slot, unsigned long long base, double* acc, int lane, int warp) {
     const int fl = op.flags;
     // the addresses are the same for every site of a phase; opaque here, or the
     // compiler computes all of them ahead of the operation loop and spills
-    int jT = L.jT;
     asm volatile("" : "+r"(jT));
-    const unsigned long long gT = base | glob(hi_off, jT);
-    unsigned long long gR[kUnitRB];
-#pragma unroll
-    for (int i = 0; i < kUnitRB; ++i) gR[i] = glob(hi_off, L.jR[i]);
-    auto off = [&](int r) {
-        unsigned long long g = gT;
-#pragma unroll
-        for (int i = 0; i < kUnitRB; ++i)
-            if (r & (1 << i)) g |= gR[i];
-        return g;
-    };
-    const float2 sc = m[0];
+    const Addr off(hi_off, ph, base | glob(hi_off, jT));
     if (fl & (FL_SAVE | FL_SAVE_FWD)) {
-        float2* const save = slot[op.ev];
+        c64* const save = reinterpret_cast<c64*>(slot[op.ev]);
 #pragma unroll
-        for (int r = 0; r < kE; ++r) __stcs(save + off(r), cmul(sc, x[r]));   // sc = 1 leaves them as they are
+        for (int r = 0; r < kE; ++r) __stcs(save + off(r), x[r]);
     }
     if (fl & FL_REDUCE) {
         // conj(f) a accumulated as A += f.x a, B += f.y a (no swapped operands):
         // conj(f) a = (A.x + B.y, A.y - B.x)
-        const float2* const phi = slot[op.ev];
-        float2 A[4], B[4];
+        const c64* const phi = reinterpret_cast<const c64*>(slot[op.ev]);
+        c64 A[4], B[4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) A[e] = B[e] = make_float2(0.f, 0.f);
+        for (int e = 0; e < 4; ++e) A[e] = B[e] = pk(0.f, 0.f);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {   // phi in two halves of eight loads in flight
-            float2 f[kE / 2];
+            c64 f[kE / 2];
             int k = 0;
 #pragma unroll
             for (int r = 0; r < kE; ++r) {
@@ -177,26 +320,26 @@ __device__ __forceinline__ void u_site(const UnitRec& op, const float2* __restri
             for (int r = 0; r < kE; ++r) {
                 if (r & (1 << I)) continue;
                 if (((r >> (I == 3 ? 2 : 3)) & 1) != h) continue;
-                const float2 f0 = f[k++], f1 = f[k++];
-                const float2 a = x[r], b = x[r | (1 << I)];
-                const float2 f0x = make_float2(f0.x, f0.x), f0y = make_float2(f0.y, f0.y);
-                const float2 f1x = make_float2(f1.x, f1.x), f1y = make_float2(f1.y, f1.y);
-                A[0] = __ffma2_rn(f0x, a, A[0]);
-                B[0] = __ffma2_rn(f0y, a, B[0]);
-                A[1] = __ffma2_rn(f0x, b, A[1]);
-                B[1] = __ffma2_rn(f0y, b, B[1]);
-                A[2] = __ffma2_rn(f1x, a, A[2]);
-                B[2] = __ffma2_rn(f1y, a, B[2]);
-                A[3] = __ffma2_rn(f1x, b, A[3]);
-                B[3] = __ffma2_rn(f1y, b, B[3]);
+                const float2 f0 = unpk(f[k]), f1 = unpk(f[k + 1]);
+                k += 2;
+                const c64 a = x[r], b = x[r | (1 << I)];
+                const c64 f0x = pk(f0.x, f0.x), f0y = pk(f0.y, f0.y), f1x = pk(f1.x, f1.x), f1y = pk(f1.y, f1.y);
+                A[0] = fma2(f0x, a, A[0]);
+                B[0] = fma2(f0y, a, B[0]);
+                A[1] = fma2(f0x, b, A[1]);
+                B[1] = fma2(f0y, b, B[1]);
+                A[2] = fma2(f1x, a, A[2]);
+                B[2] = fma2(f1y, a, B[2]);
+                A[3] = fma2(f1x, b, A[3]);
+                B[3] = fma2(f1y, b, B[3]);
             }
         }
         float v[8];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            const float2 R = cmul(sc, make_float2(A[e].x + B[e].y, A[e].y - B[e].x));
-            v[2 * e] = R.x;
-            v[2 * e + 1] = R.y;
+            const float2 a = unpk(A[e]), b = unpk(B[e]);
+            v[2 * e] = a.x + b.y;
+            v[2 * e + 1] = a.y - b.x;
         }
         // reduce-scatter over the warp: steps 16, 8, 4 halve the components a
         // lane keeps, steps 2, 1 complete the sum
@@ -220,21 +363,23 @@ __device__ __forceinline__ void u_site(const UnitRec& op, const float2* __restri
     if (fl & FL_SPAWN) {
 #pragma unroll 1
         for (int i = 0; i < op.nspawn; ++i) {
-            const float2* K = m + 2 + 4 * i;
-            const float2 k0 = K[0], k1 = K[1], k2 = K[2], k3 = K[3];
-            float2* const dst = u.spawn + ((size_t)(3 * op.sp + i) << u.n);
+            Fac K[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) K[e] = fac(m[4 * i + e]);
+            c64* const dst = reinterpret_cast<c64*>(u.spawn) + ((size_t)(3 * op.sp + i) << u.n);
 #pragma unroll
             for (int r = 0; r < kE; ++r) {
                 if (r & (1 << I)) continue;
-                const float2 a = x[r], b = x[r | (1 << I)];
-                __stcs(dst + off(r), cfma(k0, a, cmul(k1, b)));
-                __stcs(dst + off(r | (1 << I)), cfma(k2, a, cmul(k3, b)));
+                const c64 a = x[r], b = x[r | (1 << I)];
+                __stcs(dst + off(r), fmac(K[0], a, mulc(K[1], b)));
+                __stcs(dst + off(r | (1 << I)), fmac(K[2], a, mulc(K[3], b)));
             }
         }
     }
 }
 
-__global__ void __launch_bounds__(kNT, 2) unit_sweep_kernel(const SweepUnit* __restrict__ units,
+template <bool SINGLE>
+__global__ void __launch_bounds__(kNT, kBlocksPerSm) unit_sweep_kernel(const SweepUnit* __restrict__ units,
                                                             const int* __restrict__ blk, int ctas) {
     extern __shared__ __align__(128) unsigned char dyn[];
     float2* const stage = reinterpret_cast<float2*>(dyn);
@@ -243,6 +388,7 @@ __global__ void __launch_bounds__(kNT, 2) unit_sweep_kernel(const SweepUnit* __r
     __shared__ __align__(8) uint64_t bar;
     __shared__ unsigned long long hi_off[kChunks];
     __shared__ float2* slot[kUnitSlots];
+    __shared__ unsigned long long next_base;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int ui = blk ? blk[blockIdx.x] : (int)blockIdx.x / ctas;
@@ -304,67 +450,49 @@ __global__ void __launch_bounds__(kNT, 2) unit_sweep_kernel(const SweepUnit* __r
     };
 
     int t = cta;
-    unsigned long long base_next = tile_base(t);
-    if (t < n_tiles) prefetch(base_next);
+    if (t < n_tiles) {
+        const unsigned long long b = tile_base(t);
+        if (tid == 0) next_base = b;
+        prefetch(b);
+    }
     uint32_t parity = 0;
     bool failed = false;
-    float2 x[kE];
+    c64 x[kE];
     int buf = 0;   // re-layout buffer to write next
 
     for (; t < n_tiles; t += nctas) {
-        const unsigned long long base = base_next;
         const uint32_t bits = (uint32_t)tid | ((uint32_t)t << 8);
         const bool ok = mbar_wait_bounded(&bar, parity);
         if (__syncthreads_or(!ok)) {
             failed = true;
             break;
         }
+        const unsigned long long base = next_base;
         parity ^= 1u;
-        Lay L;
-        load_lay(L, phases[0], lane, warp);
-        {
-            const float2* const p = stage + stage_map(L.jT);
-            int o[kUnitRB];
-#pragma unroll
-            for (int i = 0; i < kUnitRB; ++i) o[i] = stage_map(L.jR[i]);
-#pragma unroll
-            for (int r = 0; r < kE; ++r)
-                x[r] = p[((r & 1) ? o[0] : 0) + ((r & 2) ? o[1] : 0) + ((r & 4) ? o[2] : 0) + ((r & 8) ? o[3] : 0)];
-        }
+        int jT = thread_j(phases[0], lane, warp);
+        move_tile<false>(x, stage, phases[0], jT, stage_map);
         __syncthreads();   // the staging buffer is free again
         if (t + nctas < n_tiles) {
-            base_next = tile_base(t + nctas);
-            prefetch(base_next);
+            const unsigned long long b = tile_base(t + nctas);
+            if (tid == 0) next_base = b;
+            prefetch(b);
         }
-        // pending diagonal: a scalar and a ratio per register bit
         const float2 unit1 = make_float2(1.f, 0.f);
-        float2 dsc = unit1, h0 = unit1, h1 = unit1, h2 = unit1, h3 = unit1;
+        Pend P;
+        P.d = unit1;
+#pragma unroll
+        for (int i = 0; i < kUnitRB; ++i) P.h[i][0] = P.h[i][1] = unit1;
 
 #pragma unroll 1
         for (int p = 0; p < n_phases; ++p) {
             if (p > 0) {
                 float2* const tb = relay + buf * kRelayAmps;
-                buf ^= 1;
-                {
-                    float2* const w = tb + relay_map(L.jT);
-                    int o[kUnitRB];
-#pragma unroll
-                    for (int i = 0; i < kUnitRB; ++i) o[i] = relay_map(L.jR[i]);
-#pragma unroll
-                    for (int r = 0; r < kE; ++r)
-                        w[((r & 1) ? o[0] : 0) + ((r & 2) ? o[1] : 0) + ((r & 4) ? o[2] : 0) + ((r & 8) ? o[3] : 0)] = x[r];
-                }
+                if (kRelayBufs == 2) buf ^= 1;
+                move_tile<true>(x, tb, phases[p - 1], jT, relay_map);
                 __syncthreads();
-                load_lay(L, phases[p], lane, warp);
-                {
-                    const float2* const w = tb + relay_map(L.jT);
-                    int o[kUnitRB];
-#pragma unroll
-                    for (int i = 0; i < kUnitRB; ++i) o[i] = relay_map(L.jR[i]);
-#pragma unroll
-                    for (int r = 0; r < kE; ++r)
-                        x[r] = w[((r & 1) ? o[0] : 0) + ((r & 2) ? o[1] : 0) + ((r & 4) ? o[2] : 0) + ((r & 8) ? o[3] : 0)];
-                }
+                jT = thread_j(phases[p], lane, warp);
+                move_tile<false>(x, tb, phases[p], jT, relay_map);
+                if (kRelayBufs == 1) __syncthreads();
             }
             const int oe = phases[p].op_end;
 #pragma unroll 1
@@ -372,117 +500,69 @@ __global__ void __launch_bounds__(kNT, 2) unit_sweep_kernel(const SweepUnit* __r
                 const UnitRec op = ops[o];
                 const float2* const m = mats + op.mat;
                 const int c = (bits >> op.a) & 1;
-                // one branch per family, the common ones first
-                const int code = op.code;
-                if (code < UO_FLB) {
-                    float2 m0 = m[0], m1 = m[1], m2 = m[2], m3 = m[3];
-                    const int i = code & 3;
-                    if (code >= UO_G1H) {
-                        const float2 h = i == 0 ? h0 : i == 1 ? h1 : i == 2 ? h2 : h3;
-                        m1 = cmul(m1, h);
-                        m3 = cmul(m3, h);
-                        if (i == 0) h0 = unit1;
-                        else if (i == 1) h1 = unit1;
-                        else if (i == 2) h2 = unit1;
-                        else h3 = unit1;
-                    }
-                    if (i == 0) u_g1<0>(x, m0, m1, m2, m3);
-                    else if (i == 1) u_g1<1>(x, m0, m1, m2, m3);
-                    else if (i == 2) u_g1<2>(x, m0, m1, m2, m3);
-                    else u_g1<3>(x, m0, m1, m2, m3);
-                } else if (code < UO_HP) {
-                    if (code == UO_FLB) {
-                        u_flush_bit<0>(x, h0);
-                        h0 = unit1;
-                    } else if (code == UO_FLB + 1) {
-                        u_flush_bit<1>(x, h1);
-                        h1 = unit1;
-                    } else if (code == UO_FLB + 2) {
-                        u_flush_bit<2>(x, h2);
-                        h2 = unit1;
-                    } else {
-                        u_flush_bit<3>(x, h3);
-                        h3 = unit1;
-                    }
-                } else if (code < UO_SITE) {
-                    float2 f;
-                    if (code < UO_HR) {
-                        const float4 q = *reinterpret_cast<const float4*>(m + 2 * c);
-                        dsc = cmul(make_float2(q.x, q.y), dsc);
-                        f = make_float2(q.z, q.w);
-                    } else {
-                        f = m[c];
-                    }
-                    const int i = code & 3;
-                    if (i == 0) h0 = cmul(f, h0);
-                    else if (i == 1) h1 = cmul(f, h1);
-                    else if (i == 2) h2 = cmul(f, h2);
-                    else h3 = cmul(f, h3);
-                } else if (code < UO_SC) {
-                    if (code == UO_SITE) u_site<0>(op, m, x, L, u, hi_off, slot, base, acc, lane, warp);
-                    else if (code == UO_SITE + 1) u_site<1>(op, m, x, L, u, hi_off, slot, base, acc, lane, warp);
-                    else if (code == UO_SITE + 2) u_site<2>(op, m, x, L, u, hi_off, slot, base, acc, lane, warp);
-                    else u_site<3>(op, m, x, L, u, hi_off, slot, base, acc, lane, warp);
-                } else if (code == UO_SC) {
-                    dsc = cmul(m[c + 2 * ((bits >> op.b) & 1)], dsc);
-                } else if (code == UO_FLS) {
+#define U_COMMA ,
+#define U_FOUR(F, BODY)                                  \
+    case F + 0: { constexpr int I = 0; BODY; break; }    \
+    case F + 1: { constexpr int I = 1; BODY; break; }    \
+    case F + 2: { constexpr int I = 2; BODY; break; }    \
+    case F + 3: { constexpr int I = 3; BODY; break; }
+#define U_PAIRS(F, BODY)                                      \
+    case F + 0: { constexpr int I = 0, J = 1; BODY; break; }  \
+    case F + 1: { constexpr int I = 0, J = 2; BODY; break; }  \
+    case F + 2: { constexpr int I = 0, J = 3; BODY; break; }  \
+    case F + 3: { constexpr int I = 1, J = 2; BODY; break; }  \
+    case F + 4: { constexpr int I = 1, J = 3; BODY; break; }  \
+    case F + 5: { constexpr int I = 2, J = 3; BODY; break; }
+                switch (op.code) {
+                    U_FOUR(UO_G1, (u_gate<I, SINGLE>(x, op, m, P, bits)))
+                    U_FOUR(UO_GK, const Fac k[4] = {ld_fac(m) U_COMMA ld_fac(m + 2) U_COMMA ld_fac(m + 4) U_COMMA ld_fac(m + 6)};
+                           (u_dense<I, true>(x, k)))
+                    U_FOUR(UO_KD, u_by_bit<I>(x, m[0], m[1]))
+                    U_FOUR(UO_FLB, u_by_bit<I>(x, cmul(P.d, P.h[I][0]), cmul(P.d, P.h[I][1]));
+                           P.d = P.h[I][0] = P.h[I][1] = unit1)
+                    U_FOUR(UO_FLR, u_flush_sign<I>(x, (__popc(bits & op.mask) & 1) ? -1.f : 1.f))
+                    U_FOUR(UO_HP, P.h[I][0] = cmul(P.h[I][0], m[2 * c]); P.h[I][1] = cmul(P.h[I][1], m[2 * c + 1]))
+                    U_FOUR(UO_SITE, u_site<I>(op, m, x, phases[p], jT, u, hi_off, slot, base, acc, lane, warp))
+                    U_PAIRS(UO_DN, (u_negate<I, J>(x)))
+                    U_PAIRS(UO_DG, (u_diag2<I, J>(x, m)))
+                    U_PAIRS(UO_G2, (u_g2<I, J>(x, op, m, P)))
+                    case UO_SC: P.d = cmul(P.d, m[c + 2 * ((bits >> op.b) & 1)]); break;
+                    case UO_FLS:
+                        if (op.flags & UF_REAL) {
 #pragma unroll
-                    for (int r = 0; r < kE; ++r) x[r] = cmul(dsc, x[r]);
-                    dsc = unit1;
-                } else if (code == UO_FLA) {
-                    float2 f[8];
-                    f[0] = dsc;
-                    f[1] = cmul(f[0], h0);
-                    f[2] = cmul(f[0], h1);
-                    f[3] = cmul(f[1], h1);
+                            for (int r = 0; r < kE; ++r) x[r] = mul2(pk(P.d.x, P.d.x), x[r]);
+                        } else {
+                            const Fac f = fac(P.d);
 #pragma unroll
-                    for (int r = 0; r < 4; ++r) f[4 + r] = cmul(f[r], h2);
+                            for (int r = 0; r < kE; ++r) x[r] = mulc(f, x[r]);
+                        }
+                        P.d = unit1;
+                        break;
+                    case UO_FLA:
 #pragma unroll
-                    for (int r = 0; r < 8; ++r) {
-                        x[r] = cmul(f[r], x[r]);
-                        f[r] = cmul(f[r], h3);
-                        x[8 + r] = cmul(f[r], x[8 + r]);
-                    }
-                    dsc = h0 = h1 = h2 = h3 = unit1;
-                } else if (code < UO_G2) {
-                    const float2 f = m[0];
-                    switch (code - UO_DD) {
-                        case 0: u_both<0, 1>(x, f); break;
-                        case 1: u_both<0, 2>(x, f); break;
-                        case 2: u_both<0, 3>(x, f); break;
-                        case 3: u_both<1, 2>(x, f); break;
-                        case 4: u_both<1, 3>(x, f); break;
-                        default: u_both<2, 3>(x, f); break;
-                    }
-                } else if (code < UO_DP) {
-                    switch (code - UO_G2) {
-                        case 0: u_g2<0, 1>(x, m); break;
-                        case 1: u_g2<0, 2>(x, m); break;
-                        case 2: u_g2<0, 3>(x, m); break;
-                        case 3: u_g2<1, 2>(x, m); break;
-                        case 4: u_g2<1, 3>(x, m); break;
-                        default: u_g2<2, 3>(x, m); break;
-                    }
-                } else if (code == UO_DP) {
+                        for (int g = 0; g < 4; ++g) {
+                            const float2 f2 = cmul(cmul(P.d, P.h[0][g & 1]), P.h[1][g >> 1]);
 #pragma unroll
-                    for (int r = 0; r < kE; ++r) x[r] = cmul(m[2 * c + ((r >> op.b) & 1)], x[r]);
-                } else {
+                            for (int h = 0; h < 4; ++h)
+                                x[g + 4 * h] = mulc(fac(cmul(cmul(f2, P.h[2][h & 1]), P.h[3][h >> 1])), x[g + 4 * h]);
+                        }
+                        P.d = unit1;
 #pragma unroll
-                    for (int r = 0; r < kE; ++r) x[r] = cmul(m[2 * ((r >> op.a) & 1) + ((r >> op.b) & 1)], x[r]);
+                        for (int i = 0; i < kUnitRB; ++i) P.h[i][0] = P.h[i][1] = unit1;
+                        break;
+                    default: break;
                 }
+#undef U_FOUR
+#undef U_PAIRS
+#undef U_COMMA
             }
         }
         // store the tile
         {
-            float2* const dst = u.out + (base | glob(hi_off, L.jT));
-            unsigned long long g[kUnitRB];
+            c64* const dst = reinterpret_cast<c64*>(u.out);
+            const Addr off(hi_off, phases[n_phases - 1], base | glob(hi_off, jT));
 #pragma unroll
-            for (int i = 0; i < kUnitRB; ++i) g[i] = glob(hi_off, L.jR[i]);
-#pragma unroll
-            for (int r = 0; r < kE; ++r)
-                __stcs(dst + ((r & 1) ? g[0] : 0ull) + ((r & 2) ? g[1] : 0ull) + ((r & 4) ? g[2] : 0ull) +
-                           ((r & 8) ? g[3] : 0ull),
-                       x[r]);
+            for (int r = 0; r < kE; ++r) __stcs(dst + off(r), x[r]);
         }
     }
 
@@ -523,17 +603,17 @@ size_t unit_smem_bytes(int max_words, int max_events) {
 
 int unit_blocks_per_sm(size_t smem) {
     int nb = 0;
-    cudaFuncSetAttribute(unit_sweep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, unit_sweep_kernel, kNT, smem);
+    cudaFuncSetAttribute(unit_sweep_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, unit_sweep_kernel<true>, kNT, smem);
     return nb > 0 ? nb : 1;
 }
 
-cudaError_t launch_units(const SweepUnit* units, const int* blk, int ctas, int total_ctas, size_t smem,
+cudaError_t launch_units(bool single, const SweepUnit* units, const int* blk, int ctas, int total_ctas, size_t smem,
                          cudaStream_t st) {
-    cudaError_t e =
-        cudaFuncSetAttribute(unit_sweep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    auto* const kernel = single ? unit_sweep_kernel<true> : unit_sweep_kernel<false>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    unit_sweep_kernel<<<total_ctas, kNT, smem, st>>>(units, blk, ctas);
+    kernel<<<total_ctas, kNT, smem, st>>>(units, blk, ctas);
     return cudaGetLastError();
 }
 

@@ -3,37 +3,46 @@
 
 #include <algorithm>
 #include <cmath>
-#include <complex>
 #include <cstring>
 
-#include "fp32_round.h"
 #include "nqs_internal.h"
 
 namespace nqs {
 
 namespace {
 
+// The arithmetic of every amplitude is fixed by the operation order alone: a
+// pending diagonal is a scalar and one pair of factors per register bit, a
+// gate takes the scalar and the pair of its bit into its matrix (scalar first),
+// sites and phase ends multiply what is left into the amplitudes.  Signs (CZ)
+// are exact whatever way they go, so they are kept as parities of thread and
+// tile bits and cost nothing until a gate or the end of the phase takes them.
 struct Assembler {
     const std::vector<float2>& tab;
     std::vector<UnitRec> recs;
     std::vector<float2> mats;
-    // pending diagonal of the current phase: constants known here, and flags of
-    // the factors the kernel holds (scalar; one ratio per register bit)
-    cd cs = 1.0, cp[4] = {1.0, 1.0, 1.0, 1.0};
-    bool rs = false, rh[4] = {false, false, false, false};
+    // what the kernel holds: scalar (and whether it is real), pairs; and signs
+    bool scal = false, scal_real = true;
+    bool pair[4] = {false, false, false, false};
+    uint32_t sign[4] = {0, 0, 0, 0};
 
     explicit Assembler(const std::vector<float2>& t) : tab(t) {}
 
-    cd m(int off) const { return cd(tab[off].x, tab[off].y); }
-    static bool one(cd c) {
-        const float2 f = round_c64(c);
-        return f.x == 1.f && f.y == 0.f;
-    }
-    int put(const std::vector<cd>& v) {   // matrix entries, 16-byte aligned
+    static bool is(float2 f, float re) { return f.x == re && f.y == 0.f; }
+    int put(const float2* v, int n) {   // matrices start on 16 bytes
         if (mats.size() & 1) mats.push_back(make_float2(0.f, 0.f));
         const int at = (int)mats.size();
-        for (cd c : v) mats.push_back(round_c64(c));
+        mats.insert(mats.end(), v, v + n);
         return at;
+    }
+    // a 2x2 matrix as the packed operands of the kernel: (re, re), (-im, im) per entry
+    int put_matrix(const float2* f) {
+        float2 v[8];
+        for (int e = 0; e < 4; ++e) {
+            v[2 * e] = make_float2(f[e].x, f[e].x);
+            v[2 * e + 1] = make_float2(-f[e].y, f[e].y);
+        }
+        return put(v, 8);
     }
     UnitRec& emit(int code, int a = kNoLoc, int b = kNoLoc) {
         UnitRec r{};
@@ -43,135 +52,116 @@ struct Assembler {
         recs.push_back(r);
         return recs.back();
     }
-    void ratio(int i, cd c) {   // ratio of bit i *= constant
-        const int at = put({c, c});
-        emit(UO_HR + i).mat = (unsigned short)at;
-        rh[i] = true;
+    void scalar(const float2* v, int n, int la, int lb) {   // by bit a + 2 * bit b
+        float2 w[4] = {v[0], v[1], n > 2 ? v[2] : v[0], n > 2 ? v[3] : v[1]};
+        const int at = put(w, 4);
+        emit(UO_SC, la, lb).mat = (unsigned short)at;
+        scal = true;
+        for (const float2& f : w) scal_real = scal_real && f.y == 0.f;
     }
-    void scalar_const(cd c) {
-        const int at = put({c, c});
-        emit(UO_SC).mat = (unsigned short)at;
-        rs = true;
-    }
-    // multiply everything pending into the amplitudes; keep_scalar leaves the
-    // constant scalar pending (the caller scales what it writes)
-    void flush(bool keep_scalar) {
-        for (int i = 0; i < 4; ++i)
-            if (!one(cp[i])) {
-                ratio(i, cp[i]);
-                cp[i] = 1.0;
-            }
-        int bits = 0;
-        for (int i = 0; i < 4; ++i) bits += rh[i];
-        if (!keep_scalar && !one(cs)) {
-            scalar_const(cs);
-            cs = 1.0;
-        }
-        // 8 products per ratio and 16 for the scalar one by one, 31 for all at once
-        if (8 * bits + 16 * (int)rs > 31) {
-            emit(UO_FLA);
-        } else {
-            for (int i = 0; i < 4; ++i)
-                if (rh[i]) emit(UO_FLB + i);
-            if (rs) emit(UO_FLS);
-        }
-        rs = false;
-        for (bool& r : rh) r = false;
-    }
-    void g1(int i, const cd* g) {
-        std::vector<cd> k = {g[0] * cs, g[1] * cs * cp[i], g[2] * cs, g[3] * cs * cp[i]};
-        if (mats.size() & 1) mats.push_back(make_float2(0.f, 0.f));
-        const int at = (int)mats.size();
-        float2 f[4];
-        if (cs == 1.0 && cp[i] == 1.0)
-            for (int e = 0; e < 4; ++e) f[e] = make_float2((float)g[e].real(), (float)g[e].imag());
-        else
-            round_matrix_c64(k.data(), 2, f);
-        mats.insert(mats.end(), f, f + 4);
-        cs = 1.0;
-        cp[i] = 1.0;
-        emit((rh[i] ? UO_G1H : UO_G1) + i).mat = (unsigned short)at;
-        rh[i] = false;
-    }
-    void g2(int i, int j, const cd* g) {   // first qubit on register bit i, second on j
-        for (int b : {i, j})
-            if (rh[b]) {
-                emit(UO_FLB + b);
-                rh[b] = false;
-            }
-        std::vector<cd> k(16);
-        for (int r = 0; r < 4; ++r)
-            for (int c = 0; c < 4; ++c)
-                k[4 * r + c] = g[4 * r + c] * cs * ((c & 2) ? cp[i] : cd(1.0)) * ((c & 1) ? cp[j] : cd(1.0));
-        if (i > j) {   // index by the lower register bit first
-            auto sw = [](int x) { return ((x & 1) << 1) | (x >> 1); };
-            std::vector<cd> t(16);
-            for (int r = 0; r < 4; ++r)
-                for (int c = 0; c < 4; ++c) t[4 * sw(r) + sw(c)] = k[4 * r + c];
-            k.swap(t);
-        }
-        float2 f[16];
-        round_matrix_c64(k.data(), 4, f);
-        if (mats.size() & 1) mats.push_back(make_float2(0.f, 0.f));
-        const int at = (int)mats.size();
-        mats.insert(mats.end(), f, f + 16);
-        cs = cp[i] = cp[j] = 1.0;
-        emit(UO_G2 + unit_pair(std::min(i, j), std::max(i, j))).mat = (unsigned short)at;
-    }
-    // a diagonal on register bit i whose two values depend on the bit at `loc`
-    void pair_op(int i, int loc, cd f00, cd f10, cd f01, cd f11) {   // f<bit i><bit loc>
-        if (f00 == 0.0 || f01 == 0.0) {
-            const int at = put({f00, f10, f01, f11});
-            emit(UO_DP, loc, i).mat = (unsigned short)at;
-        } else if (f00 == f01) {
-            cs *= f00;
-            const int at = put({f10 / f00, f11 / f01});
-            emit(UO_HR + i, loc).mat = (unsigned short)at;
-            rh[i] = true;
-        } else {
-            const int at = put({f00, f10 / f00, f01, f11 / f01});
-            emit(UO_HP + i, loc).mat = (unsigned short)at;
-            rh[i] = rs = true;
-        }
-    }
-    void d1(int la, const cd* g) {   // g[0], g[3]
-        if (la < kUnitRB) {
-            if (g[0] == 0.0) {
-                g1(la, g);
-            } else {
-                cs *= g[0];
-                cp[la] *= g[3] / g[0];
-            }
+    // pair of bit i *= (v0, v1) or (w0, w1) by the bit at loc
+    void pair_op(int i, int loc, float2 v0, float2 v1, float2 w0, float2 w1) {
+        if (!pair[i] && loc != kNoLoc && is(v0, 1.f) && is(v1, 1.f) && is(w0, 1.f) && is(w1, -1.f)) {
+            sign[i] ^= 1u << loc;
             return;
         }
-        const int at = put({g[0], g[3]});
-        emit(UO_SC, la - LOC_THREAD).mat = (unsigned short)at;
-        rs = true;
+        to_pair(i);
+        const float2 v[4] = {v0, v1, w0, w1};
+        const int at = put(v, 4);
+        emit(UO_HP + i, loc).mat = (unsigned short)at;
+        pair[i] = true;
     }
-    void d2(int la, int lb, const cd* d) {   // d[2 * bit a + bit b]
+    // the sign of bit i joins its pair
+    void to_pair(int i) {
+        const float2 one = make_float2(1.f, 0.f), neg = make_float2(-1.f, 0.f);
+        for (int l = 0; l < 31; ++l) {
+            if (!(sign[i] >> l & 1)) continue;
+            const float2 v[4] = {one, one, one, neg};
+            const int at = put(v, 4);
+            emit(UO_HP + i, l).mat = (unsigned short)at;
+            pair[i] = true;
+        }
+        sign[i] = 0;
+    }
+    // multiply everything pending into the amplitudes
+    void flush() {
+        int pairs = 0, which = 0;
+        for (int i = 0; i < 4; ++i)
+            if (pair[i]) {
+                ++pairs;
+                which = i;
+            }
+        if (pairs > 1) {
+            for (int i = 0; i < 4; ++i) to_pair(i);
+            emit(UO_FLA);
+        } else if (pairs == 1) {
+            to_pair(which);
+            emit(UO_FLB + which);
+        } else if (scal) {
+            emit(UO_FLS).flags = scal_real ? UF_REAL : 0;
+        }
+        for (int i = 0; i < 4; ++i) {
+            if (sign[i]) emit(UO_FLR + i).mask = sign[i];
+            pair[i] = false;
+            sign[i] = 0;
+        }
+        scal = false;
+        scal_real = true;
+    }
+    void g1(int i, const float2* m) {
+        const int at = put_matrix(m);
+        UnitRec& r = emit(UO_G1 + i);
+        r.mat = (unsigned short)at;
+        r.flags = (unsigned char)((pair[i] ? UF_PAIR : 0) | (sign[i] ? UF_SIGN : 0) | (scal ? UF_SCALAR : 0) |
+                                  (scal_real ? UF_REAL : 0));
+        r.mask = sign[i];
+        pair[i] = scal = false;
+        scal_real = true;
+        sign[i] = 0;
+    }
+    void g2(int i, int j, const float2* m) {   // first qubit on register bit i, second on j
+        // the scalar and the pairs of both bits go into the matrix on the device;
+        // stored with the lower bit first
+        to_pair(i);
+        to_pair(j);
+        float2 k[16];
+        auto sw = [](int x) { return ((x & 1) << 1) | (x >> 1); };
+        for (int r = 0; r < 4; ++r)
+            for (int c = 0; c < 4; ++c) (i < j ? k[4 * r + c] : k[4 * sw(r) + sw(c)]) = m[4 * r + c];
+        const int at = put(k, 16);
+        UnitRec& r = emit(UO_G2 + unit_pair(std::min(i, j), std::max(i, j)));
+        r.mat = (unsigned short)at;
+        r.flags = (unsigned char)((pair[i] || pair[j] ? UF_PAIR : 0) | (scal ? UF_SCALAR : 0));
+        r.a = (unsigned char)(i > j);   // the factors of the first qubit's bit come first
+        pair[i] = pair[j] = scal = false;
+        scal_real = true;
+    }
+    void d1(int la, const float2* m) {   // m[0], m[3]
+        if (la < kUnitRB) {
+            pair_op(la, kNoLoc, m[0], m[3], m[0], m[3]);
+        } else {
+            const float2 v[2] = {m[0], m[3]};
+            scalar(v, 2, la - LOC_THREAD, kNoLoc);
+        }
+    }
+    void d2(int la, int lb, const float2* m) {   // m[5 * (2 * bit a + bit b)]
+        const float2 d[4] = {m[0], m[5], m[10], m[15]};
         const bool ra = la < kUnitRB, rb = lb < kUnitRB;
         if (ra && rb) {
-            if (d[0] == 0.0 || d[1] == 0.0 || d[2] == 0.0) {
-                const int at = put({d[0], d[1], d[2], d[3]});
-                emit(UO_DG, la, lb).mat = (unsigned short)at;
+            if (is(d[0], 1.f) && is(d[1], 1.f) && is(d[2], 1.f) && is(d[3], -1.f)) {
+                emit(UO_DN + unit_pair(std::min(la, lb), std::max(la, lb)));
                 return;
             }
-            cs *= d[0];
-            cp[la] *= d[2] / d[0];
-            cp[lb] *= d[1] / d[0];
-            const cd k = d[3] * d[0] / (d[1] * d[2]);
-            if (!one(k)) {
-                const int at = put({k, k});
-                emit(UO_DD + unit_pair(std::min(la, lb), std::max(la, lb))).mat = (unsigned short)at;
-            }
+            const float2 v[4] = {d[0], la < lb ? d[1] : d[2], la < lb ? d[2] : d[1], d[3]};
+            const int at = put(v, 4);
+            emit(UO_DG + unit_pair(std::min(la, lb), std::max(la, lb))).mat = (unsigned short)at;
         } else if (ra) {
             pair_op(la, lb - LOC_THREAD, d[0], d[2], d[1], d[3]);
         } else if (rb) {
             pair_op(lb, la - LOC_THREAD, d[0], d[1], d[2], d[3]);
         } else {
-            const int at = put({d[0], d[2], d[1], d[3]});   // index bit a + 2 * bit b
-            emit(UO_SC, la - LOC_THREAD, lb - LOC_THREAD).mat = (unsigned short)at;
-            rs = true;
+            const float2 v[4] = {d[0], d[2], d[1], d[3]};
+            scalar(v, 4, la - LOC_THREAD, lb - LOC_THREAD);
         }
     }
 };
@@ -223,8 +213,6 @@ UnitProgram assemble_unit(const std::vector<DevOp>& dops, int off, int n, const 
 
     Assembler A(tab);
     std::vector<UnitPhase> phases;
-    cd carry[K];   // constant ratio pending on each tile position across phases
-    for (cd& c : carry) c = 1.0;
     for (size_t p = 0; p < ranges.size(); ++p) {
         std::vector<int> R = regs[p];
         bool used[K] = {};
@@ -266,39 +254,23 @@ UnitProgram assemble_unit(const std::vector<DevOp>& dops, int off, int n, const 
                 if (w >> i & 1) ph.warp_j[w] |= (unsigned short)(1 << T[5 + i]);
         ph.op_begin = (unsigned short)A.recs.size();
         auto at = [&](int pos, int q) { return pos >= 0 ? loc[pos] : LOC_THREAD + 8 + outer[q]; };
-        for (int i = 0; i < kUnitRB; ++i) A.cp[i] = carry[R[i]];
         for (int o = ranges[p].first; o < ranges[p].second; ++o) {
             const DevOp& d = dops[off + o];
-            cd g[16];
-            const int cnt = (d.type == OP_G2 || d.type == OP_D2) ? 16 : 4;
-            for (int e = 0; e < cnt; ++e) g[e] = A.m(d.mat + e);
+            const float2* m = tab.data() + d.mat;
             if (d.type == OP_G1) {
-                A.g1(loc[d.a], g);
+                A.g1(loc[d.a], m);
             } else if (d.type == OP_G2) {
-                A.g2(loc[d.a], loc[d.b], g);
+                A.g2(loc[d.a], loc[d.b], m);
             } else if (d.type == OP_D1) {
-                A.d1(at(d.a, d.qa), g);
+                A.d1(at(d.a, d.qa), m);
             } else if (d.type == OP_D2) {
-                const cd dd[4] = {g[0], g[5], g[10], g[15]};
-                A.d2(at(d.a, d.qa), at(d.b, d.qb), dd);
+                A.d2(at(d.a, d.qa), at(d.b, d.qb), m);
             } else if (d.type == OP_SITE) {
                 const int i = loc[d.a], fl = d.flags & 0xff;
+                A.flush();
                 if (fl & (FL_REDUCE | FL_SPAWN | FL_SAVE | FL_SAVE_FWD)) {
-                    // the state itself is seen here: constant ratios of the other
-                    // positions too
-                    for (int q = 0; q < K; ++q)
-                        if (loc[q] >= kUnitRB && !A.one(carry[q])) {
-                            const int mt = A.put({1.0, carry[q]});
-                            A.emit(UO_SC, loc[q] - LOC_THREAD).mat = (unsigned short)mt;
-                            A.rs = true;
-                            carry[q] = 1.0;
-                        }
-                    A.flush(true);
-                    std::vector<cd> k = {A.cs, A.cs};
                     const int ns = (fl & FL_SPAWN) ? (d.flags >> 16) & 0xff : 0;
-                    for (int f = 0; f < ns; ++f)
-                        for (int e = 0; e < 4; ++e) k.push_back(A.m(d.mat + 4 * (f + 1) + e) * A.cs);
-                    const int mt = A.put(k);
+                    const int mt = A.put(m + 4, 4 * ns);
                     UnitRec& r = A.emit(UO_SITE + i);
                     r.mat = (unsigned short)mt;
                     r.flags = (unsigned char)(fl & ~(FL_APPLY | FL_KDIAG));
@@ -316,25 +288,13 @@ UnitProgram assemble_unit(const std::vector<DevOp>& dops, int off, int n, const 
                     if (fl & FL_SPAWN) r.sp = (unsigned char)(d.flags >> 24);
                 }
                 if (fl & FL_APPLY) {
-                    if (fl & FL_KDIAG) A.d1(i, g);
-                    else A.g1(i, g);
+                    const float2 kd[2] = {m[0], m[3]};
+                    const int mt = (fl & FL_KDIAG) ? A.put(kd, 2) : A.put_matrix(m);
+                    A.emit(((fl & FL_KDIAG) ? UO_KD : UO_GK) + i).mat = (unsigned short)mt;
                 }
             }
         }
-        for (int i = 0; i < kUnitRB; ++i) carry[R[i]] = A.cp[i];
-        if (p + 1 == ranges.size()) {
-            for (int q = 0; q < K; ++q)
-                if (loc[q] >= kUnitRB && !A.one(carry[q])) {
-                    const int mt = A.put({1.0, carry[q]});
-                    A.emit(UO_SC, loc[q] - LOC_THREAD).mat = (unsigned short)mt;
-                    A.rs = true;
-                }
-            A.flush(false);
-        } else {
-            // constants stay with their positions; what the threads hold does not
-            for (cd& c : A.cp) c = 1.0;
-            A.flush(true);
-        }
+        A.flush();
         ph.op_end = (unsigned short)A.recs.size();
         phases.push_back(ph);
     }

@@ -21,31 +21,35 @@ constexpr int kUnitThreads = 1 << (kMaxTileQ - kUnitRB);
 constexpr int kUnitSlots = 8;                   // checkpoint pointers of a pass (reductions, saves)
 constexpr int kNoLoc = 31;                      // location of an absent bit (always 0)
 
-// Operation codes; a code in a family of four is FAMILY + register bit.
+// Operation codes; a code in a family of four is FAMILY + register bit, in a
+// family of six FAMILY + pair of register bits.
 enum UnitOp : int {
-    UO_G1 = 0,      // dense one-qubit matrix
-    UO_G1H = 4,     // the same, taking the pending ratio of its register bit
-    UO_FLB = 8,     // multiply the pending ratio of one register bit into the amplitudes
-    UO_HP = 12,     // scalar *= m[2c], ratio *= m[2c + 1], c = the bit at location a
-    UO_HR = 16,     // ratio *= m[c]
-    UO_SITE = 20,   // noise site
-    UO_SC = 24,     // scalar *= m[c], c = the bits at locations a, b
-    UO_FLS = 25,    // multiply the pending scalar into the amplitudes
-    UO_FLA = 26,    // multiply the scalar and all four ratios into the amplitudes
-    UO_DD = 27,     // + pair index: amplitudes with both register bits *= m[0]
-    UO_G2 = 33,     // + pair index: dense two-qubit matrix, index 2 * b(low) + b(high)
-    UO_DP = 39,     // amplitudes *= m[2c + bit b of r]
-    UO_DG = 40      // amplitudes *= m[2 * bit a of r + bit b of r]
+    UO_G1 = 0,      // dense one-qubit matrix; flags: UF_PAIR, UF_SIGN, UF_SCALAR, UF_REAL
+    UO_GK = 4,      // dense factor K_0 of a site
+    UO_KD = 8,      // diagonal factor K_0 of a site
+    UO_FLB = 12,    // multiply the scalar and the pair of one register bit into the amplitudes
+    UO_FLR = 16,    // multiply the sign of one register bit into the amplitudes
+    UO_HP = 20,     // pair of the bit *= m[2c], m[2c + 1], c = the bit at location a
+    UO_SITE = 24,   // noise site
+    UO_DN = 28,     // negate the amplitudes with both register bits
+    UO_DG = 34,     // amplitudes *= m[2 * (low bit) + (high bit)]
+    UO_G2 = 40,     // dense two-qubit matrix, index 2 * (low bit) + (high bit)
+    UO_SC = 46,     // scalar *= m[c], c = the bits at locations a, b
+    UO_FLS = 47,    // multiply the scalar into the amplitudes; UF_REAL: a real one
+    UO_FLA = 48     // multiply the scalar and all four pairs into the amplitudes
 };
+// A gate takes the pending pair of its bit (a factor for either value), its
+// pending sign (parity of the bits `mask`), the pending scalar; the scalar is real.
+enum : int { UF_PAIR = 1, UF_SIGN = 2, UF_SCALAR = 4, UF_REAL = 8 };
 
 // pairs of register bits (i < j) in the order 01 02 03 12 13 23
 inline int unit_pair(int i, int j) { return i == 0 ? j - 1 : i == 1 ? j + 1 : 5; }
 
 struct UnitRec {               // 16 bytes
     unsigned char code, a, b, flags;
-    unsigned char ev, nspawn, sp, pad0;   // reduction / checkpoint slot, spawned factors, spawn slot
+    unsigned char ev, nspawn, sp, pad0;     // reduction / checkpoint slot, spawned factors, spawn slot
     unsigned short mat, site;
-    unsigned int pad;
+    unsigned int mask;
 };
 
 struct UnitPhase {             // 96 bytes
@@ -91,7 +95,8 @@ struct SweepUnit {
 size_t unit_smem_bytes(int max_words, int max_events);
 int unit_blocks_per_sm(size_t smem);
 // blk: unit of every block, or null when every unit has `ctas` blocks
-cudaError_t launch_units(const SweepUnit* units, const int* blk, int ctas, int total_ctas, size_t smem,
+// single: the units are states swept alone (S = 1), not of a branch group
+cudaError_t launch_units(bool single, const SweepUnit* units, const int* blk, int ctas, int total_ctas, size_t smem,
                          cudaStream_t st);
 // Blocks per unit of a launch of n_units units of n_tiles tiles each.
 int unit_ctas(int n_units, long long n_tiles, int slots);
