@@ -32,7 +32,7 @@ struct Group {
     size_t begins = 0;     // byte offset of the block-begin array (sweeps: the unit of every block)
     int n_units = 0, total = 0;
     size_t smem = 0;
-    bool single = false;   // SWEEP: states swept alone
+    int unit_kind = 0;     // SWEEP: the kernel
     int h = -1;            // SINGLE / MEMSET: which circuit
     int li = -1;           // SINGLE: which launch
 };
@@ -96,7 +96,7 @@ int build_plan(BatchPlan& P, int first, int last, void* stream) {
     for (size_t r = 0; r < rounds; ++r) {
         // the round's sweep passes, longest blocks first (the short ones fill the
         // last wave)
-        std::vector<std::pair<const Engine*, const Launch*>> sweeps_of[2];   // branch groups, single states
+        std::vector<std::pair<const Engine*, const Launch*>> sweeps_of[kUnitKinds];   // by kernel
         std::vector<FinishUnit> fin;
         std::vector<int> fin_blocks;
         std::vector<FillUnit> fills;
@@ -107,7 +107,7 @@ int build_plan(BatchPlan& P, int first, int last, void* stream) {
             const Launch& l = E.launches[r];
             const Handle& h = *P.hs[k];
             if (l.kind == L_PASS && l.units()) {
-                sweeps_of[l.S == 1].push_back({&E, &l});
+                sweeps_of[l.unit_kind].push_back({&E, &l});
             } else if (l.kind == L_FINISH) {
                 FinishUnit u{};
                 u.partials = E.partials;
@@ -154,7 +154,7 @@ int build_plan(BatchPlan& P, int first, int last, void* stream) {
             std::vector<int> block_unit;
             Group g;
             g.kind = Group::SWEEP;
-            g.single = &sweeps == &sweeps_of[1];
+            g.unit_kind = (int)(&sweeps - sweeps_of);
             for (const auto& x : sweeps) {
                 const Launch& l = *x.second;
                 for (int k = 0; k < l.n_units; ++k) {
@@ -228,7 +228,7 @@ int run_plan(BatchPlan& P, cudaStream_t st) {
                 rc = cuda_ok(cudaMemsetAsync(P.engines[g.h]->err_dev, 0, sizeof(int), st));
                 break;
             case Group::SWEEP:
-                rc = cuda_ok(launch_units(g.single, (const SweepUnit*)(base + g.units), (const int*)(base + g.begins), 0, g.total,
+                rc = cuda_ok(launch_units(g.unit_kind, (const SweepUnit*)(base + g.units), (const int*)(base + g.begins), 0, g.total,
                                           g.smem, st));
                 break;
             case Group::FINISH:

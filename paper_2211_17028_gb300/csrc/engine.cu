@@ -25,6 +25,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -404,7 +405,7 @@ struct Builder {
     std::vector<SweepUnit> units;     // pointers into prog / partials / tables patched after layout
     std::vector<size_t> unit_prog, unit_part;
     std::vector<char> unit_bd;
-    std::map<std::pair<int, int>, UnitProgram> programs;   // by (first device op, count)
+    std::map<std::array<int, 3>, UnitProgram> programs;   // by (first device op, count, swept alone)
     size_t partial_top = 0, partial_doubles = 0;
     size_t finished = 0;              // slots already given to a finisher launch
     long long dim;
@@ -546,12 +547,19 @@ struct Builder {
             return c;
         }();
         if (kind == P_UNIT) {
-            const std::pair<int, int> key(rp.op_off + start, rp.n_ops - start);
+            const std::array<int, 3> key = {rp.op_off + start, rp.n_ops - start, S == 1};
             auto it = programs.find(key);
             if (it == programs.end())
-                it = programs.emplace(key, assemble_unit(dops, key.first, key.second, rp.local, plan.n, tab.mats, prog))
+                it = programs.emplace(key, assemble_unit(S == 1, dops, key[0], key[1], rp.local, plan.n, tab.mats, prog))
                          .first;
             const UnitProgram& pi = it->second;
+            // one kernel per launch: a group that needs another one starts a new launch
+            const int kind = unit_kind(S == 1, pi.mode);
+            if (units.size() > first_unit && cur.unit_kind != kind) {
+                close_launch();
+                open_launch();
+            }
+            cur.unit_kind = kind;
             cur.max_words = std::max(cur.max_words, pi.words);
             cur.max_events = std::max(cur.max_events, pi.n_events);
             cur.n_phases = std::max(cur.n_phases, pi.n_phases);
@@ -1348,7 +1356,7 @@ int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* 
 }
 
 static int launch_pass(const Engine& E, const Launch& l, cudaStream_t st) {
-    if (l.units()) return cuda_err(launch_units(l.S == 1, E.units_dev + l.unit_off, nullptr, l.ctas, l.grid, l.smem, st));
+    if (l.units()) return cuda_err(launch_units(l.unit_kind, E.units_dev + l.unit_off, nullptr, l.ctas, l.grid, l.smem, st));
     if (l.jit) return cuda_err(jit_launch(*l.jit, l.grid, l.args, st));
     return cuda_err(launch_tile_pass(l.S, l.grid, l.smem, l.args, st));
 }

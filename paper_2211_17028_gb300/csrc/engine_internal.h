@@ -47,6 +47,7 @@ struct Launch {
     bool seq = false;                // multi-state pass-specialised kernel sweeps its states one at a time
     // pass, unit kernel: n_units states of any number of groups, `grid` blocks in all
     int unit_off = 0, n_units = 0, ctas = 0;
+    int unit_kind = 0;               // unit_kind of their programs
     int max_words = 0, max_events = 0, n_phases = 0;
     size_t part_off = 0;             // partial sums of the launch (doubles)
     // finisher

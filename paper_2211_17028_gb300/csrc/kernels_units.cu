@@ -120,14 +120,25 @@ __device__ __forceinline__ void u_dense(c64 (&x)[kE], const Fac (&k)[4]) {
     }
 }
 
-// pending factors: a scalar and a pair per register bit
+// pending factors: a scalar and a pair or a ratio per register bit
+template <bool PAIRS>
 struct Pend {
-    float2 d, h[kUnitRB][2];
+    static constexpr int W = PAIRS ? 2 : 1;
+    float2 d, h[kUnitRB][W];
+    __device__ __forceinline__ void clear(int i) {
+#pragma unroll
+        for (int w = 0; w < W; ++w) h[i][w] = make_float2(1.f, 0.f);
+    }
+    __device__ __forceinline__ void clear() {
+        d = make_float2(1.f, 0.f);
+#pragma unroll
+        for (int i = 0; i < kUnitRB; ++i) clear(i);
+    }
 };
 
 // the dense gate of a record: its matrix with the pending factors it takes
-template <int I, bool SINGLE>
-__device__ __forceinline__ void u_gate(c64 (&x)[kE], const UnitRec& op, const float2* __restrict__ m, Pend& P,
+template <int I, bool SINGLE, bool PAIRS>
+__device__ __forceinline__ void u_gate(c64 (&x)[kE], const UnitRec& op, const float2* __restrict__ m, Pend<PAIRS>& P,
                                        uint32_t bits) {
     Fac k[4];
 #pragma unroll
@@ -142,12 +153,14 @@ __device__ __forceinline__ void u_gate(c64 (&x)[kE], const UnitRec& op, const fl
         }
         P.d = make_float2(1.f, 0.f);
     }
-    if (op.flags & UF_PAIR) {
-        k[0] = times(k[0], P.h[I][0]);
-        k[2] = times(k[2], P.h[I][0]);
-        k[1] = times(k[1], P.h[I][1]);
-        k[3] = times(k[3], P.h[I][1]);
-        P.h[I][0] = P.h[I][1] = make_float2(1.f, 0.f);
+    if (op.flags & UF_DIAG) {
+        if (PAIRS) {
+            k[0] = times(k[0], P.h[I][0]);
+            k[2] = times(k[2], P.h[I][0]);
+        }
+        k[1] = times(k[1], P.h[I][PAIRS ? 1 : 0]);
+        k[3] = times(k[3], P.h[I][PAIRS ? 1 : 0]);
+        P.clear(I);
     }
     if (op.flags & UF_SIGN) {
         const float f = (__popc(bits & op.mask) & 1) ? -1.f : 1.f;
@@ -167,13 +180,16 @@ __device__ __forceinline__ float2 lds_again(const float2* p) {
     return v;
 }
 
-template <int I0, int I1>
-__device__ __forceinline__ void u_g2(c64 (&x)[kE], const UnitRec& op, const float2* __restrict__ m, Pend& P) {
+template <int I0, int I1, bool PAIRS>
+__device__ __forceinline__ void u_g2(c64 (&x)[kE], const UnitRec& op, const float2* __restrict__ m, Pend<PAIRS>& P) {
     float2 f[4];
-    const bool pair = op.flags & UF_PAIR, scal = op.flags & UF_SCALAR;
+    const bool pair = PAIRS && (op.flags & UF_DIAG), scal = PAIRS && (op.flags & UF_SCALAR);
+    if (PAIRS) {
 #pragma unroll
-    for (int c = 0; c < 4; ++c)
-        f[c] = op.a ? cmul(P.h[I1][c & 1], P.h[I0][c >> 1]) : cmul(P.h[I0][c >> 1], P.h[I1][c & 1]);
+        for (int c = 0; c < 4; ++c) {
+            f[c] = cmul(P.h[I0][(c >> 1) & (P.W - 1)], P.h[I1][c & (P.W - 1)]);
+        }
+    }
     auto entry = [&](int q, int c) {
         float2 e = lds_again(m + 4 * q + c);
         if (scal) e = cmul(e, P.d);
@@ -190,18 +206,16 @@ __device__ __forceinline__ void u_g2(c64 (&x)[kE], const UnitRec& op, const floa
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             c64 y = mulc(entry(q, 0), v[0]);
-            if (op.a) {   // columns in the order of the gate's own qubits
-                y = fmac(entry(q, 2), v[2], y);
-                y = fmac(entry(q, 1), v[1], y);
-            } else {
-                y = fmac(entry(q, 1), v[1], y);
-                y = fmac(entry(q, 2), v[2], y);
-            }
+            y = fmac(entry(q, 1), v[1], y);
+            y = fmac(entry(q, 2), v[2], y);
             x[idx[q]] = fmac(entry(q, 3), v[3], y);
         }
     }
-    P.d = make_float2(1.f, 0.f);
-    P.h[I0][0] = P.h[I0][1] = P.h[I1][0] = P.h[I1][1] = make_float2(1.f, 0.f);
+    if (PAIRS) {
+        P.d = make_float2(1.f, 0.f);
+        P.clear(I0);
+        P.clear(I1);
+    }
 }
 
 // amplitudes *= f0 or f1 by register bit I
@@ -227,15 +241,31 @@ __device__ __forceinline__ void u_negate(c64 (&x)[kE]) {
         if ((r >> I0 & 1) && (r >> I1 & 1)) x[r] = mul2(pk(-1.f, -1.f), x[r]);
 }
 
-template <int I0, int I1>
+template <int I0, int I1, bool PAIRS>
 __device__ __forceinline__ void u_diag2(c64 (&x)[kE], const float2* __restrict__ m) {
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        const Fac f = fac(m[c]);
+    for (int c = PAIRS ? 0 : 3; c < 4; ++c) {
+        const Fac f = fac(m[PAIRS ? c : 0]);
 #pragma unroll
         for (int r = 0; r < kE; ++r)
             if (2 * (r >> I0 & 1) + (r >> I1 & 1) == c) x[r] = mulc(f, x[r]);
     }
+}
+
+// real factors of a diagonal K_0
+template <int I>
+__device__ __forceinline__ void u_by_bit_real(c64 (&x)[kE], float f0, float f1) {
+    const c64 k0 = pk(f0, f0), k1 = pk(f1, f1);
+#pragma unroll
+    for (int r = 0; r < kE; ++r) x[r] = mul2((r >> I & 1) ? k1 : k0, x[r]);
+}
+
+template <int I>
+__device__ __forceinline__ void u_ratio(c64 (&x)[kE], float2 h) {
+    const Fac k = fac(h);
+#pragma unroll
+    for (int r = 0; r < kE; ++r)
+        if (r & (1 << I)) x[r] = mulc(k, x[r]);
 }
 
 // tile index bits of the thread in a phase (those of the register bits are
@@ -283,7 +313,7 @@ struct Addr {
     __device__ __forceinline__ unsigned long long operator()(int r) const { return hi[r >> 2] + lo[r & 3]; }
 };
 
-template <int I>
+template <int I, bool SINGLE>
 __device__ __forceinline__ void u_site(const UnitRec& op, const float2* __restrict__ m, c64 (&x)[kE],
                                        const UnitPhase& ph, int jT, const SweepUnit& u, const unsigned long long* hi_off,
                                        float2* const* slot, unsigned long long base, double* acc, int lane, int warp) {
@@ -292,7 +322,7 @@ __device__ __forceinline__ void u_site(const UnitRec& op, const float2* __restri
     // compiler computes all of them ahead of the operation loop and spills
     asm volatile("" : "+r"(jT));
     const Addr off(hi_off, ph, base | glob(hi_off, jT));
-    if (fl & (FL_SAVE | FL_SAVE_FWD)) {
+    if (SINGLE && (fl & (FL_SAVE | FL_SAVE_FWD))) {   // branch groups save nothing
         c64* const save = reinterpret_cast<c64*>(slot[op.ev]);
 #pragma unroll
         for (int r = 0; r < kE; ++r) __stcs(save + off(r), x[r]);
@@ -338,8 +368,10 @@ __device__ __forceinline__ void u_site(const UnitRec& op, const float2* __restri
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             const float2 a = unpk(A[e]), b = unpk(B[e]);
-            v[2 * e] = a.x + b.y;
-            v[2 * e + 1] = a.y - b.x;
+            float2 R = make_float2(a.x + b.y, a.y - b.x);
+            if (!SINGLE) R = cmul(m[0], R);   // the scale of the state
+            v[2 * e] = R.x;
+            v[2 * e + 1] = R.y;
         }
         // reduce-scatter over the warp: steps 16, 8, 4 halve the components a
         // lane keeps, steps 2, 1 complete the sum
@@ -365,7 +397,7 @@ __device__ __forceinline__ void u_site(const UnitRec& op, const float2* __restri
         for (int i = 0; i < op.nspawn; ++i) {
             Fac K[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) K[e] = fac(m[4 * i + e]);
+            for (int e = 0; e < 4; ++e) K[e] = fac(m[2 + 4 * i + e]);
             c64* const dst = reinterpret_cast<c64*>(u.spawn) + ((size_t)(3 * op.sp + i) << u.n);
 #pragma unroll
             for (int r = 0; r < kE; ++r) {
@@ -378,7 +410,7 @@ __device__ __forceinline__ void u_site(const UnitRec& op, const float2* __restri
     }
 }
 
-template <bool SINGLE>
+template <bool SINGLE, bool PAIRS>
 __global__ void __launch_bounds__(kNT, kBlocksPerSm) unit_sweep_kernel(const SweepUnit* __restrict__ units,
                                                             const int* __restrict__ blk, int ctas) {
     extern __shared__ __align__(128) unsigned char dyn[];
@@ -478,10 +510,8 @@ __global__ void __launch_bounds__(kNT, kBlocksPerSm) unit_sweep_kernel(const Swe
             prefetch(b);
         }
         const float2 unit1 = make_float2(1.f, 0.f);
-        Pend P;
-        P.d = unit1;
-#pragma unroll
-        for (int i = 0; i < kUnitRB; ++i) P.h[i][0] = P.h[i][1] = unit1;
+        Pend<PAIRS> P;
+        P.clear();
 
 #pragma unroll 1
         for (int p = 0; p < n_phases; ++p) {
@@ -514,18 +544,23 @@ __global__ void __launch_bounds__(kNT, kBlocksPerSm) unit_sweep_kernel(const Swe
     case F + 4: { constexpr int I = 1, J = 3; BODY; break; }  \
     case F + 5: { constexpr int I = 2, J = 3; BODY; break; }
                 switch (op.code) {
-                    U_FOUR(UO_G1, (u_gate<I, SINGLE>(x, op, m, P, bits)))
+                    U_FOUR(UO_G1, (u_gate<I, SINGLE, PAIRS>(x, op, m, P, bits)))
                     U_FOUR(UO_GK, const Fac k[4] = {ld_fac(m) U_COMMA ld_fac(m + 2) U_COMMA ld_fac(m + 4) U_COMMA ld_fac(m + 6)};
                            (u_dense<I, true>(x, k)))
-                    U_FOUR(UO_KD, u_by_bit<I>(x, m[0], m[1]))
-                    U_FOUR(UO_FLB, u_by_bit<I>(x, cmul(P.d, P.h[I][0]), cmul(P.d, P.h[I][1]));
-                           P.d = P.h[I][0] = P.h[I][1] = unit1)
+                    U_FOUR(UO_KD, if (op.flags & UF_REAL) u_by_bit_real<I>(x, m[0].x, m[1].x);
+                           else u_by_bit<I>(x, m[0], m[1]))
+                    U_FOUR(UO_FLB, if (PAIRS) u_by_bit<I>(x, cmul(P.d, P.h[I][0]), cmul(P.d, P.h[I][P.W - 1]));
+                           else u_ratio<I>(x, P.h[I][0]);
+                           if (PAIRS) P.d = unit1;
+                           P.clear(I))
                     U_FOUR(UO_FLR, u_flush_sign<I>(x, (__popc(bits & op.mask) & 1) ? -1.f : 1.f))
-                    U_FOUR(UO_HP, P.h[I][0] = cmul(P.h[I][0], m[2 * c]); P.h[I][1] = cmul(P.h[I][1], m[2 * c + 1]))
-                    U_FOUR(UO_SITE, u_site<I>(op, m, x, phases[p], jT, u, hi_off, slot, base, acc, lane, warp))
+                    U_FOUR(UO_HP, const int at = c * P.W; P.h[I][0] = cmul(P.h[I][0], m[at]);
+                           if (PAIRS) P.h[I][P.W - 1] = cmul(P.h[I][P.W - 1], m[at + 1]))
+                    U_FOUR(UO_SITE, (u_site<I, SINGLE>(op, m, x, phases[p], jT, u, hi_off, slot, base, acc, lane, warp)))
                     U_PAIRS(UO_DN, (u_negate<I, J>(x)))
-                    U_PAIRS(UO_DG, (u_diag2<I, J>(x, m)))
-                    U_PAIRS(UO_G2, (u_g2<I, J>(x, op, m, P)))
+                    U_PAIRS(UO_DG, (u_diag2<I, J, PAIRS>(x, m)))
+                    U_PAIRS(UO_G2, (u_g2<I, J, PAIRS>(x, op, m, P)))
+                    U_PAIRS(UO_G2 + 6, (u_g2<J, I, PAIRS>(x, op, m, P)))
                     case UO_SC: P.d = cmul(P.d, m[c + 2 * ((bits >> op.b) & 1)]); break;
                     case UO_FLS:
                         if (op.flags & UF_REAL) {
@@ -539,16 +574,30 @@ __global__ void __launch_bounds__(kNT, kBlocksPerSm) unit_sweep_kernel(const Swe
                         P.d = unit1;
                         break;
                     case UO_FLA:
+                        if (PAIRS) {
 #pragma unroll
-                        for (int g = 0; g < 4; ++g) {
-                            const float2 f2 = cmul(cmul(P.d, P.h[0][g & 1]), P.h[1][g >> 1]);
+                            for (int g = 0; g < 4; ++g) {
+                                const float2 f2 = cmul(cmul(P.d, P.h[0][g & (P.W - 1)]), P.h[1][(g >> 1) & (P.W - 1)]);
 #pragma unroll
-                            for (int h = 0; h < 4; ++h)
-                                x[g + 4 * h] = mulc(fac(cmul(cmul(f2, P.h[2][h & 1]), P.h[3][h >> 1])), x[g + 4 * h]);
+                                for (int h = 0; h < 4; ++h)
+                                    x[g + 4 * h] = mulc(fac(cmul(cmul(f2, P.h[2][h & (P.W - 1)]), P.h[3][(h >> 1) & (P.W - 1)])),
+                                                        x[g + 4 * h]);
+                            }
+                        } else {
+                            float2 f[8];
+                            f[0] = P.d;
+                            f[1] = cmul(f[0], P.h[0][0]);
+                            f[2] = cmul(f[0], P.h[1][0]);
+                            f[3] = cmul(f[1], P.h[1][0]);
+#pragma unroll
+                            for (int r = 0; r < 4; ++r) f[4 + r] = cmul(f[r], P.h[2][0]);
+#pragma unroll
+                            for (int r = 0; r < 8; ++r) {
+                                x[r] = mulc(fac(f[r]), x[r]);
+                                x[8 + r] = mulc(fac(cmul(f[r], P.h[3][0])), x[8 + r]);
+                            }
                         }
-                        P.d = unit1;
-#pragma unroll
-                        for (int i = 0; i < kUnitRB; ++i) P.h[i][0] = P.h[i][1] = unit1;
+                        P.clear();
                         break;
                     default: break;
                 }
@@ -603,14 +652,18 @@ size_t unit_smem_bytes(int max_words, int max_events) {
 
 int unit_blocks_per_sm(size_t smem) {
     int nb = 0;
-    cudaFuncSetAttribute(unit_sweep_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, unit_sweep_kernel<true>, kNT, smem);
+    cudaFuncSetAttribute(unit_sweep_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, unit_sweep_kernel<true, true>, kNT, smem);
     return nb > 0 ? nb : 1;
 }
 
-cudaError_t launch_units(bool single, const SweepUnit* units, const int* blk, int ctas, int total_ctas, size_t smem,
+cudaError_t launch_units(int kind, const SweepUnit* units, const int* blk, int ctas, int total_ctas, size_t smem,
                          cudaStream_t st) {
-    auto* const kernel = single ? unit_sweep_kernel<true> : unit_sweep_kernel<false>;
+    // branch groups mostly keep ratios; a diagonal with zeros has none
+    auto* const kernel = kind == unit_kind(true, UM_RATIOS)  ? unit_sweep_kernel<true, false>
+                         : kind == unit_kind(true, UM_PAIRS) ? unit_sweep_kernel<true, true>
+                         : kind == unit_kind(false, UM_PAIRS) ? unit_sweep_kernel<false, true>
+                                                              : unit_sweep_kernel<false, false>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     kernel<<<total_ctas, kNT, smem, st>>>(units, blk, ctas);

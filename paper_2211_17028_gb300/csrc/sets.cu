@@ -157,8 +157,9 @@ PartLayout add_launch(Prog& G, const Plan& plan, const SetsState& S, const PassS
     if (plan.k == kMaxTileQ) {
         int local[kMaxTileQ];
         for (int j = 0; j < kMaxTileQ; ++j) local[j] = ps.local[j];
-        const UnitProgram pi = assemble_unit(ops, 0, (int)ops.size(), local, plan.n, S.tab.mats, G.prog);
+        const UnitProgram pi = assemble_unit(nstates == 1, ops, 0, (int)ops.size(), local, plan.n, S.tab.mats, G.prog);
         l.n_phases = pi.n_phases;
+        l.unit_kind = unit_kind(nstates == 1, pi.mode);
         l.smem = unit_smem_bytes(pi.words, pi.n_events);
         l.unit_off = (int)G.units.size();
         l.n_units = nstates;

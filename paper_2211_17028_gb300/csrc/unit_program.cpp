@@ -3,32 +3,26 @@
 
 #include <algorithm>
 #include <cmath>
+#include <complex>
 #include <cstring>
 
+#include "fp32_round.h"
 #include "nqs_internal.h"
 
 namespace nqs {
 
 namespace {
 
-// The arithmetic of every amplitude is fixed by the operation order alone: a
-// pending diagonal is a scalar and one pair of factors per register bit, a
-// gate takes the scalar and the pair of its bit into its matrix (scalar first),
-// sites and phase ends multiply what is left into the amplitudes.  Signs (CZ)
-// are exact whatever way they go, so they are kept as parities of thread and
-// tile bits and cost nothing until a gate or the end of the phase takes them.
-struct Assembler {
-    const std::vector<float2>& tab;
+bool is(float2 f, float re) { return f.x == re && f.y == 0.f; }
+
+// a diagonal factor pair that is a sign: 1 or (1, -1) by another bit
+bool is_sign(float2 v0, float2 v1, float2 w0, float2 w1) {
+    return is(v0, 1.f) && is(v1, 1.f) && is(w0, 1.f) && is(w1, -1.f);
+}
+
+struct Records {
     std::vector<UnitRec> recs;
     std::vector<float2> mats;
-    // what the kernel holds: scalar (and whether it is real), pairs; and signs
-    bool scal = false, scal_real = true;
-    bool pair[4] = {false, false, false, false};
-    uint32_t sign[4] = {0, 0, 0, 0};
-
-    explicit Assembler(const std::vector<float2>& t) : tab(t) {}
-
-    static bool is(float2 f, float re) { return f.x == re && f.y == 0.f; }
     int put(const float2* v, int n) {   // matrices start on 16 bytes
         if (mats.size() & 1) mats.push_back(make_float2(0.f, 0.f));
         const int at = (int)mats.size();
@@ -52,6 +46,45 @@ struct Assembler {
         recs.push_back(r);
         return recs.back();
     }
+    // K_0 of a site on register bit i, and the record of its other actions
+    void apply_site(int i, const float2* m, bool diag) {
+        if (diag) {
+            const float2 kd[2] = {m[0], m[3]};
+            const int mt = put(kd, 2);
+            UnitRec& r = emit(UO_KD + i);
+            r.mat = (unsigned short)mt;
+            if (m[0].y == 0.f && m[3].y == 0.f) r.flags = UF_REAL;
+        } else {
+            const int mt = put_matrix(m);
+            emit(UO_GK + i).mat = (unsigned short)mt;
+        }
+    }
+    UnitRec& site(int i, const float2* m, int n_spawn, cd scale) {
+        float2 k[16];
+        const float2 sc = round_c64(scale);
+        k[0] = k[1] = sc;
+        for (int e = 0; e < 4 * n_spawn; ++e)
+            k[2 + e] = is(sc, 1.f) ? m[4 + e] : round_c64(cd(m[4 + e].x, m[4 + e].y) * scale);
+        const int mt = put(k, 2 + 4 * n_spawn);
+        UnitRec& r = emit(UO_SITE + i);
+        r.mat = (unsigned short)mt;
+        r.nspawn = (unsigned char)n_spawn;
+        return r;
+    }
+};
+
+// The arithmetic of every amplitude is fixed by the operation order alone: a
+// pending diagonal is a scalar and one pair of factors per register bit, a
+// gate takes the scalar and the pair of its bit into its matrix (scalar first),
+// sites and phase ends multiply what is left into the amplitudes.  Signs (CZ)
+// are exact whatever way they go, so they are kept as parities of thread and
+// tile bits and cost nothing until a gate or the end of the phase takes them.
+struct PairAssembler : Records {
+    // what the kernel holds: scalar (and whether it is real), pairs; and signs
+    bool scal = false, scal_real = true;
+    bool pair[4] = {false, false, false, false};
+    uint32_t sign[4] = {0, 0, 0, 0};
+
     void scalar(const float2* v, int n, int la, int lb) {   // by bit a + 2 * bit b
         float2 w[4] = {v[0], v[1], n > 2 ? v[2] : v[0], n > 2 ? v[3] : v[1]};
         const int at = put(w, 4);
@@ -61,7 +94,7 @@ struct Assembler {
     }
     // pair of bit i *= (v0, v1) or (w0, w1) by the bit at loc
     void pair_op(int i, int loc, float2 v0, float2 v1, float2 w0, float2 w1) {
-        if (!pair[i] && loc != kNoLoc && is(v0, 1.f) && is(v1, 1.f) && is(w0, 1.f) && is(w1, -1.f)) {
+        if (!pair[i] && loc != kNoLoc && is_sign(v0, v1, w0, w1)) {
             sign[i] ^= 1u << loc;
             return;
         }
@@ -83,6 +116,11 @@ struct Assembler {
         }
         sign[i] = 0;
     }
+    cd scale() const { return 1.0; }   // of what a site sees
+    void at_site() { flush(); }
+    void at_end(bool) { flush(); }
+    void begin_phase(const std::vector<int>&) {}
+    void outside(int, int) {}
     // multiply everything pending into the amplitudes
     void flush() {
         int pairs = 0, which = 0;
@@ -112,7 +150,7 @@ struct Assembler {
         const int at = put_matrix(m);
         UnitRec& r = emit(UO_G1 + i);
         r.mat = (unsigned short)at;
-        r.flags = (unsigned char)((pair[i] ? UF_PAIR : 0) | (sign[i] ? UF_SIGN : 0) | (scal ? UF_SCALAR : 0) |
+        r.flags = (unsigned char)((pair[i] ? UF_DIAG : 0) | (sign[i] ? UF_SIGN : 0) | (scal ? UF_SCALAR : 0) |
                                   (scal_real ? UF_REAL : 0));
         r.mask = sign[i];
         pair[i] = scal = false;
@@ -120,19 +158,13 @@ struct Assembler {
         sign[i] = 0;
     }
     void g2(int i, int j, const float2* m) {   // first qubit on register bit i, second on j
-        // the scalar and the pairs of both bits go into the matrix on the device;
-        // stored with the lower bit first
+        // the scalar and the pairs of both bits go into the matrix on the device
         to_pair(i);
         to_pair(j);
-        float2 k[16];
-        auto sw = [](int x) { return ((x & 1) << 1) | (x >> 1); };
-        for (int r = 0; r < 4; ++r)
-            for (int c = 0; c < 4; ++c) (i < j ? k[4 * r + c] : k[4 * sw(r) + sw(c)]) = m[4 * r + c];
-        const int at = put(k, 16);
-        UnitRec& r = emit(UO_G2 + unit_pair(std::min(i, j), std::max(i, j)));
+        const int at = put(m, 16);
+        UnitRec& r = emit(UO_G2 + unit_pair(std::min(i, j), std::max(i, j)) + (i > j ? 6 : 0));
         r.mat = (unsigned short)at;
-        r.flags = (unsigned char)((pair[i] || pair[j] ? UF_PAIR : 0) | (scal ? UF_SCALAR : 0));
-        r.a = (unsigned char)(i > j);   // the factors of the first qubit's bit come first
+        r.flags = (unsigned char)((pair[i] || pair[j] ? UF_DIAG : 0) | (scal ? UF_SCALAR : 0));
         pair[i] = pair[j] = scal = false;
         scal_real = true;
     }
@@ -148,7 +180,7 @@ struct Assembler {
         const float2 d[4] = {m[0], m[5], m[10], m[15]};
         const bool ra = la < kUnitRB, rb = lb < kUnitRB;
         if (ra && rb) {
-            if (is(d[0], 1.f) && is(d[1], 1.f) && is(d[2], 1.f) && is(d[3], -1.f)) {
+            if (is_sign(d[0], d[1], d[2], d[3])) {
                 emit(UO_DN + unit_pair(std::min(la, lb), std::max(la, lb)));
                 return;
             }
@@ -166,9 +198,198 @@ struct Assembler {
     }
 };
 
+// Ratios: a diagonal on a register bit is its value at 0, a scalar, times a
+// ratio where the bit is set.  Constants fold into matrices on the host; the
+// scalar commutes with every gate, so the last gate of a phase takes it into
+// its matrix (a few products per thread instead of one per amplitude).
+struct RatioAssembler : Records {
+    cd cs = 1.0, cp[4] = {1.0, 1.0, 1.0, 1.0};   // constants: scalar, ratios
+    bool scal = false, scal_real = true;         // held by the kernel
+    bool rat[4] = {false, false, false, false};
+    uint32_t sign[4] = {0, 0, 0, 0};
+    size_t last_gate = 0;    // 1 + record of the last one-qubit gate since the pending factors were last applied
+    float2 gate[4] = {};     // its matrix
+    std::vector<cd> carry;   // constant ratio pending on each tile position across phases
+    std::vector<int> regs;
+
+    static bool one(cd c) { return is(round_c64(c), 1.f); }
+    int put_c(std::initializer_list<cd> v) {
+        float2 f[4];
+        int n = 0;
+        for (cd c : v) f[n++] = round_c64(c);
+        return put(f, n);
+    }
+    void ratio(int i, cd v0, cd v1, int loc = kNoLoc) {
+        const float2 f0 = round_c64(v0), f1 = round_c64(v1);
+        if (loc != kNoLoc && is(f0, 1.f) && is(f1, -1.f)) {
+            sign[i] ^= 1u << loc;
+            return;
+        }
+        const int at = put_c({v0, v1});
+        emit(UO_HP + i, loc).mat = (unsigned short)at;
+        rat[i] = true;
+    }
+    void scalar(cd v0, cd va, cd vb, cd vab, int la = kNoLoc, int lb = kNoLoc) {
+        const int at = put_c({v0, va, vb, vab});
+        emit(UO_SC, la, lb).mat = (unsigned short)at;
+        scal = true;
+        for (cd c : {v0, va, vb, vab}) scal_real = scal_real && round_c64(c).y == 0.f;
+    }
+    // keep_scalar leaves the constant scalar pending (the caller scales what it writes)
+    void flush(bool keep_scalar) {
+        for (int i = 0; i < 4; ++i)
+            if (!one(cp[i])) {
+                ratio(i, cp[i], cp[i]);
+                cp[i] = 1.0;
+            }
+        if (!keep_scalar && !one(cs) && last_gate > 0) take_constant();
+        int n = 0;
+        for (int i = 0; i < 4; ++i) n += rat[i];
+        if (scal && last_gate > 0 && n < 3) absorb_scalar();
+        if (!keep_scalar && !one(cs)) {
+            scalar(cs, cs, cs, cs);
+            cs = 1.0;
+        }
+        if (8 * n + 16 * (int)scal > 31) {   // 31 products for everything at once
+            emit(UO_FLA);
+        } else {
+            for (int i = 0; i < 4; ++i)
+                if (rat[i]) emit(UO_FLB + i);
+            if (scal) emit(UO_FLS).flags = scal_real ? UF_REAL : 0;
+        }
+        for (int i = 0; i < 4; ++i) {
+            if (sign[i]) emit(UO_FLR + i).mask = sign[i];
+            sign[i] = 0;
+            rat[i] = false;
+        }
+        scal = false;
+        scal_real = true;
+        last_gate = 0;
+    }
+    // The scalar's factors depend on the thread and tile alone: those that come
+    // after the last gate move ahead of it, and the gate takes them.
+    void absorb_scalar() {
+        const size_t g = last_gate - 1;
+        UnitRec r = recs[g];
+        r.flags |= (unsigned char)(UF_SCALAR | (scal_real ? UF_REAL : 0));
+        std::vector<UnitRec> before, after;
+        for (size_t k = g + 1; k < recs.size(); ++k) (recs[k].code == UO_SC ? before : after).push_back(recs[k]);
+        recs.resize(g);
+        recs.insert(recs.end(), before.begin(), before.end());
+        recs.push_back(r);
+        recs.insert(recs.end(), after.begin(), after.end());
+        scal = false;
+        scal_real = true;
+        last_gate = 0;
+    }
+    void take_constant() {   // the constant scalar goes into the last gate's matrix
+        cd k[4];
+        for (int e = 0; e < 4; ++e) k[e] = cd(gate[e].x, gate[e].y) * cs;
+        round_matrix_c64(k, 2, gate);
+        const int at = put_matrix(gate);
+        recs[last_gate - 1].mat = (unsigned short)at;
+        cs = 1.0;
+    }
+    void g1(int i, const float2* m) {
+        for (int e = 0; e < 4; ++e) gate[e] = m[e];
+        if (!one(cp[i])) {
+            cd k[4];
+            for (int e = 0; e < 4; ++e) k[e] = cd(m[e].x, m[e].y) * ((e & 1) ? cp[i] : cd(1.0));
+            round_matrix_c64(k, 2, gate);
+            cp[i] = 1.0;
+        }
+        const int at = put_matrix(gate);
+        UnitRec& r = emit(UO_G1 + i);
+        r.mat = (unsigned short)at;
+        r.flags = (unsigned char)((rat[i] ? UF_DIAG : 0) | (sign[i] ? UF_SIGN : 0));
+        r.mask = sign[i];
+        rat[i] = false;
+        sign[i] = 0;
+        last_gate = recs.size();
+    }
+    void g2(int i, int j, const float2* m) {   // first qubit on register bit i, second on j
+        for (int b : {i, j}) {
+            if (!one(cp[b])) ratio(b, cp[b], cp[b]);
+            cp[b] = 1.0;
+            if (rat[b]) emit(UO_FLB + b);
+            if (sign[b]) emit(UO_FLR + b).mask = sign[b];
+            rat[b] = false;
+            sign[b] = 0;
+        }
+        const int at = put(m, 16);
+        UnitRec& r = emit(UO_G2 + unit_pair(std::min(i, j), std::max(i, j)) + (i > j ? 6 : 0));
+        r.mat = (unsigned short)at;
+    }
+    static cd c(float2 f) { return cd(f.x, f.y); }
+    // a diagonal on register bit i whose two values depend on the bit at `loc`;
+    // one that vanishes where the bit is clear is applied as a dense gate
+    void pair_op(int i, int loc, cd f00, cd f10, cd f01, cd f11) {   // f<bit i><bit loc>
+        if (f00 == f01) cs *= f00;
+        else scalar(f00, f01, f00, f01, loc);
+        ratio(i, f10 / f00, f11 / f01, loc);
+    }
+    void d1(int la, const float2* m) {
+        if (la >= kUnitRB) {
+            scalar(c(m[0]), c(m[3]), c(m[0]), c(m[3]), la - LOC_THREAD);
+        } else {
+            cs *= c(m[0]);
+            cp[la] *= c(m[3]) / c(m[0]);
+        }
+    }
+    void d2(int la, int lb, const float2* m) {
+        const cd d[4] = {c(m[0]), c(m[5]), c(m[10]), c(m[15])};   // 2 * bit a + bit b
+        const bool ra = la < kUnitRB, rb = lb < kUnitRB;
+        if (ra && rb) {
+            cs *= d[0];
+            cp[la] *= d[2] / d[0];
+            cp[lb] *= d[1] / d[0];
+            const cd k = d[3] * d[0] / (d[1] * d[2]);
+            const int pr = unit_pair(std::min(la, lb), std::max(la, lb));
+            if (is(round_c64(k), -1.f)) {
+                emit(UO_DN + pr);
+            } else if (!one(k)) {
+                const int at = put_c({k, k});
+                emit(UO_DG + pr).mat = (unsigned short)at;
+            }
+        } else if (ra) {
+            pair_op(la, lb - LOC_THREAD, d[0], d[2], d[1], d[3]);
+        } else if (rb) {
+            pair_op(lb, la - LOC_THREAD, d[0], d[1], d[2], d[3]);
+        } else {
+            scalar(d[0], d[2], d[1], d[3], la - LOC_THREAD, lb - LOC_THREAD);
+        }
+    }
+    cd scale() const { return cs; }
+    void at_site() { flush(true); }
+    // constants stay with their positions between phases
+    void begin_phase(const std::vector<int>& R) {
+        if (carry.empty()) carry.assign(kMaxTileQ, cd(1.0));
+        regs = R;
+        for (int i = 0; i < 4; ++i) cp[i] = carry[R[i]];
+        last_gate = 0;
+    }
+    void at_end(bool last) {
+        for (int i = 0; i < 4; ++i) {
+            carry[regs[i]] = cp[i];
+            if (!last) cp[i] = 1.0;
+        }
+        flush(!last);
+        if (last)
+            for (int i = 0; i < 4; ++i) carry[regs[i]] = 1.0;
+    }
+    // the constant of a tile position outside the registers, at thread bit loc
+    void outside(int pos, int loc) {
+        if (!one(carry[pos])) scalar(1.0, carry[pos], 1.0, carry[pos], loc);
+        carry[pos] = 1.0;
+    }
+};
+
 }  // namespace
 
-UnitProgram assemble_unit(const std::vector<DevOp>& dops, int off, int n, const int* local, int n_qubits,
+namespace {
+
+template <typename Asm>
+UnitProgram assemble(const std::vector<DevOp>& dops, int off, int n, const int* local, int n_qubits,
                           const std::vector<float2>& tab, std::vector<uint4>& out) {
     static_assert(sizeof(UnitRec) == 16 && sizeof(UnitPhase) == 96 && sizeof(UnitHeader) == 64, "record sizes");
     constexpr int K = kMaxTileQ;
@@ -211,7 +432,7 @@ UnitProgram assemble_unit(const std::vector<DevOp>& dops, int off, int n, const 
     ranges.push_back({begin, n});
     regs.push_back(cur);
 
-    Assembler A(tab);
+    Asm A;
     std::vector<UnitPhase> phases;
     for (size_t p = 0; p < ranges.size(); ++p) {
         std::vector<int> R = regs[p];
@@ -253,6 +474,7 @@ UnitProgram assemble_unit(const std::vector<DevOp>& dops, int off, int n, const 
             for (int i = 0; i < 3; ++i)
                 if (w >> i & 1) ph.warp_j[w] |= (unsigned short)(1 << T[5 + i]);
         ph.op_begin = (unsigned short)A.recs.size();
+        A.begin_phase(R);
         auto at = [&](int pos, int q) { return pos >= 0 ? loc[pos] : LOC_THREAD + 8 + outer[q]; };
         for (int o = ranges[p].first; o < ranges[p].second; ++o) {
             const DevOp& d = dops[off + o];
@@ -267,14 +489,13 @@ UnitProgram assemble_unit(const std::vector<DevOp>& dops, int off, int n, const 
                 A.d2(at(d.a, d.qa), at(d.b, d.qb), m);
             } else if (d.type == OP_SITE) {
                 const int i = loc[d.a], fl = d.flags & 0xff;
-                A.flush();
                 if (fl & (FL_REDUCE | FL_SPAWN | FL_SAVE | FL_SAVE_FWD)) {
-                    const int ns = (fl & FL_SPAWN) ? (d.flags >> 16) & 0xff : 0;
-                    const int mt = A.put(m + 4, 4 * ns);
-                    UnitRec& r = A.emit(UO_SITE + i);
-                    r.mat = (unsigned short)mt;
+                    // the state itself is seen here
+                    for (int q = 0; q < K; ++q)
+                        if (loc[q] >= kUnitRB) A.outside(q, loc[q] - LOC_THREAD);
+                    A.at_site();
+                    UnitRec& r = A.site(i, m, (fl & FL_SPAWN) ? (d.flags >> 16) & 0xff : 0, A.scale());
                     r.flags = (unsigned char)(fl & ~(FL_APPLY | FL_KDIAG));
-                    r.nspawn = (unsigned char)ns;
                     r.site = (unsigned short)d.site;
                     if (fl & FL_REDUCE) {
                         r.ev = (unsigned char)((d.flags >> 8) & 0xff);
@@ -286,15 +507,16 @@ UnitProgram assemble_unit(const std::vector<DevOp>& dops, int off, int n, const 
                         hd.slot_site[r.ev] = (unsigned short)(d.site | ((fl & FL_SAVE_FWD) ? 0x8000 : 0));
                     }
                     if (fl & FL_SPAWN) r.sp = (unsigned char)(d.flags >> 24);
+                } else {
+                    A.at_site();
                 }
-                if (fl & FL_APPLY) {
-                    const float2 kd[2] = {m[0], m[3]};
-                    const int mt = (fl & FL_KDIAG) ? A.put(kd, 2) : A.put_matrix(m);
-                    A.emit(((fl & FL_KDIAG) ? UO_KD : UO_GK) + i).mat = (unsigned short)mt;
-                }
+                if (fl & FL_APPLY) A.apply_site(i, m, (fl & FL_KDIAG) != 0);
             }
         }
-        A.flush();
+        if (p + 1 == ranges.size())
+            for (int q = 0; q < K; ++q)
+                if (loc[q] >= kUnitRB) A.outside(q, loc[q] - LOC_THREAD);
+        A.at_end(p + 1 == ranges.size());
         ph.op_end = (unsigned short)A.recs.size();
         phases.push_back(ph);
     }
@@ -318,6 +540,29 @@ UnitProgram assemble_unit(const std::vector<DevOp>& dops, int off, int n, const 
     info.n_phases = (int)hd.n_phases;
     info.n_events = (int)hd.n_events;
     return info;
+}
+
+}  // namespace
+
+UnitProgram assemble_unit(bool single, const std::vector<DevOp>& dops, int off, int n, const int* local, int n_qubits,
+                          const std::vector<float2>& tab, std::vector<uint4>& out) {
+    // pairs where the order of products shows: states swept alone through
+    // diagonals that are not signs; and diagonals with zeros, which have no ratios
+    bool phases = false, zeros = false;
+    for (int o = off; o < off + n; ++o) {
+        const DevOp& d = dops[o];
+        if (d.type != OP_D1 && d.type != OP_D2) continue;
+        const int dim = d.type == OP_D1 ? 2 : 4;
+        for (int k = 0; k < dim; ++k) {
+            const float2 f = tab[d.mat + (dim + 1) * k];
+            zeros = zeros || (f.x == 0.f && f.y == 0.f);
+            phases = phases || !(is(f, 1.f) || (is(f, -1.f) && d.type == OP_D2 && k == 3));
+        }
+    }
+    UnitProgram u = (single && phases) || zeros ? assemble<PairAssembler>(dops, off, n, local, n_qubits, tab, out)
+                                                : assemble<RatioAssembler>(dops, off, n, local, n_qubits, tab, out);
+    u.mode = (single && phases) || zeros ? UM_PAIRS : UM_RATIOS;
+    return u;
 }
 
 int unit_ctas(int n_units, long long n_tiles, int slots) {

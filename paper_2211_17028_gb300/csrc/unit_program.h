@@ -21,26 +21,37 @@ constexpr int kUnitThreads = 1 << (kMaxTileQ - kUnitRB);
 constexpr int kUnitSlots = 8;                   // checkpoint pointers of a pass (reductions, saves)
 constexpr int kNoLoc = 31;                      // location of an absent bit (always 0)
 
+// How a program keeps pending diagonals:
+//   UM_PAIRS   a scalar and a pair of factors per register bit, taken by gates
+//              and multiplied into the amplitudes in a fixed order.  States
+//              swept alone (backward and main sweeps, from which levels 0 and 1
+//              come) through circuits with phases use it: their results are
+//              those of every earlier kernel, bit for bit.
+//   UM_RATIOS  a scalar and one ratio per register bit: half the products.
+//              Branch groups use it, and every program whose diagonals are
+//              signs, which are exact either way.
+enum UnitMode : int { UM_RATIOS = 0, UM_PAIRS = 1 };
+
 // Operation codes; a code in a family of four is FAMILY + register bit, in a
 // family of six FAMILY + pair of register bits.
 enum UnitOp : int {
-    UO_G1 = 0,      // dense one-qubit matrix; flags: UF_PAIR, UF_SIGN, UF_SCALAR, UF_REAL
+    UO_G1 = 0,      // dense one-qubit matrix; flags: UF_DIAG, UF_SIGN, UF_SCALAR, UF_REAL
     UO_GK = 4,      // dense factor K_0 of a site
-    UO_KD = 8,      // diagonal factor K_0 of a site
-    UO_FLB = 12,    // multiply the scalar and the pair of one register bit into the amplitudes
+    UO_KD = 8,      // diagonal factor K_0 of a site; UF_REAL: real entries
+    UO_FLB = 12,    // pairs: the scalar and the pair of one register bit into the amplitudes; ratios: the ratio
     UO_FLR = 16,    // multiply the sign of one register bit into the amplitudes
-    UO_HP = 20,     // pair of the bit *= m[2c], m[2c + 1], c = the bit at location a
+    UO_HP = 20,     // c = the bit at location a; pairs: pair of the bit *= m[2c], m[2c + 1]; ratios: ratio *= m[c]
     UO_SITE = 24,   // noise site
     UO_DN = 28,     // negate the amplitudes with both register bits
-    UO_DG = 34,     // amplitudes *= m[2 * (low bit) + (high bit)]
-    UO_G2 = 40,     // dense two-qubit matrix, index 2 * (low bit) + (high bit)
-    UO_SC = 46,     // scalar *= m[c], c = the bits at locations a, b
-    UO_FLS = 47,    // multiply the scalar into the amplitudes; UF_REAL: a real one
-    UO_FLA = 48     // multiply the scalar and all four pairs into the amplitudes
+    UO_DG = 34,     // pairs: amplitudes *= m[2 * (low bit) + (high bit)]; ratios: those with both bits *= m[0]
+    UO_G2 = 40,     // dense two-qubit matrix, its first qubit on the low bit (+ 6: on the high bit)
+    UO_SC = 52,     // scalar *= m[c], c = the bits at locations a, b
+    UO_FLS = 53,    // multiply the scalar into the amplitudes; UF_REAL: a real one
+    UO_FLA = 54     // multiply the scalar and all four pairs or ratios into the amplitudes
 };
-// A gate takes the pending pair of its bit (a factor for either value), its
-// pending sign (parity of the bits `mask`), the pending scalar; the scalar is real.
-enum : int { UF_PAIR = 1, UF_SIGN = 2, UF_SCALAR = 4, UF_REAL = 8 };
+// A gate takes the pending pair or ratio of its bit, its pending sign (parity
+// of the bits `mask`), the pending scalar; the scalar is real.
+enum : int { UF_DIAG = 1, UF_SIGN = 2, UF_SCALAR = 4, UF_REAL = 8 };
 
 // pairs of register bits (i < j) in the order 01 02 03 12 13 23
 inline int unit_pair(int i, int j) { return i == 0 ? j - 1 : i == 1 ? j + 1 : 5; }
@@ -70,13 +81,14 @@ struct UnitHeader {            // 64 bytes
 };
 
 struct UnitProgram {
+    UnitMode mode = UM_RATIOS;
     int word = 0, words = 0, n_phases = 0, n_events = 0;
 };
 
 // Assemble dops[off .. off + n) (execution order) on the tile qubits `local`
 // of an n_qubits-wide state, appending to `out`; mats is the float2 table the
-// operations index.
-UnitProgram assemble_unit(const std::vector<DevOp>& dops, int off, int n, const int* local, int n_qubits,
+// operations index; single: for a state swept alone.
+UnitProgram assemble_unit(bool single, const std::vector<DevOp>& dops, int off, int n, const int* local, int n_qubits,
                           const std::vector<float2>& mats, std::vector<uint4>& out);
 
 // One state swept through one pass: `ctas` consecutive blocks share its tiles.
@@ -92,11 +104,14 @@ struct SweepUnit {
     int n_tiles, n, cta_begin, ctas;
 };
 
+// kernel of a launch: states swept alone or of branch groups, and the mode
+inline int unit_kind(bool single, UnitMode mode) { return 2 * (int)single + (int)mode; }
+constexpr int kUnitKinds = 4;
 size_t unit_smem_bytes(int max_words, int max_events);
 int unit_blocks_per_sm(size_t smem);
 // blk: unit of every block, or null when every unit has `ctas` blocks
-// single: the units are states swept alone (S = 1), not of a branch group
-cudaError_t launch_units(bool single, const SweepUnit* units, const int* blk, int ctas, int total_ctas, size_t smem,
+// kind: unit_kind of the units' programs
+cudaError_t launch_units(int kind, const SweepUnit* units, const int* blk, int ctas, int total_ctas, size_t smem,
                          cudaStream_t st);
 // Blocks per unit of a launch of n_units units of n_tiles tiles each.
 int unit_ctas(int n_units, long long n_tiles, int slots);
