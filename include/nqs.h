@@ -276,12 +276,14 @@ int nqs_get_info(nqs_handle h, nqs_info* out);
  * nqs_fidelity call built), for profiling: one record per launch, in launch
  * order.  kind: 0 sweep pass, 1 finisher, 2 state fill, 3 state copy,
  * 4 two-state reduction, 5 level sums, 6 normalisation of the computed
- * v = U|psi> (basis psi).  For sweep passes: states swept
- * together, register qubits per thread (0: shared-memory tile kernel), phases
+ * v = U|psi> (basis psi), 7 the whole expansion of a circuit narrower than a
+ * tile (two kernels: checkpoints, then a block per prefix of insertions; with
+ * grid and algorithmic_bytes).  For sweep passes: states of a branch group
+ * (1: a state swept alone; one launch may sweep many groups), register qubits per thread (0: shared-memory tile kernel), phases
  * of the register-resident program, grid size, operation counts
  * ops[] = {dense 1-qubit, dense 2-qubit, diagonal 1-qubit, diagonal 2-qubit,
- * noise sites, site reductions, spawned states, checkpoint saves}, whether
- * the pass runs a pass-specialised kernel (NQS_OPT_JIT) and the
+ * noise sites, site reductions, spawned states, checkpoint saves} (the last two
+ * of the whole launch, the others of one group), whether the pass runs a pass-specialised kernel (NQS_OPT_JIT) and the
  * algorithmic bytes of the launch (see nqs_kernel_stats).  Call with out =
  * NULL (or cap too small) to get the count only.  No counterpart in the paper. */
 typedef struct {
@@ -308,8 +310,9 @@ int nqs_schedule_launches(nqs_handle h, nqs_launch_info* out, size_t cap, size_t
  *       block, with k chosen to hold the fewest states.  1 <= k < N forces
  *       blocks of k sites (levels <= 2, else NQS_ERR_UNSUPPORTED at the call);
  *       k >= N keeps every site.
- *   NQS_OPT_SWEEP_RB      register qubits per thread of multi-state sweep
- *       passes: 3 (512-thread blocks) or 4 (256-thread blocks).
+ *   NQS_OPT_SWEEP_RB      register qubits per thread of the multi-state passes of
+ *       pass-specialised kernels: 3 (512-thread blocks) or 4 (256-thread blocks).
+ *       The precompiled kernel sweeps one state per block with 4.
  *   NQS_OPT_MAX_OPS       fused operations per pass, 8..160 (default 96).
  *   NQS_OPT_MAX_SITES     noise sites per pass, 1..8 (default 4).
  *   NQS_OPT_SHARD_RANK, NQS_OPT_SHARD_COUNT   split one call's terms over

@@ -919,6 +919,224 @@ static int best_spacing(int N, int level) {
     return best;
 }
 
+// truncation bound: sum_{|S|>l} prod ||M-bar|| prod ||M'||
+static double truncation_bound(const std::vector<Factors>& fac, int level) {
+    std::vector<double> poly(1, 1.0);
+    for (const Factors& f : fac) {
+        std::vector<double> nx(poly.size() + 1, 0.0);
+        for (size_t i = 0; i < poly.size(); ++i) {
+            nx[i] += poly[i] * f.norm_dom;
+            nx[i + 1] += poly[i] * f.norm_rest;
+        }
+        poly.swap(nx);
+    }
+    double bnd = 0;
+    for (size_t i = level + 1; i < poly.size(); ++i) bnd += poly[i];
+    return bnd;
+}
+
+// what a schedule was built for, and what is kept of its inputs
+static void set_key(Engine& E, const nqs_state* psi, const nqs_state* v, int level, const TermIndex& ti) {
+    E.level = level;
+    E.psi_kind = psi->kind;
+    E.v_kind = v->kind;
+    E.psi_bits = psi->bits;
+    E.v_bits = v->bits;
+    E.psi_dev = psi->dev;
+    E.v_dev = v->dev;
+    E.n_terms = (long long)ti.total;
+    E.eff_level = level;
+}
+
+// Terms up to which a narrow circuit's expansion is one block per prefix
+// (small.cu); beyond it the host lists would be larger than the sweeps' savings.
+constexpr uint64_t kSmallTerms = 1ull << 24;
+
+// Circuits narrower than a tile: the whole expansion in two launches.  The
+// prefixes are all assignments of up to level - 1 kept factors whose first
+// site this shard owns.
+static int build_small(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* v, int level, const TermIndex& ti,
+                       void* stream) {
+    const Plan& plan = h.plan;
+    const int N = (int)h.factors.size(), n_ops = (int)plan.ops.size();
+    const int shard_count = std::max(1, h.opt_shard_count), shard_rank = h.opt_shard_rank;
+    const size_t sbytes = sizeof(float2) << plan.n;
+    E.n_states = 2 * (size_t)N;
+    E.buf_bytes = E.n_states * sbytes;
+    E.buf = dev_alloc(E.buf_bytes, stream);
+    if (!E.buf) {
+        E.buf_bytes = 0;
+        return NQS_ERR_NOMEM;
+    }
+    // operation lists and matrices, padded to whole chunks
+    const size_t padded = ((size_t)n_ops + 31) / 32 * 32 + 32;
+    std::vector<SmallOp> fwd(padded), bwd(padded);
+    std::vector<float2> fm(padded * 16, make_float2(0.f, 0.f)), bm(fm);
+    std::vector<int> site_op(N), n_fac(N), keep(3 * (size_t)N, 0);
+    std::vector<double> km((size_t)N * 32);
+    for (int i = 0; i < n_ops; ++i) {
+        const HostOp& o = plan.ops[i];
+        SmallOp r{};
+        r.type = (unsigned char)o.type;
+        r.a = (unsigned char)o.q0;
+        r.b = (unsigned char)(o.q1 >= 0 ? o.q1 : 0);
+        r.diag = o.diag;
+        r.site = o.site;
+        fwd[i] = bwd[n_ops - 1 - i] = r;
+        const int dim = (o.type == OP_G2 || o.type == OP_D2) ? 4 : 2;
+        cd adj[16];
+        for (int x = 0; x < dim; ++x)
+            for (int y = 0; y < dim; ++y) adj[dim * x + y] = std::conj(o.m[dim * y + x]);
+        round_matrix_c64(o.m.data(), dim, fm.data() + (size_t)i * 16);
+        round_matrix_c64(adj, dim, bm.data() + (size_t)(n_ops - 1 - i) * 16);
+        if (o.type == OP_SITE) {
+            const Factors& f = h.factors[o.site];
+            site_op[o.site] = i;
+            n_fac[o.site] = f.m;
+            for (int j = 0; j < f.m; ++j) {
+                round_matrix_c64(f.K[f.keep[j]].data(), 2, fm.data() + (size_t)i * 16 + 4 * (j + 1));
+                keep[3 * o.site + j] = f.keep[j];
+            }
+            for (int k = 0; k < 4; ++k)
+                for (int e = 0; e < 4; ++e) {
+                    km[o.site * 32 + k * 8 + 2 * e] = f.K[k][e].real();
+                    km[o.site * 32 + k * 8 + 2 * e + 1] = f.K[k][e].imag();
+                }
+        }
+    }
+    // units and the ranks of their terms
+    std::vector<SmallUnit> units;
+    std::vector<long long> ranks, pair_rank(N, -1);
+    auto first_rank = [&](int k, const int* sites, int* fp) {   // of the first factor at the last site
+        if (h.factors[sites[k - 1]].m == 0) return -1ll;
+        fp[k - 1] = 0;
+        return (long long)ti.rank(k, sites, fp);
+    };
+    int sites[NQS_MAX_LEVEL + 1], fp[NQS_MAX_LEVEL + 1];
+    if (shard_rank == 0 && level >= 1)
+        for (int s = 0; s < N; ++s) {
+            sites[0] = s;
+            pair_rank[s] = first_rank(1, sites, fp);
+        }
+    std::function<void(int, int)> extend = [&](int depth, int from) {
+        for (int s = from; s + 1 < N; ++s) {
+            if (depth == 0 && s % shard_count != shard_rank) continue;
+            sites[depth] = s;
+            for (int f = 0; f < h.factors[s].m; ++f) {
+                fp[depth] = f;
+                SmallUnit u{};
+                u.depth = depth + 1;
+                u.rank = (long long)ranks.size();
+                for (int k = 0; k <= depth; ++k) {
+                    u.site[k] = (unsigned short)sites[k];
+                    u.factor[k] = (unsigned char)fp[k];
+                }
+                for (int t = s + 1; t < N; ++t) {
+                    sites[depth + 1] = t;
+                    ranks.push_back(first_rank(depth + 2, sites, fp));
+                }
+                units.push_back(u);
+                if (depth + 2 < level) {
+                    extend(depth + 1, s + 1);
+                    sites[depth] = s;
+                    fp[depth] = f;
+                }
+            }
+        }
+    };
+    if (level >= 2) extend(0, 0);
+
+    auto align = [](size_t x) { return (x + 255) & ~(size_t)255; };
+    std::vector<long long> loff(level + 2);
+    for (int u = 0; u <= level + 1; ++u) loff[u] = (long long)ti.level_offset[u];
+    struct Part {
+        const void* src;
+        size_t bytes, off;
+    };
+    std::vector<Part> parts;
+    size_t top = 0;
+    auto add = [&](const void* src, size_t bytes) {
+        parts.push_back({src, bytes, top});
+        top = align(top + bytes + 1);
+        return parts.back().off;
+    };
+    const size_t o_fwd = add(fwd.data(), fwd.size() * sizeof(SmallOp)), o_fm = add(fm.data(), fm.size() * sizeof(float2));
+    const size_t o_bwd = add(bwd.data(), bwd.size() * sizeof(SmallOp)), o_bm = add(bm.data(), bm.size() * sizeof(float2));
+    const size_t o_site = add(site_op.data(), N * sizeof(int)), o_nf = add(n_fac.data(), N * sizeof(int));
+    const size_t o_keep = add(keep.data(), keep.size() * sizeof(int)), o_km = add(km.data(), km.size() * sizeof(double));
+    const size_t o_unit = add(units.data(), units.size() * sizeof(SmallUnit));
+    const size_t o_rank = add(ranks.data(), ranks.size() * sizeof(long long));
+    const size_t o_pair = add(pair_rank.data(), N * sizeof(long long));
+    const size_t o_loff = add(loff.data(), loff.size() * sizeof(long long));
+    const size_t uploaded = top, o_err = top, o_vals = align(o_err + sizeof(int));
+    const size_t o_res = align(o_vals + std::max<uint64_t>(ti.total, 1) * sizeof(double));
+    E.aux_bytes = align(o_res + sizeof(nqs_result));
+    E.aux = dev_alloc(E.aux_bytes, stream);
+    if (!E.aux) {
+        E.aux_bytes = 0;
+        engine_release(E, stream);
+        return NQS_ERR_NOMEM;
+    }
+    std::vector<char> blob(uploaded, 0);
+    for (const Part& q : parts)
+        if (q.bytes) std::memcpy(blob.data() + q.off, q.src, q.bytes);
+    cudaStream_t st = (cudaStream_t)stream;
+    char* ab = (char*)E.aux;
+    int rc = cuda_err(cudaMemcpyAsync(ab, blob.data(), uploaded, cudaMemcpyHostToDevice, st));
+    if (rc == NQS_OK) rc = cuda_err(cudaMemsetAsync(ab + o_err, 0, o_res - o_err, st));   // status word and term values
+    if (rc == NQS_OK) rc = cuda_err(cudaStreamSynchronize(st));   // pageable source
+    if (rc != NQS_OK) {
+        engine_release(E, stream);
+        return rc;
+    }
+    E.upload_bytes = uploaded;
+    SmallArgs& a = E.small;
+    a = SmallArgs{};
+    a.n = plan.n;
+    a.n_sites = N;
+    a.n_units = (int)units.size();
+    a.fwd_ops = plan.site_pos[N - 1] + 1;
+    a.bwd_ops = n_ops - plan.site_pos[0];
+    a.all_ops = n_ops;
+    a.fwd = (const SmallOp*)(ab + o_fwd);
+    a.fwd_mats = (const float2*)(ab + o_fm);
+    a.bwd = (const SmallOp*)(ab + o_bwd);
+    a.bwd_mats = (const float2*)(ab + o_bm);
+    a.site_op = (const int*)(ab + o_site);
+    a.n_factors = (const int*)(ab + o_nf);
+    a.kmats = (const double*)(ab + o_km);
+    a.keep = (const int*)(ab + o_keep);
+    a.phi = (float2*)E.buf;
+    a.chi = a.phi + ((size_t)N << plan.n);
+    a.units = (const SmallUnit*)(ab + o_unit);
+    a.ranks = (const long long*)(ab + o_rank);
+    a.pair_rank = (const long long*)(ab + o_pair);
+    a.level0 = shard_rank == 0 ? 0 : -1;
+    E.term_vals = a.term_vals = (double*)(ab + o_vals);
+    E.err_dev = (int*)(ab + o_err);
+    E.level_off_dev = (long long*)(ab + o_loff);
+    E.res_dev = (nqs_result*)(ab + o_res);
+    a.psi_kind = psi->kind;
+    a.v_kind = v->kind;
+    a.psi_bits = psi->bits;
+    a.v_bits = v->bits;
+    a.psi_dev = (const float2*)psi->dev;
+    a.v_dev = (const float2*)v->dev;
+    Launch l;
+    l.kind = L_SMALL;
+    l.grid = N + a.n_units;
+    const double dim = std::pow(2.0, plan.n);
+    l.bytes = 8.0 * dim * (4.0 * N + (double)ranks.size() + a.n_units);
+    E.launches.push_back(l);
+    l = Launch();
+    l.kind = L_SUM;
+    E.launches.push_back(l);
+    E.spacing = 0;
+    set_key(E, psi, v, level, ti);
+    E.bound = truncation_bound(h.factors, level);
+    return NQS_OK;
+}
+
 // Build (or reuse) the schedule for this level and state kinds.
 int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* v, int level, void* stream,
                    bool allow_jit) {
@@ -944,6 +1162,10 @@ int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* 
     for (int s = 0; s < N; ++s) m[s] = h.factors[s].m;
     B.ti.build(m, level);
 
+    // a circuit narrower than a tile: one block per prefix, whole states on chip.
+    // (The tile kernel remains for spaced checkpoints, huge expansions and N = 0.)
+    if (plan.n <= kSmallMaxQ && N > 0 && !(h.opt_spacing > 0 && h.opt_spacing < N) && B.ti.total <= kSmallTerms)
+        return build_small(h, E, psi, v, level, B.ti, stream);
     const bool rt = plan.k == kMaxTileQ || E.wide;
     const bool use_jit = want_jit && rt && jit_available() && !E.jit_failed;
     if (want_jit && rt && !use_jit) E.jit_state = -1;   // NVRTC missing: the precompiled kernel runs
@@ -1330,28 +1552,8 @@ int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* 
     }
     E.launches = std::move(B.L);
     E.units = std::move(B.units);
-    E.level = level;
-    E.psi_kind = psi->kind;
-    E.v_kind = v->kind;
-    E.psi_bits = psi->bits;
-    E.v_bits = v->bits;
-    E.psi_dev = psi->dev;
-    E.v_dev = v->dev;
-    E.n_terms = (long long)B.ti.total;
-    E.eff_level = level;
-    // truncation bound: sum_{|S|>l} prod ||M-bar|| prod ||M'||
-    std::vector<double> poly(1, 1.0);
-    for (int s = 0; s < N; ++s) {
-        std::vector<double> nx(poly.size() + 1, 0.0);
-        for (size_t i = 0; i < poly.size(); ++i) {
-            nx[i] += poly[i] * h.factors[s].norm_dom;
-            nx[i + 1] += poly[i] * h.factors[s].norm_rest;
-        }
-        poly.swap(nx);
-    }
-    double bnd = 0;
-    for (size_t i = level + 1; i < poly.size(); ++i) bnd += poly[i];
-    E.bound = bnd;
+    set_key(E, psi, v, level, B.ti);
+    E.bound = truncation_bound(h.factors, level);
     return NQS_OK;
 }
 
@@ -1378,6 +1580,7 @@ int run_launch(Handle& h, Engine& E, const Launch& l, cudaStream_t st) {
         case L_SUM:
             return cuda_err(launch_level_sum(E.term_vals, E.level_off_dev, E.eff_level, E.res_dev, E.bound, E.n_terms,
                                              E.err_dev, st));
+        case L_SMALL: return cuda_err(launch_small(E.small, st));
         case L_NORMALIZE:
             return cuda_err(launch_normalize(l.dst, dim, E.partials, l.fin_grid, fill_grid, st));
     }
@@ -1385,11 +1588,14 @@ int run_launch(Handle& h, Engine& E, const Launch& l, cudaStream_t st) {
 }
 
 int run_schedule(Handle& h, Engine& E, cudaStream_t st) {
-    int rc = cuda_err(cudaMemsetAsync(E.err_dev, 0, sizeof(int), st));
+    // the status word (the kernels of narrow circuits wait for nothing and leave it 0)
+    int rc = NQS_OK;
+    if (E.launches.empty() || E.launches[0].kind != L_SMALL)
+        rc = cuda_err(cudaMemsetAsync(E.err_dev, 0, sizeof(int), st));
     if (rc != NQS_OK) return rc;
     for (const Launch& l : E.launches) {
         cudaEvent_t e0 = nullptr, e1 = nullptr;
-        int kind = (l.kind == L_PASS) ? 0 : (l.kind == L_FINISH || l.kind == L_SUM || l.kind == L_REDUCE2) ? 1 : 2;
+        int kind = (l.kind == L_PASS || l.kind == L_SMALL) ? 0 : (l.kind == L_FINISH || l.kind == L_SUM || l.kind == L_REDUCE2) ? 1 : 2;
         const bool timed = h.profiling && l.kind != L_COPY;
         if (timed) {
             if (E.ev_next >= E.ev_pool.size()) {
@@ -1400,7 +1606,7 @@ int run_schedule(Handle& h, Engine& E, cudaStream_t st) {
             }
             e0 = E.ev_pool[E.ev_next].first;
             e1 = E.ev_pool[E.ev_next].second;
-            E.ev_used.push_back({kind, l.kind == L_PASS ? (l.S > 1 ? 3 : 4) : -1, l.bytes});
+            E.ev_used.push_back({kind, l.kind == L_PASS ? (l.S > 1 ? 3 : 4) : l.kind == L_SMALL ? 4 : -1, l.bytes});
             ++E.ev_next;
             cudaEventRecord(e0, st);
         }
@@ -1504,6 +1710,9 @@ int engine_launch_list(const Handle& h, nqs_launch_info* out, size_t cap, size_t
             for (int c = 0; c < 8; ++c) o.ops[c] = l.op_counts[c];
             o.jit = l.jit ? 1 : 0;
             o.algorithmic_bytes = l.bytes;
+        } else if (l.kind == L_SMALL) {
+            o.grid = l.grid;
+            o.algorithmic_bytes = l.bytes;
         }
     }
     return NQS_OK;
@@ -1575,7 +1784,7 @@ int engine_spacing(const Handle& h, int* n_states) {
 uint64_t engine_launches_per_call(const Handle& h) {
     if (!h.eng) return 0;
     uint64_t n = 0;
-    for (const auto& l : h.eng->launches) n += (l.kind != L_COPY) ? 1 : 0;
+    for (const auto& l : h.eng->launches) n += l.kind == L_SMALL ? 2 : l.kind != L_COPY ? 1 : 0;
     return n;
 }
 

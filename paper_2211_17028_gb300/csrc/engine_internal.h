@@ -10,6 +10,7 @@
 #include "fp32_round.h"
 #include "jit.h"
 #include "nqs_internal.h"
+#include "small.h"
 #include "sweep_types.h"
 #include "unit_program.h"
 
@@ -30,7 +31,7 @@ struct Run {
     std::vector<RunPass> passes;     // in execution order
 };
 
-enum LaunchKind { L_PASS, L_FINISH, L_FILL, L_COPY, L_REDUCE2, L_SUM, L_NORMALIZE };
+enum LaunchKind { L_PASS, L_FINISH, L_FILL, L_COPY, L_REDUCE2, L_SUM, L_NORMALIZE, L_SMALL };
 
 struct Launch {
     LaunchKind kind;
@@ -79,6 +80,7 @@ struct Engine {
     const void* psi_dev = nullptr;
     const void* v_dev = nullptr;
     std::vector<Launch> launches;
+    SmallArgs small{};               // narrow circuits: the whole expansion (L_SMALL)
     double bound = 0;
     long long n_terms = 0;
     int eff_level = 0;
