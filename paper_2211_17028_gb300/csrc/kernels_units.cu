@@ -606,8 +606,8 @@ __global__ void __launch_bounds__(kNT, kBlocksPerSm) unit_sweep_kernel(const Swe
 #undef U_COMMA
             }
         }
-        // store the tile
-        {
+        // store the tile, unless only its reductions or spawned states were wanted
+        if (u.out) {
             c64* const dst = reinterpret_cast<c64*>(u.out);
             const Addr off(hi_off, phases[n_phases - 1], base | glob(hi_off, jT));
 #pragma unroll

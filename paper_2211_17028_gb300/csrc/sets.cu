@@ -5,13 +5,27 @@
 //
 // nqs_prepare_sets stores phi_s (backward sweep from v) and chi_s (forward
 // sweep from psi, saved before K_0 is applied) at every site.  A set is then
-// evaluated from its first site's checkpoint: w_i = K_i chi_{s_1} is spawned
-// (three states), swept to s_2 (K_0 at the sites in between), spawned again
-// into three groups of three, swept to s_3 and reduced against phi_{s_3};
-// k = 1 reduces chi_{s_1} against phi_{s_1} directly.  Sets are taken in
-// lexicographic order so that sets with a common first site share the sweep
-// of w_i, and sets with a common first pair share the sweeps of the nine
-// states, each of which reduces at every third site its sets need.
+// evaluated between its sites' checkpoints.
+//   k = 1: chi_{s_1} is reduced against phi_{s_1}.
+//   k = 2: w_i = K_i chi_{s_1} is spawned (three states), swept to s_2 (K_0 at
+//     the sites in between) and reduced against phi_{s_2}.
+//   k = 3, meeting at s_2: u_j = K_j^dagger phi_{s_3} is spawned too and swept
+//     backward to s_2, where each w_i is reduced against each u_j: six states
+//     swept, and the nine 2x2 matrices give all 27 terms.
+//   k = 3, forward: at s_2 the w_i spawn nine states, which are swept on and
+//     reduced at s_3, at every third site of the sets that share s_1 and s_2.
+// Sets are taken in lexicographic order so that sets with a common first site
+// share the sweep of w_i.  A common pair meets while the third sites' backward
+// sweeps (three states each) are together no longer than the nine forward
+// states' sweep to the last of them, that is up to about three third sites.
+//
+// The sets of one first site are a chain of passes, each of which needs the
+// one before; chains are independent.  They are dealt to lanes, each with its
+// own states, and the r-th passes of all lanes are one launch: three states of
+// a 20-qubit circuit are 768 tiles (2.5 rounds of the resident blocks), of a
+// 14-qubit one twelve.  40 triples of a 20-qubit circuit with 200 noises:
+// 66.6 ms with nine states swept by three launches of three each, one chain
+// after another; @@ms.
 //
 // When the 2N checkpoints do not fit in device memory (or the handle's
 // checkpoint-spacing option asks for it), chi is kept only at the first site
@@ -53,8 +67,10 @@ struct SetsState {
     std::vector<std::pair<int, int>> mat_pass;   // (first op in mat_ops, count) per pass, reversed order
     std::vector<int> mat_seg;         // segment index of each entry of mat_pass
     std::vector<int> mat_block;       // block of each entry of mat_pass
-    float2* g1 = nullptr;             // three states spawned at the first site
-    float2* g2 = nullptr;             // nine spawned at the second
+    float2* g1 = nullptr;             // lane 0: three states spawned at the first site
+    float2* g2 = nullptr;             // and nine spawned at the second (or three at the third)
+    int lanes = 1;                    // lane l: the same 12 states, 12 l states further on
+    float2** lane_tab = nullptr;      // the first three states of g2 of every lane
     float2** phi_tab = nullptr;
     float2** chi_tab = nullptr;
     double* kmats = nullptr;
@@ -63,6 +79,8 @@ struct SetsState {
     int* err = nullptr;
     Tables tab;
     std::vector<int> fwd_mat;        // forward matrix offset of every linear op
+    std::vector<int> bwd_mat;        // adjoints
+    std::vector<int> spawn_adj;      // per site: K_0 (unused), then the adjoints of the kept factors
     int sm_count = 0;
     bool ready = false;
 };
@@ -71,12 +89,35 @@ namespace {
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
+// states of the lanes beyond the first, held from nqs_prepare_sets on
+constexpr size_t kLaneBytes = (size_t)1 << 30;
+constexpr int kMaxLanes = 96;         // three one-tile states each: the resident blocks
+constexpr int kLaneStates = 12;
+
+enum CkptTable : char { CT_PHI, CT_BOUNDARY, CT_LANE };   // what a unit's reductions and saves refer to
+
+// One pass of a lane: its units, and the finisher slots of its reductions.
+struct Step {
+    int kind = 0, n_phases = 0, n_events = 0, lane = 0;
+    size_t smem = 0, word = 0;
+    CkptTable table = CT_PHI;
+    std::vector<SweepUnit> units;
+    struct Slot {
+        int ev, state;
+        FinishSlot f;
+    };
+    std::vector<Slot> slots;
+};
+
 struct Prog {
+    int sm_count = 0;
     std::vector<DevOp> dops;          // shared-memory tile kernel
     std::vector<uint4> prog;          // unit kernel
     std::vector<SweepUnit> units;
     std::vector<size_t> unit_prog, unit_part;
-    std::vector<char> unit_bd;
+    std::vector<char> unit_table, unit_lane;
+    std::vector<std::vector<Step>> lanes = std::vector<std::vector<Step>>(1);   // passes not launched yet
+    int lane = 0;                     // where passes are added
     std::vector<FinishSlot> slots;
     std::vector<Launch> L;
     size_t partial_doubles = 8, partial_top = 0, finished = 0;
@@ -98,18 +139,74 @@ struct Prog {
         partial_top = 0;
         L.push_back(f);
     }
+    // launches for the passes collected so far: round r takes the r-th pass of
+    // every lane, one launch per kernel, the longest programs first
+    void settle() {
+        size_t rounds = 0;
+        for (const auto& l : lanes) rounds = std::max(rounds, l.size());
+        for (size_t r = 0; r < rounds; ++r)
+            for (int kind = 0; kind < kUnitKinds; ++kind) {
+                std::vector<const Step*> steps;
+                for (const auto& l : lanes)
+                    if (r < l.size() && l[r].kind == kind) steps.push_back(&l[r]);
+                if (steps.empty()) continue;
+                std::stable_sort(steps.begin(), steps.end(),
+                                 [](const Step* x, const Step* y) { return x->n_phases > y->n_phases; });
+                Launch l;
+                l.kind = L_PASS;
+                l.unit_kind = kind;
+                l.unit_off = (int)units.size();
+                for (const Step* s : steps) {
+                    l.n_units += (int)s->units.size();
+                    l.smem = std::max(l.smem, s->smem);
+                    l.n_phases = std::max(l.n_phases, s->n_phases);
+                }
+                l.ctas = unit_ctas(l.n_units, steps[0]->units[0].n_tiles, unit_blocks_per_sm(l.smem) * sm_count);
+                l.grid = l.ctas * l.n_units;
+                size_t need = 0;
+                for (const Step* s : steps) need += s->units.size() * s->n_events * l.ctas * 8;
+                size_t at = take_partials(need);
+                int cta = 0;
+                for (const Step* s : steps) {
+                    const size_t event = (size_t)l.ctas * 8, state = event * s->n_events;
+                    for (size_t u = 0; u < s->units.size(); ++u) {
+                        units.push_back(s->units[u]);
+                        units.back().ctas = l.ctas;
+                        units.back().cta_begin = cta;
+                        cta += l.ctas;
+                        unit_prog.push_back(s->word);
+                        unit_part.push_back(at + u * state);
+                        unit_table.push_back(s->table);
+                        unit_lane.push_back((char)s->lane);
+                    }
+                    for (const Step::Slot& x : s->slots) {
+                        slots.push_back(x.f);
+                        slots.back().part = at + x.state * state + x.ev * event;
+                        slots.back().grid = l.ctas;
+                    }
+                    at += s->units.size() * state;
+                }
+                L.push_back(l);
+            }
+        for (auto& l : lanes) l.clear();
+    }
+    void push(const Launch& l) {   // a launch that is no unit pass
+        settle();
+        L.push_back(l);
+    }
 };
 
-// DevOps of the forward direction for linear ops [a, b) of pass `ps`, with
-// site flags chosen by `flag_of(site)`.
+// DevOps for linear ops [a, b) of pass `ps`, with site flags chosen by
+// `flag_of(site)`; back: the adjoints in reverse order.
 template <typename F>
 std::vector<DevOp> emit_range(const Plan& plan, const SetsState& S, const PassSpec& ps, int a, int b, F flag_of,
-                              const std::vector<Factors>& fac) {
+                              const std::vector<Factors>& fac, bool back = false) {
     std::vector<int> pos(plan.n, -1);
     for (int j = 0; j < plan.k; ++j) pos[ps.local[j]] = j;
     std::vector<DevOp> out;
     int events = 0;
-    for (int i = a; i < b; ++i) {
+    for (int e = a; e < b; ++e) {
+        const int i = back ? a + b - 1 - e : e;
         const HostOp& o = plan.ops[i];
         DevOp d{};
         d.type = o.type;
@@ -118,11 +215,14 @@ std::vector<DevOp> emit_range(const Plan& plan, const SetsState& S, const PassSp
         d.a = o.q0 >= 0 ? pos[o.q0] : -1;
         d.b = o.q1 >= 0 ? pos[o.q1] : -1;
         d.site = o.site;
-        d.mat = S.fwd_mat[i];
+        d.mat = back ? S.bwd_mat[i] : S.fwd_mat[i];
         if (o.type == OP_SITE) {
             int fl = flag_of(o.site);
             if (fl & FL_REDUCE) fl |= (events++) << 8;
-            if (fl & FL_SPAWN) fl |= fac[o.site].m << 16;
+            if (fl & FL_SPAWN) {
+                fl |= fac[o.site].m << 16;
+                if (back) d.mat = S.spawn_adj[o.site];
+            }
             if (o.diag) fl |= FL_KDIAG;
             d.flags = fl;
         }
@@ -137,55 +237,50 @@ int pass_of(const std::vector<PassSpec>& segs, int lin) {
     return -1;
 }
 
-// One sweep launch over custom DevOps of one pass; the states and the buffers
-// they spawn into are consecutive from in, out and spawn on.  Returns the
-// offset of the partial sums of state 0, event 0; `step` receives the distance
-// between states and between events, `grid` the blocks of a state.
-struct PartLayout {
-    size_t base = 0, state = 0, event = 0;
+// One sweep pass over custom DevOps; the states and the buffers they spawn
+// into are consecutive from in, out and spawn on.  out null: the swept states
+// are not needed any more.  Returns what add_slot needs.
+struct PassRef {
+    int step = -1;                              // unit kernel: pass of the current lane
+    size_t base = 0, state = 0, event = 0;      // tile kernel: layout of the partial sums
     int grid = 0;
 };
 
-PartLayout add_launch(Prog& G, const Plan& plan, const SetsState& S, const PassSpec& ps, int nstates,
-                      const std::vector<DevOp>& ops, const float2* in, float2* out, float2* spawn, bool bd_table) {
+PassRef add_launch(Prog& G, const Plan& plan, const SetsState& S, const PassSpec& ps, int nstates,
+                   const std::vector<DevOp>& ops, const float2* in, float2* out, float2* spawn,
+                   CkptTable table = CT_PHI) {
     const size_t dim = (size_t)1 << plan.n;
-    Launch l;
-    PartLayout pl;
-    l.kind = L_PASS;
-    l.S = nstates;
+    PassRef pl;
     const long long n_tiles = 1ll << (plan.n - plan.k);
     if (plan.k == kMaxTileQ) {
         int local[kMaxTileQ];
         for (int j = 0; j < kMaxTileQ; ++j) local[j] = ps.local[j];
         const UnitProgram pi = assemble_unit(nstates == 1, ops, 0, (int)ops.size(), local, plan.n, S.tab.mats, G.prog);
-        l.n_phases = pi.n_phases;
-        l.unit_kind = unit_kind(nstates == 1, pi.mode);
-        l.smem = unit_smem_bytes(pi.words, pi.n_events);
-        l.unit_off = (int)G.units.size();
-        l.n_units = nstates;
-        l.ctas = unit_ctas(nstates, n_tiles, unit_blocks_per_sm(l.smem) * S.sm_count);
-        l.grid = l.ctas * nstates;
-        pl.grid = l.ctas;
-        pl.event = (size_t)l.ctas * 8;
-        pl.state = pl.event * pi.n_events;
-        pl.base = G.take_partials(pl.state * nstates);
+        Step st;
+        st.n_phases = pi.n_phases;
+        st.n_events = pi.n_events;
+        st.kind = unit_kind(nstates == 1, pi.mode);
+        st.smem = unit_smem_bytes(pi.words, pi.n_events);
+        st.word = (size_t)pi.word;
+        st.table = table;
+        st.lane = G.lane;
         for (int s = 0; s < nstates; ++s) {
             SweepUnit u{};
             u.in = in + s * dim;
-            u.out = out + s * dim;
+            u.out = out ? out + s * dim : nullptr;
             u.spawn = spawn ? spawn + 3 * s * dim : nullptr;
             u.n_tiles = (int)n_tiles;
             u.n = plan.n;
-            u.ctas = l.ctas;
-            u.cta_begin = s * l.ctas;
-            G.units.push_back(u);
-            G.unit_prog.push_back((size_t)pi.word);
-            G.unit_part.push_back(pl.base + s * pl.state);
-            G.unit_bd.push_back(bd_table);
+            st.units.push_back(u);
         }
-        G.L.push_back(l);
+        pl.step = (int)G.lanes[G.lane].size();
+        G.lanes[G.lane].push_back(std::move(st));
         return pl;
     }
+    Launch l;
+    l.kind = L_PASS;
+    l.S = nstates;
+    if (!out) out = S.scratch;   // single states only
     PassArgs& a = l.args;
     a.n = plan.n;
     a.k = plan.k;
@@ -209,7 +304,7 @@ PartLayout add_launch(Prog& G, const Plan& plan, const SetsState& S, const PassS
         if (spawn)
             for (int i = 0; i < 3; ++i) a.spawn[3 * s + i] = spawn + (3 * s + i) * dim;
     }
-    l.bd_table = bd_table;
+    l.bd_table = table == CT_BOUNDARY;
     l.op_index = (int)G.dops.size();
     G.dops.insert(G.dops.end(), ops.begin(), ops.end());
     a.n_ops = (int)ops.size();
@@ -223,25 +318,27 @@ PartLayout add_launch(Prog& G, const Plan& plan, const SetsState& S, const PassS
     return pl;
 }
 
-// slot of one reduction (site, state): factor position f -> value index rank_of(f)
+// slot of one reduction (event ev of a pass, state st) at a site: factor
+// position f -> value index rank_of(f)
 template <typename R>
-void add_slot(Prog& G, size_t part, int grid, int site, const std::vector<Factors>& fac, R rank_of) {
+void add_slot(Prog& G, const PassRef& pl, int ev, int st, int site, const std::vector<Factors>& fac, R rank_of) {
     const Factors& ft = fac[site];
     FinishSlot f{};
-    f.part = part;
-    f.grid = grid;
+    f.part = pl.base + ev * pl.event + st * pl.state;
+    f.grid = pl.grid;
     for (int i = 0; i < 4; ++i) {
         f.d[i] = FinishDesc{-1, 0, 0};
         if (i >= 1 && i <= ft.m) f.d[i] = FinishDesc{(long long)rank_of(i - 1), site * 32 + ft.keep[i - 1] * 8, 0};
     }
-    G.slots.push_back(f);
+    if (pl.step >= 0) G.lanes[G.lane][pl.step].slots.push_back({ev, st, f});
+    else G.slots.push_back(f);
 }
 
 // sweep `nstates` states over the linear ops (a, b]; site t gets flag_of(t)
-// (which may spawn only at b); every launch with reductions gets its finisher
+// (which may spawn only at b); last: the states are not needed afterwards
 template <typename FlagFn, typename RankFn>
 void sweep_range(Prog& G, const Handle& h, const SetsState& S, int a, int b, FlagFn flag_of, int nstates,
-                 float2* states, float2* spawn, RankFn rank_of) {
+                 float2* states, float2* spawn, bool last, RankFn rank_of) {
     const Plan& plan = h.plan;
     for (int p = pass_of(S.fsegs, a + 1); p >= 0 && p < (int)S.fsegs.size(); ++p) {
         const PassSpec& ps = S.fsegs[p];
@@ -260,13 +357,14 @@ void sweep_range(Prog& G, const Handle& h, const SetsState& S, int a, int b, Fla
             }
             auto ops = emit_range(plan, S, ps, c0, c1, flag_of, h.factors);
             const bool last_chunk = has_last && c1 == hi;
-            const PartLayout pl = add_launch(G, plan, S, ps, nstates, ops, states, states, last_chunk ? spawn : nullptr, false);
+            const bool drop = last && last_chunk && plan.k == kMaxTileQ;
+            const PassRef pl = add_launch(G, plan, S, ps, nstates, ops, states, drop ? nullptr : states,
+                                          last_chunk ? spawn : nullptr);
             int ev = 0;
             for (const DevOp& d : ops) {
                 if (d.type != OP_SITE || !(d.flags & FL_REDUCE)) continue;
                 for (int st = 0; st < nstates; ++st)
-                    add_slot(G, pl.base + ev * pl.event + st * pl.state, pl.grid, d.site, h.factors,
-                             [&](int f) { return rank_of(d.site, st, f); });
+                    add_slot(G, pl, ev, st, d.site, h.factors, [&](int f) { return rank_of(d.site, st, f); });
                 ++ev;
             }
             c0 = c1;
@@ -275,7 +373,48 @@ void sweep_range(Prog& G, const Handle& h, const SetsState& S, int a, int b, Fla
     }
 }
 
+// sweep `nstates` states backward over the linear ops (a, b), K_0^dagger at sites
+void sweep_back(Prog& G, const Handle& h, const SetsState& S, int a, int b, int nstates, float2* states) {
+    for (int p = pass_of(S.fsegs, b - 1); p >= 0; --p) {
+        const PassSpec& ps = S.fsegs[p];
+        const int lo = std::max(ps.op_begin, a + 1), hi = std::min(ps.op_end, b);
+        if (lo >= hi) break;
+        add_launch(G, h.plan, S, ps, nstates, emit_range(h.plan, S, ps, lo, hi, [](int) { return FL_APPLY; }, h.factors, true),
+                   states, states, nullptr);
+    }
+}
+
+// sweep `nstates` states forward over the linear ops [a, b), b a site, and
+// reduce each against the lane's n_back backward states on the site's qubit
+template <typename RankFn>
+void sweep_and_meet(Prog& G, const Handle& h, const SetsState& S, int a, int b, int nstates, float2* states,
+                    int n_back, bool last, RankFn rank_of) {
+    const Plan& plan = h.plan;
+    const int end = pass_of(S.fsegs, b);
+    const auto apply = [](int) { return FL_APPLY; };
+    for (int p = pass_of(S.fsegs, a); p < end; ++p) {
+        const PassSpec& ps = S.fsegs[p];
+        const int lo = std::max(ps.op_begin, a);
+        if (lo < ps.op_end)
+            add_launch(G, plan, S, ps, nstates, emit_range(plan, S, ps, lo, ps.op_end, apply, h.factors), states, states,
+                       nullptr);
+    }
+    const PassSpec& ps = S.fsegs[end];
+    auto ops = emit_range(plan, S, ps, std::max(ps.op_begin, a), b, apply, h.factors);
+    const auto at = emit_range(plan, S, ps, b, b + 1, [](int) { return FL_REDUCE; }, h.factors);
+    for (int j = 0; j < n_back; ++j) {
+        ops.push_back(at[0]);
+        ops.back().site = j;                              // of the lane's table
+        ops.back().flags = FL_REDUCE | (j << 8);
+    }
+    const PassRef pl = add_launch(G, plan, S, ps, nstates, ops, states, last ? nullptr : states, nullptr, CT_LANE);
+    for (int j = 0; j < n_back; ++j)
+        for (int st = 0; st < nstates; ++st)
+            add_slot(G, pl, j, st, plan.ops[b].site, h.factors, [&](int f) { return rank_of(j, st, f); });
+}
+
 int upload_and_run(Handle& h, SetsState& S, Prog& G, size_t extra_bytes, void** extra, cudaStream_t st) {
+    G.settle();
     G.flush_finish();
     // per-call buffer: device ops, programs, units, finisher slots, partials, extra
     const size_t o_prog = align256(G.dops.size() * sizeof(DevOp) + 1);
@@ -304,7 +443,9 @@ int upload_and_run(Handle& h, SetsState& S, Prog& G, size_t extra_bytes, void** 
     for (size_t u = 0; u < G.units.size(); ++u) {
         SweepUnit& x = G.units[u];
         x.prog = (const uint4*)(base + o_prog) + G.unit_prog[u];
-        x.ckpt = G.unit_bd[u] ? S.phi_bd_tab : S.phi_tab;
+        x.ckpt = G.unit_table[u] == CT_LANE       ? S.lane_tab + 3 * G.unit_lane[u]
+                 : G.unit_table[u] == CT_BOUNDARY ? S.phi_bd_tab
+                                                  : S.phi_tab;
         x.ckpt_fwd = S.chi_tab;
         x.partials = E.partials + G.unit_part[u];
         x.err = S.err;
@@ -371,8 +512,17 @@ int engine_prepare_sets(Handle& h, const nqs_state* psi, const nqs_state* v, voi
     auto spaced_states = [&](int k) { return 2 * (size_t)((N + k - 1) / k) + (size_t)k + 5 + 12; };
     int k = (h.opt_spacing > 0 && h.opt_spacing < N) ? h.opt_spacing : 0;
     if (k == 0) {
-        S.buf_bytes = (2 * (size_t)N + 2 + 3 + 9) * sbytes;
+        const size_t own = 2 * (size_t)N + 2 + kLaneStates;
+        // further lanes where they fit; narrow circuits' tile kernel and spaced
+        // checkpoints have one
+        S.lanes = plan.k == kMaxTileQ ? 1 + (int)std::min<size_t>(std::min(kMaxLanes, N) - 1, kLaneBytes / (kLaneStates * sbytes)) : 1;
+        S.buf_bytes = (own + (size_t)(S.lanes - 1) * kLaneStates) * sbytes;
         S.buf = dev_alloc(S.buf_bytes, stream);
+        if (!S.buf && S.lanes > 1) {
+            S.lanes = 1;
+            S.buf_bytes = own * sbytes;
+            S.buf = dev_alloc(S.buf_bytes, stream);
+        }
         if (!S.buf && h.opt_spacing == 0 && N > 1) {
             k = 1;
             for (int c = 2; c < N; ++c)
@@ -380,6 +530,7 @@ int engine_prepare_sets(Handle& h, const nqs_state* psi, const nqs_state* v, voi
         }
     }
     if (k > 0) {
+        S.lanes = 1;
         S.buf_bytes = spaced_states(k) * sbytes;
         S.buf = dev_alloc(S.buf_bytes, stream);
     }
@@ -426,6 +577,17 @@ int engine_prepare_sets(Handle& h, const nqs_state* psi, const nqs_state* v, voi
     S.fwd_mat.assign(plan.ops.size(), -1);
     for (const RunPass& rp : run_fwd.passes)
         for (int o = 0; o < rp.n_ops; ++o) S.fwd_mat[rp.lin[o]] = run_ops[rp.op_off + o].mat;
+    S.bwd_mat.assign(plan.ops.size(), -1);
+    for (const RunPass& rp : run_bwd.passes)
+        for (int o = 0; o < rp.n_ops; ++o) S.bwd_mat[rp.lin[o]] = run_ops[rp.op_off + o].mat;
+    for (int s = 0; s < N; ++s) {
+        const Factors& f = h.factors[s];
+        S.spawn_adj.push_back(S.tab.add(f.K[0].data(), 4, true, 2));
+        for (int j = 0; j < 3; ++j) {
+            const Mat2 z{};
+            S.tab.add((j < f.m ? f.K[f.keep[j]] : z).data(), 4, true, 2);
+        }
+    }
     Run run_ideal;
     if (v->kind == NQS_STATE_IDEAL) run_ideal = make_run(plan, plan.free_passes, RT_IDEAL, false, false, false, h.factors,
                                                          S.tab, run_ops);
@@ -454,7 +616,8 @@ int engine_prepare_sets(Handle& h, const nqs_state* psi, const nqs_state* v, voi
     const size_t o_err = align256(o_kmat + (size_t)N * 32 * sizeof(double));
     const size_t o_mats = align256(o_err + sizeof(int));
     const size_t o_bd = align256(o_mats + S.tab.mats.size() * sizeof(float2) + 1);
-    S.aux_bytes = align256(o_bd + N * sizeof(float2*));
+    const size_t o_lane = align256(o_bd + N * sizeof(float2*));
+    S.aux_bytes = align256(o_lane + 3 * (size_t)S.lanes * sizeof(float2*));
     S.aux = dev_alloc(S.aux_bytes, stream);
     if (!S.aux) {
         S.aux_bytes = 0;
@@ -467,6 +630,7 @@ int engine_prepare_sets(Handle& h, const nqs_state* psi, const nqs_state* v, voi
     S.kmats = (double*)(ab + o_kmat);
     S.err = (int*)(ab + o_err);
     S.phi_bd_tab = (float2**)(ab + o_bd);
+    S.lane_tab = (float2**)(ab + o_lane);
     float2* mats_dev = (float2*)(ab + o_mats);
     std::vector<double> kh((size_t)N * 32);
     for (int s = 0; s < N; ++s)
@@ -481,10 +645,14 @@ int engine_prepare_sets(Handle& h, const nqs_state* psi, const nqs_state* v, voi
         chi_t[s] = k ? S.chi[s / k] : S.chi[s];
         bd_t[s] = k ? S.phi[s / k] : S.phi[s];
     }
+    std::vector<float2*> lane_t;
+    for (int l = 0; l < S.lanes; ++l)
+        for (int j = 0; j < 3; ++j) lane_t.push_back(S.g2 + ((size_t)l * kLaneStates + j) * dim);
     int rc = NQS_OK;
     auto up = [&](void* dst, const void* src, size_t bytes) {
         if (bytes && rc == NQS_OK) rc = cuda_err(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st));
     };
+    up(S.lane_tab, lane_t.data(), lane_t.size() * sizeof(float2*));
     up(S.phi_tab, phi_t.data(), N * sizeof(float2*));
     up(S.chi_tab, chi_t.data(), N * sizeof(float2*));
     up(S.phi_bd_tab, bd_t.data(), N * sizeof(float2*));
@@ -499,6 +667,7 @@ int engine_prepare_sets(Handle& h, const nqs_state* psi, const nqs_state* v, voi
 
     // checkpoint sweeps: (ideal v) -> backward saving phi -> forward saving chi
     Prog G;
+    G.sm_count = S.sm_count;
     auto run_passes = [&](const Run& run, const std::vector<PassSpec>& segs, const float2* first_in, bool bwd,
                           bool save_fwd) {
         for (size_t p = 0; p < run.passes.size(); ++p) {
@@ -514,7 +683,8 @@ int engine_prepare_sets(Handle& h, const nqs_state* psi, const nqs_state* v, voi
                 if (d.type == OP_SITE && save_fwd)
                     d.flags = FL_APPLY | ((!k || block_first[d.site]) ? FL_SAVE_FWD : 0) | (d.flags & FL_KDIAG);
             const PassSpec& ps = segs[bwd ? run.passes.size() - 1 - p : p];
-            add_launch(G, plan, S, ps, 1, ops, (p == 0 && first_in) ? first_in : S.main, S.main, nullptr, bwd);
+            add_launch(G, plan, S, ps, 1, ops, (p == 0 && first_in) ? first_in : S.main, S.main, nullptr,
+                       bwd ? CT_BOUNDARY : CT_PHI);
         }
     };
     auto fill = [&](const nqs_state* st8, const float2*& ext) {
@@ -524,7 +694,7 @@ int engine_prepare_sets(Handle& h, const nqs_state* psi, const nqs_state* v, voi
             l.kind = L_FILL;
             l.dst = S.main;
             l.bits = st8->bits;
-            G.L.push_back(l);
+            G.push(l);
         } else {
             ext = (const float2*)st8->dev;
         }
@@ -540,6 +710,7 @@ int engine_prepare_sets(Handle& h, const nqs_state* psi, const nqs_state* v, voi
     run_passes(run_bwd, bsegs, ext, true, false);
     fill(psi, ext);
     run_passes(run_fwd, plan.free_passes, ext, false, true);
+    G.settle();
     // the matrices of the device table: programs index their own copies, the
     // shared-memory tile kernel reads the table
     for (Launch& l : G.L)
@@ -566,6 +737,7 @@ int engine_eval_sets(Handle& h, int k, const int* sets, size_t m, double* W_out,
             if (s < 0 || s >= S.N || (r > 0 && s <= sets[j * k + r - 1])) return NQS_ERR_ARG;
         }
     Prog G;
+    G.sm_count = S.sm_count;
     const float2* mats_dev = nullptr;
     {
         // the matrix table sits at the end of aux (see engine_prepare_sets)
@@ -590,8 +762,7 @@ int engine_eval_sets(Handle& h, int k, const int* sets, size_t m, double* W_out,
             if (S.mat_block[p] != c) continue;
             std::vector<DevOp> ops(S.mat_ops.begin() + S.mat_pass[p].first,
                                    S.mat_ops.begin() + S.mat_pass[p].first + S.mat_pass[p].second);
-            add_launch(G, plan, S, S.segs[S.mat_seg[p]], 1, ops, first_in ? S.phi[c] : S.work_mat, S.work_mat, nullptr,
-                       false);
+            add_launch(G, plan, S, S.segs[S.mat_seg[p]], 1, ops, first_in ? S.phi[c] : S.work_mat, S.work_mat, nullptr);
             first_in = false;
         }
         ring_block = c;
@@ -606,15 +777,15 @@ int engine_eval_sets(Handle& h, int k, const int* sets, size_t m, double* W_out,
         c.kind = L_COPY;
         c.dst = S.work;
         c.src = S.chi[s1 / K];
-        G.L.push_back(c);
+        G.push(c);
         sweep_range(G, h, S, plan.site_pos[first] - 1, plan.site_pos[s1] - 1, [](int) { return FL_APPLY; }, 1, S.work,
-                    nullptr, [](int, int, int) { return -1ll; });
+                    nullptr, false, [](int, int, int) { return -1ll; });
         return S.work;
     };
     // sweep `states` from linear op `from` through the reduction sites of
     // `slots` (site -> value slot base), one checkpoint block at a time
     auto reduce_through = [&](int from, const std::map<int, long long>& slots, int nst, float2* states,
-                              int mult) {
+                              bool drop) {
         int pos = from;
         for (auto it = slots.begin(); it != slots.end();) {
             const int blk = K ? it->first / K : 0;
@@ -624,81 +795,101 @@ int engine_eval_sets(Handle& h, int k, const int* sets, size_t m, double* W_out,
             const int last = std::prev(end)->first;
             sweep_range(G, h, S, pos, plan.site_pos[last],
                         [&](int t) { return FL_APPLY | (slots.count(t) ? FL_REDUCE : 0); }, nst, states, nullptr,
-                        [&](int t, int st, int f) { return slots.at(t) + st * mult + f; });
+                        drop && end == slots.end(),
+                        [&](int t, int st, int f) { return slots.at(t) + 3 * st + f; });
             pos = plan.site_pos[last];
             it = end;
         }
     };
-    for (size_t i = 0; i < m;) {
-        const int s1 = at(i, 0);
-        size_t i1 = i;
-        while (i1 < m && at(i1, 0) == s1) ++i1;
-        if (k == 1) {
+    if (k == 1) {
+        for (size_t r = 0; r < m; ++r) {
+            const int s1 = at(r, 0);
             const float2* chi = chi_of(s1);
             materialize(K ? s1 / K : 0);
-            for (size_t r = i; r < i1; ++r) {
-                const long long base = (long long)order[r] * 27;
-                Launch l;
-                l.kind = L_REDUCE2;
-                l.src = phi_of(s1);
-                l.dst = const_cast<float2*>(chi);   // read only
-                l.bits = (unsigned long long)h.circ.noises[s1].qubit;
-                const long long npairs = 1ll << (plan.n - 1);
-                l.grid = (int)std::max<long long>(
-                    1, std::min<long long>((long long)S.sm_count * 4, (npairs + 16ll * kThreads - 1) / (16ll * kThreads)));
-                l.part_off = G.take_partials((size_t)l.grid * 8);
-                G.L.push_back(l);
-                add_slot(G, l.part_off, l.grid, s1, h.factors, [&](int f) { return base + f; });
-            }
-            i = i1;
-            continue;
+            const long long base = (long long)order[r] * 27;
+            Launch l;
+            l.kind = L_REDUCE2;
+            l.src = phi_of(s1);
+            l.dst = const_cast<float2*>(chi);   // read only
+            l.bits = (unsigned long long)h.circ.noises[s1].qubit;
+            const long long npairs = 1ll << (plan.n - 1);
+            PassRef pl;
+            G.settle();
+            pl.grid = l.grid = (int)std::max<long long>(
+                1, std::min<long long>((long long)S.sm_count * 4, (npairs + 16ll * kThreads - 1) / (16ll * kThreads)));
+            pl.base = l.part_off = G.take_partials((size_t)l.grid * 8);
+            G.push(l);
+            add_slot(G, pl, 0, 0, s1, h.factors, [&](int f) { return base + f; });
         }
+    }
+    // sets [i, i1) of the first site at(i, 0), as passes of the current lane
+    auto chain = [&](size_t i, size_t i1) {
+        float2* const g1 = S.g1 + (size_t)G.lane * kLaneStates * ((size_t)1 << plan.n);
+        float2* const g2 = g1 + (S.g2 - S.g1);
+        const size_t dim = (size_t)1 << plan.n;
+        const int s1 = at(i, 0), p1 = plan.site_pos[s1], m1 = h.factors[s1].m;
+        if (m1 == 0) return;   // every term is zero
         // spawn K_i chi_{s1} into the first group (shared by every set starting at s1)
-        const int p1 = plan.site_pos[s1];
-        const int m1 = h.factors[s1].m;
         const PassSpec& ps1 = S.fsegs[pass_of(S.fsegs, p1)];
-        {
-            auto ops = emit_range(plan, S, ps1, p1, p1 + 1, [&](int) { return FL_SPAWN; }, h.factors);
-            const float2* chi = chi_of(s1);
-            add_launch(G, plan, S, ps1, 1, ops, chi, S.scratch, S.g1, false);
-        }
+        const float2* chi = chi_of(s1);
+        add_launch(G, plan, S, ps1, 1, emit_range(plan, S, ps1, p1, p1 + 1, [](int) { return FL_SPAWN; }, h.factors), chi,
+                   nullptr, g1);
         if (k == 2) {
             std::map<int, long long> base2;   // second site -> value slots of its set
             for (size_t r = i; r < i1; ++r) base2[at(r, 1)] = (long long)order[r] * 27;
-            reduce_through(p1, base2, m1, S.g1, 3);
-            i = i1;
-            continue;
+            reduce_through(p1, base2, m1, g1, true);
+            return;
         }
-        int pos = p1;
+        int pos = p1;   // operations up to here are applied to the first group
         for (size_t r = i; r < i1;) {
-            const int s2 = at(r, 1), p2 = plan.site_pos[s2];
+            const int s2 = at(r, 1), p2 = plan.site_pos[s2], m2 = h.factors[s2].m;
             size_t r2 = r;
             while (r2 < i1 && at(r2, 1) == s2) ++r2;
+            std::map<int, long long> base3;   // third site -> value slots of its set
+            long long back = 0;
+            for (size_t q = r; q < r2; ++q) {
+                base3[at(q, 2)] = (long long)order[q] * 27;
+                back += (long long)h.factors[at(q, 2)].m * (plan.site_pos[at(q, 2)] - p2);
+            }
+            const long long fwd = (long long)m1 * m2 * (plan.site_pos[base3.rbegin()->first] - p2);
+            if (m2 == 0) {
+                r = r2;
+                continue;
+            }
+            if (!K && plan.k == kMaxTileQ && back <= fwd) {
+                for (auto it = base3.begin(); it != base3.end(); ++it) {
+                    const int s3 = it->first, p3 = plan.site_pos[s3], m3 = h.factors[s3].m;
+                    if (m3 == 0) continue;
+                    const PassSpec& ps3 = S.fsegs[pass_of(S.fsegs, p3)];
+                    add_launch(G, plan, S, ps3, 1,
+                               emit_range(plan, S, ps3, p3, p3 + 1, [](int) { return FL_SPAWN; }, h.factors, true), S.phi[s3],
+                               nullptr, g2);
+                    sweep_back(G, h, S, p2, p3, m3, g2);
+                    sweep_and_meet(G, h, S, pos + 1, p2, m1, g1, m3, r2 == i1 && std::next(it) == base3.end(),
+                                   [&](int j, int st, int f) { return it->second + 9 * st + 3 * f + j; });
+                    pos = p2 - 1;
+                }
+                r = r2;
+                continue;
+            }
             // carry the first group to s2 (K_0 there), spawning the nine states
-            sweep_range(G, h, S, pos, p2, [&](int t) { return FL_APPLY | (t == s2 ? FL_SPAWN : 0); }, m1, S.g1, S.g2,
+            sweep_range(G, h, S, pos, p2, [&](int t) { return FL_APPLY | (t == s2 ? FL_SPAWN : 0); }, m1, g1, g2, false,
                         [](int, int, int) { return -1ll; });
             pos = p2;
-            std::map<int, long long> base3;   // third site -> value slots of its set
-            for (size_t q = r; q < r2; ++q) base3[at(q, 2)] = (long long)order[q] * 27;
-            const int m2 = h.factors[s2].m;
-            if (!K) {
-                for (int g = 0; g < m1; ++g) {
-                    std::map<int, long long> bg = base3;
-                    for (auto& e : bg) e.second += g * 9;
-                    reduce_through(p2, bg, m2, S.g2 + (size_t)3 * g * ((size_t)1 << plan.n), 3);
-                }
+            if (m2 == 3 && plan.k == kMaxTileQ) {
+                reduce_through(p2, base3, 3 * m1, g2, true);
             } else {
-                // one block at a time for all three groups, so each block's phi is recomputed once
+                // one checkpoint block at a time for all groups, so each block's phi is recomputed once
                 int gpos[3] = {p2, p2, p2};
                 for (auto it = base3.begin(); it != base3.end();) {
-                    const int blk = it->first / K;
+                    const int blk = K ? it->first / K : 0;
                     auto end = it;
-                    while (end != base3.end() && end->first / K == blk) ++end;
+                    while (end != base3.end() && (!K || end->first / K == blk)) ++end;
                     std::map<int, long long> part(it, end);
                     for (int g = 0; g < m1; ++g) {
                         std::map<int, long long> bg = part;
                         for (auto& e : bg) e.second += g * 9;
-                        reduce_through(gpos[g], bg, m2, S.g2 + (size_t)3 * g * ((size_t)1 << plan.n), 3);
+                        reduce_through(gpos[g], bg, m2, g2 + (size_t)3 * g * dim, false);
                         gpos[g] = plan.site_pos[std::prev(end)->first];
                     }
                     it = end;
@@ -706,8 +897,36 @@ int engine_eval_sets(Handle& h, int k, const int* sets, size_t m, double* W_out,
             }
             r = r2;
         }
-        i = i1;
+    };
+    if (k > 1) {
+        // chains, the longest first, each to the lane with the least work
+        struct Chain {
+            size_t begin, end;
+            long long ops;
+        };
+        std::vector<Chain> chains;
+        for (size_t i = 0; i < m;) {
+            Chain c{i, i, 0};
+            while (c.end < m && at(c.end, 0) == at(i, 0)) {
+                const size_t r = c.end++;
+                c.ops += plan.site_pos[at(r, k - 1)] - plan.site_pos[at(r, 0)];
+            }
+            chains.push_back(c);
+            i = c.end;
+        }
+        const int lanes = std::min<int>(S.lanes, (int)chains.size());
+        if (lanes > 1)
+            std::stable_sort(chains.begin(), chains.end(), [](const Chain& x, const Chain& y) { return x.ops > y.ops; });
+        G.lanes.resize(lanes);
+        for (const Chain& c : chains) {
+            G.lane = 0;
+            for (int l = 1; l < lanes; ++l)
+                if (G.lanes[l].size() < G.lanes[G.lane].size()) G.lane = l;
+            chain(c.begin, c.end);
+        }
+        G.lane = 0;
     }
+    G.settle();
     for (Launch& l : G.L)
         if (l.kind == L_PASS && !l.units()) l.args.mats = mats_dev;
     void* vals = nullptr;

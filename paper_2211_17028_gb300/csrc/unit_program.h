@@ -94,7 +94,7 @@ UnitProgram assemble_unit(bool single, const std::vector<DevOp>& dops, int off, 
 // One state swept through one pass: `ctas` consecutive blocks share its tiles.
 struct SweepUnit {
     const float2* in;
-    float2* out;
+    float2* out;               // null: the swept state is not kept
     float2* spawn;             // spawned state (slot k, factor i) at spawn + ((3 k + i) << n)
     const uint4* prog;
     float2* const* ckpt;       // phi_s
