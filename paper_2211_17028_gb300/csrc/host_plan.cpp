@@ -177,56 +177,6 @@ void lookahead_order(Plan& p, int max_sites, int max_ops, std::vector<PassSpec>&
         if (p.ops[i].type == OP_SITE) p.site_pos[p.ops[i].site] = i;
 }
 
-// Orders the operations of every pass so that they fall into few phases (runs
-// whose dense qubits fit in the four register qubits of the unit kernel): every
-// phase costs a trip of the tile through shared memory, about as much time as
-// three gates.  Phase by phase, the registers take the qubit of the first
-// remaining dense operation and then, one at a time, the qubits that let the
-// phase take the most operations.  In circuit order a sweep of the 20-qubit grid
-// (16 layers, 20 noises) has 64 phases, in this order 30: its level-2 call takes
-// 6.05 instead of 6.58 ms, 25 qubits level 1 13.8 instead of 15.4 ms.
-void phase_order(Plan& p, const std::vector<PassSpec>& passes) {
-    constexpr int kRegs = 4;
-    for (const PassSpec& ps : passes) {
-        std::vector<HostOp> ops(p.ops.begin() + ps.op_begin, p.ops.begin() + ps.op_end);
-        std::vector<OpMask> masks(ops.size());
-        std::vector<int> rest(ops.size()), order, keep;
-        for (size_t i = 0; i < ops.size(); ++i) {
-            masks[i].q = (1ull << ops[i].q0) | (ops[i].q1 >= 0 ? 1ull << ops[i].q1 : 0ull);
-            masks[i].diag = op_is_diag(ops[i]);
-            masks[i].site = ops[i].type == OP_SITE;
-            rest[i] = (int)i;
-        }
-        while (!rest.empty()) {
-            uint64_t tile = 0, cand = 0;
-            for (int i : rest)
-                if (!masks[i].diag) {
-                    if (!tile) tile = masks[i].q;
-                    cand |= masks[i].q;
-                }
-            while (__builtin_popcountll(tile) < kRegs && (cand & ~tile)) {
-                uint64_t best = 0;
-                int best_v = -1;
-                for (uint64_t left = cand & ~tile; left; left &= left - 1) {
-                    const uint64_t q = left & (~left + 1);
-                    const int v = take_pass(masks, rest, tile | q, 1 << 30, 1 << 30, nullptr, nullptr);
-                    if (v > best_v) {
-                        best_v = v;
-                        best = q;
-                    }
-                }
-                tile |= best;
-            }
-            keep.clear();
-            take_pass(masks, rest, tile, 1 << 30, 1 << 30, &order, &keep);
-            rest.swap(keep);
-        }
-        for (size_t i = 0; i < ops.size(); ++i) p.ops[ps.op_begin + i] = ops[order[i]];
-    }
-    for (int i = 0; i < (int)p.ops.size(); ++i)
-        if (p.ops[i].type == OP_SITE) p.site_pos[p.ops[i].site] = i;
-}
-
 }  // namespace
 
 void build_plan(const Circuit& c, const std::vector<Factors>& f, int tile_qubits, Plan& p) {
@@ -372,7 +322,6 @@ void build_plan(const Circuit& c, const std::vector<Factors>& f, int tile_qubits
         const char* e = std::getenv("NQS_PLAN_REORDER");   // 0: keep the circuit order
         if (!(e && e[0] == '0')) {
             lookahead_order(p, 4, 96, p.grouped_passes);
-            phase_order(p, p.grouped_passes);
             p.free_passes = p.grouped_passes;
         } else {
             p.free_passes = segment(p, false, 4, 96);
