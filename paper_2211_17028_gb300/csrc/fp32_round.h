@@ -54,6 +54,8 @@ inline double distance2(const float* x, const cdr* m, int n) {
 inline float2 round_c64(std::complex<double> c) {
     float re = (float)c.real(), im = (float)c.imag();
     if (std::fabs(std::abs(c) - 1.0) > 1e-9) return make_float2(re, im);
+    // 1, i, -1, -i are their own best neighbours (nearly every call of the program assembler)
+    if (c.real() * c.imag() == 0.0 && std::fabs(c.real()) + std::fabs(c.imag()) == 1.0) return make_float2(re, im);
     float best_re = re, best_im = im;
     double best = 1e300;
     for (int a = -1; a <= 1; ++a)

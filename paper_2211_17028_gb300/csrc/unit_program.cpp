@@ -212,7 +212,10 @@ struct RatioAssembler : Records {
     std::vector<cd> carry;   // constant ratio pending on each tile position across phases
     std::vector<int> regs;
 
-    static bool one(cd c) { return is(round_c64(c), 1.f); }
+    static bool one(cd c) {
+        if (c == cd(1.0)) return true;
+        return std::fabs(c.real() - 1.0) < 1e-7 && std::fabs(c.imag()) < 1e-7 && is(round_c64(c), 1.f);
+    }
     int put_c(std::initializer_list<cd> v) {
         float2 f[4];
         int n = 0;
@@ -409,24 +412,21 @@ UnitProgram assemble(const std::vector<DevOp>& dops, int off, int n, const int* 
         }
     // phases: runs of operations whose dense qubits fit in the register bits
     std::vector<std::pair<int, int>> ranges;
-    std::vector<std::vector<int>> regs;
-    std::vector<int> cur;
+    std::vector<unsigned> regs;      // their tile positions
+    unsigned cur = 0;
     int begin = 0;
     for (int o = 0; o < n; ++o) {
         const DevOp& d = dops[off + o];
-        int need[2], cnt = 0;
-        if (d.type == OP_G1 || d.type == OP_SITE || d.type == OP_G2) need[cnt++] = d.a;
-        if (d.type == OP_G2) need[cnt++] = d.b;
-        std::vector<int> u = cur;
-        for (int c = 0; c < cnt; ++c)
-            if (std::find(u.begin(), u.end(), need[c]) == u.end()) u.push_back(need[c]);
-        if ((int)u.size() > kUnitRB) {
+        unsigned need = 0;
+        if (d.type == OP_G1 || d.type == OP_SITE || d.type == OP_G2) need |= 1u << d.a;
+        if (d.type == OP_G2) need |= 1u << d.b;
+        if (__builtin_popcount(cur | need) > kUnitRB) {
             ranges.push_back({begin, o});
             regs.push_back(cur);
-            cur.assign(need, need + cnt);
+            cur = need;
             begin = o;
         } else {
-            cur.swap(u);
+            cur |= need;
         }
     }
     ranges.push_back({begin, n});
@@ -435,9 +435,13 @@ UnitProgram assemble(const std::vector<DevOp>& dops, int off, int n, const int* 
     Asm A;
     std::vector<UnitPhase> phases;
     for (size_t p = 0; p < ranges.size(); ++p) {
-        std::vector<int> R = regs[p];
+        std::vector<int> R;
         bool used[K] = {};
-        for (int q : R) used[q] = true;
+        for (int q = 0; q < K; ++q)
+            if (regs[p] >> q & 1) {
+                R.push_back(q);
+                used[q] = true;
+            }
         for (int q = K - 1; q >= 0 && (int)R.size() < kUnitRB; --q)
             if (!used[q]) {
                 R.push_back(q);
