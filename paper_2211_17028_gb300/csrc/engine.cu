@@ -635,7 +635,7 @@ struct Builder {
             too_big = true;
             return;
         }
-        const int per_sm = unit_blocks_per_sm(cur.smem);
+        const int per_sm = unit_blocks_per_sm(cur.unit_kind, cur.smem);
         cur.ctas = unit_ctas(cur.n_units, units[first_unit].n_tiles, per_sm * E.sm_count);
         cur.grid = cur.ctas * cur.n_units;
         size_t need = 0;

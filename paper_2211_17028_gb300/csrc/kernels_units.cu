@@ -7,22 +7,29 @@
 // TMA bulk copies (256-byte runs of the five low qubits) while the current one
 // is processed; every wait on the copies' mbarrier is bounded.
 //
-// What bounds it: issue slots (a dense one-qubit gate is 8 FP32 multiply-adds
-// per amplitude) wherever the launch fills the chip, the latency of one tile
-// where it does not.  Hence
-// * one state per block and two blocks per SM, instead of the three states of
-//   a branch group in one block of 512 threads: three times as many blocks on
-//   a narrow circuit, and twice the amplitudes per decoded operation;
+// What bounds it: issue slots wherever the launch fills the chip (a quarter of
+// the instructions are packed FP32; the rest decode, swap halves and form
+// addresses), the latency of one tile where it does not.  Hence
+// * one state per block and two or three blocks per SM, instead of the three
+//   states of a branch group in one block of 512 threads: three times as many
+//   blocks on a narrow circuit, and twice the amplitudes per decoded operation;
 // * the program says what to do with pending diagonal factors (unit_program.h),
 //   so an operation is a record, a jump and its arithmetic: no flags, no
 //   loops over register bits;
+// * the gates of a layer, up to one per register bit, share a record, and that
+//   record is tested for first: decoding is a tree of compares (no jump table),
+//   ten branches per operation;
 // * thread bits and the bits of the tile's number sit in one word, so a
 //   diagonal on any qubit outside the registers is one indexed table read;
-// * the re-layout buffers alternate (one barrier per re-layout) and are padded
-//   (index j at j + j/16 + j/256: additive, and lanes on positions of distinct
-//   residue mod 4 meet distinct banks).
-// One pass of 2^20 amplitudes x 60 states with 24 dense gates: see the figures
-// at launch_units.
+// * the re-layout buffers are padded (index j at j + j/16 + j/256: additive, and
+//   lanes on positions of distinct residue mod 4 meet distinct banks).
+// The order of an amplitude's operations is the circuit's: the lowest level of
+// a basis test state is one amplitude, whose error of about 1e-6 is the rounding
+// of this order.  Gates as a phase and a real rotation (a third of the products)
+// in an order of half as many phases ran 20 qubits level 2 in 5.4 ms, and rounded
+// that amplitude up to three times worse on some inputs.
+#include <algorithm>
+
 #include "mbar.cuh"
 #include "nqs_internal.h"
 #include "unit_program.h"
@@ -43,9 +50,14 @@ __device__ __forceinline__ int relay_map(int j) { return j + (j >> 4) + (j >> 8)
 __device__ __forceinline__ int stage_map(int j) { return j + 2 * (j >> 5) + 2 * (j >> 9); }
 constexpr int kRelayAmps = kAmps + (kAmps >> 4) + (kAmps >> 8);
 constexpr int kStageAmps = kAmps + 2 * (kAmps >> 5) + 2 * (kAmps >> 9);
-constexpr int kRelayBufs = 2;
-constexpr int kBlocksPerSm = 2;
-constexpr size_t kFixedSmem = ((size_t)kStageAmps + kRelayBufs * kRelayAmps) * sizeof(float2);
+// Two forms of the kernel.  Two blocks per SM: 128 registers, two alternating
+// re-layout buffers.  Three blocks: 80 registers (30 words spilled) and one
+// buffer with a second barrier per re-layout; half as many warps again hide more
+// of the latency of decoding and of the sites' loads, so it is used where the
+// launch has blocks for it and the program leaves room (5 % less time on 20
+// qubits at level 2; 7 % more on 13 qubits, whose 66 tiles do not fill the chip).
+constexpr int relay_bufs(int blocks) { return blocks == 2 ? 2 : 1; }
+constexpr size_t fixed_smem(int blocks) { return ((size_t)kStageAmps + relay_bufs(blocks) * kRelayAmps) * sizeof(float2); }
 
 // An amplitude is one 64-bit register pair (re in the low word) and every
 // product on it a packed FP32x2 operation written as such: kept as two floats,
@@ -138,13 +150,16 @@ struct Pend {
 
 // the dense gate of a record: its matrix with the pending factors it takes
 template <int I, bool SINGLE, bool PAIRS>
-__device__ __forceinline__ void u_gate(c64 (&x)[kE], const UnitRec& op, const float2* __restrict__ m, Pend<PAIRS>& P,
+__device__ __forceinline__ void u_gate(c64 (&x)[kE], const UnitRec& op, const float2* __restrict__ mats, Pend<PAIRS>& P,
                                        uint32_t bits) {
+    const int fl = (int)(op.mask >> (8 * I));
+    if (!(fl & UF_HERE)) return;
+    const float2* const m = mats + op.off[I] + 2;
     Fac k[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) k[e] = ld_fac(m + 2 * e);
-    if (op.flags & UF_SCALAR) {
-        if (op.flags & UF_REAL) {
+    if (fl & UF_SCALAR) {
+        if (fl & UF_REAL) {
 #pragma unroll
             for (int e = 0; e < 4; ++e) k[e] = times_real(k[e], P.d.x);
         } else {
@@ -153,7 +168,7 @@ __device__ __forceinline__ void u_gate(c64 (&x)[kE], const UnitRec& op, const fl
         }
         P.d = make_float2(1.f, 0.f);
     }
-    if (op.flags & UF_DIAG) {
+    if (fl & UF_DIAG) {
         if (PAIRS) {
             k[0] = times(k[0], P.h[I][0]);
             k[2] = times(k[2], P.h[I][0]);
@@ -162,8 +177,8 @@ __device__ __forceinline__ void u_gate(c64 (&x)[kE], const UnitRec& op, const fl
         k[3] = times(k[3], P.h[I][PAIRS ? 1 : 0]);
         P.clear(I);
     }
-    if (op.flags & UF_SIGN) {
-        const float f = (__popc(bits & op.mask) & 1) ? -1.f : 1.f;
+    if (fl & UF_SIGN) {
+        const float f = (__popc(bits & __float_as_uint(m[-2].x)) & 1) ? -1.f : 1.f;
         k[1] = times_real(k[1], f);
         k[3] = times_real(k[3], f);
     }
@@ -239,6 +254,15 @@ __device__ __forceinline__ void u_negate(c64 (&x)[kE]) {
 #pragma unroll
     for (int r = 0; r < kE; ++r)
         if ((r >> I0 & 1) && (r >> I1 & 1)) x[r] = mul2(pk(-1.f, -1.f), x[r]);
+}
+
+__device__ __forceinline__ void u_negate_pairs(c64 (&x)[kE], int pairs) {
+    if (pairs & 1) u_negate<0, 1>(x);
+    if (pairs & 2) u_negate<0, 2>(x);
+    if (pairs & 4) u_negate<0, 3>(x);
+    if (pairs & 8) u_negate<1, 2>(x);
+    if (pairs & 16) u_negate<1, 3>(x);
+    if (pairs & 32) u_negate<2, 3>(x);
 }
 
 template <int I0, int I1, bool PAIRS>
@@ -328,8 +352,9 @@ __device__ __forceinline__ void u_site(const UnitRec& op, const float2* __restri
         for (int r = 0; r < kE; ++r) __stcs(save + off(r), x[r]);
     }
     if (fl & FL_REDUCE) {
-        // conj(f) a accumulated as A += f.x a, B += f.y a (no swapped operands):
-        // conj(f) a = (A.x + B.y, A.y - B.x)
+        // conj(f) a accumulated as A += (f.x a.x, f.y a.y), B += (f.x a.y, f.y a.x):
+        // conj(f) a = (A.x + A.y, B.x - B.y).  The swapped amplitudes serve both
+        // values of phi, and phi is used as it was loaded.
         const c64* const phi = reinterpret_cast<const c64*>(slot[op.ev]);
         c64 A[4], B[4];
 #pragma unroll
@@ -350,25 +375,24 @@ __device__ __forceinline__ void u_site(const UnitRec& op, const float2* __restri
             for (int r = 0; r < kE; ++r) {
                 if (r & (1 << I)) continue;
                 if (((r >> (I == 3 ? 2 : 3)) & 1) != h) continue;
-                const float2 f0 = unpk(f[k]), f1 = unpk(f[k + 1]);
+                const c64 f0 = f[k], f1 = f[k + 1];
                 k += 2;
-                const c64 a = x[r], b = x[r | (1 << I)];
-                const c64 f0x = pk(f0.x, f0.x), f0y = pk(f0.y, f0.y), f1x = pk(f1.x, f1.x), f1y = pk(f1.y, f1.y);
-                A[0] = fma2(f0x, a, A[0]);
-                B[0] = fma2(f0y, a, B[0]);
-                A[1] = fma2(f0x, b, A[1]);
-                B[1] = fma2(f0y, b, B[1]);
-                A[2] = fma2(f1x, a, A[2]);
-                B[2] = fma2(f1y, a, B[2]);
-                A[3] = fma2(f1x, b, A[3]);
-                B[3] = fma2(f1y, b, B[3]);
+                const c64 a = x[r], b = x[r | (1 << I)], as = swp(a), bs = swp(b);
+                A[0] = fma2(f0, a, A[0]);
+                B[0] = fma2(f0, as, B[0]);
+                A[1] = fma2(f0, b, A[1]);
+                B[1] = fma2(f0, bs, B[1]);
+                A[2] = fma2(f1, a, A[2]);
+                B[2] = fma2(f1, as, B[2]);
+                A[3] = fma2(f1, b, A[3]);
+                B[3] = fma2(f1, bs, B[3]);
             }
         }
         float v[8];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             const float2 a = unpk(A[e]), b = unpk(B[e]);
-            float2 R = make_float2(a.x + b.y, a.y - b.x);
+            float2 R = make_float2(a.x + a.y, b.x - b.y);
             if (!SINGLE) R = cmul(m[0], R);   // the scale of the state
             v[2 * e] = R.x;
             v[2 * e + 1] = R.y;
@@ -410,17 +434,18 @@ __device__ __forceinline__ void u_site(const UnitRec& op, const float2* __restri
     }
 }
 
-template <bool SINGLE, bool PAIRS>
-__global__ void __launch_bounds__(kNT, kBlocksPerSm) unit_sweep_kernel(const SweepUnit* __restrict__ units,
-                                                            const int* __restrict__ blk, int ctas) {
+template <bool SINGLE, bool PAIRS, int BLOCKS>
+__global__ void __launch_bounds__(kNT, BLOCKS) unit_sweep_kernel(const SweepUnit* __restrict__ units,
+                                                                const int* __restrict__ blk, int ctas) {
+    constexpr int kRelayBufs = relay_bufs(BLOCKS);
+    constexpr size_t kFixedSmem = fixed_smem(BLOCKS);
     extern __shared__ __align__(128) unsigned char dyn[];
     float2* const stage = reinterpret_cast<float2*>(dyn);
-    float2* const relay = stage + kStageAmps;                                  // two buffers
+    float2* const relay = stage + kStageAmps;                                  // one or two buffers
     __shared__ __align__(16) SweepUnit u;
     __shared__ __align__(8) uint64_t bar;
     __shared__ unsigned long long hi_off[kChunks];
     __shared__ float2* slot[kUnitSlots];
-    __shared__ unsigned long long next_base;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int ui = blk ? blk[blockIdx.x] : (int)blockIdx.x / ctas;
@@ -481,34 +506,30 @@ __global__ void __launch_bounds__(kNT, kBlocksPerSm) unit_sweep_kernel(const Swe
             bulk_prefetch_l2(slot[q / kChunks] + (b | hi_off[q % kChunks]), kChunk * sizeof(float2));
     };
 
-    int t = cta;
-    if (t < n_tiles) {
-        const unsigned long long b = tile_base(t);
-        if (tid == 0) next_base = b;
-        prefetch(b);
-    }
+    // the next tile's base: the tile number's bits lie on the set bits of nl, so
+    // with ones everywhere else a carry runs from one of them to the next
+    const unsigned long long step = tile_base(nctas);
+    unsigned long long base = tile_base(cta), next = base;
+    if (cta < n_tiles) prefetch(base);
     uint32_t parity = 0;
     bool failed = false;
     c64 x[kE];
     int buf = 0;   // re-layout buffer to write next
 
-    for (; t < n_tiles; t += nctas) {
+    for (int t = cta; t < n_tiles; t += nctas) {
         const uint32_t bits = (uint32_t)tid | ((uint32_t)t << 8);
         const bool ok = mbar_wait_bounded(&bar, parity);
         if (__syncthreads_or(!ok)) {
             failed = true;
             break;
         }
-        const unsigned long long base = next_base;
+        base = next;
+        next = ((base | ~nl) + step) & nl;
         parity ^= 1u;
         int jT = thread_j(phases[0], lane, warp);
         move_tile<false>(x, stage, phases[0], jT, stage_map);
         __syncthreads();   // the staging buffer is free again
-        if (t + nctas < n_tiles) {
-            const unsigned long long b = tile_base(t + nctas);
-            if (tid == 0) next_base = b;
-            prefetch(b);
-        }
+        if (t + nctas < n_tiles) prefetch(next);
         const float2 unit1 = make_float2(1.f, 0.f);
         Pend<PAIRS> P;
         P.clear();
@@ -543,8 +564,15 @@ __global__ void __launch_bounds__(kNT, kBlocksPerSm) unit_sweep_kernel(const Swe
     case F + 3: { constexpr int I = 1, J = 2; BODY; break; }  \
     case F + 4: { constexpr int I = 1, J = 3; BODY; break; }  \
     case F + 5: { constexpr int I = 2, J = 3; BODY; break; }
+                if (op.code == UO_G1) {   // the most frequent one, ahead of the tree of the others
+                    if (op.a) u_negate_pairs(x, op.a);
+                    u_gate<0, SINGLE, PAIRS>(x, op, mats, P, bits);
+                    u_gate<1, SINGLE, PAIRS>(x, op, mats, P, bits);
+                    u_gate<2, SINGLE, PAIRS>(x, op, mats, P, bits);
+                    u_gate<3, SINGLE, PAIRS>(x, op, mats, P, bits);
+                    continue;
+                }
                 switch (op.code) {
-                    U_FOUR(UO_G1, (u_gate<I, SINGLE, PAIRS>(x, op, m, P, bits)))
                     U_FOUR(UO_GK, const Fac k[4] = {ld_fac(m) U_COMMA ld_fac(m + 2) U_COMMA ld_fac(m + 4) U_COMMA ld_fac(m + 6)};
                            (u_dense<I, true>(x, k)))
                     U_FOUR(UO_KD, if (op.flags & UF_REAL) u_by_bit_real<I>(x, m[0].x, m[1].x);
@@ -557,7 +585,7 @@ __global__ void __launch_bounds__(kNT, kBlocksPerSm) unit_sweep_kernel(const Swe
                     U_FOUR(UO_HP, const int at = c * P.W; P.h[I][0] = cmul(P.h[I][0], m[at]);
                            if (PAIRS) P.h[I][P.W - 1] = cmul(P.h[I][P.W - 1], m[at + 1]))
                     U_FOUR(UO_SITE, (u_site<I, SINGLE>(op, m, x, phases[p], jT, u, hi_off, slot, base, acc, lane, warp)))
-                    U_PAIRS(UO_DN, (u_negate<I, J>(x)))
+                    case UO_DN: u_negate_pairs(x, op.a); break;
                     U_PAIRS(UO_DG, (u_diag2<I, J, PAIRS>(x, m)))
                     U_PAIRS(UO_G2, (u_g2<I, J, PAIRS>(x, op, m, P)))
                     U_PAIRS(UO_G2 + 6, (u_g2<J, I, PAIRS>(x, op, m, P)))
@@ -647,24 +675,59 @@ __global__ void bounded_wait_probe_kernel(int* status) {
 }  // namespace
 
 size_t unit_smem_bytes(int max_words, int max_events) {
-    return kFixedSmem + (size_t)max_words * 16 + (size_t)max_events * kNW * 8 * sizeof(double);
+    return fixed_smem(2) + (size_t)max_words * 16 + (size_t)max_events * kNW * 8 * sizeof(double);
 }
 
-int unit_blocks_per_sm(size_t smem) {
+namespace {
+
+using UnitKernel = void (*)(const SweepUnit*, const int*, int);
+
+// branch groups mostly keep ratios; a diagonal with zeros has none
+UnitKernel unit_kernel(int kind, int blocks) {
+    if (kind == unit_kind(true, UM_PAIRS)) return unit_sweep_kernel<true, true, 2>;
+    if (kind == unit_kind(false, UM_PAIRS)) return unit_sweep_kernel<false, true, 2>;
+    if (kind == unit_kind(true, UM_RATIOS)) return blocks == 3 ? unit_sweep_kernel<true, false, 3> : unit_sweep_kernel<true, false, 2>;
+    return blocks == 3 ? unit_sweep_kernel<false, false, 3> : unit_sweep_kernel<false, false, 2>;
+}
+
+// shared memory of the three-block form for a program that needs `smem` in the other
+size_t smem_of(int blocks, size_t smem) { return smem - fixed_smem(2) + fixed_smem(blocks); }
+
+int attribute(cudaDeviceAttr a) {
+    int dev = 0, v = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&v, a, dev);
+    return v;
+}
+
+// whether three blocks of such a program fit an SM (1 KB per block is the
+// system's; pairs in 80 registers would spill 900 bytes)
+bool three_fit(int kind, size_t smem) {
+    if (kind == unit_kind(true, UM_PAIRS) || kind == unit_kind(false, UM_PAIRS)) return false;
+    static const size_t fixed = [] {
+        cudaFuncAttributes a{};
+        return cudaFuncGetAttributes(&a, unit_sweep_kernel<true, false, 3>) == cudaSuccess ? a.sharedSizeBytes : (size_t)2048;
+    }();
+    return 3 * (smem_of(3, smem) + fixed + 1024) <= (size_t)attribute(cudaDevAttrMaxSharedMemoryPerMultiprocessor);
+}
+
+}  // namespace
+
+int unit_blocks_per_sm(int kind, size_t smem) {
+    if (three_fit(kind, smem)) return 3;
     int nb = 0;
-    cudaFuncSetAttribute(unit_sweep_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, unit_sweep_kernel<true, true>, kNT, smem);
+    const UnitKernel k = unit_kernel(kind, 2);
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, kNT, smem);
     return nb > 0 ? nb : 1;
 }
 
 cudaError_t launch_units(int kind, const SweepUnit* units, const int* blk, int ctas, int total_ctas, size_t smem,
                          cudaStream_t st) {
-    // branch groups mostly keep ratios; a diagonal with zeros has none
-    auto* const kernel = kind == unit_kind(true, UM_RATIOS)  ? unit_sweep_kernel<true, false>
-                         : kind == unit_kind(true, UM_PAIRS) ? unit_sweep_kernel<true, true>
-                         : kind == unit_kind(false, UM_PAIRS) ? unit_sweep_kernel<false, true>
-                                                              : unit_sweep_kernel<false, false>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const int blocks = total_ctas > 2 * attribute(cudaDevAttrMultiProcessorCount) && three_fit(kind, smem) ? 3 : 2;
+    const UnitKernel kernel = unit_kernel(kind, blocks);
+    smem = smem_of(blocks, smem);
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     kernel<<<total_ctas, kNT, smem, st>>>(units, blk, ctas);
     return cudaGetLastError();

@@ -161,7 +161,7 @@ struct Prog {
                     l.smem = std::max(l.smem, s->smem);
                     l.n_phases = std::max(l.n_phases, s->n_phases);
                 }
-                l.ctas = unit_ctas(l.n_units, steps[0]->units[0].n_tiles, unit_blocks_per_sm(l.smem) * sm_count);
+                l.ctas = unit_ctas(l.n_units, steps[0]->units[0].n_tiles, unit_blocks_per_sm(kind, l.smem) * sm_count);
                 l.grid = l.ctas * l.n_units;
                 size_t need = 0;
                 for (const Step* s : steps) need += s->units.size() * s->n_events * l.ctas * 8;

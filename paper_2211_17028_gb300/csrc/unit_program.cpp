@@ -30,12 +30,15 @@ struct Records {
         return at;
     }
     // a 2x2 matrix as the packed operands of the kernel: (re, re), (-im, im) per entry
-    int put_matrix(const float2* f) {
-        float2 v[8];
+    static void packed(const float2* f, float2* v) {
         for (int e = 0; e < 4; ++e) {
             v[2 * e] = make_float2(f[e].x, f[e].x);
             v[2 * e + 1] = make_float2(-f[e].y, f[e].y);
         }
+    }
+    int put_matrix(const float2* f) {
+        float2 v[8];
+        packed(f, v);
         return put(v, 8);
     }
     UnitRec& emit(int code, int a = kNoLoc, int b = kNoLoc) {
@@ -45,6 +48,56 @@ struct Records {
         r.b = (unsigned char)b;
         recs.push_back(r);
         return recs.back();
+    }
+    // Dense gates that nothing on their bit separates share a record, in the
+    // order of their bits (so every amplitude sees the same arithmetic as with a
+    // record each): decoding a record costs about as much as a third of a gate.
+    size_t joint = 0;        // 1 + record that more gates may join
+    size_t first = 0;        // first record of the phase
+    int last_bit = 0;        // bit of the last gate
+    static int pairs_of(int i) {
+        int m = 0;
+        for (int j = 0; j < 4; ++j)
+            if (j != i) m |= 1 << unit_pair(std::min(i, j), std::max(i, j));
+        return m;
+    }
+    bool joins(int i, int flags) const {
+        if (joint == 0 || (recs[joint - 1].mask >> (8 * i)) != 0) return false;   // a bit below the ones there
+        for (size_t k = joint; k < recs.size(); ++k) {
+            const int code = recs[k].code;
+            if (!((code >= UO_HP && code < UO_HP + 4 && code != UO_HP + i) || (code == UO_SC && !(flags & UF_SCALAR)) ||
+                  (code == UO_DN && !(recs[k].a & pairs_of(i)))))
+                return false;
+        }
+        return true;
+    }
+    void gate_record(int i, const float2* f, int flags, uint32_t sign) {
+        float2 v[10] = {};
+        std::memcpy(&v[0].x, &sign, sizeof(sign));
+        packed(f, v + 2);
+        const int at = put(v, 10);
+        if (!joins(i, flags)) {
+            unsigned char before = 0;
+            if (recs.size() > first && recs.back().code == UO_DN) {
+                before = recs.back().a;
+                recs.pop_back();
+            }
+            emit(UO_G1, before);
+            joint = recs.size();
+        }
+        UnitRec& r = recs[joint - 1];
+        r.off[i] = (unsigned short)at;
+        r.mask |= (unsigned)(flags | UF_HERE) << (8 * i);
+        last_bit = i;
+    }
+    // negate where both bits of a pair are set
+    void negate(int pair) {
+        if (recs.size() <= first || recs.back().code != UO_DN) emit(UO_DN, 0);
+        recs.back().a ^= (unsigned char)(1 << pair);
+    }
+    void start_phase() {
+        joint = 0;
+        first = recs.size();
     }
     // K_0 of a site on register bit i, and the record of its other actions
     void apply_site(int i, const float2* m, bool diag) {
@@ -119,7 +172,7 @@ struct PairAssembler : Records {
     cd scale() const { return 1.0; }   // of what a site sees
     void at_site() { flush(); }
     void at_end(bool) { flush(); }
-    void begin_phase(const std::vector<int>&) {}
+    void begin_phase(const std::vector<int>&) { start_phase(); }
     void outside(int, int) {}
     // multiply everything pending into the amplitudes
     void flush() {
@@ -145,14 +198,12 @@ struct PairAssembler : Records {
         }
         scal = false;
         scal_real = true;
+        joint = 0;
     }
     void g1(int i, const float2* m) {
-        const int at = put_matrix(m);
-        UnitRec& r = emit(UO_G1 + i);
-        r.mat = (unsigned short)at;
-        r.flags = (unsigned char)((pair[i] ? UF_DIAG : 0) | (sign[i] ? UF_SIGN : 0) | (scal ? UF_SCALAR : 0) |
-                                  (scal_real ? UF_REAL : 0));
-        r.mask = sign[i];
+        gate_record(i, m,
+                    (pair[i] ? UF_DIAG : 0) | (sign[i] ? UF_SIGN : 0) | (scal ? UF_SCALAR : 0) | (scal_real ? UF_REAL : 0),
+                    sign[i]);
         pair[i] = scal = false;
         scal_real = true;
         sign[i] = 0;
@@ -181,7 +232,7 @@ struct PairAssembler : Records {
         const bool ra = la < kUnitRB, rb = lb < kUnitRB;
         if (ra && rb) {
             if (is_sign(d[0], d[1], d[2], d[3])) {
-                emit(UO_DN + unit_pair(std::min(la, lb), std::max(la, lb)));
+                negate(unit_pair(std::min(la, lb), std::max(la, lb)));
                 return;
             }
             const float2 v[4] = {d[0], la < lb ? d[1] : d[2], la < lb ? d[2] : d[1], d[3]};
@@ -267,14 +318,14 @@ struct RatioAssembler : Records {
         }
         scal = false;
         scal_real = true;
-        last_gate = 0;
+        last_gate = joint = 0;
     }
     // The scalar's factors depend on the thread and tile alone: those that come
     // after the last gate move ahead of it, and the gate takes them.
     void absorb_scalar() {
         const size_t g = last_gate - 1;
         UnitRec r = recs[g];
-        r.flags |= (unsigned char)(UF_SCALAR | (scal_real ? UF_REAL : 0));
+        r.mask |= (unsigned)(UF_SCALAR | (scal_real ? UF_REAL : 0)) << (8 * last_bit);
         std::vector<UnitRec> before, after;
         for (size_t k = g + 1; k < recs.size(); ++k) (recs[k].code == UO_SC ? before : after).push_back(recs[k]);
         recs.resize(g);
@@ -283,14 +334,13 @@ struct RatioAssembler : Records {
         recs.insert(recs.end(), after.begin(), after.end());
         scal = false;
         scal_real = true;
-        last_gate = 0;
+        last_gate = joint = 0;
     }
     void take_constant() {   // the constant scalar goes into the last gate's matrix
         cd k[4];
         for (int e = 0; e < 4; ++e) k[e] = cd(gate[e].x, gate[e].y) * cs;
         round_matrix_c64(k, 2, gate);
-        const int at = put_matrix(gate);
-        recs[last_gate - 1].mat = (unsigned short)at;
+        packed(gate, mats.data() + recs[last_gate - 1].off[last_bit] + 2);
         cs = 1.0;
     }
     void g1(int i, const float2* m) {
@@ -301,14 +351,10 @@ struct RatioAssembler : Records {
             round_matrix_c64(k, 2, gate);
             cp[i] = 1.0;
         }
-        const int at = put_matrix(gate);
-        UnitRec& r = emit(UO_G1 + i);
-        r.mat = (unsigned short)at;
-        r.flags = (unsigned char)((rat[i] ? UF_DIAG : 0) | (sign[i] ? UF_SIGN : 0));
-        r.mask = sign[i];
+        gate_record(i, gate, (rat[i] ? UF_DIAG : 0) | (sign[i] ? UF_SIGN : 0), sign[i]);
         rat[i] = false;
         sign[i] = 0;
-        last_gate = recs.size();
+        last_gate = joint;
     }
     void g2(int i, int j, const float2* m) {   // first qubit on register bit i, second on j
         for (int b : {i, j}) {
@@ -349,7 +395,7 @@ struct RatioAssembler : Records {
             const cd k = d[3] * d[0] / (d[1] * d[2]);
             const int pr = unit_pair(std::min(la, lb), std::max(la, lb));
             if (is(round_c64(k), -1.f)) {
-                emit(UO_DN + pr);
+                negate(pr);
             } else if (!one(k)) {
                 const int at = put_c({k, k});
                 emit(UO_DG + pr).mat = (unsigned short)at;
@@ -368,8 +414,9 @@ struct RatioAssembler : Records {
     void begin_phase(const std::vector<int>& R) {
         if (carry.empty()) carry.assign(kMaxTileQ, cd(1.0));
         regs = R;
+        start_phase();
         for (int i = 0; i < 4; ++i) cp[i] = carry[R[i]];
-        last_gate = 0;
+        last_gate = joint = 0;
     }
     void at_end(bool last) {
         for (int i = 0; i < 4; ++i) {

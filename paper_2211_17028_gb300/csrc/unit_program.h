@@ -35,14 +35,15 @@ enum UnitMode : int { UM_RATIOS = 0, UM_PAIRS = 1 };
 // Operation codes; a code in a family of four is FAMILY + register bit, in a
 // family of six FAMILY + pair of register bits.
 enum UnitOp : int {
-    UO_G1 = 0,      // dense one-qubit matrix; flags: UF_DIAG, UF_SIGN, UF_SCALAR, UF_REAL
+    UO_G1 = 0,      // dense one-qubit matrices of register bits, ascending, after UO_DN of the pairs in a:
+                    // mask = their flags (8 bits each), off[i] = {sign mask}, 0, matrix of bit i
     UO_GK = 4,      // dense factor K_0 of a site
     UO_KD = 8,      // diagonal factor K_0 of a site; UF_REAL: real entries
     UO_FLB = 12,    // pairs: the scalar and the pair of one register bit into the amplitudes; ratios: the ratio
     UO_FLR = 16,    // multiply the sign of one register bit into the amplitudes
     UO_HP = 20,     // c = the bit at location a; pairs: pair of the bit *= m[2c], m[2c + 1]; ratios: ratio *= m[c]
     UO_SITE = 24,   // noise site
-    UO_DN = 28,     // negate the amplitudes with both register bits
+    UO_DN = 28,     // negate the amplitudes with both register bits, for every pair in a
     UO_DG = 34,     // pairs: amplitudes *= m[2 * (low bit) + (high bit)]; ratios: those with both bits *= m[0]
     UO_G2 = 40,     // dense two-qubit matrix, its first qubit on the low bit (+ 6: on the high bit)
     UO_SC = 52,     // scalar *= m[c], c = the bits at locations a, b
@@ -51,15 +52,20 @@ enum UnitOp : int {
 };
 // A gate takes the pending pair or ratio of its bit, its pending sign (parity
 // of the bits `mask`), the pending scalar; the scalar is real.
-enum : int { UF_DIAG = 1, UF_SIGN = 2, UF_SCALAR = 4, UF_REAL = 8 };
+enum : int { UF_DIAG = 1, UF_SIGN = 2, UF_SCALAR = 4, UF_REAL = 8, UF_HERE = 64 };
 
 // pairs of register bits (i < j) in the order 01 02 03 12 13 23
 inline int unit_pair(int i, int j) { return i == 0 ? j - 1 : i == 1 ? j + 1 : 5; }
 
 struct UnitRec {               // 16 bytes
     unsigned char code, a, b, flags;
-    unsigned char ev, nspawn, sp, pad0;     // reduction / checkpoint slot, spawned factors, spawn slot
-    unsigned short mat, site;
+    union {
+        struct {
+            unsigned char ev, nspawn, sp, pad0;   // reduction / checkpoint slot, spawned factors, spawn slot
+            unsigned short mat, site;
+        };
+        unsigned short off[4];                    // UO_G1: matrices of the register bits
+    };
     unsigned int mask;
 };
 
@@ -108,7 +114,7 @@ struct SweepUnit {
 inline int unit_kind(bool single, UnitMode mode) { return 2 * (int)single + (int)mode; }
 constexpr int kUnitKinds = 4;
 size_t unit_smem_bytes(int max_words, int max_events);
-int unit_blocks_per_sm(size_t smem);
+int unit_blocks_per_sm(int kind, size_t smem);
 // blk: unit of every block, or null when every unit has `ctas` blocks
 // kind: unit_kind of the units' programs
 cudaError_t launch_units(int kind, const SweepUnit* units, const int* blk, int ctas, int total_ctas, size_t smem,
