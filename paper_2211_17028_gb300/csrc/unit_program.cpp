@@ -273,6 +273,20 @@ struct RatioAssembler : Records {
         for (cd c : v) f[n++] = round_c64(c);
         return put(f, n);
     }
+    // Rounded phases are off modulus 1 by up to 1e-8, and a circuit repeats its
+    // phases (every edge of a QAOA layer has the same one), so the errors add up:
+    // what the entries f of v have in common is taken out of the constants, in
+    // full for a factor of all amplitudes, by half for one of those with a set
+    // bit.  Signs are exact and change nothing.
+    void keep_norm(int at, std::initializer_list<cd> v, double weight) {
+        double s = 0.0;   // sum of the relative errors of the moduli
+        const float2* f = mats.data() + at;
+        for (const cd& c : v) {
+            s += 0.5 * (std::norm(cd(f->x, f->y)) / std::norm(c) - 1.0);
+            ++f;
+        }
+        if (std::fabs(s) < 1e-6) cs *= 1.0 - weight * s / (double)v.size();
+    }
     void ratio(int i, cd v0, cd v1, int loc = kNoLoc) {
         const float2 f0 = round_c64(v0), f1 = round_c64(v1);
         if (loc != kNoLoc && is(f0, 1.f) && is(f1, -1.f)) {
@@ -282,11 +296,13 @@ struct RatioAssembler : Records {
         const int at = put_c({v0, v1});
         emit(UO_HP + i, loc).mat = (unsigned short)at;
         rat[i] = true;
+        keep_norm(at, {v0, v1}, 0.5);
     }
     void scalar(cd v0, cd va, cd vb, cd vab, int la = kNoLoc, int lb = kNoLoc) {
         const int at = put_c({v0, va, vb, vab});
         emit(UO_SC, la, lb).mat = (unsigned short)at;
         scal = true;
+        keep_norm(at, {v0, va, vb, vab}, 1.0);
         for (cd c : {v0, va, vb, vab}) scal_real = scal_real && round_c64(c).y == 0.f;
     }
     // keep_scalar leaves the constant scalar pending (the caller scales what it writes)
@@ -301,8 +317,9 @@ struct RatioAssembler : Records {
         for (int i = 0; i < 4; ++i) n += rat[i];
         if (scal && last_gate > 0 && n < 3) absorb_scalar();
         if (!keep_scalar && !one(cs)) {
-            scalar(cs, cs, cs, cs);
+            const cd all = cs;
             cs = 1.0;
+            scalar(all, all, all, all);
         }
         if (8 * n + 16 * (int)scal > 31) {   // 31 products for everything at once
             emit(UO_FLA);
