@@ -203,7 +203,7 @@ ProgInfo build_program(const std::vector<DevOp>& dops, int off, int n, int RB, c
             r.qb = (unsigned char)(d.qb >= 0 ? d.qb : 0xff);
             r.ev = (unsigned char)((d.flags >> 8) & 0xff);
             r.nspawn = (unsigned char)((d.flags >> 16) & 0xff);
-            r.site = (unsigned short)(d.site >= 0 ? d.site : 0);
+            r.site = (unsigned)(d.site >= 0 ? d.site : 0);
             int cnt = (d.type == OP_G2 || d.type == OP_D2) ? 16 : 4;
             if (d.type == OP_SITE && (d.flags & FL_SPAWN)) cnt = 16;
             r.mat = (unsigned short)mats.size();
@@ -1028,7 +1028,7 @@ static int build_small(Handle& h, Engine& E, const nqs_state* psi, const nqs_sta
                 u.depth = depth + 1;
                 u.rank = (long long)ranks.size();
                 for (int k = 0; k <= depth; ++k) {
-                    u.site[k] = (unsigned short)sites[k];
+                    u.site[k] = sites[k];
                     u.factor[k] = (unsigned char)fp[k];
                 }
                 for (int t = s + 1; t < N; ++t) {

@@ -27,7 +27,7 @@ struct SmallOp {
 struct SmallUnit {
     long long rank;                   // index in the rank table of the term of the first site after the last
     int depth;
-    unsigned short site[kSmallDepth];
+    int site[kSmallDepth];
     unsigned char factor[kSmallDepth];   // kept-factor positions
     int pad;
 };

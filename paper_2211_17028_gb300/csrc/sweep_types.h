@@ -61,8 +61,8 @@ struct DevPhase {
 struct OpRec {
     unsigned char type, la, lb, flags;   // la, lb: location codes (register bit, LOC_THREAD + bit, 0xff outside)
     unsigned char qa, qb, ev, nspawn;    // qubits; reduction event; spawned factors
-    unsigned short site, mat;            // site index; matrix offset (float2) in the program
-    unsigned int pad;
+    unsigned short mat, pad;             // matrix offset (float2) in the program
+    unsigned int site;
 };
 
 struct PassArgs {

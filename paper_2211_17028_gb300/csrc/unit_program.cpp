@@ -458,7 +458,7 @@ namespace {
 template <typename Asm>
 UnitProgram assemble(const std::vector<DevOp>& dops, int off, int n, const int* local, int n_qubits,
                           const std::vector<float2>& tab, std::vector<uint4>& out) {
-    static_assert(sizeof(UnitRec) == 16 && sizeof(UnitPhase) == 96 && sizeof(UnitHeader) == 64, "record sizes");
+    static_assert(sizeof(UnitRec) == 16 && sizeof(UnitPhase) == 96 && sizeof(UnitHeader) == 80, "record sizes");
     constexpr int K = kMaxTileQ;
     UnitHeader hd{};
     bool in_tile[64] = {};
@@ -564,15 +564,14 @@ UnitProgram assemble(const std::vector<DevOp>& dops, int off, int n, const int* 
                     A.at_site();
                     UnitRec& r = A.site(i, m, (fl & FL_SPAWN) ? (d.flags >> 16) & 0xff : 0, A.scale());
                     r.flags = (unsigned char)(fl & ~(FL_APPLY | FL_KDIAG));
-                    r.site = (unsigned short)d.site;
                     if (fl & FL_REDUCE) {
                         r.ev = (unsigned char)((d.flags >> 8) & 0xff);
-                        hd.slot_site[r.ev] = (unsigned short)d.site;
+                        hd.slot_site[r.ev] = (unsigned)d.site;
                         hd.n_events = std::max(hd.n_events, (unsigned)r.ev + 1);
                         hd.n_slots = std::max<unsigned char>(hd.n_slots, r.ev + 1);
                     } else if (fl & (FL_SAVE | FL_SAVE_FWD)) {
                         r.ev = hd.n_slots++;
-                        hd.slot_site[r.ev] = (unsigned short)(d.site | ((fl & FL_SAVE_FWD) ? 0x8000 : 0));
+                        hd.slot_site[r.ev] = (unsigned)d.site | ((fl & FL_SAVE_FWD) ? kSlotFwd : 0u);
                     }
                     if (fl & FL_SPAWN) r.sp = (unsigned char)(d.flags >> 24);
                 } else {
@@ -597,7 +596,7 @@ UnitProgram assemble(const std::vector<DevOp>& dops, int off, int n, const int* 
     info.word = (int)out.size();
     hd.n_phases = (unsigned)phases.size();
     hd.n_ops = (unsigned)A.recs.size();
-    hd.ops_word = 4 + 6 * hd.n_phases;
+    hd.ops_word = kHeaderWords + 6 * hd.n_phases;
     hd.mats_word = hd.ops_word + hd.n_ops;
     hd.words = hd.mats_word + (unsigned)((A.mats.size() + 1) / 2);
     words(&hd, sizeof(hd));

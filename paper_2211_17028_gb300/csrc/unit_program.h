@@ -62,7 +62,7 @@ struct UnitRec {               // 16 bytes
     union {
         struct {
             unsigned char ev, nspawn, sp, pad0;   // reduction / checkpoint slot, spawned factors, spawn slot
-            unsigned short mat, site;
+            unsigned short mat, pad1;
         };
         unsigned short off[4];                    // UO_G1: matrices of the register bits
     };
@@ -77,14 +77,16 @@ struct UnitPhase {             // 96 bytes
     unsigned short pad[2];
 };
 
-struct UnitHeader {            // 64 bytes
+struct UnitHeader {            // 80 bytes
     unsigned int n_phases, n_ops, ops_word, mats_word;
     unsigned long long nl_mask;             // qubits outside the tile
     unsigned int n_events, words;
     unsigned char local[12];                // tile qubits, ascending
     unsigned char n_slots, pad[3];
-    unsigned short slot_site[kUnitSlots];   // site of each checkpoint slot (bit 15: forward table)
+    unsigned int slot_site[kUnitSlots];     // site of each checkpoint slot (kSlotFwd: in the forward table)
 };
+constexpr unsigned int kSlotFwd = 1u << 31;
+constexpr int kHeaderWords = sizeof(UnitHeader) / 16;
 
 struct UnitProgram {
     UnitMode mode = UM_RATIOS;
