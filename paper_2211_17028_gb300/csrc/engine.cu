@@ -32,6 +32,8 @@
 #include <cstring>
 #include <functional>
 #include <map>
+#include <mutex>
+#include <set>
 #include <vector>
 
 #include "engine_internal.h"
@@ -40,6 +42,23 @@ namespace nqs {
 
 
 int cuda_err(cudaError_t e) { return e == cudaSuccess ? NQS_OK : NQS_ERR_CUDA; }
+
+cudaError_t allow_dynamic_smem(const void* kernel) {
+    static std::mutex mu;
+    static std::set<std::pair<const void*, int>> done;   // kernel, device
+    int dev = 0, optin = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lock(mu);
+    if (done.count({kernel, dev})) return cudaSuccess;
+    cudaFuncAttributes a{};
+    e = cudaFuncGetAttributes(&a, kernel);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)a.sharedSizeBytes);
+    if (e == cudaSuccess) done.insert({kernel, dev});
+    return e;
+}
 
 // NQS_JIT=0 in the environment turns the automatic choice of pass-specialised kernels off
 static bool jit_env_enabled() {

@@ -265,9 +265,8 @@ cudaError_t launch_generic_small(const GSmallArgs& a, cudaStream_t st) {
     const size_t smem = sizeof(float2) << a.n;
     cudaError_t e = cudaSuccess;
     if (smem > (size_t)(32 << 10)) {
-        e = cudaFuncSetAttribute(gs_checkpoints_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(gs_units_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = allow_dynamic_smem((const void*)gs_checkpoints_kernel);
+        if (e == cudaSuccess) e = allow_dynamic_smem((const void*)gs_units_kernel);
         if (e != cudaSuccess) return e;
     }
     gs_checkpoints_kernel<<<2, threads, smem, st>>>(a);

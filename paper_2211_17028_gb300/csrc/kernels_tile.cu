@@ -213,28 +213,16 @@ __global__ void __launch_bounds__(kThreads) tile_pass_kernel(const PassArgs P) {
 }
 
 
-namespace {
-template <int S>
-void set_attr() {
-    static bool done = false;
-    if (!done) {
-        cudaFuncSetAttribute(tile_pass_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             S * (1 << kMaxTileQ) * (int)sizeof(float2));
-        done = true;
-    }
-}
-}  // namespace
-
 int tile_pass_blocks_per_sm(int S, size_t smem) {
     int nb = 0;
     if (S == 1) {
-        set_attr<1>();
+        allow_dynamic_smem((const void*)tile_pass_kernel<1>);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, tile_pass_kernel<1>, kThreads, smem);
     } else if (S == 2) {
-        set_attr<2>();
+        allow_dynamic_smem((const void*)tile_pass_kernel<2>);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, tile_pass_kernel<2>, kThreads, smem);
     } else {
-        set_attr<3>();
+        allow_dynamic_smem((const void*)tile_pass_kernel<3>);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, tile_pass_kernel<3>, kThreads, smem);
     }
     return nb > 0 ? nb : 1;

@@ -717,7 +717,7 @@ int unit_blocks_per_sm(int kind, size_t smem) {
     if (three_fit(kind, smem)) return 3;
     int nb = 0;
     const UnitKernel k = unit_kernel(kind, 2);
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_dynamic_smem((const void*)k);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, kNT, smem);
     return nb > 0 ? nb : 1;
 }
@@ -727,7 +727,7 @@ cudaError_t launch_units(int kind, const SweepUnit* units, const int* blk, int c
     const int blocks = total_ctas > 2 * attribute(cudaDevAttrMultiProcessorCount) && three_fit(kind, smem) ? 3 : 2;
     const UnitKernel kernel = unit_kernel(kind, blocks);
     smem = smem_of(blocks, smem);
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_dynamic_smem((const void*)kernel);
     if (e != cudaSuccess) return e;
     kernel<<<total_ctas, kNT, smem, st>>>(units, blk, ctas);
     return cudaGetLastError();

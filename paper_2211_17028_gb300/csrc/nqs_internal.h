@@ -221,6 +221,12 @@ int mlp_loss_grad(Mlp* m, const float* X, const float* y, int B, double* loss, f
 int mlp_train(Mlp* m, const float* X, const float* y, int n, int batch, int steps, float lr, unsigned long long seed,
               double* final_loss, void* stream);
 
+// Let launches of `kernel` on the current device have as much dynamic shared
+// memory as a block can (engine.cu).  The limit belongs to the kernel, not to a
+// launch: set to what one call needs, it would be too low for the launch of a
+// call on another thread that needs more.
+cudaError_t allow_dynamic_smem(const void* kernel);
+
 // allocator (capi.cpp)
 void* dev_alloc(size_t bytes, void* stream);
 void dev_free(void* p, size_t bytes, void* stream);
