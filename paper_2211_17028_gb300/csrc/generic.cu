@@ -778,6 +778,7 @@ int general_fidelity(Handle& h, const nqs_state* psi, const nqs_state* v, int le
     int rc = cu(cudaMemcpyAsync(fac_dev, fh.data(), fh.size() * sizeof(float2), cudaMemcpyHostToDevice, st));
     if (!rc) rc = cu(cudaMemcpyAsync(kdevA, kh.data(), kh.size() * sizeof(double2), cudaMemcpyHostToDevice, st));
     if (!rc) rc = cu(cudaMemcpyAsync(loff, lo.data(), lo.size() * sizeof(long long), cudaMemcpyHostToDevice, st));
+    if (!rc) rc = cu(cudaStreamSynchronize(st));   // pageable sources
     if (!rc) rc = cu(cudaMemsetAsync(ampsA, 0, (two_sided ? 2 : 1) * (size_t)ti.total * sizeof(double2), st));
     // psi, v
     const int fill_grid = (int)std::max<long long>(1, std::min<long long>((long long)sms * 8, dim / kT));
