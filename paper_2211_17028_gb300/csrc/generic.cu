@@ -41,6 +41,7 @@ struct GEngine {
     size_t buf_bytes = 0;
     void* aux = nullptr;
     size_t aux_bytes = 0;
+    bool one_sibling = false;      // the buffers hold one sibling per depth: more did not fit
     long long n_terms = 0;
     bool has_result = false;
     cudaStream_t last = nullptr;
@@ -393,6 +394,7 @@ void release(GEngine& G, void* stream) {
     if (G.aux) dev_free(G.aux, G.aux_bytes, stream);
     G.buf = G.aux = nullptr;
     G.buf_bytes = G.aux_bytes = 0;
+    G.one_sibling = false;
     G.small_level = -1;
 }
 
@@ -703,8 +705,6 @@ int general_fidelity(Handle& h, const nqs_state* psi, const nqs_state* v, int le
     // deeper one, psi, v; aux: factors, partials, amps, values, tables
     const size_t sb = (size_t)dim * sizeof(float2);
     const int depths = std::max(0, level - 1);
-    const int width = (int)std::max<size_t>(1, std::min<size_t>(15, kSiblingBytes / sb));
-    const size_t n_states = (size_t)N + 1 + (size_t)depths * width + 2;
     const size_t kcount = [&] {
         size_t c = 0;
         for (const auto& f : h.gfac) c += (size_t)f.m * (f.nq == 1 ? 4 : 16);
@@ -715,25 +715,43 @@ int general_fidelity(Handle& h, const nqs_state* psi, const nqs_state* v, int le
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int grid = (int)std::max<long long>(1, std::min<long long>((long long)sms * 4, (dim / 2 + kT - 1) / kT));
     auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
+    int width = (int)std::max<size_t>(1, std::min<size_t>(15, kSiblingBytes / sb));
+    size_t n_states, o_part, o_amps, o_vals, o_loff, o_res, o_fac, aux_bytes;
     const size_t o_k = 0;
-    const size_t o_part = al(o_k + 2 * kcount * sizeof(double2));
-    const size_t o_amps = al(o_part + (size_t)width * grid * 32 * sizeof(double));
-    const size_t o_vals = al(o_amps + (two_sided ? 2 : 1) * (size_t)ti.total * sizeof(double2));
-    const size_t o_loff = al(o_vals + (size_t)ti.total * sizeof(double));
-    const size_t o_res = al(o_loff + (size_t)(level + 2) * sizeof(long long));
-    const size_t o_fac = al(o_res + sizeof(nqs_result));
-    const size_t aux_bytes = al(o_fac + 2 * (size_t)N * 256 * sizeof(float2));
+    auto lay_out = [&] {
+        n_states = (size_t)N + 1 + (size_t)depths * width + 2;
+        o_part = al(o_k + 2 * kcount * sizeof(double2));
+        o_amps = al(o_part + (size_t)width * grid * 32 * sizeof(double));
+        o_vals = al(o_amps + (two_sided ? 2 : 1) * (size_t)ti.total * sizeof(double2));
+        o_loff = al(o_vals + (size_t)ti.total * sizeof(double));
+        o_res = al(o_loff + (size_t)(level + 2) * sizeof(long long));
+        o_fac = al(o_res + sizeof(nqs_result));
+        aux_bytes = al(o_fac + 2 * (size_t)N * 256 * sizeof(float2));
+    };
+    auto held = [&] { return G.buf_bytes >= n_states * sb && G.aux_bytes >= aux_bytes; };
+    lay_out();
     G.small_level = -1;   // its tables are written over
-    if (G.buf_bytes < n_states * sb || G.aux_bytes < aux_bytes) {
+    if (G.one_sibling && !held()) {
+        const int all = width;
+        width = 1;
+        lay_out();
+        if (!held()) width = all;
+        lay_out();
+    }
+    if (!held()) {
         release(G, stream);
-        G.buf = dev_alloc(n_states * sb, stream);
-        G.aux = dev_alloc(aux_bytes, stream);
-        if (!G.buf || !G.aux) {
+        // all siblings together where they fit, else one after another
+        for (;; width = 1, lay_out()) {
+            G.buf_bytes = n_states * sb;
+            G.aux_bytes = aux_bytes;
+            G.buf = dev_alloc(G.buf_bytes, stream);
+            G.aux = dev_alloc(G.aux_bytes, stream);
+            if (G.buf && G.aux) break;
+            const bool last = width == 1;
             release(G, stream);
-            return NQS_ERR_NOMEM;
+            if (last) return NQS_ERR_NOMEM;
+            G.one_sibling = true;
         }
-        G.buf_bytes = n_states * sb;
-        G.aux_bytes = aux_bytes;
     }
     char* ab = (char*)G.aux;
     double2* kdevA = (double2*)(ab + o_k);

@@ -48,3 +48,38 @@ def test_uploads_are_read_before_the_call_returns():
     side.synchronize()
     assert out.F == want["F"] and out.status == 0
     circ.close()
+
+
+def test_one_sibling_where_fifteen_do_not_fit():
+    """N + level + 3 states of 256 KiB fit, the siblings' 15 per depth do not."""
+    import torch
+    from paper_2211_17028_gb300 import nqs
+    w = _workload()
+    text, psi = W.to_ir_text(w), nqs.basis(w.psi["bits"])
+    circ = nqs.NoisyCircuit(text)
+    want = circ.fidelity(psi, nqs.ideal(), 2)
+    terms = circ.term_values()
+    circ.close()
+    refused = []
+
+    def alloc(nbytes, stream, ctx):
+        if nbytes > (3 + 2 + 3) * (8 << 15):
+            refused.append(nbytes)
+            return None
+        return torch.cuda.caching_allocator_alloc(int(nbytes), 0, int(stream or 0))
+
+    def free(ptr, nbytes, stream, ctx):
+        torch.cuda.caching_allocator_delete(int(ptr))
+
+    hooks = nqs.ALLOC_FN(alloc), nqs.FREE_FN(free)
+    nqs.nqs_set_allocator(*hooks)
+    try:
+        circ = nqs.NoisyCircuit(text)
+        got = circ.fidelity(psi, nqs.ideal(), 2)
+        assert refused and got["F"] == want["F"] and got["T"] == want["T"]
+        assert list(circ.term_values()) == list(terms)
+        asked = len(refused)   # the next call keeps what it has
+        assert circ.fidelity(psi, nqs.ideal(), 2)["F"] == want["F"] and len(refused) == asked
+        circ.close()
+    finally:
+        nqs.use_torch_allocator()
