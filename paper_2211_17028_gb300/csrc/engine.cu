@@ -1481,9 +1481,12 @@ int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* 
             if (!todo.empty()) {
                 // 12-qubit tiles first, then the precompiled kernel
                 if (std::getenv("NQS_JIT_VERBOSE")) std::fprintf(stderr, "nqs jit: %s\n", err.c_str());
-                (E.wide ? E.wide_failed : E.jit_failed) = true;
+                const bool wide = E.wide;
+                (wide ? E.wide_failed : E.jit_failed) = true;
                 engine_release(E, stream);
-                return build_schedule(h, E, psi, v, level, stream, allow_jit);
+                const int rc = build_schedule(h, E, psi, v, level, stream, allow_jit);
+                if (!wide) E.jit_failed = false;   // the next schedule tries again
+                return rc;
             }
         }
     }

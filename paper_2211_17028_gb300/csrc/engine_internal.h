@@ -113,7 +113,7 @@ struct Engine {
     Plan wide_plan;                  // the plan re-cut for 13-qubit tiles (generated kernels)
     bool wide = false;               // the current schedule runs on wide_plan
     bool wide_failed = false;        // a wide schedule's kernels could not be built: 12-qubit tiles
-    bool jit_failed = false;         // the generated kernels could not be built: the precompiled one
+    bool jit_failed = false;         // this schedule's generated kernels could not be built: the precompiled one
 };
 
 

@@ -35,6 +35,7 @@
 #include <atomic>
 #include <cmath>
 #include <complex>
+#include <condition_variable>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -1132,13 +1133,14 @@ Nvrtc& nvrtc() {
 struct CacheEntry {
     std::vector<char> cubin;
     std::string error;
-    bool done = false;
+    bool done = false;             // compiled or failed (under g_cache_mu)
     std::map<int, void*> kernel;   // per device: cudaKernel_t (libraries load into every context)
     cudaLibrary_t lib = nullptr;
     int smem_set = 0;
 };
 
 std::mutex g_cache_mu;
+std::condition_variable g_cache_cv;   // an entry is done
 std::map<std::string, CacheEntry*>& cache() {
     static std::map<std::string, CacheEntry*> c;
     return c;
@@ -1196,7 +1198,8 @@ bool jit_available() { return nvrtc().ok; }
 long long jit_compile_count() { return g_compiles.load(); }
 
 int jit_compile(std::vector<JitPass*>& passes, std::string* error) {
-    // distinct sources, compiled in parallel
+    // distinct sources, compiled in parallel; one that another thread compiles is
+    // waited for below
     std::vector<std::pair<std::string, CacheEntry*>> todo;
     {
         std::lock_guard<std::mutex> g(g_cache_mu);
@@ -1221,14 +1224,17 @@ int jit_compile(std::vector<JitPass*>& passes, std::string* error) {
                     const size_t i = next++;
                     if (i >= todo.size()) break;
                     compile_one(todo[i].first, *todo[i].second);
+                    std::lock_guard<std::mutex> g(g_cache_mu);
                     todo[i].second->done = true;
+                    g_cache_cv.notify_all();
                 }
             });
         for (auto& t : th) t.join();
     }
-    std::lock_guard<std::mutex> g(g_cache_mu);
+    std::unique_lock<std::mutex> g(g_cache_mu);
     for (JitPass* p : passes) {
         CacheEntry* ce = cache()[p->source];
+        g_cache_cv.wait(g, [&] { return ce->done; });
         if (ce->cubin.empty()) {
             if (error) *error = ce->error;
             return -1;

@@ -1,7 +1,7 @@
 """Two handles on two threads: what one call sets for its own launches must not
 reach the launches of another.  The calls have different needs of shared
 memory (13 and 14 qubits of general noises; unit programs of different
-lengths)."""
+lengths) or want the same generated kernels at the same time."""
 
 import ctypes
 import threading
@@ -73,3 +73,28 @@ def test_two_threads_do_not_disturb_each_other(make, widths):
     assert not failed, (len(failed), failed[:4])
     for a in work:
         a[0].close()
+
+
+def test_generated_kernels_wanted_by_two_threads_at_once():
+    """The second thread waits for the kernels that the first one compiles."""
+    from paper_2211_17028_gb300 import nqs
+    w = W.random_circuit(640, 14, 60, 4, v_kind="ideal")
+    circs = [nqs.NoisyCircuit(W.to_ir_text(w)) for _ in range(2)]
+    psi = nqs.basis(w.psi["bits"])
+    start = threading.Barrier(2)
+    got = [None, None]
+
+    def call(i):
+        nqs.nqs_set_option(circs[i].h, nqs.NQS_OPT_JIT, 1)
+        start.wait()
+        F = circs[i].fidelity(psi, nqs.ideal(), 2)["F"]
+        got[i] = (F, nqs.nqs_get_info(circs[i].h)["jit_state"])
+
+    threads = [threading.Thread(target=call, args=(i,)) for i in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert got[0] == got[1] and got[0][1] == 1, got
+    for c in circs:
+        c.close()
