@@ -65,10 +65,13 @@ void free_plan(BatchPlan* p, void* stream) {
     delete p;
 }
 
-size_t state_bytes_needed(const Handle& h, int level) {
+// Device bytes that circuit k's schedule takes if it has to be built: its states
+// and about 16 MiB of tables (programs, partial sums, term values).
+size_t new_bytes(const Handle& h, const nqs_state& psi, const nqs_state& v, int level) {
     const int N = (int)h.factors.size();
     const int lvl = std::min(level, N);
-    return ((size_t)std::max(N, 1) + 1 + group_states(h, lvl, false)) * ((size_t)8 << h.plan.n);
+    if (h.eng && schedule_current(*h.eng, &psi, &v, lvl)) return 0;
+    return ((size_t)std::max(N, 1) + 1 + group_states(h, lvl, false)) * ((size_t)8 << h.plan.n) + ((size_t)16 << 20);
 }
 
 // Build the round-grouped launch sequence of the circuits [first, last) and
@@ -281,44 +284,44 @@ int engine_batch_fidelity(Handle** hs, size_t count, const nqs_state* psis, cons
     P->engines.assign(count, nullptr);
     P->gens.assign(count, 0);
 
-    // waves of circuits whose state buffers fit in the free device memory
-    size_t free_b = 0, total_b = 0;
+    // waves of circuits whose buffers fit in the device memory: a wave takes
+    // circuits, each with the schedule that it has on its own, until the next one's
+    // buffers are refused.  A twentieth of the device is kept out of that, for the
+    // unit arrays and for others, unless the batch leaves it anyway.
+    size_t free_b = 0, total_b = 0, need = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
         free_plan(P, stream);
         return NQS_ERR_CUDA;
     }
-    size_t held = 0;
-    for (size_t k = 0; k < count; ++k) held += engine_workspace_bytes(*hs[k]);
-    const size_t budget = (size_t)(0.9 * (double)(free_b + held));
-    std::vector<std::pair<int, int>> waves;
-    {
-        size_t acc = 0;
-        int first = 0;
-        for (size_t k = 0; k < count; ++k) {
-            const size_t need = state_bytes_needed(*hs[k], levels[k]) + (64u << 20);
-            if (acc > 0 && acc + need > budget) {
-                waves.push_back({first, (int)k});
-                first = (int)k;
-                acc = 0;
-            }
-            acc += need;
-        }
-        waves.push_back({first, (int)count});
-    }
-    const bool single_wave = waves.size() == 1;
+    for (size_t k = 0; k < count; ++k) need += new_bytes(*hs[k], psis[k], vs[k], levels[k]);
+    const size_t reserve_bytes = total_b / 20;
+    const bool reserving = need + reserve_bytes > free_b;
+    bool single_wave = false;
 
     int rc = NQS_OK;
-    for (const auto& w : waves) {
-        for (int k = w.first; k < w.second && rc == NQS_OK; ++k) {
+    for (std::pair<int, int> w(0, 0); w.second < (int)count && rc == NQS_OK;) {
+        w.first = w.second;
+        void* reserve = nullptr;
+        for (int k = w.first; k < (int)count && rc == NQS_OK; ++k) {
             Handle& h = *hs[k];
+            const int level = std::min(levels[k], (int)h.factors.size());
             if (!h.eng) h.eng = new Engine();
             rc = engine_init(*h.eng);
-            if (rc == NQS_OK) rc = build_schedule(h, *h.eng, &psis[k], &vs[k], std::min(levels[k], (int)h.factors.size()),
-                                                  stream, false);
+            if (rc == NQS_OK && !schedule_current(*h.eng, &psis[k], &vs[k], level)) {
+                if (reserving && !reserve) reserve = dev_alloc(reserve_bytes, stream);
+                rc = build_schedule(h, *h.eng, &psis[k], &vs[k], level, stream, false, k == w.first);
+                if (rc == NQS_ERR_NOMEM && k > w.first) {   // the next wave begins with it
+                    rc = NQS_OK;
+                    break;
+                }
+            }
             P->engines[k] = h.eng;
             P->gens[k] = h.eng->gen;
+            w.second = k + 1;
         }
+        if (reserve) dev_free(reserve, reserve_bytes, stream);
         if (rc != NQS_OK) break;
+        single_wave = w.first == 0 && w.second == (int)count;
         // results array and unit arrays (build_plan asks once for a larger buffer)
         if (!P->dev) {
             const size_t res_bytes = ((count * sizeof(nqs_result)) + 255) & ~(size_t)255;

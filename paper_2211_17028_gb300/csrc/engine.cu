@@ -339,13 +339,18 @@ Run make_run(const Plan& plan, const std::vector<PassSpec>& segs, RunType rt, bo
 // swept together, all their states in one launch per pass (a 20-qubit
 // state has 256 tiles: three states alone fill the chip 1.3 times, and a
 // 13-qubit one has two tiles).  256 MiB of states is 8192 tiles, 27 times the
-// resident blocks: more groups at once gain nothing.
+// resident blocks: more groups at once gain nothing, and half of it costs 6 % at
+// 20 qubits, level 2 (6.17 -> 6.57 ms).
 constexpr size_t kGroupBytes = (size_t)256 << 20;
-// the passes of a sweep that spawns may hold several sites (fewer passes) when
-// the children of a whole pass fit in this much
-constexpr size_t kSpawnBytes = (size_t)2 << 30;
-// per-block partial sums held before a finisher launch is put in
-constexpr size_t kPartialDoubles = (size_t)4 << 20;
+// The passes of a sweep that spawns may hold several sites (fewer passes) when
+// the children of a whole pass fit in this much.  A handle keeps these states as
+// long as its checkpoints, and a study keeps hundreds of handles: with 2 GiB here
+// 512 circuits of 12 to 24 qubits held 275 GiB, all of the device (235 with the
+// three states of one site each; 255 so).  Wider states are many tiles each, and
+// their spawning sweep is one of many: 2 to 5 % at 23 and 24 qubits.
+constexpr size_t kSpawnBytes = (size_t)512 << 20;
+// per-block partial sums held before a finisher launch is put in (8 MiB)
+constexpr size_t kPartialDoubles = (size_t)1 << 20;
 
 // Sizes of the branch-group buffers: states per depth (1 .. level - 1).
 struct GroupPlan {
@@ -1156,17 +1161,20 @@ static int build_small(Handle& h, Engine& E, const nqs_state* psi, const nqs_sta
     return NQS_OK;
 }
 
+bool schedule_current(const Engine& E, const nqs_state* psi, const nqs_state* v, int level) {
+    return E.level == level && E.psi_kind == psi->kind && E.v_kind == v->kind && E.psi_bits == psi->bits &&
+           E.v_bits == v->bits && E.psi_dev == psi->dev && E.v_dev == v->dev;
+}
+
 // Build (or reuse) the schedule for this level and state kinds.
 int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* v, int level, void* stream,
-                   bool allow_jit) {
+                   bool allow_jit, bool make_do) {
     const int N = (int)h.factors.size();
     // automatic: circuits of 26 qubits or more, where one call's sweeps outlast
     // the compilation of its distinct passes
     const bool want_jit =
         allow_jit && (h.opt_jit == 1 || (h.opt_jit == 0 && h.plan.n >= 26 && jit_env_enabled()));
-    if (E.level == level && E.psi_kind == psi->kind && E.v_kind == v->kind && E.psi_bits == psi->bits &&
-        E.v_bits == v->bits && E.psi_dev == psi->dev && E.v_dev == v->dev && !(want_jit && E.jit_state == 0))
-        return NQS_OK;
+    if (schedule_current(E, psi, v, level) && !(want_jit && E.jit_state == 0)) return NQS_OK;
     engine_release(E, stream);
     ++E.gen;
 
@@ -1203,8 +1211,8 @@ int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* 
     }
 
     // state buffers.  Every site keeps its phi when the states fit (or the
-    // option asks for it): phi slots, main, group buffers (3 at depth 1, 9
-    // deeper).  Otherwise (levels <= 2) phi is kept only at the last site of
+    // option asks for it): phi slots, main, group buffers (group_plan; 3 at depth
+    // 1, 9 deeper where those do not fit).  Otherwise (levels <= 2) phi is kept only at the last site of
     // each block of `spacing` sites and a block's phi are recomputed into a
     // ring of `spacing` slots whenever a sweep enters the block.
     const size_t sbytes = (size_t)B.dim * sizeof(float2);
@@ -1217,7 +1225,8 @@ int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* 
     size_t n_states = 0;
     if (spacing == 0) {
         // groups swept together when the memory allows, else one at a time
-        for (int small = B.kind != P_UNIT; small < 2 && !E.buf; ++small) {
+        const int first = B.kind != P_UNIT;
+        for (int small = first; small <= (make_do ? 1 : first) && !E.buf; ++small) {
             B.gp = group_plan(plan, h.factors, level, B.kind != P_UNIT, small != 0);
             n_states = (size_t)n_phi + 1 + B.gp.total();
             E.buf_bytes = n_states * sbytes;
@@ -1225,7 +1234,7 @@ int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* 
         }
         if (!E.buf) {
             E.buf_bytes = 0;
-            if (h.opt_spacing != 0 || level > 2 || N < 2) return NQS_ERR_NOMEM;
+            if (!make_do || h.opt_spacing != 0 || level > 2 || N < 2) return NQS_ERR_NOMEM;
             spacing = best_spacing(N, level);
         }
     }
@@ -1484,7 +1493,7 @@ int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* 
                 const bool wide = E.wide;
                 (wide ? E.wide_failed : E.jit_failed) = true;
                 engine_release(E, stream);
-                const int rc = build_schedule(h, E, psi, v, level, stream, allow_jit);
+                const int rc = build_schedule(h, E, psi, v, level, stream, allow_jit, make_do);
                 if (!wide) E.jit_failed = false;   // the next schedule tries again
                 return rc;
             }

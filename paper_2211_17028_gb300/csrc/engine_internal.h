@@ -154,13 +154,16 @@ Run make_run(const Plan& plan, const std::vector<PassSpec>& segs, RunType rt, bo
 int engine_init(Engine& E);
 void engine_release(Engine& E, void* stream);
 // allow_jit: the schedule may use pass-specialised kernels (the batch executor
-// launches passes through its own multi-circuit kernel and passes false)
+// launches passes through its own multi-circuit kernel and passes false);
+// make_do: where the states do not fit, a schedule with fewer of them, else
+// NQS_ERR_NOMEM
 int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* v, int level, void* stream,
-                   bool allow_jit = true);
+                   bool allow_jit = true, bool make_do = true);
 int run_schedule(Handle& h, Engine& E, cudaStream_t st);
 int run_launch(Handle& h, Engine& E, const Launch& l, cudaStream_t st);
-// device bytes of the branch-group state buffers a schedule allocates beside
-// its checkpoints and main state (the batch executor packs waves with it)
+// whether E's schedule is the one for these states and this level
+bool schedule_current(const Engine& E, const nqs_state* psi, const nqs_state* v, int level);
+// branch-group states a schedule holds beside its checkpoints and main state
 size_t group_states(const Handle& h, int level, bool generated);
 
 }  // namespace nqs
