@@ -97,9 +97,12 @@ int build_plan(BatchPlan& P, int first, int last, void* stream) {
     size_t rounds = 0;
     for (int k = first; k < last; ++k) rounds = std::max(rounds, P.engines[k]->launches.size());
     for (size_t r = 0; r < rounds; ++r) {
-        // the round's sweep passes, longest blocks first (the short ones fill the
-        // last wave)
-        std::vector<std::pair<const Engine*, const Launch*>> sweeps_of[kUnitKinds];   // by kernel
+        // the round's sweep passes by kernel, and apart those whose programs leave room
+        // for three blocks per SM: a launch reserves the shared memory of its longest
+        // program for every block, and one circuit's long pass would leave all others
+        // two blocks (512 circuits of 12 to 24 qubits: 5.28 s in one launch per kernel,
+        // 4.74 s so; 5.27 s one circuit after another)
+        std::vector<std::pair<const Engine*, const Launch*>> sweeps_of[2 * kUnitKinds];
         std::vector<FinishUnit> fin;
         std::vector<int> fin_blocks;
         std::vector<FillUnit> fills;
@@ -110,7 +113,7 @@ int build_plan(BatchPlan& P, int first, int last, void* stream) {
             const Launch& l = E.launches[r];
             const Handle& h = *P.hs[k];
             if (l.kind == L_PASS && l.units()) {
-                sweeps_of[l.unit_kind].push_back({&E, &l});
+                sweeps_of[2 * l.unit_kind + unit_three_blocks(l.unit_kind, l.smem)].push_back({&E, &l});
             } else if (l.kind == L_FINISH) {
                 FinishUnit u{};
                 u.partials = E.partials;
@@ -147,6 +150,7 @@ int build_plan(BatchPlan& P, int first, int last, void* stream) {
         }
         for (auto& sweeps : sweeps_of) {
             if (sweeps.empty()) continue;
+            // longest blocks first (the short ones fill the last wave)
             auto tiles_per_block = [](const std::pair<const Engine*, const Launch*>& x) {
                 return x.first->units[x.second->unit_off].n_tiles / x.second->ctas;
             };
@@ -157,7 +161,7 @@ int build_plan(BatchPlan& P, int first, int last, void* stream) {
             std::vector<int> block_unit;
             Group g;
             g.kind = Group::SWEEP;
-            g.unit_kind = (int)(&sweeps - sweeps_of);
+            g.unit_kind = (int)(&sweeps - sweeps_of) / 2;
             for (const auto& x : sweeps) {
                 const Launch& l = *x.second;
                 for (int k = 0; k < l.n_units; ++k) {

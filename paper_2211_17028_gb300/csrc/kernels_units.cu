@@ -700,9 +700,11 @@ int attribute(cudaDeviceAttr a) {
     return v;
 }
 
+}  // namespace
+
 // whether three blocks of such a program fit an SM (1 KB per block is the
 // system's; pairs in 80 registers would spill 900 bytes)
-bool three_fit(int kind, size_t smem) {
+bool unit_three_blocks(int kind, size_t smem) {
     if (kind == unit_kind(true, UM_PAIRS) || kind == unit_kind(false, UM_PAIRS)) return false;
     static const size_t fixed = [] {
         cudaFuncAttributes a{};
@@ -711,10 +713,8 @@ bool three_fit(int kind, size_t smem) {
     return 3 * (smem_of(3, smem) + fixed + 1024) <= (size_t)attribute(cudaDevAttrMaxSharedMemoryPerMultiprocessor);
 }
 
-}  // namespace
-
 int unit_blocks_per_sm(int kind, size_t smem) {
-    if (three_fit(kind, smem)) return 3;
+    if (unit_three_blocks(kind, smem)) return 3;
     int nb = 0;
     const UnitKernel k = unit_kernel(kind, 2);
     allow_dynamic_smem((const void*)k);
@@ -724,7 +724,7 @@ int unit_blocks_per_sm(int kind, size_t smem) {
 
 cudaError_t launch_units(int kind, const SweepUnit* units, const int* blk, int ctas, int total_ctas, size_t smem,
                          cudaStream_t st) {
-    const int blocks = total_ctas > 2 * attribute(cudaDevAttrMultiProcessorCount) && three_fit(kind, smem) ? 3 : 2;
+    const int blocks = total_ctas > 2 * attribute(cudaDevAttrMultiProcessorCount) && unit_three_blocks(kind, smem) ? 3 : 2;
     const UnitKernel kernel = unit_kernel(kind, blocks);
     smem = smem_of(blocks, smem);
     const cudaError_t e = allow_dynamic_smem((const void*)kernel);

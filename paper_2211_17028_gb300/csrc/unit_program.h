@@ -117,6 +117,8 @@ inline int unit_kind(bool single, UnitMode mode) { return 2 * (int)single + (int
 constexpr int kUnitKinds = 4;
 size_t unit_smem_bytes(int max_words, int max_events);
 int unit_blocks_per_sm(int kind, size_t smem);
+// whether a launch of such programs can use the form with three blocks per SM
+bool unit_three_blocks(int kind, size_t smem);
 // blk: unit of every block, or null when every unit has `ctas` blocks
 // kind: unit_kind of the units' programs
 cudaError_t launch_units(int kind, const SweepUnit* units, const int* blk, int ctas, int total_ctas, size_t smem,
