@@ -915,6 +915,7 @@ void engine_release(Engine& E, void* stream) {
     E.buf = E.aux = nullptr;
     E.buf_bytes = E.aux_bytes = 0;
     E.level = -1;
+    E.has_result = false;   // the term values went with it
     E.launches.clear();
     E.units.clear();
     E.jit.clear();

@@ -396,6 +396,7 @@ void release(GEngine& G, void* stream) {
     G.buf_bytes = G.aux_bytes = 0;
     G.one_sibling = false;
     G.small_level = -1;
+    G.has_result = false;   // the term values went with it
 }
 
 double dropped_bound(const std::vector<GFactors>& fac, int level) {

@@ -49,6 +49,10 @@ def test_waves_give_the_plain_results():
                 got = outs[k].to_dict()
                 assert got["F"] == plain[k]["F"] and got["T"] == plain[k]["T"], (call, k)
         assert len(refused) >= 2
+        # a wave's buffers are given back for the next one, the term values with them
+        with pytest.raises(nqs.NqsError) as e:
+            circs[0].term_values()
+        assert e.value.code == nqs.NQS_ERR_ORDER
         for c in circs:
             c.close()
     finally:
