@@ -428,6 +428,7 @@ struct Builder {
     std::vector<Launch> L;
     std::vector<SweepUnit> units;     // pointers into prog / partials / tables patched after layout
     std::vector<size_t> unit_prog, unit_part;
+    std::vector<int> unit_base;       // first site of its checkpoint table
     std::vector<char> unit_bd;
     std::map<std::array<int, 3>, UnitProgram> programs;   // by (first device op, count, swept alone)
     size_t partial_top = 0, partial_doubles = 0;
@@ -598,6 +599,7 @@ struct Builder {
                 u.n = plan.n;
                 units.push_back(u);
                 unit_prog.push_back((size_t)pi.word);
+                unit_base.push_back(pi.site_base);
                 unit_part.push_back((size_t)pi.n_events);   // events until the launch is closed
                 unit_bd.push_back(bd_table);
                 if (rank) reqs.push_back({units.size() - 1, &rp, start, s, rank});
@@ -1542,7 +1544,7 @@ int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* 
     for (size_t u = 0; u < B.units.size(); ++u) {
         SweepUnit& x = B.units[u];
         x.prog = prog_dev + B.unit_prog[u];
-        x.ckpt = ckpt_dev + (B.unit_bd[u] ? N : 0);
+        x.ckpt = ckpt_dev + (B.unit_bd[u] ? N : 0) + B.unit_base[u];
         x.ckpt_fwd = nullptr;
         x.partials = E.partials + B.unit_part[u];
         x.err = E.err_dev;

@@ -472,11 +472,11 @@ __global__ void __launch_bounds__(kNT, BLOCKS) unit_sweep_kernel(const SweepUnit
     }
     if (tid < (int)ghd->n_slots) {
         const unsigned s = ghd->slot_site[tid];
-        slot[tid] = (s & kSlotFwd) ? u.ckpt_fwd[s & ~kSlotFwd] : u.ckpt[s];
+        slot[tid] = (s & 0x8000) ? u.ckpt_fwd[s & 0x7fff] : u.ckpt[s];
     }
     __syncthreads();
     const UnitHeader& hd = *reinterpret_cast<const UnitHeader*>(prog);
-    const UnitPhase* const phases = reinterpret_cast<const UnitPhase*>(prog + kHeaderWords);
+    const UnitPhase* const phases = reinterpret_cast<const UnitPhase*>(prog + 4);
     const UnitRec* const ops = reinterpret_cast<const UnitRec*>(prog + hd.ops_word);
     const float2* const mats = reinterpret_cast<const float2*>(prog + hd.mats_word);
     const int n_phases = (int)hd.n_phases, n_tiles = u.n_tiles, nctas = u.ctas;

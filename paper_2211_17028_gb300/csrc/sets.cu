@@ -100,6 +100,7 @@ enum CkptTable : char { CT_PHI, CT_BOUNDARY, CT_LANE };   // what a unit's reduc
 struct Step {
     int kind = 0, n_phases = 0, n_events = 0, lane = 0;
     size_t smem = 0, word = 0;
+    int site_base = 0;
     CkptTable table = CT_PHI;
     std::vector<SweepUnit> units;
     struct Slot {
@@ -116,6 +117,7 @@ struct Prog {
     std::vector<SweepUnit> units;
     std::vector<size_t> unit_prog, unit_part;
     std::vector<char> unit_table, unit_lane;
+    std::vector<int> unit_base;
     std::vector<std::vector<Step>> lanes = std::vector<std::vector<Step>>(1);   // passes not launched yet
     int lane = 0;                     // where passes are added
     std::vector<FinishSlot> slots;
@@ -175,6 +177,7 @@ struct Prog {
                         units.back().cta_begin = cta;
                         cta += l.ctas;
                         unit_prog.push_back(s->word);
+                        unit_base.push_back(s->site_base);
                         unit_part.push_back(at + u * state);
                         unit_table.push_back(s->table);
                         unit_lane.push_back((char)s->lane);
@@ -262,6 +265,7 @@ PassRef add_launch(Prog& G, const Plan& plan, const SetsState& S, const PassSpec
         st.kind = unit_kind(nstates == 1, pi.mode);
         st.smem = unit_smem_bytes(pi.words, pi.n_events);
         st.word = (size_t)pi.word;
+        st.site_base = pi.site_base;
         st.table = table;
         st.lane = G.lane;
         for (int s = 0; s < nstates; ++s) {
@@ -446,7 +450,8 @@ int upload_and_run(Handle& h, SetsState& S, Prog& G, size_t extra_bytes, void** 
         x.ckpt = G.unit_table[u] == CT_LANE       ? S.lane_tab + 3 * G.unit_lane[u]
                  : G.unit_table[u] == CT_BOUNDARY ? S.phi_bd_tab
                                                   : S.phi_tab;
-        x.ckpt_fwd = S.chi_tab;
+        x.ckpt += G.unit_base[u];
+        x.ckpt_fwd = S.chi_tab + G.unit_base[u];
         x.partials = E.partials + G.unit_part[u];
         x.err = S.err;
     }

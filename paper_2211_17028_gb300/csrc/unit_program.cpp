@@ -2,6 +2,7 @@
 #include "unit_program.h"
 
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <complex>
 #include <cstring>
@@ -458,9 +459,11 @@ namespace {
 template <typename Asm>
 UnitProgram assemble(const std::vector<DevOp>& dops, int off, int n, const int* local, int n_qubits,
                           const std::vector<float2>& tab, std::vector<uint4>& out) {
-    static_assert(sizeof(UnitRec) == 16 && sizeof(UnitPhase) == 96 && sizeof(UnitHeader) == 80, "record sizes");
+    static_assert(sizeof(UnitRec) == 16 && sizeof(UnitPhase) == 96 && sizeof(UnitHeader) == 64, "record sizes");
     constexpr int K = kMaxTileQ;
     UnitHeader hd{};
+    int slot_site[kUnitSlots] = {};
+    bool slot_used[kUnitSlots] = {}, slot_fwd[kUnitSlots] = {};
     bool in_tile[64] = {};
     for (int j = 0; j < K; ++j) {
         hd.local[j] = (unsigned char)local[j];
@@ -566,12 +569,15 @@ UnitProgram assemble(const std::vector<DevOp>& dops, int off, int n, const int* 
                     r.flags = (unsigned char)(fl & ~(FL_APPLY | FL_KDIAG));
                     if (fl & FL_REDUCE) {
                         r.ev = (unsigned char)((d.flags >> 8) & 0xff);
-                        hd.slot_site[r.ev] = (unsigned)d.site;
+                        slot_site[r.ev] = d.site;
+                        slot_used[r.ev] = true;
                         hd.n_events = std::max(hd.n_events, (unsigned)r.ev + 1);
                         hd.n_slots = std::max<unsigned char>(hd.n_slots, r.ev + 1);
                     } else if (fl & (FL_SAVE | FL_SAVE_FWD)) {
                         r.ev = hd.n_slots++;
-                        hd.slot_site[r.ev] = (unsigned)d.site | ((fl & FL_SAVE_FWD) ? kSlotFwd : 0u);
+                        slot_site[r.ev] = d.site;
+                        slot_used[r.ev] = true;
+                        slot_fwd[r.ev] = (fl & FL_SAVE_FWD) != 0;
                     }
                     if (fl & FL_SPAWN) r.sp = (unsigned char)(d.flags >> 24);
                 } else {
@@ -596,9 +602,22 @@ UnitProgram assemble(const std::vector<DevOp>& dops, int off, int n, const int* 
     info.word = (int)out.size();
     hd.n_phases = (unsigned)phases.size();
     hd.n_ops = (unsigned)A.recs.size();
-    hd.ops_word = kHeaderWords + 6 * hd.n_phases;
+    hd.ops_word = 4 + 6 * hd.n_phases;
     hd.mats_word = hd.ops_word + hd.n_ops;
     hd.words = hd.mats_word + (unsigned)((A.mats.size() + 1) / 2);
+    // The sites of a pass are neighbours, however many the circuit has: slots keep
+    // 15 bits, counted from the lowest one.  (The same with 32 bits a slot, in the
+    // header or behind the matrices, made the sweeps 0.1 to 0.9 % slower.)
+    int low = INT_MAX, high = 0;
+    for (int k = 0; k < kUnitSlots; ++k)
+        if (slot_used[k]) {
+            low = std::min(low, slot_site[k]);
+            high = std::max(high, slot_site[k]);
+        }
+    if (low <= high) info.site_base = low;
+    for (int k = 0; k < kUnitSlots; ++k)
+        if (slot_used[k]) hd.slot_site[k] = (unsigned short)((slot_site[k] - info.site_base) | (slot_fwd[k] ? 0x8000 : 0));
+    if (high - info.site_base > 0x7fff) hd.words = 1u << 24;   // no planner makes one; no launch takes it
     words(&hd, sizeof(hd));
     words(phases.data(), phases.size() * sizeof(UnitPhase));
     words(A.recs.data(), A.recs.size() * sizeof(UnitRec));

@@ -77,20 +77,19 @@ struct UnitPhase {             // 96 bytes
     unsigned short pad[2];
 };
 
-struct UnitHeader {            // 80 bytes
+struct UnitHeader {            // 64 bytes
     unsigned int n_phases, n_ops, ops_word, mats_word;
     unsigned long long nl_mask;             // qubits outside the tile
     unsigned int n_events, words;
     unsigned char local[12];                // tile qubits, ascending
     unsigned char n_slots, pad[3];
-    unsigned int slot_site[kUnitSlots];     // site of each checkpoint slot (kSlotFwd: in the forward table)
+    unsigned short slot_site[kUnitSlots];   // site of each checkpoint slot from site_base on (bit 15: forward table)
 };
-constexpr unsigned int kSlotFwd = 1u << 31;
-constexpr int kHeaderWords = sizeof(UnitHeader) / 16;
 
 struct UnitProgram {
     UnitMode mode = UM_RATIOS;
     int word = 0, words = 0, n_phases = 0, n_events = 0;
+    int site_base = 0;           // the units' checkpoint tables start at this site
 };
 
 // Assemble dops[off .. off + n) (execution order) on the tile qubits `local`
@@ -105,7 +104,7 @@ struct SweepUnit {
     float2* out;               // null: the swept state is not kept
     float2* spawn;             // spawned state (slot k, factor i) at spawn + ((3 k + i) << n)
     const uint4* prog;
-    float2* const* ckpt;       // phi_s
+    float2* const* ckpt;       // phi_s, s from the program's site_base on
     float2* const* ckpt_fwd;   // chi_s
     double* partials;          // [event][cta][8]
     int* err;

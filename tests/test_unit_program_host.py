@@ -50,11 +50,12 @@ def run_host(tmp_path, body):
 
 
 def test_checkpoint_slots_hold_any_site(tmp_path):
-    """A slot names its site and its table (phi or chi) whatever the number of
-    sites of the circuit; the other records with a site index do as well."""
+    """A slot names its site, counted from the program's first one, and its table
+    (phi or chi) whatever the number of sites of the circuit; the other records
+    with a site index do as well."""
     out = run_host(tmp_path, r'''
 int main() {
-    const int sites[4] = {5, 32768, 40000, 70000};
+    for (int from : {0, 32766, 70000})
     for (int fwd = 0; fwd < 3; ++fwd) {   // reductions and saves of phi, saves of chi
         std::vector<float2> table = {{1, 0}, {0, 0}, {0, 0}, {1, 0}};
         std::vector<DevOp> ops;
@@ -63,15 +64,14 @@ int main() {
             d.type = OP_SITE;
             d.a = d.qa = k;
             d.b = d.qb = -1;
-            d.site = sites[k];
+            d.site = from + k;
             d.flags = FL_APPLY | (fwd == 0 ? FL_REDUCE | (k << 8) : fwd == 1 ? FL_SAVE : FL_SAVE_FWD);
             ops.push_back(d);
         }
         Program p(true, ops, table, 12);
-        for (int k = 0; k < 4; ++k) {   // as the kernel reads it: the top bit selects the table
-            const auto s = p.hd.slot_site[k];
-            const auto top = (decltype(s))(1ull << (8 * sizeof(s) - 1));
-            printf("%lld %d\n", (long long)(s & (decltype(s))~top), (s & top) != 0);
+        for (int k = 0; k < 4; ++k) {   // as the kernel reads it from tables that start at site_base
+            const unsigned s = p.hd.slot_site[k];
+            printf("%d %d\n", p.info.site_base + (int)(s & 0x7fff), (s & 0x8000) != 0);
         }
     }
     OpRec r{};
@@ -82,9 +82,8 @@ int main() {
 }
 ''')
     got = [(int(a), int(b)) for a, b in zip(out[::2], out[1::2])]
-    sites = [5, 32768, 40000, 70000]
-    assert got[:12] == [(s, int(t == 2)) for t in range(3) for s in sites]
-    assert got[12] == (70000, 70000)
+    assert got[:36] == [(s + k, int(t == 2)) for s in (0, 32766, 70000) for t in range(3) for k in range(4)]
+    assert got[36] == (70000, 70000)
 
 
 def test_repeated_phases_keep_the_norm(tmp_path):
