@@ -97,7 +97,7 @@ int build_plan(BatchPlan& P, int first, int last, void* stream) {
     size_t rounds = 0;
     for (int k = first; k < last; ++k) rounds = std::max(rounds, P.engines[k]->launches.size());
     for (size_t r = 0; r < rounds; ++r) {
-        // the round's sweep passes by kernel, and apart those whose programs leave room
+        // The round's sweep passes by kernel, and apart those whose programs leave room
         // for three blocks per SM: a launch reserves the shared memory of its longest
         // program for every block, and one circuit's long pass would leave all others
         // two blocks (512 circuits of 12 to 24 qubits: 5.28 s in one launch per kernel,
@@ -147,6 +147,15 @@ int build_plan(BatchPlan& P, int first, int last, void* stream) {
                 g.li = (int)r;
                 P.seq.push_back(g);
             }
+        }
+        for (int k = 0; k < kUnitKinds; ++k) {
+            auto &two = sweeps_of[2 * k], &three = sweeps_of[2 * k + 1];
+            long long blocks = 0;
+            for (const auto* form : {&two, &three})
+                for (const auto& x : *form) blocks += x.second->grid;
+            if (two.empty() || blocks >= 24ll * P.engines[first]->sm_count) continue;
+            two.insert(two.end(), three.begin(), three.end());
+            three.clear();
         }
         for (auto& sweeps : sweeps_of) {
             if (sweeps.empty()) continue;
