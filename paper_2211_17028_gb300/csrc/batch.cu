@@ -101,7 +101,9 @@ int build_plan(BatchPlan& P, int first, int last, void* stream) {
         // for three blocks per SM: a launch reserves the shared memory of its longest
         // program for every block, and one circuit's long pass would leave all others
         // two blocks (512 circuits of 12 to 24 qubits: 5.28 s in one launch per kernel,
-        // 4.74 s so; 5.27 s one circuit after another)
+        // 4.74 s so; 5.25 s one circuit after another).  Together where two launches
+        // would fill the chip less often than eight times (eight circuits of 12 to 16
+        // qubits: 1.75 ms, apart 2.28).
         std::vector<std::pair<const Engine*, const Launch*>> sweeps_of[2 * kUnitKinds];
         std::vector<FinishUnit> fin;
         std::vector<int> fin_blocks;
@@ -315,14 +317,16 @@ int engine_batch_fidelity(Handle** hs, size_t count, const nqs_state* psis, cons
     for (std::pair<int, int> w(0, 0); w.second < (int)count && rc == NQS_OK;) {
         w.first = w.second;
         void* reserve = nullptr;
+        bool asked = !reserving;   // for it, before the wave's first new buffers
         for (int k = w.first; k < (int)count && rc == NQS_OK; ++k) {
             Handle& h = *hs[k];
             const int level = std::min(levels[k], (int)h.factors.size());
             if (!h.eng) h.eng = new Engine();
             rc = engine_init(*h.eng);
             if (rc == NQS_OK && !schedule_current(*h.eng, &psis[k], &vs[k], level)) {
-                if (reserving && !reserve) reserve = dev_alloc(reserve_bytes, stream);
-                rc = build_schedule(h, *h.eng, &psis[k], &vs[k], level, stream, false, k == w.first);
+                if (!asked) reserve = dev_alloc(reserve_bytes, stream);
+                asked = true;
+                rc = build_schedule(h, *h.eng, &psis[k], &vs[k], level, stream, false, k == w.first, reserving);
                 if (rc == NQS_ERR_NOMEM && k > w.first) {   // the next wave begins with it
                     rc = NQS_OK;
                     break;

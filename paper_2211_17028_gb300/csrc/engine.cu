@@ -343,12 +343,13 @@ Run make_run(const Plan& plan, const std::vector<PassSpec>& segs, RunType rt, bo
 // 20 qubits, level 2 (6.17 -> 6.57 ms).
 constexpr size_t kGroupBytes = (size_t)256 << 20;
 // The passes of a sweep that spawns may hold several sites (fewer passes) when
-// the children of a whole pass fit in this much.  A handle keeps these states as
-// long as its checkpoints, and a study keeps hundreds of handles: with 2 GiB here
-// 512 circuits of 12 to 24 qubits held 275 GiB, all of the device (235 with the
-// three states of one site each; 255 so).  Wider states are many tiles each, and
-// their spawning sweep is one of many: 2 to 5 % at 23 and 24 qubits.
+// the children of a whole pass fit in this much, or in the larger one while half of
+// the device stays free.  A handle keeps these states as long as its checkpoints,
+// and a study keeps hundreds of handles: with 2 GiB in any case 512 circuits of 12
+// to 24 qubits held 275 GiB, all of the device (235 with the three states of one
+// site each).  One site a pass costs 4 to 6 % at 23 and 24 qubits, level 2.
 constexpr size_t kSpawnBytes = (size_t)512 << 20;
+constexpr size_t kSpawnBytesFree = (size_t)2 << 30;
 // per-block partial sums held before a finisher launch is put in (8 MiB)
 constexpr size_t kPartialDoubles = (size_t)1 << 20;
 
@@ -356,6 +357,7 @@ constexpr size_t kPartialDoubles = (size_t)1 << 20;
 struct GroupPlan {
     bool grouped = false;              // spawning sweeps use passes of several sites
     int sites = 1;                     // most spawning sites of such a pass
+    size_t pass_bytes = 0;             // children of a whole pass
     std::vector<size_t> cap;           // states of depth d
     size_t chunk = 1;                  // groups of one depth that may spawn together
     size_t total() const {
@@ -366,7 +368,7 @@ struct GroupPlan {
 };
 
 static GroupPlan group_plan(const Plan& plan, const std::vector<Factors>& fac, int level, bool generated,
-                            bool small) {
+                            bool small, size_t spawn_bytes) {
     GroupPlan g;
     g.cap.assign(std::max(1, level), 0);
     if (level < 2) return g;
@@ -380,7 +382,8 @@ static GroupPlan group_plan(const Plan& plan, const std::vector<Factors>& fac, i
     }
     const size_t pass_states = 3 * (size_t)g.sites + 9 * (size_t)g.sites * (level - 2);
     // generated kernels spawn at one site per pass and sweep one group per launch
-    g.grouped = !generated && !small && pass_states * sb <= kSpawnBytes;
+    g.pass_bytes = pass_states * sb;
+    g.grouped = !generated && !small && g.pass_bytes <= spawn_bytes;
     if (!g.grouped) g.sites = 1;
     const size_t room = (generated || small) ? 0 : kGroupBytes / sb;
     // C(N, d) 3^d states of depth d exist in all
@@ -396,7 +399,7 @@ static GroupPlan group_plan(const Plan& plan, const std::vector<Factors>& fac, i
 }
 
 size_t group_states(const Handle& h, int level, bool generated) {
-    return group_plan(h.plan, h.factors, std::min(level, (int)h.factors.size()), generated, false).total();
+    return group_plan(h.plan, h.factors, std::min(level, (int)h.factors.size()), generated, false, kSpawnBytesFree).total();
 }
 
 namespace {
@@ -1171,7 +1174,7 @@ bool schedule_current(const Engine& E, const nqs_state* psi, const nqs_state* v,
 
 // Build (or reuse) the schedule for this level and state kinds.
 int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* v, int level, void* stream,
-                   bool allow_jit, bool make_do) {
+                   bool allow_jit, bool make_do, bool close) {
     const int N = (int)h.factors.size();
     // automatic: circuits of 26 qubits or more, where one call's sweeps outlast
     // the compilation of its distinct passes
@@ -1229,8 +1232,16 @@ int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* 
     if (spacing == 0) {
         // groups swept together when the memory allows, else one at a time
         const int first = B.kind != P_UNIT;
+        size_t spawn_bytes = kSpawnBytes;
+        const GroupPlan wide = group_plan(plan, h.factors, level, first, false, kSpawnBytesFree);
+        if (!close && wide.grouped && wide.pass_bytes > kSpawnBytes) {
+            size_t free_b = 0, total_b = 0;
+            if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess &&
+                free_b >= total_b / 2 + ((size_t)n_phi + 1 + wide.total()) * sbytes)
+                spawn_bytes = kSpawnBytesFree;
+        }
         for (int small = first; small <= (make_do ? 1 : first) && !E.buf; ++small) {
-            B.gp = group_plan(plan, h.factors, level, B.kind != P_UNIT, small != 0);
+            B.gp = group_plan(plan, h.factors, level, first, small != 0, spawn_bytes);
             n_states = (size_t)n_phi + 1 + B.gp.total();
             E.buf_bytes = n_states * sbytes;
             E.buf = dev_alloc(E.buf_bytes, stream);
@@ -1496,7 +1507,7 @@ int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* 
                 const bool wide = E.wide;
                 (wide ? E.wide_failed : E.jit_failed) = true;
                 engine_release(E, stream);
-                const int rc = build_schedule(h, E, psi, v, level, stream, allow_jit, make_do);
+                const int rc = build_schedule(h, E, psi, v, level, stream, allow_jit, make_do, close);
                 if (!wide) E.jit_failed = false;   // the next schedule tries again
                 return rc;
             }

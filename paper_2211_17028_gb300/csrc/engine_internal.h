@@ -156,14 +156,14 @@ void engine_release(Engine& E, void* stream);
 // allow_jit: the schedule may use pass-specialised kernels (the batch executor
 // launches passes through its own multi-circuit kernel and passes false);
 // make_do: where the states do not fit, a schedule with fewer of them, else
-// NQS_ERR_NOMEM
+// NQS_ERR_NOMEM; close: one of many, which together fill the device
 int build_schedule(Handle& h, Engine& E, const nqs_state* psi, const nqs_state* v, int level, void* stream,
-                   bool allow_jit = true, bool make_do = true);
+                   bool allow_jit = true, bool make_do = true, bool close = false);
 int run_schedule(Handle& h, Engine& E, cudaStream_t st);
 int run_launch(Handle& h, Engine& E, const Launch& l, cudaStream_t st);
 // whether E's schedule is the one for these states and this level
 bool schedule_current(const Engine& E, const nqs_state* psi, const nqs_state* v, int level);
-// branch-group states a schedule holds beside its checkpoints and main state
+// most branch-group states a schedule holds beside its checkpoints and main state
 size_t group_states(const Handle& h, int level, bool generated);
 
 }  // namespace nqs

@@ -1,6 +1,6 @@
 """What a handle holds beside its checkpoints: hundreds of handles of a study
 live side by side, so branch groups are held together only as far as that
-fills the chip."""
+fills the chip, and wide ones only while the device is free."""
 
 import pytest
 
@@ -9,14 +9,16 @@ import workloads as W
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n,level,most", [(20, 2, 36), (23, 2, 3), (20, 3, 96)])
-def test_states_held_for_branch_groups(n, level, most):
-    """Wide states: the three of one site at a time, as they are many tiles
-    each.  Narrower ones: at most 256 MiB per depth, or the children of one pass."""
+@pytest.mark.parametrize("n,level,full,most", [(20, 2, False, 36), (20, 3, False, 96), (23, 2, False, 12), (23, 2, True, 3)])
+def test_states_held_for_branch_groups(n, level, full, most):
+    """At most 256 MiB per depth or the children of one pass; on a device that is
+    half full, three states of 64 MiB at a time."""
     import torch
     from paper_2211_17028_gb300 import nqs
     torch.cuda.set_device(0)
     nqs.use_torch_allocator()
+    torch.cuda.empty_cache()
+    other = torch.empty(torch.cuda.mem_get_info()[1] * 11 // 20 if full else 1, dtype=torch.uint8, device="cuda")
     w = W.random_circuit(900 + n, n, 60, 12, v_kind="ideal")
     circ = nqs.NoisyCircuit(W.to_ir_text(w))
     assert circ.fidelity(nqs.basis(w.psi["bits"]), nqs.ideal(), level)["status"] == 0
@@ -26,4 +28,5 @@ def test_states_held_for_branch_groups(n, level, most):
     # tables, programs, partial sums and term values
     assert info["workspace_bytes"] - info["n_states"] * (8 << n) <= 24 << 20
     circ.close()
+    del other
     torch.cuda.empty_cache()
