@@ -142,7 +142,8 @@ int nqs_fidelity(nqs_handle h, const nqs_state* psi, const nqs_state* v, int lev
  * Circuits are packed into waves whose buffers fit in free device memory;
  * a batch that fits in one wave is captured as a CUDA graph and replayed by
  * later calls with the same handles, states and levels (the handles keep
- * their workspaces).  Errors as nqs_fidelity, checked for every entry before
+ * their workspaces).  With several waves each one's workspaces are given back
+ * before the next, term values included (nqs_term_values: NQS_ERR_ORDER).  Errors as nqs_fidelity, checked for every entry before
  * anything runs; NQS_ERR_ARG also for a handle listed twice. */
 int nqs_batch_fidelity(const nqs_handle* hs, size_t count, const nqs_state* psis,
                        const nqs_state* vs, const int* levels, nqs_result* outs, void* stream);
@@ -178,7 +179,8 @@ int nqs_general_factors(nqs_handle h, uint32_t site, int32_t* m, int32_t* dim, i
                         double* KB);
 
 /* Term values X of the last nqs_fidelity on this handle, in canonical order,
- * copied to host memory `out` (synchronises the stream of that call). */
+ * copied to host memory `out` (synchronises the stream of that call).
+ * NQS_ERR_ORDER when there is none, or its buffers have been given back. */
 int nqs_term_values(nqs_handle h, double* out, size_t cap, size_t* count);
 
 /* Truncation bound of level l: sum over site sets S with |S| > l of
@@ -418,7 +420,8 @@ int nqs_reduced_matrix_noalloc(const void* phi, const void* chi, int n, int qubi
  * S (dominant factor elsewhere) -- the summand of T_k grouped by site set
  * (Sec. IV, Algorithm 1's inner loop over factor tuples).
  * nqs_prepare_sets runs the backward sweep from v and a forward sweep from
- * psi, keeping phi_s and chi_s for every site (2N + 14 device states); it must
+ * psi, keeping phi_s and chi_s for every site (2N + 14 device states, and up to
+ * 1 GiB of further work states where there is room); it must
  * precede nqs_eval_sets and be repeated after nqs_prepare_noise.
  * nqs_eval_sets: `sets` is m x k site indices (ascending within a set),
  * W_out receives m doubles on the host (the call synchronises `stream`).

@@ -4,10 +4,10 @@
 // rounds: round r executes the r-th launch of every circuit that has one.
 // Launches of one round belong to different circuits and never depend on one
 // another, so each launch kind of a round becomes a single multi-circuit
-// launch (sweep passes grouped by state count, finishers, fills, level sums)
+// launch (sweep passes grouped by kernel and form, finishers, fills, level sums)
 // with no grid-wide waiting.  Small circuits, whose single-circuit passes
 // would occupy a handful of SMs, then share the GPU.  Circuits are packed
-// into waves whose state buffers fit in the free device memory; when the
+// into waves whose buffers fit in the free device memory; when the
 // whole batch fits in one wave, its launch sequence is captured once as a
 // CUDA graph and replayed on later calls with the same inputs.
 #include <cuda_runtime.h>

@@ -1,32 +1,30 @@
 // Pass-specialised sweep kernels, generated from a launch's program and
 // compiled at run time with NVRTC for sm_103a.
 //
-// The register-resident sweep kernel (kernels_sweep.cu) interprets a
-// per-launch program: for every operation it loads a record, dispatches on
-// its type and register qubit, loads the matrix from shared memory and works
-// out layouts and addresses at run time.  Here the same program becomes
-// straight-line code: operations, register positions, tile layouts, global
-// offsets and matrix entries are compile-time constants, zero matrix entries
-// drop out, pending diagonal factors that are known when the code is
+// The unit sweep kernel (kernels_units.cu) interprets a program: for every
+// operation it loads a record, dispatches on its code, loads the matrix from
+// shared memory and works out addresses at run time.  Here the operations of a
+// pass become straight-line code: operations, register positions, tile layouts,
+// global offsets and matrix entries are compile-time constants, zero matrix
+// entries drop out, pending diagonal factors that are known when the code is
 // generated (one-qubit diagonals, diagonals between register qubits,
 // diagonal K_0) are multiplied together on the host, and only factors that
 // depend on the thread or the tile stay run-time values.  Amplitudes whose
 // addresses are adjacent (the site's qubit or a register qubit being qubit 0)
-// move as 16-byte vectors.  The semantics are those of the interpreted
-// kernel: same tile (12 qubits; 13 with 512-thread blocks as an option), same
-// TMA bulk prefetch with bounded mbarrier waits, same phases and XOR-swizzled
-// re-layouts, same site actions and the same per-block FP64 partials, so the
-// finishers and term sums are shared.  The organisation differs: each kernel
-// holds one state of 16 amplitudes per thread, and a pass over the three (or
-// nine) states of a branch group sweeps a tile's states one after another
-// (twice the resident warps of holding them together; the tile's phi values
-// come from DRAM once and from L2 for the later states, under L2 eviction
-// policies), consecutive re-layouts alternate between two buffers, and site
-// reductions accumulate with split real/imaginary partners.
+// move as 16-byte vectors.  The semantics are those of the unit kernel: tiles of
+// 12 qubits (13 with 512-thread blocks as an option), TMA bulk prefetch with
+// bounded mbarrier waits, phases of four register qubits, the same site actions
+// and per-block FP64 partials, so the finishers and term sums are shared.  The
+// organisation differs: a pass over the three (or nine) states of a branch group
+// is one launch whose blocks sweep a tile's states one after another, 16
+// amplitudes per thread (the tile's phi values come from DRAM once and from L2
+// for the later states, under L2 eviction policies), re-layouts are XOR-swizzled
+// and alternate between two buffers, and site reductions accumulate with split
+// real/imaginary partners.
 //
 // Kernels are cached by their source text for the life of the process;
 // the distinct kernels of a schedule are compiled in parallel.  When NVRTC
-// cannot be loaded the engine keeps the interpreted kernel (still on the GPU)
+// cannot be loaded the engine keeps the unit kernel (still on the GPU)
 // and reports it through nqs_info.jit_state == -1 (jit_launches == 0).
 #include <cuda_runtime.h>
 #include <dlfcn.h>

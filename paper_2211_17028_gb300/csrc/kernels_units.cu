@@ -7,9 +7,12 @@
 // TMA bulk copies (256-byte runs of the five low qubits) while the current one
 // is processed; every wait on the copies' mbarrier is bounded.
 //
-// What bounds it: issue slots wherever the launch fills the chip (a quarter of
-// the instructions are packed FP32; the rest decode, swap halves and form
-// addresses), the latency of one tile where it does not.  Hence
+// What bounds it: instructions wherever the launch fills the chip (24 qubits: an
+// instruction issued in 51 to 54 % of the cycles of a scheduler with 5.6 warps, three
+// in ten of them FMA-pipe instructions, the rest decoding, swapping halves and
+// forming addresses; the largest stalls are fixed latencies, phi loads, barriers
+// and instruction fetches; DRAM at 17 to 27 % of its peak), the latency of one
+// tile where it does not.  Hence
 // * one state per block and two or three blocks per SM, instead of the three
 //   states of a branch group in one block of 512 threads: three times as many
 //   blocks on a narrow circuit, and twice the amplitudes per decoded operation;

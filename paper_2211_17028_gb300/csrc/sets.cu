@@ -24,8 +24,8 @@
 // own states, and the r-th passes of all lanes are one launch: three states of
 // a 20-qubit circuit are 768 tiles (2.5 rounds of the resident blocks), of a
 // 14-qubit one twelve.  40 triples of a 20-qubit circuit with 200 noises:
-// 66.6 ms with nine states swept by three launches of three each, one chain
-// after another; @@ms.
+// 110 ms with nine states swept by three launches of three each, one chain
+// after another; 24.5 ms.
 //
 // When the 2N checkpoints do not fit in device memory (or the handle's
 // checkpoint-spacing option asks for it), chi is kept only at the first site

@@ -25,8 +25,10 @@ constexpr int kNoLoc = 31;                      // location of an absent bit (al
 //   UM_PAIRS   a scalar and a pair of factors per register bit, taken by gates
 //              and multiplied into the amplitudes in a fixed order.  States
 //              swept alone (backward and main sweeps, from which levels 0 and 1
-//              come) through circuits with phases use it: their results are
-//              those of every earlier kernel, bit for bit.
+//              come) through circuits with phases use it: the order of an
+//              amplitude's products, and so its rounding, is fixed by the order
+//              of the operations, whichever kernel sweeps it.  (Reductions add
+//              the amplitudes up in an order of their own.)
 //   UM_RATIOS  a scalar and one ratio per register bit: half the products.
 //              Branch groups use it, and every program whose diagonals are
 //              signs, which are exact either way.
